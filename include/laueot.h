@@ -205,7 +205,11 @@ int laue_create(laue_handle** h, int device);
 int laue_destroy(laue_handle* h);
 const char* laue_last_error(const laue_handle* h);
 
-/* Workspace bytes needed for problems bounded by *dims. */
+/* Workspace bytes for problems bounded by *dims.  The Sinkhorn passes list the
+ * pairs whose plan entry can be nonzero in what the workspace holds beyond
+ * the calls' own needs; the size includes room for those lists (at most 3 GB).
+ * A smaller workspace, down to the calls' own needs, is accepted: the passes
+ * then evaluate those pairs anew in every iteration, with the same results. */
 int laue_workspace_size(laue_handle* h, const LaueProblemDims* dims, size_t* bytes);
 
 /* Hands the library a device buffer of `bytes` bytes (256-byte aligned) to
@@ -353,9 +357,9 @@ int laue_cost_sinkhorn_noalloc(const LaueGeometry* geom, const LaueObsSpots* obs
 
 /* Autotuner of the pair passes (no counterpart in the paper): times each
  * launch shape of the row and column passes of laue_cost_sinkhorn on this
- * problem (shape v: {256, 128, 128 with a 128-register cap, 64 with a
- * 128-register cap} threads per CTA, one row/column pair per thread; the tile
- * size follows the CTA width), n_iter passes each after one warm-up
+ * problem (shape v: tiles of {256, 128, 128, 64} row/column pairs, whose
+ * partial sums the dustbins are merged from; shapes 1 and 2 are the same),
+ * n_iter passes each after one warm-up
  * iteration, and keeps the fastest row and column shapes in the handle for
  * later calls.  choice_host (optional, 2 ints): the chosen row and column
  * shapes; ms_host (optional, 2 x 4 floats): mean milliseconds per row and
@@ -372,18 +376,20 @@ int laue_autotune(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* 
  * sum, shifted by the angle block's largest potential, fell below 1e-30
  * (modulo 2^32); [2] pair evaluations (one cost and one exponential each) of
  * laue_single_fit; [3] pair evaluations of the row and column passes of
- * laue_cost_sinkhorn (after the exact skipping); [4] pairs the M-step pair
+ * laue_cost_sinkhorn (after the exact skipping; listed entries count with
+ * their padding); [4] pairs the M-step pair
  * passes of laue_mstep, laue_mstep_adjoint and laue_objective_grad visit
  * (after the exact skipping).  Synchronises `stream`. */
 int laue_read_counters(laue_handle* h, void* stream, long long* counts_host, int n);
 
 /* Exact underflow skipping in the Sinkhorn pair passes (no counterpart in the
  * paper; on by default): within each angle block the spots are ordered by
- * direction, each run of 32 pairs (a quarter of a staged chunk of 128)
- * carries a cone bounding its directions, and a pass skips a (tile, granule)
- * combination when the cones prove that every shifted exponent is below
- * -130, i.e. every plan entry flushes to exactly 0; the potentials are
- * bit-identical either way.  The M-step pair passes skip, by the same cone
+ * direction, each run of 32 pairs and of 8 pairs carries a cone bounding its
+ * directions, and the passes leave out the pairs for which the cones, or the
+ * cost itself, prove that the shifted exponent is below -126, i.e. the plan
+ * entry flushes to exactly 0; the potentials are bit-identical either way.
+ * Where the workspace has room (laue_workspace_size), the pairs that stay are
+ * listed once per E-step.  The M-step pair passes skip, by the same cone
  * bounds, the granules whose every plan entry is below 2^-40 (entries their
  * sums leave out), so their results are bit-identical too.  enable = 0 turns
  * the skipping off (the ordering stays).  Read the evaluated pairs with

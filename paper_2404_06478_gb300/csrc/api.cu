@@ -139,9 +139,12 @@ extern "C" int laue_create(laue_handle** h, int device) {
     int prev = 0;
     cudaGetDevice(&prev);
     cudaSetDevice(device);
-    if (sinkhorn_occupancy(H->row_occ, H->col_occ) != 0)
-        for (int v = 0; v < kSkVariants; ++v) H->row_occ[v] = H->col_occ[v] = 1;
+    const cudaError_t e = sinkhorn_setup();
     cudaSetDevice(prev);
+    if (e != cudaSuccess) {
+        free(H);
+        return LAUE_ERR_CUDA;
+    }
     H->row_variant = H->col_variant = kSkDefaultVariant;
     H->skip = 1;
     H->err[0] = 0;
@@ -160,7 +163,7 @@ extern "C" int laue_workspace_size(laue_handle* h, const LaueProblemDims* dims, 
     if (!h || !dims || !bytes) return laue_fail(h, LAUE_ERR_INVALID_ARG, "null argument");
     if (dims->T < 0 || dims->n_obs < 0 || dims->n_model < 0 || dims->n_grains < 0 || dims->n_planes < 0)
         return laue_fail(h, LAUE_ERR_INVALID_ARG, "negative dimension");
-    *bytes = make_layout(*dims, h->sm_count).total;
+    *bytes = make_layout(*dims, h->sm_count).total + list_bytes(*dims);
     return LAUE_OK;
 }
 
@@ -464,7 +467,7 @@ extern "C" int laue_refresh(laue_handle* h, const LaueGeometry* geom, const Laue
 // ------------------------------------------------------------- Sinkhorn
 
 int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* obs, const LaueModelSpots* model,
-                 const LaueOTParams* prm, const Layout& L, SkArgs* out, SkLaunch* lc) {
+                 const LaueOTParams* prm, const Layout& L, SkArgs* out, SkLaunch* lc, size_t list_from) {
     char* ws = (char*)h->ws;
     SkArgs a{};
     a.T = obs->T;
@@ -501,6 +504,15 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
         a.obs_ext = (float*)(a.mod_cone + L.max_mod_gran);
         a.mod_ext = a.obs_ext + L.max_obs_gran;
         a.skip = h->skip;
+        // the sort buffers, once the sort is done: compact potentials, sub-granule cones
+        char* b = ws + L.sortbuf;
+        a.obs_sub = (float4*)b;
+        a.mod_sub = a.obs_sub + (size_t)kSubs * L.max_obs_gran;
+        a.obs_subext = (float*)(a.mod_sub + (size_t)kSubs * L.max_mod_gran);
+        a.mod_subext = a.obs_subext + (size_t)kSubs * L.max_obs_gran;
+        a.Gc = (float*)(((uintptr_t)(a.mod_subext + (size_t)kSubs * L.max_mod_gran) + 15) / 16 * 16);
+        a.Fc = a.Gc + 2 * (size_t)L.max_mod_pairs;
+        a.pmax = (unsigned*)(a.Fc + 2 * (size_t)L.max_obs_pairs);
     }
     a.row_tiles = (int4*)(ws + L.row_tiles);
     a.col_tiles = (int4*)(ws + L.col_tiles);
@@ -525,6 +537,8 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
             if (k < G.n_det && Dk < dmin) dmin = Dk;
         }
         a.skipK = (float)(dmin * dmin * 1.4426950408889634 / eps);
+        a.uniK = 1;
+        for (int k = 0; k < G.n_det; ++k) a.uniK &= a.negK_det[k] == a.negKD2;
     }
     a.kc = (float)((double)prm->c_out * 1.4426950408889634 / eps);
     a.frac = prm->unmatched_frac;
@@ -533,16 +547,33 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
     a.tau_row = a.mode == 2 ? (float)((double)prm->kappa / ((double)prm->kappa + eps)) : 1.0f;
     a.tau_col = a.mode == 2 ? (float)((double)prm->lambda / ((double)prm->lambda + eps)) : 1.0f;
     a.warm = prm->warm_start ? 1 : 0;
-    *out = a;
     lc->row_variant = h->row_variant;
     lc->col_variant = h->col_variant;
-    int rt = std::max(1, std::min(h->sm_count * h->row_occ[h->row_variant], L.max_row_tiles));
-    int ct = std::max(1, std::min(h->sm_count * h->col_occ[h->col_variant], L.max_col_tiles));
-    lc->row_grid = rt;
-    lc->col_grid = ct;
-    // harvest passes: CTAs as wide as the tiles, about 768 threads per SM
-    lc->hrv_grid = std::max(1, std::min(h->sm_count * (768 / a.tile_rows), L.max_row_tiles));
-    lc->hcol_grid = std::max(1, std::min(h->sm_count * (768 / a.tile_cols), L.max_col_tiles));
+    // as many tiles to a CTA as it takes to have two CTAs per SM
+    auto ctas = [&](int tiles, int tile, int* per_cta) {
+        *per_cta = std::min(kPassThreads / tile, (tiles + 2 * h->sm_count - 1) / (2 * h->sm_count));
+        return std::max(1, (tiles + *per_cta - 1) / *per_cta);
+    };
+    lc->row_ctas = ctas(a.T + a.n_obs / 2 / a.tile_rows + 1, a.tile_rows, &lc->row_per_cta);
+    lc->col_ctas = ctas(a.T + a.n_model / 2 / a.tile_cols + 1, a.tile_cols, &lc->col_per_cta);
+    lc->row_slices = (int)list_slices(a.T, a.n_obs, a.tile_rows);
+    lc->col_slices = (int)list_slices(a.T, a.n_model, a.tile_cols);
+    // the M-step pair kernel runs one thread per column pair of the column
+    // pass's tiles (narrow tiles skip more), about 768 threads per SM
+    lc->col_grid = std::max(1, std::min(h->sm_count * (768 / a.tile_cols), L.max_col_tiles));
+    // pair lists in the workspace beyond the layout (skipping off: every pair is evaluated)
+    size_t from = align_up(std::max(L.total, list_from), 256);
+    size_t fixed = list_fixed_bytes(a.T, a.n_obs, a.n_model, a.tile_rows, a.tile_cols);
+    if (a.skip && a.skipK > 0.0f && from + fixed + kListChunkBytes <= h->ws_bytes) {
+        a.row_hdr = (int*)(ws + from);
+        a.col_hdr = a.row_hdr + lc->row_slices;
+        a.row_tab = a.col_hdr + lc->col_slices;
+        a.col_tab = a.row_tab + (size_t)kListChunks * lc->row_slices;
+        a.pool = ws + from + fixed;
+        size_t chunks = (h->ws_bytes - from - fixed) / kListChunkBytes;
+        a.pool_chunks = (int)std::min(chunks, kListPoolMax);
+    }
+    *out = a;
     return LAUE_OK;
 }
 
@@ -733,23 +764,25 @@ extern "C" int laue_autotune(laue_handle* h, const LaueGeometry* geom, const Lau
         h->col_variant = v;
         SkArgs a;
         SkLaunch lc;
-        laue_fill_sk(h, geom, obs, model, prm, L, &a, &lc);
+        laue_fill_sk(h, geom, obs, model, prm, L, &a, &lc, need);
         a.f = f_tmp;
         a.g = g_tmp;
         a.dust_out = d_tmp;
         a.warm = 0;
         if ((rc = laue_cuda_check(h, sinkhorn_prepare(a, s), "autotune prepare"))) break;
-        sinkhorn_iterate(a, lc, 1, s);
+        if ((rc = laue_cuda_check(h, sinkhorn_build_lists(a, lc, s), "autotune lists"))) break;
+        rc = laue_cuda_check(h, sinkhorn_iterate(a, lc, 1, s), "autotune passes");
+        if (rc) break;
         float ms = 0.0f;
         cudaEventRecord(e0, s);
-        for (int k = 0; k < n_iter; ++k) sinkhorn_row_pass(a, lc, s);
+        for (int k = 0; k < n_iter; ++k) sinkhorn_row_pass(a, lc, 1, s);
         cudaEventRecord(e1, s);
         cudaEventSynchronize(e1);
         cudaEventElapsedTime(&ms, e0, e1);
         if (ms_host) ms_host[2 * v] = ms / n_iter;
         if (ms < best_row) { best_row = ms; row_v = v; }
         cudaEventRecord(e0, s);
-        for (int k = 0; k < n_iter; ++k) sinkhorn_col_pass(a, lc, s);
+        for (int k = 0; k < n_iter; ++k) sinkhorn_col_pass(a, lc, 1, s);
         cudaEventRecord(e1, s);
         cudaEventSynchronize(e1);
         cudaEventElapsedTime(&ms, e0, e1);
@@ -797,9 +830,6 @@ static int mstep_entry(laue_handle* h, const LaueGeometry* geom, const LaueLatti
     SkLaunch lc;
     LaueOTParams op{0.4, prm->eps, 0.0f, 0, 0, 1, 0};
     laue_fill_sk(h, geom, obs, model, &op, L, &m.sk, &lc);
-    // the M-step pair kernel runs one thread per column pair of the column
-    // pass's tiles (narrow tiles skip more), about 768 threads per SM
-    lc.col_grid = std::max(1, std::min(h->sm_count * (768 / m.sk.tile_cols), L.max_col_tiles));
     m.sk.f = const_cast<float*>(f);
     m.sk.g = const_cast<float*>(g);
     m.sk.dust_out = nullptr;
@@ -875,9 +905,6 @@ extern "C" int laue_objective_grad(laue_handle* h, const LaueGeometry* geom, con
     SkLaunch lc;
     LaueOTParams op{0.4, eps, 0.0f, 0, 0, 1, 0};
     laue_fill_sk(h, geom, obs, model, &op, L, &m.sk, &lc);
-    // the M-step pair kernel runs one thread per column pair of the column
-    // pass's tiles (narrow tiles skip more), about 768 threads per SM
-    lc.col_grid = std::max(1, std::min(h->sm_count * (768 / m.sk.tile_cols), L.max_col_tiles));
     m.sk.f = const_cast<float*>(f);
     m.sk.g = const_cast<float*>(g);
     m.sk.dust_out = nullptr;

@@ -10,7 +10,6 @@
 struct laue_handle {
     int device;
     int sm_count;
-    int row_occ[laue::kSkVariants], col_occ[laue::kSkVariants];  // resident CTAs per SM of each launch shape
     int row_variant, col_variant;  // launch shapes in use (the autotuner's choice)
     int skip;                      // exact underflow skipping in the pair passes (default on)
     void* ws;
@@ -26,4 +25,5 @@ int laue_check_obs(laue_handle* h, const LaueObsSpots* o);
 int laue_check_model(laue_handle* h, const LaueModelSpots* m);
 int laue_need_ws(laue_handle* h, const LaueProblemDims& d, laue::Layout* L);
 int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* obs, const LaueModelSpots* model,
-                 const LaueOTParams* prm, const laue::Layout& L, laue::SkArgs* out, laue::SkLaunch* lc);
+                 const LaueOTParams* prm, const laue::Layout& L, laue::SkArgs* out, laue::SkLaunch* lc,
+                 size_t list_from = 0);

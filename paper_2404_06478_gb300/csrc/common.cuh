@@ -35,6 +35,9 @@ enum CtrlSlot {
     CTRL_SK_PAIRS = 20,   // 64-bit count (slots 20-21) of pair evaluations of the Sinkhorn passes
     CTRL_SP_DONE = 22,    // finished-CTA ticket of the sparse passes
     CTRL_MS_PAIRS = 24,   // 64-bit count (slots 24-25) of staged pairs the M-step pair kernel visits
+    CTRL_POOL_NEXT = 26,  // chunks handed out of the pair-list pool
+    CTRL_ROW_EVAL = 28,   // 64-bit pair evaluations of one row pass (slots 28-29) and
+    CTRL_COL_EVAL = 30,   // of one column pass (slots 30-31), counted when the lists are built
     CTRL_SLOTS = 64
 };
 
@@ -55,6 +58,16 @@ inline size_t sf_near_cap(int n_obs) {
     return (c + 3) / 4 * 4;  // keeps every CTA's slice 16-byte aligned
 }
 constexpr int kConeGran = 32;  // pairs per cone granule of the pair passes' exact skipping (kGran)
+constexpr int kSubGran = 8;    // pairs per sub-granule: the finer cones of the streamed side
+constexpr int kSubs = kConeGran / kSubGran;
+
+// Pair lists of the Sinkhorn passes (sinkhorn.cu).  A slice is the 32 spot
+// pairs of one warp; its listed entries sit in chunks of the pool, kListDepth
+// entries deep for each of its 64 spots: kListDepth x 64 costs (float), then
+// as many slots of the other side (16 bits).
+constexpr int kListDepth = 8;
+constexpr int kListChunks = 128;  // chunks a slice can hold (1024 entries per spot)
+constexpr size_t kListChunkBytes = (size_t)kListDepth * 64 * 6;
 constexpr size_t kCtrlBytes = 4096;  // status + counters + small scalars
 
 // ---------------------------------------------------------------------------
@@ -70,7 +83,8 @@ struct Layout {
     size_t modX, modY, modZ, modW;// pair-interleaved model spots
     size_t pairoff;               // int: I2_off[T+1], J2_off[T+1] (pair offsets), granule bases (2 x (T+1))
     size_t perm;                  // int: observed and model sort permutations (order -> caller, caller -> order)
-    size_t sortbuf;               // sort keys and indices (two buffers each)
+    size_t sortbuf;               // sort keys and indices (two buffers each); after the sort the compact
+                                  // potentials and the sub-granule cones
     size_t cone;                  // float4 + float per granule of 32 pairs, observed then model
     size_t fwd_blocks;            // int per forward block (count, then offset)
     size_t jsum;                  // float per model spot x 12 (M-step sums)
@@ -121,9 +135,14 @@ inline Layout make_layout(const LaueProblemDims& d, int sm_count) {
     L.pairoff = take(sizeof(int) * (size_t)(4 * T + 8));
     size_t nsp = (size_t)d.n_obs + d.n_model + 2;
     L.perm = take(sizeof(int) * 2 * nsp);
-    L.sortbuf = take(sizeof(int) * 4 * nsp);
     L.max_obs_gran = (int)((ip + kConeGran - 1) / kConeGran) + T + 1;  // cone granules of kConeGran pairs
     L.max_mod_gran = (int)((jp + kConeGran - 1) / kConeGran) + T + 1;
+    {
+        size_t sort_bytes = sizeof(int) * 4 * nsp;
+        size_t reuse = sizeof(float) * 2 * (ip + jp) + sizeof(unsigned) * 4 * T + 64 +
+                       (sizeof(float4) + sizeof(float)) * kSubs * (size_t)(L.max_obs_gran + L.max_mod_gran);
+        L.sortbuf = take(sort_bytes > reuse ? sort_bytes : reuse);
+    }
     L.cone = take((sizeof(float4) + sizeof(float)) * (size_t)(L.max_obs_gran + L.max_mod_gran) + 64);
     L.fwd_blocks = take(sizeof(int) * (size_t)(2 * L.max_fwd_blocks + 2));
     L.jsum = take(sizeof(float) * 12 * (size_t)(d.n_model + 1));
@@ -138,6 +157,31 @@ inline Layout make_layout(const LaueProblemDims& d, int sm_count) {
                                      : 0);
     L.total = off;
     return L;
+}
+
+// Pair lists: they take whatever the workspace holds beyond the layout (and
+// stay off where that is too little), so a workspace of the layout's size
+// still runs every call.  Slices of one side of a problem, for tiles of `tile`
+// pairs:
+inline size_t list_slices(int T, int n_spots, int tile) {
+    return (size_t)T * (tile / 32 + 1) + (size_t)n_spots / 64 + 2;
+}
+inline size_t list_fixed_bytes(int T, int n_obs, int n_model, int tile_rows, int tile_cols) {
+    size_t s = list_slices(T, n_obs, tile_rows) + list_slices(T, n_model, tile_cols);
+    return align_up(s * sizeof(int) * (1 + (size_t)kListChunks), 256);
+}
+// Bytes the lists can use: room for every same-angle pair of both sides with a
+// quarter more for padding, and at most kListPoolMax chunks (3 GB; 400 million
+// entries: the 1000-grain configuration's passes hold 81 million at 1 mm^2).
+constexpr size_t kListPoolMax = 1u << 20;
+inline size_t list_bytes(const LaueProblemDims& d) {
+    if (d.n_obs <= 0 || d.n_model <= 0) return 0;
+    int T = d.T > 0 ? d.T : 1;
+    double pairs = (double)d.n_obs * (double)d.n_model / T;
+    double slices = (double)list_slices(T, d.n_obs, 256) + (double)list_slices(T, d.n_model, 256);
+    double chunks = 2.5 * pairs / (kListDepth * 64) + 2.0 * slices;
+    size_t pool = chunks < (double)kListPoolMax ? (size_t)chunks + 1 : kListPoolMax;
+    return list_fixed_bytes(T, d.n_obs, d.n_model, 256, 256) + pool * kListChunkBytes;
 }
 
 // ---------------------------------------------------------------------------

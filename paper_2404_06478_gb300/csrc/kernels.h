@@ -88,7 +88,19 @@ struct SkArgs {
     float4 *obs_cone, *mod_cone;
     float *obs_ext, *mod_ext;
     int *obs_gbase, *mod_gbase;  // T+1 first granule of each block
-    int skip;              // skip (tile, chunk) pairs whose plan entries all underflow
+    int skip;              // skip pairs whose plan entries all underflow
+    // cones of the sub-granules (kSubGran pairs), kSubs per granule
+    float4 *obs_sub, *mod_sub;
+    float *obs_subext, *mod_subext;
+    // potentials of the passes by ordered slot: pair offset of the block x 2 + rank
+    float *Fc, *Gc;
+    unsigned* pmax;        // 4T: maxima per angle of the last passes (passes.cu)
+    // pair lists (pool_chunks = 0: none): chunks per slice (-1: the slice is not
+    // listed), chunk numbers of each slice, the pool
+    int *row_hdr, *col_hdr, *row_tab, *col_tab;
+    char* pool;
+    int pool_chunks;
+    int uniK;              // every detector has the same cost length: K_j = -negKD2
     int4* row_tiles;
     int4* col_tiles;
     int4* ang_tiles;       // per angle: {first row tile, #row tiles, first col tile, #col tiles}
@@ -175,10 +187,14 @@ void sparse_carve(SpArgs& a, char* base, int T, int n_obs, int n_model, int rho)
 cudaError_t sparse_sinkhorn_run(const SpArgs& a, int n_iter, bool rows, bool cols, cudaStream_t s);
 
 constexpr int kSkVariants = 4;       // launch shapes of the pair passes (see sinkhorn.cu)
+constexpr int kPassThreads = 512;     // CTA of the pair passes: at most kPassThreads / tile tiles
 constexpr int kSkDefaultVariant = 3;  // 64-pair tiles: the autotuner's usual pick
 
 struct SkLaunch {
-    int row_grid, col_grid, hrv_grid, hcol_grid;
+    int row_ctas, col_ctas;        // CTAs of the pair passes
+    int row_per_cta, col_per_cta;  // tiles of a CTA
+    int row_slices, col_slices;  // bound on the slices of each side
+    int col_grid;                // CTAs of the M-step's pair kernel
     int row_variant, col_variant;
 };
 
@@ -186,11 +202,14 @@ cudaError_t sinkhorn_run(const SkArgs& a, const SkLaunch& l, int n_iter, bool wa
                          cudaStream_t s);
 cudaError_t sinkhorn_prepare(const SkArgs& a, cudaStream_t s);
 cudaError_t sinkhorn_iterate(const SkArgs& a, const SkLaunch& l, int n_iter, cudaStream_t s);
-cudaError_t sinkhorn_finish(const SkArgs& a, const SkLaunch& l, bool want_rows, bool want_cols, cudaStream_t s);
-int sinkhorn_occupancy(int* row_blocks_per_sm, int* col_blocks_per_sm);  // kSkVariants entries each
+cudaError_t sinkhorn_finish(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols, cudaStream_t s);
+cudaError_t sinkhorn_harvest(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols,
+                             cudaStream_t s);
+cudaError_t sinkhorn_setup();
+cudaError_t sinkhorn_build_lists(const SkArgs& a, const SkLaunch& l, cudaStream_t s);
 int sk_variant_threads(int v);
-void sinkhorn_row_pass(const SkArgs& a, const SkLaunch& l, cudaStream_t s);
-void sinkhorn_col_pass(const SkArgs& a, const SkLaunch& l, cudaStream_t s);
+cudaError_t sinkhorn_row_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s);
+cudaError_t sinkhorn_col_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s);
 
 // ------------------------------------------------------------------ M-step
 struct MsArgs {

@@ -31,14 +31,13 @@ struct StaticDevice {
     int device;     // CUDA ordinal this entry describes
     void* scratch;  // device address of g_static_scratch on this device
     int sm_count;
-    int row_occ[kSkVariants], col_occ[kSkVariants];
 };
 
 StaticDevice g_devices[kMaxDevices];
 std::mutex g_setup_mutex;
 
 // One-time set-up for the current device: the device address of the static
-// scratch, the SM count and the occupancy of the pair passes.
+// scratch and the SM count.
 int static_device(StaticDevice** out) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return LAUE_ERR_CUDA;
@@ -49,8 +48,7 @@ int static_device(StaticDevice** out) {
         if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || p == nullptr) return LAUE_ERR_CUDA;
         int sm = 0;
         if (cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return LAUE_ERR_CUDA;
-        if (sinkhorn_occupancy(d.row_occ, d.col_occ) != 0)
-            for (int v = 0; v < kSkVariants; ++v) d.row_occ[v] = d.col_occ[v] = 1;
+        if (sinkhorn_setup() != cudaSuccess) return LAUE_ERR_CUDA;
         d.device = dev;
         d.scratch = p;
         d.sm_count = sm;
@@ -85,10 +83,6 @@ extern "C" int laue_cost_sinkhorn_noalloc(const LaueGeometry* geom, const LaueOb
     laue_handle h{};  // a view of the static scratch; nothing is allocated
     h.device = d->device;
     h.sm_count = d->sm_count;
-    for (int v = 0; v < kSkVariants; ++v) {
-        h.row_occ[v] = d->row_occ[v];
-        h.col_occ[v] = d->col_occ[v];
-    }
     h.row_variant = h.col_variant = kSkDefaultVariant;
     h.skip = 1;
     h.ws = d->scratch;

@@ -1,0 +1,1322 @@
+// passes.cu — the pair passes of the fused E-step (see sinkhorn.cu): the pair
+// lists, the row and column updates, and the plan read-out.
+//
+// A pass runs one warp per SLICE: 32 consecutive spot pairs of a tile, each
+// lane holding the two spots a and b of its pair.  A slice is either LISTED
+// (see sk_list_kernel: the pairs whose plan entry can be nonzero, with their
+// costs) or SWEPT: the warp walks the sub-granules of the block that its cone
+// can see, stages their spots in shared memory and evaluates every pair of
+// them.
+//
+// Both forms add the same nonzero terms in the same order (ascending slot of
+// the other side, even and odd slots in two accumulators), and every term
+// they leave out is exactly 0, so a potential has the same bits either way.
+//
+// CTAs are kPassThreads wide: the last one of a pass merges the tiles' partial
+// sums into the dustbin potentials, and needs the threads.  Where there are few
+// tiles a CTA takes fewer of them than it has warps for, so that they spread
+// over the SMs.
+#include <type_traits>
+
+#include "pairs.cuh"
+
+namespace laue {
+
+constexpr float kListLog2 = 127.0f;   // K e2 beyond which ex2.approx.ftz gives exactly 0 (potentials <= shift)
+constexpr float kTinySum = 1.0e-30f;  // below ~2^-100 the fast sum is recomputed exactly
+constexpr float kFarLog2 = 60.0f;     // see the read-out kernels
+
+// Walk over the sub-granules of a streamed block that a slice's cone can see,
+// in order; every call is warp-uniform.
+struct SubWalk {
+    const float4* sub;
+    const float* ext;
+    int nsub, s0;
+    unsigned mask;
+    __device__ __forceinline__ void init(const float4* sub_, const float* ext_, int n_pairs) {
+        sub = sub_;
+        ext = ext_;
+        nsub = (n_pairs + kSubGran - 1) / kSubGran;
+        s0 = -32;
+        mask = 0u;
+    }
+    // next sub-granule, -1 past the end
+    __device__ __forceinline__ int next(const Cone& own, bool own_obs, int skip, float K) {
+        while (!mask) {
+            s0 += 32;
+            if (s0 >= nsub) return -1;
+            const int s = s0 + (threadIdx.x & 31);
+            bool need = s < nsub;
+            if (need && skip) {
+                const Cone c = load_cone(sub, ext, s);
+                need = (own_obs ? min_scaled_cost(own, c, K) : min_scaled_cost(c, own, K)) <= kSkipLog2;
+            }
+            mask = __ballot_sync(0xffffffffu, need);
+        }
+        const int s = s0 + __ffs(mask) - 1;
+        mask &= mask - 1;
+        return s;
+    }
+};
+
+// Pairs of the sub-granules a slice can see.
+__device__ __forceinline__ int count_pairs(const Cone& own, bool own_obs, const float4* sub, const float* ext,
+                                           int n_pairs, int skip, float K) {
+    SubWalk w;
+    w.init(sub, ext, n_pairs);
+    int n = 0;
+    for (int s = w.next(own, own_obs, skip, K); s >= 0; s = w.next(own, own_obs, skip, K))
+        n += min(kSubGran, n_pairs - s * kSubGran);
+    return n;
+}
+
+// A warp's staging buffer: two batches of 32 streamed pairs (four
+// sub-granules) that cp.async fills while the other is evaluated.
+struct WarpStage {
+    float4 X[2][32];         // {-cx, -cy} or {px, py} of a pair
+    float4 Z[2][32], W[2][32];  // model pairs: {-rx, -ry}, {-rz, -K}
+    float2 Y[2][32], P[2][32];  // {-cz} or {pz}; the potentials
+};
+
+__device__ __forceinline__ void cp16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp8(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+// Streams the pairs of the sub-granules that the slice can see (skip = 0: of
+// the whole block) through the warp's buffer; per batch fn(stage, pairs,
+// first pair of each of its sub-granules).  The streamed block: n_pairs pairs
+// from pair b0 of the model spots (MODEL) or the observed spots; pot their
+// potentials (nullptr: not staged).
+template <bool MODEL, class Fn>
+__device__ __forceinline__ void sweep(const SkArgs& a, WarpStage& S, const Cone& own, const float4* sub, const float* ext,
+                                      int b0, int n_pairs, int skip, const float* pot, Fn fn) {
+    const int lane = threadIdx.x & 31;
+    SubWalk walk;
+    walk.init(sub, ext, n_pairs);
+    auto fetch = [&](int st, int4& first) {  // issues the copies of the next batch; its pairs
+        int n = 0;
+        int f[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int s = walk.next(own, MODEL, skip, a.skipK);
+            if (s < 0) break;
+            f[c] = s * kSubGran;
+            n = c * kSubGran + min(kSubGran, n_pairs - f[c]);
+        }
+        first = make_int4(f[0], f[1], f[2], f[3]);
+        if (lane < n) {
+            const int g = lane / kSubGran;
+            const int q = b0 + (g == 0 ? f[0] : g == 1 ? f[1] : g == 2 ? f[2] : f[3]) + lane % kSubGran;
+            cp16(&S.X[st][lane], (MODEL ? a.modX : a.obsX) + q);
+            cp8(&S.Y[st][lane], (MODEL ? a.modY : a.obsY) + q);
+            if (MODEL) {
+                cp16(&S.Z[st][lane], a.modZ + q);
+                cp16(&S.W[st][lane], a.modW + q);
+            }
+            if (pot) cp8(&S.P[st][lane], pot + 2 * (size_t)q);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        return n;
+    };
+    int4 first, first_n;
+    int st = 0, n = fetch(0, first);
+    while (n > 0) {
+        const int n_next = fetch(st ^ 1, first_n);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        fn(st, n, first);
+        __syncwarp();
+        st ^= 1;
+        n = n_next;
+        first = first_n;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+}
+
+// |rhat - r|^2 of two packed pairs, the arithmetic of pair_v2.
+__device__ __forceinline__ f2 pair_e2(f2 px, f2 py, f2 pz, f2 ncx, f2 ncy, f2 ncz, f2 nrx, f2 nry, f2 nrz) {
+    f2 dx = add2(px, ncx), dy = add2(py, ncy), dz = add2(pz, ncz);
+    f2 q = mul2(dx, dx);
+    q = fma2(dy, dy, q);
+    q = fma2(dz, dz, q);
+    f2 s = pk(rsq(lo(q)), rsq(hi(q)));
+    f2 ex = fma2(dx, s, nrx), ey = fma2(dy, s, nry), ez = fma2(dz, s, nrz);
+    f2 e2 = mul2(ex, ex);
+    e2 = fma2(ey, ey, e2);
+    return fma2(ez, ez, e2);
+}
+
+// A slice's place in its pass.
+struct Slice {
+    int tile, w;     // tile, and which slice of the tile
+    int id;          // slice number (header and chunk table)
+    int t, q, lane;  // angle, the lane's own pair, lane
+    bool valid;
+    int n_own;       // pairs of the slice
+};
+
+template <int TILE>
+__device__ __forceinline__ Slice slice_of(const int4* tiles, int n_tiles, int per_cta) {
+    constexpr int kW = TILE / 32;
+    Slice s;
+    const int warp = threadIdx.x >> 5;
+    s.lane = threadIdx.x & 31;
+    s.tile = warp / kW < per_cta ? blockIdx.x * per_cta + warp / kW : n_tiles;
+    s.w = warp % kW;
+    s.id = s.tile * kW + s.w;
+    s.t = 0;
+    s.q = 0;
+    s.n_own = 0;
+    if (s.tile < n_tiles) {
+        const int4 td = tiles[s.tile];
+        s.t = td.x;
+        s.q = td.y + 32 * s.w + s.lane;
+        s.n_own = min(32, max(0, td.z - 32 * s.w));
+    }
+    s.valid = s.lane < s.n_own;
+    return s;
+}
+
+// Observed pair of a lane, duplicated for the packed arithmetic.
+struct RowPair {
+    f2 pxa, pya, pza, pxb, pyb, pzb;
+};
+
+__device__ __forceinline__ RowPair load_row_pair(const SkArgs& a, int q, bool valid) {
+    float4 X = valid ? a.obsX[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+    float2 Y = valid ? *(const float2*)&a.obsY[q] : make_float2(kPadFar, kPadFar);
+    return RowPair{dup(X.x), dup(X.z), dup(Y.x), dup(X.y), dup(X.w), dup(Y.y)};
+}
+
+
+// ------------------------------------------------------------- pair lists
+// For fixed poses and temperature the pairs whose plan entry can be nonzero
+// do not change over the iterations of an E-step: with the potentials at most
+// the shift, a term is 2^(G_j - shift - K e2) <= 2^(-K e2), which
+// ex2.approx.ftz flushes to 0 beyond K e2 = 126.  So each slice's pairs with
+// K e2 <= kListLog2 are listed once per E-step, with the cost e2 that the
+// passes would recompute: 0.44 % of the 9.2e9 same-angle pairs of the
+// 1000-grain configuration at 1 mm^2, where the passes used to evaluate
+// 28.9 %.  A pass then streams 6 bytes per entry (HBM) instead of spending 13
+// packed instructions and two MUFU per evaluated pair.
+//
+// One warp lists one slice; chunks come from the pool as the longest of the
+// slice's 64 lists grows (a chunk's place in the pool is not reproducible, its
+// contents are).  A slice is left to the sweep when its chunks run out, when a
+// block has more than 65536 spots (16-bit slots), or when more than half of
+// the pairs it evaluates would be listed: a listed entry costs about as much
+// as two swept pairs.
+//
+// Most of the pairs that the cones let through are still too far apart, so a
+// cheap test comes first: the angle between p (seen from the origin) and r is
+// at most the angle of the cost bound plus the parallax asin(|c| / |p|), three
+// packed multiply-adds per two pairs against thirteen and two MUFU.  Only the
+// pairs that pass it (a bit mask per spot and batch) have their cost taken.
+struct ListStage {
+    WarpStage S;
+    float2 nx[32], ny[32], nz[32];  // unit directions of the streamed pairs
+    int tab[kListChunks];
+};
+
+__device__ __forceinline__ int nth(const int4& f, int g) { return g == 0 ? f.x : g == 1 ? f.y : g == 2 ? f.z : f.w; }
+
+constexpr int kListWarps = 4;
+
+template <int TILE, bool ROWS>
+__global__ void __launch_bounds__(32 * kListWarps) sk_list_kernel(SkArgs a) {
+    __shared__ __align__(16) ListStage stage[kListWarps];
+    constexpr int kW = TILE / 32;
+    const int lane = threadIdx.x & 31;
+    const int id = blockIdx.x * kListWarps + (threadIdx.x >> 5);
+    const int tile = id / kW, w = id % kW;
+    if (tile >= a.ctrl[ROWS ? CTRL_N_ROW_TILES : CTRL_N_COL_TILES]) return;
+    ListStage& L = stage[threadIdx.x >> 5];
+    const int4 td = (ROWS ? a.row_tiles : a.col_tiles)[tile];
+    const int t = td.x, first = td.y + 32 * w, n_own = min(32, max(0, td.z - 32 * w));
+    int* hdr = (ROWS ? a.row_hdr : a.col_hdr) + id;
+    if (n_own == 0) {
+        if (lane == 0 && a.pool_chunks > 0) *hdr = 0;
+        return;
+    }
+    const int q = first + lane;
+    const bool valid = lane < n_own;
+    const int o0 = (ROWS ? a.I2_off : a.J2_off)[t], b0 = (ROWS ? a.J2_off : a.I2_off)[t];
+    const int np = (ROWS ? a.J2_off : a.I2_off)[t + 1] - b0;
+    const int* own_off = ROWS ? a.I_off : a.J_off;
+    const int* str_off = ROWS ? a.J_off : a.I_off;
+    const int n_str = str_off[t + 1] - str_off[t];
+    const bool vb = valid && 2 * (q - o0) + 1 < own_off[t + 1] - own_off[t];
+    const int* own_g = ROWS ? a.obs_gbase : a.mod_gbase;
+    const int* str_g = ROWS ? a.mod_gbase : a.obs_gbase;
+    const Cone own = load_cone(ROWS ? a.obs_cone : a.mod_cone, ROWS ? a.obs_ext : a.mod_ext,
+                               own_g[t] + (first - o0) / kGran);
+    const float4* sub = (ROWS ? a.mod_sub : a.obs_sub) + (size_t)kSubs * str_g[t];
+    const float* subext = (ROWS ? a.mod_subext : a.obs_subext) + (size_t)kSubs * str_g[t];
+    const int evaluated = count_pairs(own, ROWS, sub, subext, np, a.skip, a.skipK);
+    bool fail = a.pool_chunks == 0 || n_str > 65536;
+    int ca = 0, cb = 0, nch = 0;
+    if (!fail) {
+        RowPair R{};
+        ColPair C;
+        if (ROWS) R = load_row_pair(a, q, valid);
+        else load_col_pair(a, valid ? q : first, C);
+        // unit directions of the lane's spots, and the parallax of its pairs
+        float da[3], db[3];
+        if (ROWS) {
+            const float x[6] = {lo(R.pxa), lo(R.pya), lo(R.pza), lo(R.pxb), lo(R.pyb), lo(R.pzb)};
+            const float ra = rsqrtf(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]);
+            const float rb = rsqrtf(x[3] * x[3] + x[4] * x[4] + x[5] * x[5]);
+            for (int k = 0; k < 3; ++k) {
+                da[k] = x[k] * ra;
+                db[k] = x[3 + k] * rb;
+            }
+        } else {
+            da[0] = -lo(C.nrxa), da[1] = -lo(C.nrya), da[2] = -lo(C.nrza);
+            db[0] = -lo(C.nrxb), db[1] = -lo(C.nryb), db[2] = -lo(C.nrzb);
+        }
+        const f2 dax = dup(da[0]), day = dup(da[1]), daz = dup(da[2]);
+        const f2 dbx = dup(db[0]), dby = dup(db[1]), dbz = dup(db[2]);
+        // the angle of the largest listed cost of any spot, K 4 sin^2(th / 2) = kListLog2
+        const float h = kListLog2 / (4.0f * a.skipK);
+        const float th = h < 1.0f ? 2.0f * asinf(sqrtf(h)) : 7.0f;
+        auto put = [&](int& cnt, int ab, float e2, int slot) {
+            char* p = a.pool + (size_t)L.tab[cnt / kListDepth] * kListChunkBytes;
+            const int at = (cnt % kListDepth) * 64 + 2 * lane + ab;
+            ((float*)p)[at] = e2;
+            ((unsigned short*)(p + kListDepth * 64 * 4))[at] = (unsigned short)slot;
+            ++cnt;
+        };
+        sweep<ROWS>(a, L.S, own, sub, subext, b0, np, a.skip, nullptr, [&](int st, int n, const int4& f) {
+            if (fail || kListDepth * nch > evaluated) {
+                fail = true;  // mostly nonzero: the sweep is as good
+                return;
+            }
+            // the batch's unit directions; the largest parallax of the slice with it
+            float ext = ROWS ? 0.0f : 3.0e38f;
+            {
+                const float4 X = L.S.X[st][lane];
+                const float2 Y = L.S.Y[st][lane];
+                float2 ux = make_float2(X.x, X.y), uy = make_float2(X.z, X.w), uz = Y;
+                if (ROWS) {
+                    const float4 Z = L.S.Z[st][lane], W = L.S.W[st][lane];
+                    ux = make_float2(-Z.x, -Z.y), uy = make_float2(-Z.z, -Z.w), uz = make_float2(-W.x, -W.y);
+                } else {
+                    const float r0 = rsqrtf(ux.x * ux.x + uy.x * uy.x + uz.x * uz.x);
+                    const float r1 = rsqrtf(ux.y * ux.y + uy.y * uy.y + uz.y * uz.y);
+                    ux = make_float2(ux.x * r0, ux.y * r1);
+                    uy = make_float2(uy.x * r0, uy.y * r1);
+                    uz = make_float2(uz.x * r0, uz.y * r1);
+                }
+                L.nx[lane] = ux;
+                L.ny[lane] = uy;
+                L.nz[lane] = uz;
+                if (lane < n) ext = subext[(nth(f, lane / kSubGran)) / kSubGran];
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float y = __shfl_xor_sync(0xffffffffu, ext, o);
+                ext = ROWS ? fmaxf(ext, y) : fminf(ext, y);
+            }
+            const float cmax = ROWS ? ext : own.ext, pmin = ROWS ? own.ext : ext;
+            const float reach = th + (pmin > cmax ? asinf(cmax / pmin) : 7.0f) + 1e-4f;
+            const float least = reach < 3.1f ? cosf(reach) - 4e-6f : -3.0f;
+            __syncwarp();
+            unsigned ma[2] = {0u, 0u}, mb[2] = {0u, 0u};
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                const int j1 = min(16, n - 16 * hf);
+#pragma unroll 4
+                for (int j = 0; j < j1; ++j) {
+                    const f2 x = *(const f2*)&L.nx[16 * hf + j], y = *(const f2*)&L.ny[16 * hf + j],
+                             z = *(const f2*)&L.nz[16 * hf + j];
+                    const f2 ta = fma2(daz, z, fma2(day, y, mul2(dax, x)));
+                    const f2 tb = fma2(dbz, z, fma2(dby, y, mul2(dbx, x)));
+                    // not less, so that a spot that is not a number stays
+                    ma[hf] |= (!(lo(ta) < least) ? 1u : 0u) << (2 * j) | (!(hi(ta) < least) ? 2u : 0u) << (2 * j);
+                    mb[hf] |= (!(lo(tb) < least) ? 1u : 0u) << (2 * j) | (!(hi(tb) < least) ? 2u : 0u) << (2 * j);
+                }
+            }
+            for (int hf = 0; hf < 2; ++hf) {
+                unsigned m0 = valid ? ma[hf] : 0u, m1 = vb ? mb[hf] : 0u;
+                // room for the half batch
+                while (!fail && __any_sync(0xffffffffu, max(ca + __popc(m0), cb + __popc(m1)) > kListDepth * nch)) {
+                    int c = a.pool_chunks;
+                    if (nch < kListChunks) {
+                        if (lane == 0) c = atomicAdd(a.ctrl + CTRL_POOL_NEXT, 1);
+                        c = __shfl_sync(0xffffffffu, c, 0);
+                    }
+                    fail = c >= a.pool_chunks;
+                    if (!fail) {
+                        if (lane == 0) L.tab[nch] = c;
+                        __syncwarp();
+                        ++nch;
+                    }
+                }
+                if (fail) return;
+                while (__any_sync(0xffffffffu, m0 | m1)) {
+#pragma unroll
+                    for (int ab = 0; ab < 2; ++ab) {
+                        unsigned& m = ab ? m1 : m0;
+                        if (!m) continue;
+                        const int bit = __ffs(m) - 1;
+                        m &= m - 1;
+                        const int j = 16 * hf + (bit >> 1);
+                        const int slot = 2 * (nth(f, j / kSubGran) + j % kSubGran) + (bit & 1);
+                        const ulonglong2 X = *(const ulonglong2*)&L.S.X[st][j];
+                        const f2 Y = *(const f2*)&L.S.Y[st][j];
+                        f2 e;
+                        float k;
+                        if (ROWS) {
+                            const ulonglong2 Z = *(const ulonglong2*)&L.S.Z[st][j], W = *(const ulonglong2*)&L.S.W[st][j];
+                            e = pair_e2(ab ? R.pxb : R.pxa, ab ? R.pyb : R.pya, ab ? R.pzb : R.pza, X.x, X.y, Y, Z.x, Z.y,
+                                        W.x);
+                            k = bit & 1 ? hi(W.y) : lo(W.y);
+                        } else {
+                            e = pair_e2(X.x, X.y, Y, ab ? C.ncxb : C.ncxa, ab ? C.ncyb : C.ncya, ab ? C.nczb : C.ncza,
+                                        ab ? C.nrxb : C.nrxa, ab ? C.nryb : C.nrya, ab ? C.nrzb : C.nrza);
+                            k = lo(ab ? C.kb : C.ka);
+                        }
+                        const float e2 = bit & 1 ? hi(e) : lo(e);
+                        // the padding spot of an odd block is no entry
+                        if (slot < n_str && !(e2 * k < -kListLog2)) put(ab ? cb : ca, ab, e2, slot);
+                    }
+                }
+            }
+        });
+    }
+    int most = max(ca, cb);
+    for (int o = 16; o > 0; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+    nch = fail ? 0 : (most + kListDepth - 1) / kListDepth;
+    // entries of the slice (with padding) against the spot pairs of the sweep
+    if (!fail && nch * kListDepth > evaluated) fail = true;
+    if (!fail) {
+        int* to = (ROWS ? a.row_tab : a.col_tab) + (size_t)kListChunks * id;
+        for (int c = lane; c < nch; c += 32) to[c] = L.tab[c];
+        // pad every list to the slice's depth (2^-inf adds nothing)
+        for (int ab = 0; ab < 2; ++ab)
+            for (int c = ab ? cb : ca; c < kListDepth * nch; ++c) {
+                char* p = a.pool + (size_t)L.tab[c / kListDepth] * kListChunkBytes;
+                const int at = (c % kListDepth) * 64 + 2 * lane + ab;
+                ((float*)p)[at] = 3.0e38f;
+                ((unsigned short*)(p + kListDepth * 64 * 4))[at] = 0;
+            }
+    }
+    if (lane == 0) {
+        if (a.pool_chunks > 0) *hdr = fail ? -1 : nch;
+        const long long n = fail ? 4LL * n_own * evaluated : 64LL * kListDepth * nch;
+        atomicAdd((unsigned long long*)(a.ctrl + (ROWS ? CTRL_ROW_EVAL : CTRL_COL_EVAL)), (unsigned long long)n);
+    }
+}
+
+// ---------------------------------------------------- entries of a listed slice
+// Half a chunk (four entries of each of the lane's spots) in registers; the
+// next half is loaded while one is used.  The lists are read once per pass:
+// they stay out of L1.
+constexpr int kHalf = kListDepth / 2;
+struct Entries {
+    float2 e2[kHalf];     // costs of the lane's spots a and b
+    unsigned slot[kHalf];  // slots: a in the low half, b in the high half
+};
+
+__device__ __forceinline__ void load_entries(Entries& E, const char* chunk, int half, int lane) {
+#pragma unroll
+    for (int k = 0; k < kHalf; ++k) {
+        E.e2[k] = __ldcg((const float2*)chunk + 32 * (kHalf * half + k) + lane);
+        E.slot[k] = __ldcg((const unsigned*)(chunk + kListDepth * 64 * 4) + 32 * (kHalf * half + k) + lane);
+    }
+}
+
+// A listed slice: its number of chunks (-1: swept), the lane's share of the
+// first 32 chunk numbers and the first half chunk, which a pass loads before
+// it waits for the pass before it.
+struct ListHead {
+    int nch, mine;
+    Entries E;
+};
+
+__device__ __forceinline__ ListHead list_head(const SkArgs& a, const int* hdr, const int* tab, int id, int lane) {
+    ListHead h;
+    h.nch = a.pool_chunks > 0 ? __ldcg(hdr + id) : -1;
+    h.mine = lane < h.nch ? __ldcg(tab + (size_t)kListChunks * id + lane) : 0;
+    if (h.nch > 0)
+        load_entries(h.E, a.pool + (size_t)__shfl_sync(0xffffffffu, h.mine, 0) * kListChunkBytes, 0, lane);
+    return h;
+}
+
+// fn(entries) for every half chunk of the slice, in order.
+template <class Fn>
+__device__ __forceinline__ void for_each_half(const SkArgs& a, ListHead& h, const int* tab, int id, int lane, Fn fn) {
+    Entries N;
+    const char* p = a.pool + (size_t)__shfl_sync(0xffffffffu, h.mine, 0) * kListChunkBytes;
+    for (int c = 0; c < h.nch; ++c) {
+        load_entries(N, p, 1, lane);
+        fn(h.E);
+        if (c + 1 < h.nch) {
+            if (((c + 1) & 31) == 0)
+                h.mine = c + 1 + lane < h.nch ? __ldcg(tab + (size_t)kListChunks * id + c + 1 + lane) : 0;
+            p = a.pool + (size_t)__shfl_sync(0xffffffffu, h.mine, (c + 1) & 31) * kListChunkBytes;
+            load_entries(h.E, p, 0, lane);
+        }
+        fn(N);
+    }
+}
+
+// Sums of 2^(pot_slot - shift - K e2) over a listed slice's entries for the
+// lane's two spots: even slots into e, odd slots into o.  GATHER_K: -K comes
+// with the slot's model spot (rows of a geometry with several cost lengths).
+struct ListSum {
+    float ea, oa, eb, ob;
+};
+
+template <bool GATHER_K>
+__device__ __forceinline__ void list_sum(const SkArgs& a, ListHead& h, const int* tab, int id, int lane, const float* pot,
+                                         float shift, float ka, float kb, const float4* modW, ListSum& S) {
+    for_each_half(a, h, tab, id, lane, [&](const Entries& E) {
+        float pa[kHalf], pb[kHalf];
+#pragma unroll
+        for (int k = 0; k < kHalf; ++k) {
+            pa[k] = pot[E.slot[k] & 0xffffu];
+            pb[k] = pot[E.slot[k] >> 16];
+        }
+#pragma unroll
+        for (int k = 0; k < kHalf; ++k) {
+            if (GATHER_K) {
+                const unsigned ja = E.slot[k] & 0xffffu, jb = E.slot[k] >> 16;
+                const float2 wa = *((const float2*)&modW[ja >> 1] + 1), wb = *((const float2*)&modW[jb >> 1] + 1);
+                ka = ja & 1u ? wa.y : wa.x;
+                kb = jb & 1u ? wb.y : wb.x;
+            }
+            const float ta = ex2(fmaf(E.e2[k].x, ka, pa[k] - shift)), tb = ex2(fmaf(E.e2[k].y, kb, pb[k] - shift));
+            const bool oa = E.slot[k] & 1u, ob = E.slot[k] & 0x10000u;
+            S.ea += oa ? 0.0f : ta;
+            S.oa += oa ? ta : 0.0f;
+            S.eb += ob ? 0.0f : tb;
+            S.ob += ob ? tb : 0.0f;
+        }
+    });
+}
+
+// ------------------------------------------------------------ swept slices
+__device__ __forceinline__ void row_pair_v(const RowPair& R, const WarpStage& S, int st, int j, f2 base, f2& va, f2& vb) {
+    const ulonglong2 X = *(const ulonglong2*)&S.X[st][j], Z = *(const ulonglong2*)&S.Z[st][j],
+                     W = *(const ulonglong2*)&S.W[st][j];
+    const f2 ncz = *(const f2*)&S.Y[st][j];
+    va = pair_v2(R.pxa, R.pya, R.pza, X.x, X.y, ncz, Z.x, Z.y, W.x, W.y, base);
+    vb = pair_v2(R.pxb, R.pyb, R.pzb, X.x, X.y, ncz, Z.x, Z.y, W.x, W.y, base);
+}
+
+__device__ __forceinline__ void col_pair_v(const ColPair& C, const WarpStage& S, int st, int j, f2 base, f2& va, f2& vb) {
+    const ulonglong2 X = *(const ulonglong2*)&S.X[st][j];
+    const f2 pz = *(const f2*)&S.Y[st][j];
+    va = pair_v2(X.x, X.y, pz, C.ncxa, C.ncya, C.ncza, C.nrxa, C.nrya, C.nrza, C.ka, base);
+    vb = pair_v2(X.x, X.y, pz, C.ncxb, C.ncyb, C.nczb, C.nrxb, C.nryb, C.nrzb, C.kb, base);
+}
+
+// What the slices of either side need to sweep the other.
+struct Sweep {
+    Cone own;
+    const float4* sub;
+    const float* ext;
+    int b0, n;
+};
+
+template <bool ROWS>
+__device__ __forceinline__ Sweep sweep_of(const SkArgs& a, const Slice& sl) {
+    const int first = sl.q - sl.lane, t = sl.t;
+    Sweep w;
+    if (ROWS) {
+        w.own = load_cone(a.obs_cone, a.obs_ext, a.obs_gbase[t] + (first - a.I2_off[t]) / kGran);
+        w.sub = a.mod_sub + (size_t)kSubs * a.mod_gbase[t];
+        w.ext = a.mod_subext + (size_t)kSubs * a.mod_gbase[t];
+        w.b0 = a.J2_off[t];
+        w.n = a.J2_off[t + 1] - w.b0;
+    } else {
+        w.own = load_cone(a.mod_cone, a.mod_ext, a.mod_gbase[t] + (first - a.J2_off[t]) / kGran);
+        w.sub = a.obs_sub + (size_t)kSubs * a.obs_gbase[t];
+        w.ext = a.obs_subext + (size_t)kSubs * a.obs_gbase[t];
+        w.b0 = a.I2_off[t];
+        w.n = a.I2_off[t + 1] - w.b0;
+    }
+    return w;
+}
+
+// fn(stage, pair of the stage, base potentials' packed pair, pair of the block)
+// over the slice's sweep; skip = 0: over the whole block.
+template <bool ROWS, class Fn>
+__device__ __forceinline__ void for_each_swept(const SkArgs& a, WarpStage& S, const Slice& sl, int skip, Fn fn) {
+    const Sweep w = sweep_of<ROWS>(a, sl);
+    sweep<ROWS>(a, S, w.own, w.sub, w.ext, w.b0, w.n, skip, ROWS ? a.Gc : a.Fc, [&](int st, int n, const int4& f) {
+#pragma unroll 4
+        for (int j = 0; j < n; ++j) fn(st, j, S.P[st][j], nth(f, j / kSubGran) + j % kSubGran);
+    });
+}
+
+// Shifted sums over a swept slice.
+template <bool ROWS>
+__device__ __forceinline__ void swept_sum(const SkArgs& a, WarpStage& S, const Slice& sl, float shift, ListSum& out) {
+    f2 Sa = pk(out.ea, out.oa), Sb = pk(out.eb, out.ob);
+    auto add = [&](f2 va, f2 vb) {
+        Sa = add2(Sa, pk(ex2(lo(va)), ex2(hi(va))));
+        Sb = add2(Sb, pk(ex2(lo(vb)), ex2(hi(vb))));
+    };
+    if (ROWS) {
+        const RowPair R = load_row_pair(a, sl.q, sl.valid);
+        for_each_swept<ROWS>(a, S, sl, a.skip, [&](int st, int j, float2 P, int) {
+            f2 va, vb;
+            row_pair_v(R, S, st, j, pk(P.x - shift, P.y - shift), va, vb);
+            add(va, vb);
+        });
+    } else {
+        ColPair C;
+        load_col_pair(a, sl.valid ? sl.q : sl.q - sl.lane, C);
+        for_each_swept<ROWS>(a, S, sl, a.skip, [&](int st, int j, float2 P, int) {
+            f2 va, vb;
+            col_pair_v(C, S, st, j, pk(P.x - shift, P.y - shift), va, vb);
+            add(va, vb);
+        });
+    }
+    out = ListSum{lo(Sa), hi(Sa), lo(Sb), hi(Sb)};
+}
+
+// Exact log-sum-exps (running maximum) of the lanes' two spots over the whole
+// block, where a shifted sum underflowed: four streamed pairs to a group.
+template <bool ROWS>
+__device__ __noinline__ void exact_lse(const SkArgs& a, WarpStage& S, const Slice& sl, float dust, float& va_out,
+                                       float& vb_out) {
+    RowLse A, B;
+    A.init(dust);
+    B.init(dust);
+    RowPair R{};
+    ColPair C;
+    if (ROWS) R = load_row_pair(a, sl.q, sl.valid);
+    else load_col_pair(a, sl.valid ? sl.q : sl.q - sl.lane, C);
+    const Sweep w = sweep_of<ROWS>(a, sl);
+    sweep<ROWS>(a, S, w.own, w.sub, w.ext, w.b0, w.n, 0, ROWS ? a.Gc : a.Fc, [&](int st, int n, const int4&) {
+        auto pair = [&](int j, f2& va, f2& vb) {
+            const f2 base = *(const f2*)&S.P[st][j];
+            if (ROWS) row_pair_v(R, S, st, j, base, va, vb);
+            else col_pair_v(C, S, st, j, base, va, vb);
+        };
+        int j = 0;
+        for (; j + kGroup <= n; j += kGroup) {
+            f2 va[kGroup], vb[kGroup];
+#pragma unroll
+            for (int g = 0; g < kGroup; ++g) pair(j + g, va[g], vb[g]);
+            A.add4(va);
+            B.add4(vb);
+        }
+        for (; j < n; ++j) {
+            f2 va, vb;
+            pair(j, va, vb);
+            A.add1(va);
+            B.add1(vb);
+        }
+    });
+    va_out = A.value();
+    vb_out = B.value();
+}
+
+// ----------------------------------------------------- ends of the passes
+// Largest potential of each angle block, kept by the passes as the maximum of
+// the tile partials in an order-preserving code (0: none yet).  Rows and
+// columns have two sets each: pass `it` fills set it & 1, and the last CTA of
+// the pass clears the other side's set that the next pass fills, whose readers
+// are done.
+__device__ __forceinline__ unsigned max_code(float v) {
+    const unsigned b = __float_as_uint(v);
+    return b & 0x80000000u ? ~b : b | 0x80000000u;
+}
+__device__ __forceinline__ float angle_max(const unsigned* set, int t, float add) {
+    const unsigned k = __ldcg(set + t);
+    const float m = k == 0u ? kNegHuge : __uint_as_float(k & 0x80000000u ? k & 0x7fffffffu : ~k);
+    return m > kNegHuge ? m + add : kNegHuge;
+}
+__device__ __forceinline__ unsigned* row_max(const SkArgs& a, int it) { return a.pmax + (it & 1) * a.T; }
+__device__ __forceinline__ unsigned* col_max(const SkArgs& a, int it) { return a.pmax + (2 + (it & 1)) * a.T; }
+// after n_iter iterations (0: the maxima of the starting potentials)
+__device__ __forceinline__ float final_row_max(const SkArgs& a, const DustPtrs& D, int t, int n_iter) {
+    return n_iter > 0 ? angle_max(row_max(a, n_iter - 1), t, a.kc) : D.Fmax[t];
+}
+__device__ __forceinline__ float final_col_max(const SkArgs& a, const DustPtrs& D, int t, int n_iter) {
+    return n_iter > 0 ? angle_max(col_max(a, n_iter - 1), t, 0.0f) : D.Gmax[t];
+}
+
+// Lanes' partial log-sum-exps of a CTA's tiles into part[tile] and the angle
+// maxima: the warps of a tile in order.
+template <int TILE>
+__device__ __forceinline__ void store_parts(float m, float s, int per_cta, int n_tiles, int my_angle, float2* part,
+                                            unsigned* maxima, float* sm, float* ss) {
+    constexpr int kW = TILE / 32;
+    const int warp = threadIdx.x >> 5;
+    warp_lse_reduce(m, s);
+    if ((threadIdx.x & 31) == 0) {
+        sm[warp] = m;
+        ss[warp] = s;
+    }
+    __syncthreads();
+    const int tile = blockIdx.x * per_cta + threadIdx.x;
+    if ((int)threadIdx.x < per_cta && tile < n_tiles) {
+        Lse2 L;
+        L.m = kNegHuge;
+        L.s = 0.0f;
+        for (int k = 0; k < kW; ++k) L.merge(sm[threadIdx.x * kW + k], ss[threadIdx.x * kW + k]);
+        part[tile] = make_float2(L.m, L.s);
+        if (L.m > kNegHuge) atomicMax(maxima + my_angle, max_code(L.m));
+    }
+}
+
+// True in exactly one CTA, the last one to get here.
+__device__ __forceinline__ bool last_block(int* done, int* flag) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        *flag = atomicAdd(done, 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    const bool last = *flag != 0;
+    if (last) __threadfence();
+    return last;
+}
+
+// Log-sum-exp of the n tile partials by the last CTA: TILE chains (chain c
+// takes the tiles c, c + TILE, ... in order), then the chains by warp and the
+// warps in order.  A chain's running maxima are known before its sum (a prefix
+// maximum), so every exponential is taken in parallel and only the sum's
+// multiply-adds are serial: kPassThreads / TILE segments of a chain hold their
+// elements in registers and hand the sum on.  Thread 0 gets (m, s).
+template <int TILE>
+__device__ void merge_parts(const float2* part, int n, float& m_out, float& s_out, float* sm, float* ss,
+                            float (*segmax)[TILE], float* cm, float* cs) {
+    constexpr int kSeg = kPassThreads / TILE, kR = 8;
+    const int c = threadIdx.x % TILE, seg = threadIdx.x / TILE;
+    if (seg == 0) {
+        cm[c] = kNegHuge;
+        cs[c] = 0.0f;
+    }
+    for (int r0 = 0; r0 * TILE < n; r0 += kSeg * kR) {
+        float2 v[kR];
+        float top = kNegHuge;
+#pragma unroll
+        for (int i = 0; i < kR; ++i) {
+            const int k = c + TILE * (r0 + seg * kR + i);
+            v[i] = k < n ? __ldcg(&part[k]) : make_float2(kNegHuge, 0.0f);
+            if (v[i].y != 0.0f) top = fmaxf(top, v[i].x);
+        }
+        segmax[seg][c] = top;
+        __syncthreads();
+        float m = cm[c];
+        for (int g = 0; g < seg; ++g) m = fmaxf(m, segmax[g][c]);
+        float e[kR];
+        unsigned fresh = 0u;
+#pragma unroll
+        for (int i = 0; i < kR; ++i) {
+            const bool nw = v[i].y != 0.0f && v[i].x > m;
+            e[i] = nw ? ex2(m - v[i].x) : ex2(v[i].x - m);
+            if (nw) {
+                fresh |= 1u << i;
+                m = v[i].x;
+            }
+        }
+        for (int g = 0; g < kSeg; ++g) {
+            if (seg == g) {
+                float s = cs[c];
+#pragma unroll
+                for (int i = 0; i < kR; ++i)
+                    if (v[i].y != 0.0f) s = (fresh >> i) & 1u ? fmaf(s, e[i], v[i].y) : fmaf(v[i].y, e[i], s);
+                cs[c] = s;
+                if (g == kSeg - 1) cm[c] = m;
+            }
+            __syncthreads();
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < TILE) {
+        float m = cm[c], s = cs[c];
+        warp_lse_reduce(m, s);
+        if ((threadIdx.x & 31) == 0) {
+            sm[threadIdx.x >> 5] = m;
+            ss[threadIdx.x >> 5] = s;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        Lse2 L;
+        L.m = kNegHuge;
+        L.s = 0.0f;
+        for (int k = 0; k < TILE / 32; ++k) L.merge(sm[k], ss[k]);
+        m_out = L.m;
+        s_out = L.s;
+    }
+}
+
+// (m, s) merged with the partials [first, first + cnt) in order, by one warp:
+// the exponentials in parallel, the sum's multiply-adds in order.
+__device__ __forceinline__ void warp_merge_parts(const float2* part, int first, int cnt, float& m, float& s) {
+    const int lane = threadIdx.x & 31;
+    for (int k0 = 0; k0 < cnt; k0 += 32) {
+        const float2 p = k0 + lane < cnt ? __ldcg(&part[first + k0 + lane]) : make_float2(kNegHuge, 0.0f);
+        const bool live = p.y != 0.0f;
+        float top = live ? p.x : kNegHuge;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float y = __shfl_up_sync(0xffffffffu, top, o);
+            if (lane >= o) top = fmaxf(top, y);
+        }
+        float before = __shfl_up_sync(0xffffffffu, top, 1);
+        before = lane == 0 ? m : fmaxf(m, before);
+        const bool nw = live && p.x > before;
+        const float e = nw ? ex2(before - p.x) : ex2(p.x - before);
+        const unsigned lives = __ballot_sync(0xffffffffu, live), fresh = __ballot_sync(0xffffffffu, nw);
+        for (int l = 0; l < min(32, cnt - k0); ++l) {
+            const float el = __shfl_sync(0xffffffffu, e, l), yl = __shfl_sync(0xffffffffu, p.y, l);
+            if ((lives >> l) & 1u) s = (fresh >> l) & 1u ? fmaf(s, el, yl) : fmaf(yl, el, s);
+        }
+        m = fmaxf(m, __shfl_sync(0xffffffffu, top, 31));
+    }
+}
+
+
+template <int TILE>
+struct PassShared {
+    WarpStage stage[kPassThreads / 32];
+    float sm[kPassThreads / 32], ss[kPassThreads / 32];
+    float segmax[kPassThreads / TILE][TILE];
+    float cm[TILE], cs[TILE];
+    int last;
+};
+
+// Programmatic dependent launch: a pass starts while the one before it ends.
+// What it reads before pass_wait is what the list kernels and the scheduler
+// left, and those were complete before the pass before it (which waited for
+// its own predecessor before it let this one start) went on.
+__device__ __forceinline__ void pass_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pass_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// --------------------------------------------------- row and column passes
+// Iteration `it` of the row (ROWS) or column update.  What bounds it: at the
+// 1000-grain density the lists (HBM), below that the chain of a pass: the
+// potentials' gathers, the tickets and the merge of the tiles.
+template <int TILE, bool ROWS>
+__global__ void __launch_bounds__(kPassThreads, 2) sk_pass_kernel(SkArgs a, int it, int per_cta) {
+    extern __shared__ __align__(128) char pass_smem[];
+    PassShared<TILE>& H = *(PassShared<TILE>*)pass_smem;
+    if (ROWS && it == 0) pass_wait();  // the first pass follows the kernels that write the lists
+    DustPtrs D = dust_ptrs(a.dust, a.T);
+    const int n_tiles = __ldcg(a.ctrl + (ROWS ? CTRL_N_ROW_TILES : CTRL_N_COL_TILES));
+    const int4* tiles = ROWS ? a.row_tiles : a.col_tiles;
+    const Slice sl = slice_of<TILE>(tiles, n_tiles, per_cta);
+    const int t = sl.t, lane = sl.lane;
+    const int* tab = ROWS ? a.row_tab : a.col_tab;
+    ListHead h;
+    h.nch = 0;
+    if (sl.n_own > 0) h = list_head(a, ROWS ? a.row_hdr : a.col_hdr, tab, sl.id, lane);
+    const int* own_off = ROWS ? a.I_off : a.J_off;
+    const int* own2 = ROWS ? a.I2_off : a.J2_off;
+    const int* str2 = ROWS ? a.J2_off : a.I2_off;
+    const bool vb = sl.valid && 2 * (sl.q - own2[t]) + 1 < own_off[t + 1] - own_off[t];
+    const int s0 = str2[t], ns = str2[t + 1] - s0;
+    float2 K = make_float2(a.negKD2, a.negKD2);  // -K of the lane's own spots (columns)
+    if (!ROWS && sl.valid) K = *((const float2*)&a.modW[sl.q] + 1);
+    if (!vb) K.y = -1.0f;
+    int my_angle = 0;
+    {
+        const int tile = blockIdx.x * per_cta + threadIdx.x;
+        if ((int)threadIdx.x < per_cta && tile < n_tiles) my_angle = tiles[tile].x;
+    }
+    const float* pot = ROWS ? a.Gc : a.Fc;
+    float* out = ROWS ? a.Fc : a.Gc;
+    if (!(ROWS && it == 0)) pass_wait();
+    pass_release();
+    const bool ub = a.mode == 2;  // unbalanced OT: no dustbins, scaled update
+    const int d = a.mode ? t : 0;
+    float pm = kNegHuge, ps = 0.0f;
+    if (sl.n_own > 0) {
+        // the dustbin's term: the outlier column (rows), the unmatched-model row with C_0j = 0 (columns)
+        const float dust = ub ? kNegHuge : ROWS ? __ldcg(D.G0 + d) - a.kc : __ldcg(D.F0 + d);
+        const float top = ROWS ? (it > 0 ? angle_max(col_max(a, it - 1), t, 0.0f) : D.Gmax[t])
+                               : angle_max(row_max(a, it), t, a.kc);
+        const float shift = ub ? top : fmaxf(top, dust);
+        const float e0 = ub ? 0.0f : ex2(dust - shift);
+        ListSum S{e0, 0.0f, e0, 0.0f};
+        if (h.nch < 0)
+            swept_sum<ROWS>(a, H.stage[threadIdx.x >> 5], sl, shift, S);
+        else if (!ROWS || a.uniK)
+            list_sum<false>(a, h, tab, sl.id, lane, pot + 2 * s0, shift, K.x, ROWS ? a.negKD2 : K.y, nullptr, S);
+        else
+            list_sum<ROWS>(a, h, tab, sl.id, lane, pot + 2 * s0, shift, 0.0f, 0.0f, a.modW + s0, S);
+        const float sa = S.ea + S.oa, sb = S.eb + S.ob;
+        float va = -(shift + lg2(sa)), vv = vb ? -(shift + lg2(sb)) : 0.0f;
+        const unsigned low_a = __ballot_sync(0xffffffffu, sl.valid && !(sa > kTinySum));
+        const unsigned low_b = __ballot_sync(0xffffffffu, vb && !(sb > kTinySum));
+        if (low_a | low_b) {
+            float xa, xb;
+            exact_lse<ROWS>(a, H.stage[threadIdx.x >> 5], sl, dust, xa, xb);
+            if ((low_a >> lane) & 1u) va = -xa;
+            if ((low_b >> lane) & 1u) vv = -xb;
+            if (lane == 0)
+                atomicAdd((unsigned*)a.ctrl + (ROWS ? CTRL_EXACT_ROWS : CTRL_EXACT_COLS),
+                          (unsigned)(__popc(low_a) + __popc(low_b)));
+        }
+        if (sl.valid) {
+            if (ub) {  // Algorithm UnbalancedOT: the balanced update raised to kappa / (kappa + eps)
+                const float tau = ROWS ? a.tau_row : a.tau_col;
+                va = ns > 0 ? tau * va : 0.0f;
+                vv = ns > 0 ? tau * vv : 0.0f;
+            }
+            *(float2*)&out[2 * (size_t)sl.q] = make_float2(va, vb ? vv : kNegHuge);
+            // tile partial of LSE2(F_i - kc) for the outlier column, of LSE2(G_j) for the unmatched row
+            const float off = ROWS ? a.kc : 0.0f;
+            pm = va - off;
+            ps = 1.0f;
+            if (vb) lse_merge_into(pm, ps, vv - off, 1.0f);
+        }
+    }
+    float2* part = ROWS ? a.row_part : a.col_part;
+    store_parts<TILE>(pm, ps, per_cta, n_tiles, my_angle, part, ROWS ? row_max(a, it) : col_max(a, it), H.sm, H.ss);
+    if (!last_block(a.ctrl + (ROWS ? CTRL_ROW_DONE : CTRL_COL_DONE), &H.last)) return;
+    // rows: promote F_0, then G_0 from the new F; columns: next F_0 from the new G and the current G_0
+    if (a.mode == 1) {
+        for (int u = threadIdx.x >> 5; u < a.T; u += kPassThreads / 32) {
+            const int4 at = a.ang_tiles[u];
+            const float F0 = ROWS ? __ldcg(D.F0n + u) : 0.0f;
+            float m = (ROWS ? F0 : __ldcg(D.G0 + u)) - a.kc, s = 1.0f;
+            warp_merge_parts(part, ROWS ? at.x : at.z, ROWS ? at.y : at.w, m, s);
+            if (lane == 0) {
+                const float v = (ROWS ? D.log2O[u] : D.log2U[u]) - (m + lg2(s));
+                if (ROWS) {
+                    D.F0[u] = F0;
+                    D.G0[u] = v;
+                } else {
+                    D.F0n[u] = v;
+                }
+            }
+        }
+    } else if (a.mode == 0) {
+        float m, s;
+        const float at = threadIdx.x == 0 ? __ldcg(ROWS ? D.F0n : D.G0) : 0.0f;
+        merge_parts<TILE>(part, n_tiles, m, s, H.sm, H.ss, H.segmax, H.cm, H.cs);
+        if (threadIdx.x == 0) {
+            Lse2 L;
+            L.init(at - a.kc);
+            L.merge(m, s);
+            const float v = (ROWS ? D.log2O[0] : D.log2U[0]) - L.value();
+            if (ROWS) {
+                D.F0[0] = at;
+                D.G0[0] = v;
+            } else {
+                D.F0n[0] = v;
+            }
+        }
+    }
+    // the set of maxima that the other side's next pass fills
+    unsigned* clear = ROWS ? col_max(a, it) : row_max(a, it + 1);
+    for (int u = threadIdx.x; u < a.T; u += kPassThreads) clear[u] = 0u;
+    if (threadIdx.x == 0) {
+        a.ctrl[ROWS ? CTRL_ROW_DONE : CTRL_COL_DONE] = 0;
+        *(unsigned long long*)(a.ctrl + CTRL_SK_PAIRS) +=
+            *(const unsigned long long*)(a.ctrl + (ROWS ? CTRL_ROW_EVAL : CTRL_COL_EVAL));
+    }
+}
+
+// ------------------------------------------------------------- read-out
+// Largest of the CTA's non-negative values into *out.
+__device__ __forceinline__ void block_err(float v, float* red, int* out) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < kPassThreads / 32; ++k) v = fmaxf(v, red[k]);
+        atomicMax(out, __float_as_int(v));
+    }
+}
+
+// Plan read-out per observed spot with the final potentials: argmax over the
+// block's model spots and the outlier column (ties to the lowest index, the
+// outlier column only when strictly larger), top1 - top2 margin in plan
+// units, and the row-marginal error.  Once per E-step.
+//
+// Listed slices read their lists, swept ones the sub-granules that their
+// cones see.  A pair left out has an exponent of at most the largest
+// potential less kListLog2; a row whose best entry (the outlier column
+// included) does not stand kFarLog2 above that is read again over its whole
+// block, the lanes of the warp sharing its pairs, so the ranking and the sums
+// are those of every pair.
+struct Top2 {
+    float m, s, b1, b2;
+    int arg;
+    __device__ __forceinline__ void init() {
+        m = kNegHuge;
+        s = 0.0f;
+        b1 = kNegHuge;
+        b2 = kNegHuge;
+        arg = -1;
+    }
+    // j: the spot's slot in the spatial order; perm maps slots to the caller's
+    // indices, and ties go to the lowest caller index
+    __device__ __forceinline__ void add(float v, int j, const int* perm) {
+        if (v > m) {
+            s = s * ex2(m - v) + 1.0f;
+            m = v;
+        } else {
+            s += ex2(v - m);
+        }
+        if (v > b1 || (v == b1 && v > kNegHuge && perm[j] < perm[arg])) {
+            b2 = b1;
+            b1 = v;
+            arg = j;
+        } else if (v > b2) {
+            b2 = v;
+        }
+    }
+    // the same of two disjoint sets of entries
+    __device__ __forceinline__ void merge(const Top2& o, const int* perm) {
+        const float top = fmaxf(m, o.m);
+        s = (s == 0.0f ? 0.0f : s * ex2(m - top)) + (o.s == 0.0f ? 0.0f : o.s * ex2(o.m - top));
+        m = top;
+        b2 = fmaxf(fminf(b1, o.b1), fmaxf(b2, o.b2));
+        if (o.b1 > b1 || (o.b1 == b1 && o.b1 > kNegHuge && perm[o.arg] < perm[arg])) {
+            b1 = o.b1;
+            arg = o.arg;
+        }
+    }
+};
+
+// Top2 of one observed spot over its whole block, by the warp together.
+__device__ __noinline__ Top2 whole_row(const SkArgs& a, int t, float px, float py, float pz) {
+    const int lane = threadIdx.x & 31, j0 = a.J2_off[t], nj = a.J2_off[t + 1] - j0, jbase = a.J_off[t];
+    const f2 x = dup(px), y = dup(py), z = dup(pz);
+    Top2 P;
+    P.init();
+    for (int k = lane; k < nj; k += 32) {
+        const ulonglong2 X = *(const ulonglong2*)&a.modX[j0 + k], Z = *(const ulonglong2*)&a.modZ[j0 + k],
+                         W = *(const ulonglong2*)&a.modW[j0 + k];
+        const f2 v = pair_v2(x, y, z, X.x, X.y, *(const f2*)&a.modY[j0 + k], Z.x, Z.y, W.x, W.y,
+                             *(const f2*)&a.Gc[2 * (size_t)(j0 + k)]);
+        P.add(lo(v), jbase + 2 * k, a.mod_perm);
+        P.add(hi(v), jbase + 2 * k + 1, a.mod_perm);  // padding slots have -3e38 and never win
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        Top2 Q;
+        Q.m = __shfl_xor_sync(0xffffffffu, P.m, o);
+        Q.s = __shfl_xor_sync(0xffffffffu, P.s, o);
+        Q.b1 = __shfl_xor_sync(0xffffffffu, P.b1, o);
+        Q.b2 = __shfl_xor_sync(0xffffffffu, P.b2, o);
+        Q.arg = __shfl_xor_sync(0xffffffffu, P.arg, o);
+        P.merge(Q, a.mod_perm);
+    }
+    return P;
+}
+
+// Log-sum-exp of one model spot's column over its whole block, by the warp together.
+__device__ __noinline__ Lse2 whole_col(const SkArgs& a, int t, int q, int odd) {
+    const int lane = threadIdx.x & 31, i0 = a.I2_off[t], ni = a.I2_off[t + 1] - i0;
+    ColPair C;
+    load_col_pair(a, q, C);
+    Lse2 L;
+    L.m = kNegHuge;
+    L.s = 0.0f;
+    for (int k = lane; k < ni; k += 32) {
+        const ulonglong2 X = *(const ulonglong2*)&a.obsX[i0 + k];
+        const f2 pz = *(const f2*)&a.obsY[i0 + k], F = *(const f2*)&a.Fc[2 * (size_t)(i0 + k)];
+        const f2 v = odd ? pair_v2(X.x, X.y, pz, C.ncxb, C.ncyb, C.nczb, C.nrxb, C.nryb, C.nrzb, C.kb, F)
+                         : pair_v2(X.x, X.y, pz, C.ncxa, C.ncya, C.ncza, C.nrxa, C.nrya, C.nrza, C.ka, F);
+        L.merge(lo(v), 1.0f);
+        L.merge(hi(v), 1.0f);
+    }
+    warp_lse_reduce(L.m, L.s);
+    return L;
+}
+
+// Padding entries of a list (their cost is 3e38; a spot that is not a number stays an entry).
+__device__ __forceinline__ bool is_entry(float e2) { return !(e2 > 2.0e38f); }
+
+template <int TILE>
+__global__ void __launch_bounds__(kPassThreads, 2) sk_harvest_row_kernel(SkArgs a, int n_iter, int per_cta) {
+    extern __shared__ __align__(128) char pass_smem[];
+    PassShared<TILE>& H = *(PassShared<TILE>*)pass_smem;
+    DustPtrs D = dust_ptrs(a.dust, a.T);
+    const Slice sl = slice_of<TILE>(a.row_tiles, a.ctrl[CTRL_N_ROW_TILES], per_cta);
+    const int t = sl.t, lane = sl.lane;
+    float my_err = 0.0f;
+    if (sl.n_own > 0) {
+        WarpStage& S = H.stage[threadIdx.x >> 5];
+        const int lrow = 2 * (sl.q - a.I2_off[t]);
+        const bool vb = sl.valid && lrow + 1 < a.I_off[t + 1] - a.I_off[t];
+        const int jbase = a.J_off[t], j0 = a.J2_off[t];
+        const float dustv = a.mode == 2 ? kNegHuge : D.G0[a.mode ? t : 0] - a.kc;
+        Top2 A, B;
+        A.init();
+        B.init();
+        const RowPair R = load_row_pair(a, sl.q, sl.valid);
+        auto sweep_all = [&](int skip) {
+            for_each_swept<true>(a, S, sl, skip, [&](int st, int j, float2 P, int k) {
+                f2 va, vv;
+                row_pair_v(R, S, st, j, pk(P.x, P.y), va, vv);
+                const int at = jbase + 2 * k;
+                if (!sl.valid) return;
+                A.add(lo(va), at, a.mod_perm);
+                A.add(hi(va), at + 1, a.mod_perm);  // padding slots have -3e38 and never win
+                B.add(lo(vv), at, a.mod_perm);
+                B.add(hi(vv), at + 1, a.mod_perm);
+            });
+        };
+        ListHead h = list_head(a, a.row_hdr, a.row_tab, sl.id, lane);
+        if (h.nch >= 0) {
+            const float* pot = a.Gc + 2 * j0;
+            for_each_half(a, h, a.row_tab, sl.id, lane, [&](const Entries& E) {
+#pragma unroll
+                for (int k = 0; k < kHalf; ++k) {
+                    const int ja = E.slot[k] & 0xffffu, jb = E.slot[k] >> 16;
+                    float ka = a.negKD2, kb = a.negKD2;
+                    if (!a.uniK) {
+                        ka = ((const float*)&a.modW[j0 + (ja >> 1)])[2 + (ja & 1)];
+                        kb = ((const float*)&a.modW[j0 + (jb >> 1)])[2 + (jb & 1)];
+                    }
+                    if (is_entry(E.e2[k].x)) A.add(fmaf(E.e2[k].x, ka, pot[ja]), jbase + ja, a.mod_perm);
+                    if (is_entry(E.e2[k].y)) B.add(fmaf(E.e2[k].y, kb, pot[jb]), jbase + jb, a.mod_perm);
+                }
+            });
+        } else {
+            sweep_all(a.skip);
+        }
+        const float far = final_col_max(a, D, t, n_iter) - kListLog2 + kFarLog2;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            unsigned low = __ballot_sync(0xffffffffu, e ? vb && !(fmaxf(B.b1, dustv) >= far)
+                                                        : sl.valid && !(fmaxf(A.b1, dustv) >= far));
+            for (; low; low &= low - 1) {
+                const int l = __ffs(low) - 1;
+                const Top2 P = whole_row(a, t, __shfl_sync(0xffffffffu, e ? lo(R.pxb) : lo(R.pxa), l),
+                                         __shfl_sync(0xffffffffu, e ? lo(R.pyb) : lo(R.pya), l),
+                                         __shfl_sync(0xffffffffu, e ? lo(R.pzb) : lo(R.pza), l));
+                if (lane == l) (e ? B : A) = P;
+            }
+        }
+        if (sl.valid) {
+            int i = a.I_off[t] + lrow;
+            const float2 Fp = *(const float2*)&a.Fc[2 * (size_t)sl.q];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if (e == 1 && !vb) break;
+                Top2& P = e ? B : A;
+                float F = e ? Fp.y : Fp.x;
+                if (dustv > P.b1) {  // outlier column last, only when strictly larger
+                    P.b2 = P.b1;
+                    P.b1 = dustv;
+                    P.arg = -1;
+                } else if (dustv > P.b2) {
+                    P.b2 = dustv;
+                }
+                Lse2 L;
+                L.m = P.m;
+                L.s = P.s;
+                L.merge(dustv, 1.0f);
+                float rs = ex2(F + L.value());
+                my_err = fmaxf(my_err, fabsf(rs - 1.0f));
+                // unbalanced plan: a spot that keeps most of its mass is an outlier
+                if (a.mode == 2 && !(rs >= 0.5f)) P.arg = -1;
+                int ic = a.obs_perm[i + e];  // the caller's index of this observed spot
+                if (a.assign) a.assign[ic] = P.arg >= 0 ? a.mod_perm[P.arg] : -1;
+                if (a.margin) a.margin[ic] = ex2(F + P.b1) - (P.b2 > kNegHuge ? ex2(F + P.b2) : 0.0f);
+            }
+        }
+    }
+    block_err(my_err, H.sm, (int*)(D.err + 2));
+    if (!last_block(a.ctrl + CTRL_HRV_DONE, &H.last)) return;
+    if (threadIdx.x == 0) {
+        float err = __int_as_float(__ldcg((const int*)(D.err + 2)));
+        int nd = a.mode == 2 ? 0 : (a.mode ? a.T : 1);
+        for (int d = 0; d < nd; ++d) {
+            if (D.log2U[d] > kNegHuge) err = fmaxf(err, fabsf(ex2(D.F0[d] - D.F0n[d]) - 1.0f));
+        }
+        D.err[0] = err;
+        a.ctrl[CTRL_HRV_DONE] = 0;
+    }
+}
+
+// Column mass q_j = sum_i Q_ij over observed rows and the column-marginal
+// error with the final potentials, in base 2 with a running maximum.  Pairs
+// are left out, and columns read again, as for the rows.
+template <int TILE>
+__global__ void __launch_bounds__(kPassThreads, 2) sk_harvest_col_kernel(SkArgs a, int n_iter, int per_cta) {
+    extern __shared__ __align__(128) char pass_smem[];
+    PassShared<TILE>& H = *(PassShared<TILE>*)pass_smem;
+    DustPtrs D = dust_ptrs(a.dust, a.T);
+    const Slice sl = slice_of<TILE>(a.col_tiles, a.ctrl[CTRL_N_COL_TILES], per_cta);
+    const int t = sl.t, lane = sl.lane;
+    float my_err = 0.0f;
+    if (sl.n_own > 0) {
+        WarpStage& S = H.stage[threadIdx.x >> 5];
+        const int lcol = 2 * (sl.q - a.J2_off[t]);
+        const bool vb = sl.valid && lcol + 1 < a.J_off[t + 1] - a.J_off[t];
+        const int i0 = a.I2_off[t];
+        const float F0 = a.mode == 2 ? kNegHuge : D.F0[a.mode ? t : 0];
+        Lse2 A, B;
+        A.m = B.m = kNegHuge;
+        A.s = B.s = 0.0f;
+        auto add = [](Lse2& L, float v) {
+            if (v > L.m) {
+                L.s = L.s * ex2(L.m - v) + 1.0f;
+                L.m = v;
+            } else {
+                L.s += ex2(v - L.m);
+            }
+        };
+        ColPair C;
+        load_col_pair(a, sl.valid ? sl.q : sl.q - lane, C);
+        auto sweep_all = [&](int skip) {
+            for_each_swept<false>(a, S, sl, skip, [&](int st, int j, float2 P, int) {
+                f2 va, vv;
+                col_pair_v(C, S, st, j, pk(P.x, P.y), va, vv);
+                add(A, lo(va));
+                add(A, hi(va));
+                add(B, lo(vv));
+                add(B, hi(vv));
+            });
+        };
+        ListHead h = list_head(a, a.col_hdr, a.col_tab, sl.id, lane);
+        if (h.nch >= 0) {
+            const float* pot = a.Fc + 2 * i0;
+            const float ka = lo(C.ka), kb = lo(C.kb);
+            for_each_half(a, h, a.col_tab, sl.id, lane, [&](const Entries& E) {
+#pragma unroll
+                for (int k = 0; k < kHalf; ++k) {
+                    if (is_entry(E.e2[k].x)) add(A, fmaf(E.e2[k].x, ka, pot[E.slot[k] & 0xffffu]));
+                    if (is_entry(E.e2[k].y)) add(B, fmaf(E.e2[k].y, kb, pot[E.slot[k] >> 16]));
+                }
+            });
+        } else {
+            sweep_all(a.skip);
+        }
+        const float far = final_row_max(a, D, t, n_iter) - kListLog2 + kFarLog2;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            unsigned low = __ballot_sync(0xffffffffu, e ? vb && !(B.m >= far) : sl.valid && !(A.m >= far));
+            for (; low; low &= low - 1) {
+                const int l = __ffs(low) - 1;
+                const Lse2 P = whole_col(a, t, sl.q - lane + l, e);
+                if (lane == l) (e ? B : A) = P;
+            }
+        }
+        if (sl.valid) {
+            const float2 Gp = *(const float2*)&a.Gc[2 * (size_t)sl.q];
+            for (int e = 0; e < 2; ++e) {
+                if (e == 1 && !vb) break;
+                const Lse2& L = e ? B : A;
+                const float G = e ? Gp.y : Gp.x;
+                const float qj = L.s > 0.0f ? ex2(G + L.m + lg2(L.s)) : 0.0f;
+                if (a.q) a.q[a.mod_perm[a.J_off[t] + lcol + e]] = qj;
+                my_err = fmaxf(my_err, fabsf(qj + ex2(G + F0) - 1.0f));
+            }
+        }
+    }
+    block_err(my_err, H.sm, (int*)(D.err + 3));
+    if (!last_block(a.ctrl + CTRL_HCOL_DONE, &H.last)) return;
+    if (threadIdx.x == 0) {
+        D.err[1] = __int_as_float(__ldcg((const int*)(D.err + 3)));
+        a.ctrl[CTRL_HCOL_DONE] = 0;
+    }
+}
+
+// ------------------------------------------------------------ launches
+// Launch shapes of the pair passes the autotuner chooses from: the pairs of a
+// tile.  (Shapes 1 and 2 are the same kernels.)
+int sk_variant_threads(int v) { return v == 0 ? 256 : (v == 3 ? 64 : 128); }
+
+namespace {
+
+// Calls fn(tile width as an integral constant) for shape v.
+template <class Fn>
+cudaError_t with_tile(int v, Fn fn) {
+    if (v == 0) return fn(std::integral_constant<int, 256>{});
+    if (v == 3) return fn(std::integral_constant<int, 64>{});
+    return fn(std::integral_constant<int, 128>{});
+}
+
+template <class Kernel, class... Args>
+cudaError_t launch_pass(Kernel k, int ctas, size_t smem, bool overlap, cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(ctas);
+    c.blockDim = dim3(kPassThreads);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&c, k, args...);
+}
+
+template <int TILE>
+cudaError_t allow_smem() {
+    const int n = (int)sizeof(PassShared<TILE>);
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(sk_pass_kernel<TILE, true>, at, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_pass_kernel<TILE, false>, at, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_harvest_row_kernel<TILE>, at, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_harvest_col_kernel<TILE>, at, n);
+    return e;
+}
+
+}  // namespace
+
+// Once per device (the current one), before the first launch.
+cudaError_t sinkhorn_setup() {
+    cudaError_t e = allow_smem<64>();
+    if (e == cudaSuccess) e = allow_smem<128>();
+    if (e == cudaSuccess) e = allow_smem<256>();
+    return e;
+}
+
+cudaError_t sinkhorn_row_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s) {
+    return with_tile(l.row_variant, [&](auto tile) {
+        constexpr int t = decltype(tile)::value;
+        return launch_pass(sk_pass_kernel<t, true>, l.row_ctas, sizeof(PassShared<t>), true, s, a, it, l.row_per_cta);
+    });
+}
+
+cudaError_t sinkhorn_col_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s) {
+    return with_tile(l.col_variant, [&](auto tile) {
+        constexpr int t = decltype(tile)::value;
+        return launch_pass(sk_pass_kernel<t, false>, l.col_ctas, sizeof(PassShared<t>), true, s, a, it, l.col_per_cta);
+    });
+}
+
+cudaError_t sinkhorn_build_lists(const SkArgs& a, const SkLaunch& l, cudaStream_t s) {
+    const int rg = (l.row_slices + kListWarps - 1) / kListWarps, cg = (l.col_slices + kListWarps - 1) / kListWarps;
+    cudaError_t e = with_tile(l.row_variant, [&](auto tile) {
+        sk_list_kernel<decltype(tile)::value, true><<<rg, 32 * kListWarps, 0, s>>>(a);
+        return cudaGetLastError();
+    });
+    if (e != cudaSuccess) return e;
+    return with_tile(l.col_variant, [&](auto tile) {
+        sk_list_kernel<decltype(tile)::value, false><<<cg, 32 * kListWarps, 0, s>>>(a);
+        return cudaGetLastError();
+    });
+}
+
+cudaError_t sinkhorn_harvest(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols,
+                             cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    if (want_rows)
+        e = with_tile(l.row_variant, [&](auto tile) {
+            constexpr int t = decltype(tile)::value;
+            return launch_pass(sk_harvest_row_kernel<t>, l.row_ctas, sizeof(PassShared<t>), false, s, a, n_iter,
+                               l.row_per_cta);
+        });
+    if (e == cudaSuccess && want_cols)
+        e = with_tile(l.col_variant, [&](auto tile) {
+            constexpr int t = decltype(tile)::value;
+            return launch_pass(sk_harvest_col_kernel<t>, l.col_ctas, sizeof(PassShared<t>), false, s, a, n_iter,
+                               l.col_per_cta);
+        });
+    return e;
+}
+
+}  // namespace laue

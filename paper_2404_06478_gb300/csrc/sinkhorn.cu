@@ -109,6 +109,8 @@ __global__ void __launch_bounds__(1024) sk_schedule_kernel(SkArgs a) {
         a.ctrl[CTRL_N_COL_TILES] = nc;
         for (int k = CTRL_ROW_NEXT; k <= CTRL_GEN_DONE; ++k)
             if (k != CTRL_N_ROW_TILES && k != CTRL_N_COL_TILES && k != CTRL_FWD_TOTAL) a.ctrl[k] = 0;
+        a.ctrl[CTRL_POOL_NEXT] = 0;
+        for (int k = CTRL_ROW_EVAL; k < CTRL_COL_EVAL + 2; ++k) a.ctrl[k] = 0;
     }
     __syncthreads();
     for (int t = threadIdx.x; t < T; t += blockDim.x) {
@@ -126,6 +128,7 @@ __global__ void __launch_bounds__(1024) sk_schedule_kernel(SkArgs a) {
                 a.col_tiles[idx] = make_int4(t, j0 + k * a.tile_cols, min(a.tile_cols, nj - k * a.tile_cols), 0);
         }
     }
+    for (int u = threadIdx.x; u < 4 * T; u += blockDim.x) a.pmax[u] = 0u;
     // dustbin masses (paper: T_a = T_b - b^T 1 + a^T 1), in double precision
     DustPtrs D = dust_ptrs(a.dust, T);
     int nd = a.mode ? T : 1;
@@ -282,12 +285,12 @@ __global__ void __launch_bounds__(256) sk_cone_kernel(SkArgs a) {
     const int nspots = off[t + 1] - off[t];
     const int l0 = 2 * kGran * (g - gb[t]);            // first spot rank of the granule
     const int l1 = min(nspots, l0 + 2 * kGran);
-    float d[2 * kGran / 32][3];
+    float d[2 * kGran / 32][3], dx[2 * kGran / 32];
     float sx = 0.f, sy = 0.f, sz = 0.f, ext = mod ? 0.0f : 3.0e38f;
-    int cntv = 0;
     for (int k = 0; k < 2 * kGran / 32; ++k) {
         int l = l0 + lane + 32 * k;
         d[k][0] = d[k][1] = d[k][2] = 0.0f;
+        dx[k] = mod ? 0.0f : 3.0e38f;
         if (l >= l1) continue;
         int q = poff[t] + (l >> 1), ln = l & 1;
         float x, y, z;
@@ -297,13 +300,15 @@ __global__ void __launch_bounds__(256) sk_cone_kernel(SkArgs a) {
             y = -(ln ? Z.w : Z.z);
             z = -(ln ? W.y : W.x);
             float cx = ln ? X.y : X.x, cy = ln ? X.w : X.z, cz = ln ? Y.y : Y.x;
-            ext = fmaxf(ext, sqrtf(cx * cx + cy * cy + cz * cz));
+            dx[k] = sqrtf(cx * cx + cy * cy + cz * cz);
+            ext = fmaxf(ext, dx[k]);
         } else {
             float4 X = a.obsX[q], Y = a.obsY[q];
             x = ln ? X.y : X.x;
             y = ln ? X.w : X.z;
             z = ln ? Y.y : Y.x;
             float r = sqrtf(x * x + y * y + z * z);
+            dx[k] = r;
             ext = fminf(ext, r);
         }
         float r = rsqrtf(fmaxf(x * x + y * y + z * z, 1e-30f));
@@ -313,7 +318,31 @@ __global__ void __launch_bounds__(256) sk_cone_kernel(SkArgs a) {
         sx += d[k][0];
         sy += d[k][1];
         sz += d[k][2];
-        ++cntv;
+    }
+    // cones of the sub-granules: 2 kSubGran = 16 spots, half a warp
+    for (int k = 0; k < 2 * kGran / 32; ++k) {
+        const bool have = l0 + lane + 32 * k < l1;
+        float mx = d[k][0], my = d[k][1], mz = d[k][2], e = dx[k];
+        for (int o = 8; o > 0; o >>= 1) {
+            mx += __shfl_xor_sync(0xffffffffu, mx, o);
+            my += __shfl_xor_sync(0xffffffffu, my, o);
+            mz += __shfl_xor_sync(0xffffffffu, mz, o);
+            float y = __shfl_xor_sync(0xffffffffu, e, o);
+            e = mod ? fmaxf(e, y) : fminf(e, y);
+        }
+        const float m2 = mx * mx + my * my + mz * mz;
+        const bool none = !(m2 > 1e-12f);  // no axis (or a spot that is not a number): no bound
+        const float r = rsqrtf(fmaxf(m2, 1e-30f));
+        mx = none ? 0.0f : mx * r;
+        my = none ? 0.0f : my * r;
+        mz = none ? 1.0f : mz * r;
+        float beta = have ? angle_between(mx, my, mz, d[k][0], d[k][1], d[k][2]) : 0.0f;
+        for (int o = 8; o > 0; o >>= 1) beta = fmaxf(beta, __shfl_xor_sync(0xffffffffu, beta, o));
+        const int sub = 2 * k + (lane >> 4);
+        if ((lane & 15) == 0) {
+            (mod ? a.mod_sub : a.obs_sub)[kSubs * (size_t)g + sub] = make_float4(mx, my, mz, none ? 3.2f : beta + 1e-5f);
+            (mod ? a.mod_subext : a.obs_subext)[kSubs * (size_t)g + sub] = e;
+        }
     }
     for (int o = 16; o > 0; o >>= 1) {
         sx += __shfl_xor_sync(0xffffffffu, sx, o);
@@ -363,12 +392,15 @@ __global__ void sk_pack_kernel(SkArgs a) {
         X[lane] = p.x;
         X[2 + lane] = p.y;
         Y[lane] = p.z;
-        Y[2 + lane] = a.warm ? a.f[k] * s : 0.0f;
+        const float F = a.warm ? a.f[k] * s : 0.0f;
+        Y[2 + lane] = F;
+        a.Fc[2 * q + lane] = F;
         if (lane == 0 && l + 1 == a.I_off[t + 1] - a.I_off[t]) {
             X[1] = 0.0f;
             X[3] = 0.0f;
             Y[1] = kPadFar;
             Y[3] = kNegHuge;
+            a.Fc[2 * q + 1] = kNegHuge;
         }
     }
     if (k < a.n_model) {
@@ -384,7 +416,9 @@ __global__ void sk_pack_kernel(SkArgs a) {
         X[lane] = -c.x;
         X[2 + lane] = -c.y;
         Y[lane] = -c.z;
-        Y[2 + lane] = a.warm ? a.g[k] * s : 0.0f;
+        const float G = a.warm ? a.g[k] * s : 0.0f;
+        Y[2 + lane] = G;
+        a.Gc[2 * q + lane] = G;
         Z[lane] = -r.x;
         Z[2 + lane] = -r.y;
         W[lane] = -r.z;
@@ -395,6 +429,7 @@ __global__ void sk_pack_kernel(SkArgs a) {
             X[3] = 0.0f;
             Y[1] = 0.0f;
             Y[3] = kNegHuge;
+            a.Gc[2 * q + 1] = kNegHuge;
             Z[1] = 0.0f;
             Z[3] = 0.0f;
             W[1] = -1.0f;
@@ -448,545 +483,6 @@ __global__ void __launch_bounds__(1024) sk_init_dust_kernel(SkArgs a) {
     }
 }
 
-// Row pair (two observed spots) against the staged model pairs of one chunk.
-struct RowPair {
-    f2 pxa, pya, pza, pxb, pyb, pzb;
-    RowLse A, B;
-};
-
-__device__ __forceinline__ void col_chunk(ColPair& C, const float4* __restrict__ sX, const float4* __restrict__ sY,
-                                          int n) {
-    int k = 0;
-    for (; k + kGroup <= n; k += kGroup) {
-        f2 va[kGroup], vb[kGroup];
-#pragma unroll
-        for (int g = 0; g < kGroup; ++g) {
-            ulonglong2 X = *(const ulonglong2*)&sX[k + g];
-            ulonglong2 Y = *(const ulonglong2*)&sY[k + g];
-            va[g] = pair_v2(X.x, X.y, Y.x, C.ncxa, C.ncya, C.ncza, C.nrxa, C.nrya, C.nrza, C.ka, Y.y);
-            vb[g] = pair_v2(X.x, X.y, Y.x, C.ncxb, C.ncyb, C.nczb, C.nrxb, C.nryb, C.nrzb, C.kb, Y.y);
-        }
-        C.A.add4(va);
-        C.B.add4(vb);
-    }
-    for (; k < n; ++k) {
-        ulonglong2 X = *(const ulonglong2*)&sX[k];
-        ulonglong2 Y = *(const ulonglong2*)&sY[k];
-        C.A.add1(pair_v2(X.x, X.y, Y.x, C.ncxa, C.ncya, C.ncza, C.nrxa, C.nrya, C.nrza, C.ka, Y.y));
-        C.B.add1(pair_v2(X.x, X.y, Y.x, C.ncxb, C.ncyb, C.nczb, C.nrxb, C.nryb, C.nrzb, C.kb, Y.y));
-    }
-}
-
-// Fast path of the passes: the staged potentials are shifted by the block's
-// maximum (prep step), so every exponent is <= 0 and the sums need no running
-// maximum: per staged pair, 2 x 13 packed instructions, 4 MUFU ex2 and 2
-// packed adds for 4 pair evaluations.
-__device__ __forceinline__ void row_chunk_sum(const RowPair& R, const float4* __restrict__ sX,
-                                              const float4* __restrict__ sY, const float4* __restrict__ sZ,
-                                              const float4* __restrict__ sW, int n, f2& Sa, f2& Sb) {
-#pragma unroll 4
-    for (int k = 0; k < n; ++k) {
-        ulonglong2 X = *(const ulonglong2*)&sX[k];
-        ulonglong2 Y = *(const ulonglong2*)&sY[k];
-        ulonglong2 Z = *(const ulonglong2*)&sZ[k];
-        ulonglong2 W = *(const ulonglong2*)&sW[k];
-        f2 va = pair_v2(R.pxa, R.pya, R.pza, X.x, X.y, Y.x, Z.x, Z.y, W.x, W.y, Y.y);
-        f2 vb = pair_v2(R.pxb, R.pyb, R.pzb, X.x, X.y, Y.x, Z.x, Z.y, W.x, W.y, Y.y);
-        Sa = add2(Sa, pk(ex2(lo(va)), ex2(hi(va))));
-        Sb = add2(Sb, pk(ex2(lo(vb)), ex2(hi(vb))));
-    }
-}
-
-__device__ __forceinline__ void col_chunk_sum(const ColPair& C, const float4* __restrict__ sX,
-                                              const float4* __restrict__ sY, int n, f2& Sa, f2& Sb) {
-#pragma unroll 4
-    for (int k = 0; k < n; ++k) {
-        ulonglong2 X = *(const ulonglong2*)&sX[k];
-        ulonglong2 Y = *(const ulonglong2*)&sY[k];
-        f2 va = pair_v2(X.x, X.y, Y.x, C.ncxa, C.ncya, C.ncza, C.nrxa, C.nrya, C.nrza, C.ka, Y.y);
-        f2 vb = pair_v2(X.x, X.y, Y.x, C.ncxb, C.ncyb, C.nczb, C.nrxb, C.nryb, C.nrzb, C.kb, Y.y);
-        Sa = add2(Sa, pk(ex2(lo(va)), ex2(hi(va))));
-        Sb = add2(Sb, pk(ex2(lo(vb)), ex2(hi(vb))));
-    }
-}
-
-constexpr float kTinySum = 1.0e-30f;  // below ~2^-100 the fast sum is recomputed exactly
-
-// Exact row log-sum-exp from global memory (running maximum), for rows whose
-// shifted sum underflowed.
-__device__ float row_exact(const SkArgs& a, int t, f2 px, f2 py, f2 pz, float dustv) {
-    atomicAdd((unsigned*)a.ctrl + CTRL_EXACT_ROWS, 1u);
-    RowLse L;
-    L.init(dustv);
-    for (int q = a.J2_off[t]; q < a.J2_off[t + 1]; ++q) {
-        float4 x = a.modX[q], y = a.modY[q], z = a.modZ[q], w = a.modW[q];
-        L.add1(pair_v2(px, py, pz, pk(x.x, x.y), pk(x.z, x.w), pk(y.x, y.y), pk(z.x, z.y), pk(z.z, z.w),
-                       pk(w.x, w.y), pk(w.z, w.w), pk(y.z, y.w)));
-    }
-    return L.value();
-}
-
-__device__ float col_exact(const SkArgs& a, int t, f2 ncx, f2 ncy, f2 ncz, f2 nrx, f2 nry, f2 nrz, float dz, f2 K2) {
-    atomicAdd((unsigned*)a.ctrl + CTRL_EXACT_COLS, 1u);
-    RowLse L;
-    L.init(dz);
-    for (int q = a.I2_off[t]; q < a.I2_off[t + 1]; ++q) {
-        float4 x = a.obsX[q], y = a.obsY[q];
-        L.add1(pair_v2(pk(x.x, x.y), pk(x.z, x.w), pk(y.x, y.y), ncx, ncy, ncz, nrx, nry, nrz, K2, pk(y.z, y.w)));
-    }
-    return L.value();
-}
-
-// Per-angle maximum of the potentials written by a pass, from the per-tile
-// partial log-sum-exps (their running maxima).
-__device__ void block_maxima(const float2* part, const int4* ang, int T, bool rows, float add, float* out) {
-    for (int t = threadIdx.x; t < T; t += blockDim.x) {
-        int4 at = ang[t];
-        int first = rows ? at.x : at.z, cnt = rows ? at.y : at.w;
-        float m = kNegHuge;
-        for (int k = 0; k < cnt; ++k) m = fmaxf(m, part[first + k].x);
-        out[t] = m > kNegHuge ? m + add : kNegHuge;
-    }
-}
-
-// --------------------------------------------------------------- row pass
-template <int TPB, int MINB>
-__global__ void __launch_bounds__(TPB, MINB) sk_row_kernel(SkArgs a) {
-    __shared__ __align__(128) Stage S;
-    init_stage(S);
-    uint32_t parity[2] = {0u, 0u};
-    DustPtrs D = dust_ptrs(a.dust, a.T);
-    const int n_tiles = a.ctrl[CTRL_N_ROW_TILES];
-    const Srcs src{{a.modX, a.modY, a.modZ, a.modW}, 4};
-    while (true) {
-        int tile = next_tile(S, a.ctrl + CTRL_ROW_NEXT, n_tiles);
-        if (tile < 0) break;
-        int4 td = a.row_tiles[tile];
-        int t = td.x;
-        int q = td.y + threadIdx.x;
-        bool valid = (int)threadIdx.x < td.z;
-        int ni = a.I_off[t + 1] - a.I_off[t];
-        bool vb = valid && 2 * (q - a.I2_off[t]) + 1 < ni;
-        int j0 = a.J2_off[t], nj = a.J2_off[t + 1] - j0;
-        const bool ub = a.mode == 2;  // unbalanced OT: no dustbins, scaled update
-        float dustv = ub ? kNegHuge : D.G0[a.mode ? t : 0] - a.kc;
-        float4 X = valid ? a.obsX[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 Y = valid ? a.obsY[q] : make_float4(0.f, 0.f, kPadFar, kPadFar);
-        RowPair R;
-        R.pxa = dup(X.x);
-        R.pya = dup(X.z);
-        R.pza = dup(Y.x);
-        R.pxb = dup(X.y);
-        R.pyb = dup(X.w);
-        R.pzb = dup(Y.y);
-        const float shift = ub ? D.Gmax[t] : fmaxf(D.Gmax[t], dustv);
-        f2 Sa = pk(ub ? 0.0f : ex2(dustv - shift), 0.0f), Sb = Sa;
-        auto prep = [&](int st, int n) {
-            for (int k = threadIdx.x; k < n; k += TPB) {
-                float4& y = S.s[1][st][k];
-                y.z -= shift;
-                y.w -= shift;
-            }
-        };
-        // the granules of a staged chunk selected by mask
-        auto body = [&](int st, int n, int, int mask = (1 << kParts) - 1) {
-            if (!valid) return;
-            for_each_run(mask, n, [&](int h, int m) {
-                row_chunk_sum(R, S.s[0][st] + h, S.s[1][st] + h, S.s[2][st] + h, S.s[3][st] + h, m, Sa, Sb);
-            });
-        };
-        // the model granules this tile of observed spots can see (exact underflow skipping)
-        const int nch = (nj + kChunk - 1) / kChunk;
-        const bool use_list = a.skip && nch > 0 && nch <= kMaxList;
-        int n_list = nch;
-        if (use_list) {
-            const Cone O = tile_cone(a.obs_cone, a.obs_ext, a.obs_gbase[t], a.I2_off[t], td.y, td.z, true);
-            const float K = a.skipK;  // the smallest cost factor of any spot
-            const int mg = a.mod_gbase[t], ng = (nj + kGran - 1) / kGran;
-            n_list = build_chunk_list(S, nch, [&](int c) {
-                int m = 0;
-                for (int hh = 0; hh < kParts; ++hh)
-                    if (kParts * c + hh < ng &&
-                        min_scaled_cost(O, load_cone(a.mod_cone, a.mod_ext, mg + kParts * c + hh), K) <= kSkipLog2)
-                        m |= 1 << hh;
-                return m;
-            });
-        }
-        bool ok = use_list ? stream_list_prep(S, parity, src, j0, nj, n_list, prep, body)
-                           : stream_tile_prep(S, parity, src, j0, nj, prep, body);
-        if (threadIdx.x == 0) {
-            long long np = 0;
-            if (use_list)
-                for (int c = 0; c < n_list; ++c) np += list_pairs(S.list[c] & 0xffffff, (int)((unsigned)S.list[c] >> 24), nj);
-            else
-                np = nj;
-            atomicAdd((unsigned long long*)(a.ctrl + CTRL_SK_PAIRS), (unsigned long long)(4LL * td.z * np));
-        }
-        if (!ok) {
-            if (threadIdx.x == 0) set_status(a.ctrl, LAUE_ERR_TIMEOUT);
-            break;
-        }
-        float sa = lo(Sa) + hi(Sa), sb = lo(Sb) + hi(Sb);
-        float Fa = valid ? (sa > kTinySum ? -(shift + lg2(sa)) : -row_exact(a, t, R.pxa, R.pya, R.pza, dustv)) : 0.0f;
-        float Fb = vb ? (sb > kTinySum ? -(shift + lg2(sb)) : -row_exact(a, t, R.pxb, R.pyb, R.pzb, dustv)) : 0.0f;
-        if (ub) {  // Algorithm UnbalancedOT: the balanced update raised to kappa / (kappa + eps)
-            Fa = nj > 0 ? a.tau_row * Fa : 0.0f;
-            Fb = nj > 0 ? a.tau_row * Fb : 0.0f;
-        }
-        if (valid) *(float2*)&a.obsY[q].z = make_float2(Fa, vb ? Fb : kNegHuge);
-        // tile partial of LSE2(F_i - kc) for the outlier column update
-        float pm = kNegHuge, ps = 0.0f;
-        if (valid) {
-            pm = Fa - a.kc;
-            ps = 1.0f;
-            if (vb) lse_merge_into(pm, ps, Fb - a.kc, 1.0f);
-        }
-        block_lse(S, pm, ps);
-        if (threadIdx.x == 0) a.row_part[tile] = make_float2(pm, ps);
-    }
-    if (!last_cta(S, a.ctrl + CTRL_ROW_DONE)) return;
-    // finalise: promote F_0 and compute G_0 from the new F
-    if (a.mode == 2) {
-        // no dustbins
-    } else if (a.mode) {
-        for (int t = threadIdx.x; t < a.T; t += blockDim.x) {
-            D.F0[t] = D.F0n[t];
-            int4 at = a.ang_tiles[t];
-            Lse2 L;
-            L.init(D.F0[t] - a.kc);
-            for (int k = 0; k < at.y; ++k) {
-                float2 pp = a.row_part[at.x + k];
-                L.merge(pp.x, pp.y);
-            }
-            D.G0[t] = D.log2O[t] - L.value();
-        }
-    } else {
-        float m = kNegHuge, s = 0.0f;
-        for (int k = threadIdx.x; k < n_tiles; k += blockDim.x) {
-            float2 pp = a.row_part[k];
-            lse_merge_into(m, s, pp.x, pp.y);
-        }
-        block_lse(S, m, s);
-        if (threadIdx.x == 0) {
-            D.F0[0] = D.F0n[0];
-            Lse2 L;
-            L.init(D.F0[0] - a.kc);
-            L.merge(m, s);
-            D.G0[0] = D.log2O[0] - L.value();
-        }
-    }
-    block_maxima(a.row_part, a.ang_tiles, a.T, true, a.kc, D.Fmax);
-    if (threadIdx.x == 0) {
-        a.ctrl[CTRL_ROW_NEXT] = 0;
-        a.ctrl[CTRL_ROW_DONE] = 0;
-    }
-}
-
-// ------------------------------------------------------------ column pass
-template <int TPB, int MINB>
-__global__ void __launch_bounds__(TPB, MINB) sk_col_kernel(SkArgs a) {
-    __shared__ __align__(128) Stage S;
-    init_stage(S);
-    uint32_t parity[2] = {0u, 0u};
-    DustPtrs D = dust_ptrs(a.dust, a.T);
-    const int n_tiles = a.ctrl[CTRL_N_COL_TILES];
-    const Srcs src{{a.obsX, a.obsY, nullptr, nullptr}, 2};
-    while (true) {
-        int tile = next_tile(S, a.ctrl + CTRL_COL_NEXT, n_tiles);
-        if (tile < 0) break;
-        int4 td = a.col_tiles[tile];
-        int t = td.x;
-        int q = td.y + threadIdx.x;
-        bool valid = (int)threadIdx.x < td.z;
-        int nj = a.J_off[t + 1] - a.J_off[t];
-        bool vb = valid && 2 * (q - a.J2_off[t]) + 1 < nj;
-        int i0 = a.I2_off[t], ni = a.I2_off[t + 1] - i0;
-        ColPair C;
-        if (valid) load_col_pair(a, q, C);
-        const bool ub = a.mode == 2;
-        float dz = ub ? kNegHuge : D.F0[a.mode ? t : 0];  // unmatched-model row, C_0j = 0
-        const float shift = ub ? D.Fmax[t] : fmaxf(D.Fmax[t], dz);
-        f2 Sa = pk(ub ? 0.0f : ex2(dz - shift), 0.0f), Sb = Sa;
-        auto prep = [&](int st, int n) {
-            for (int k = threadIdx.x; k < n; k += TPB) {
-                float4& y = S.s[1][st][k];
-                y.z -= shift;
-                y.w -= shift;
-            }
-        };
-        auto body = [&](int st, int n, int, int mask = (1 << kParts) - 1) {
-            if (!valid) return;
-            for_each_run(mask, n, [&](int h, int m) { col_chunk_sum(C, S.s[0][st] + h, S.s[1][st] + h, m, Sa, Sb); });
-        };
-        // the observed granules this tile of model spots can see (exact underflow skipping)
-        const int nch = (ni + kChunk - 1) / kChunk;
-        const bool use_list = a.skip && nch > 0 && nch <= kMaxList;
-        int n_list = nch;
-        if (use_list) {
-            const Cone M = tile_cone(a.mod_cone, a.mod_ext, a.mod_gbase[t], a.J2_off[t], td.y, td.z, false);
-            const float K = a.skipK;  // the smallest cost factor of any spot
-            const int og = a.obs_gbase[t], ng = (ni + kGran - 1) / kGran;
-            n_list = build_chunk_list(S, nch, [&](int c) {
-                int m = 0;
-                for (int hh = 0; hh < kParts; ++hh)
-                    if (kParts * c + hh < ng &&
-                        min_scaled_cost(load_cone(a.obs_cone, a.obs_ext, og + kParts * c + hh), M, K) <= kSkipLog2)
-                        m |= 1 << hh;
-                return m;
-            });
-        }
-        bool ok = use_list ? stream_list_prep(S, parity, src, i0, ni, n_list, prep, body)
-                           : stream_tile_prep(S, parity, src, i0, ni, prep, body);
-        if (threadIdx.x == 0) {
-            long long np = 0;
-            if (use_list)
-                for (int c = 0; c < n_list; ++c) np += list_pairs(S.list[c] & 0xffffff, (int)((unsigned)S.list[c] >> 24), ni);
-            else
-                np = ni;
-            atomicAdd((unsigned long long*)(a.ctrl + CTRL_SK_PAIRS), (unsigned long long)(4LL * td.z * np));
-        }
-        if (!ok) {
-            if (threadIdx.x == 0) set_status(a.ctrl, LAUE_ERR_TIMEOUT);
-            break;
-        }
-        float sa = lo(Sa) + hi(Sa), sb = lo(Sb) + hi(Sb);
-        float Ga = valid ? (sa > kTinySum ? -(shift + lg2(sa))
-                                          : -col_exact(a, t, C.ncxa, C.ncya, C.ncza, C.nrxa, C.nrya, C.nrza, dz, C.ka))
-                         : 0.0f;
-        float Gb = vb ? (sb > kTinySum ? -(shift + lg2(sb))
-                                       : -col_exact(a, t, C.ncxb, C.ncyb, C.nczb, C.nrxb, C.nryb, C.nrzb, dz, C.kb))
-                      : 0.0f;
-        if (ub) {  // raised to lambda / (lambda + eps)
-            Ga = ni > 0 ? a.tau_col * Ga : 0.0f;
-            Gb = ni > 0 ? a.tau_col * Gb : 0.0f;
-        }
-        if (valid) *(float2*)&a.modY[q].z = make_float2(Ga, vb ? Gb : kNegHuge);
-        float pm = kNegHuge, ps = 0.0f;
-        if (valid) {
-            pm = Ga;
-            ps = 1.0f;
-            if (vb) lse_merge_into(pm, ps, Gb, 1.0f);
-        }
-        block_lse(S, pm, ps);
-        if (threadIdx.x == 0) a.col_part[tile] = make_float2(pm, ps);
-    }
-    if (!last_cta(S, a.ctrl + CTRL_COL_DONE)) return;
-    // finalise: next F_0 from the new G and the current G_0
-    if (a.mode == 2) {
-        // no dustbins
-    } else if (a.mode) {
-        for (int t = threadIdx.x; t < a.T; t += blockDim.x) {
-            int4 at = a.ang_tiles[t];
-            Lse2 L;
-            L.init(D.G0[t] - a.kc);
-            for (int k = 0; k < at.w; ++k) {
-                float2 pp = a.col_part[at.z + k];
-                L.merge(pp.x, pp.y);
-            }
-            D.F0n[t] = D.log2U[t] - L.value();
-        }
-    } else {
-        float m = kNegHuge, s = 0.0f;
-        for (int k = threadIdx.x; k < n_tiles; k += blockDim.x) {
-            float2 pp = a.col_part[k];
-            lse_merge_into(m, s, pp.x, pp.y);
-        }
-        block_lse(S, m, s);
-        if (threadIdx.x == 0) {
-            Lse2 L;
-            L.init(D.G0[0] - a.kc);
-            L.merge(m, s);
-            D.F0n[0] = D.log2U[0] - L.value();
-        }
-    }
-    block_maxima(a.col_part, a.ang_tiles, a.T, false, 0.0f, D.Gmax);
-    if (threadIdx.x == 0) {
-        a.ctrl[CTRL_COL_NEXT] = 0;
-        a.ctrl[CTRL_COL_DONE] = 0;
-    }
-}
-
-// ------------------------------------------------------------ row harvest
-// Plan read-out per observed spot with the final potentials: argmax over the
-// block's model spots and the outlier column (ties to the lowest index, the
-// outlier column only when strictly larger), top1 - top2 margin in plan
-// units, and the row-marginal error.  Scalar bookkeeping; once per E-step.
-struct Top2 {
-    float m, s, b1, b2;
-    int arg;
-    __device__ __forceinline__ void init() {
-        m = kNegHuge;
-        s = 0.0f;
-        b1 = kNegHuge;
-        b2 = kNegHuge;
-        arg = -1;
-    }
-    // j: the spot's slot in the spatial order; perm maps slots to the caller's
-    // indices, and ties go to the lowest caller index
-    __device__ __forceinline__ void add(float v, int j, const int* perm) {
-        if (v > m) {
-            s = s * ex2(m - v) + 1.0f;
-            m = v;
-        } else {
-            s += ex2(v - m);
-        }
-        if (v > b1 || (v == b1 && v > kNegHuge && perm[j] < perm[arg])) {
-            b2 = b1;
-            b1 = v;
-            arg = j;
-        } else if (v > b2) {
-            b2 = v;
-        }
-    }
-};
-
-__global__ void __launch_bounds__(kTPB) sk_harvest_row_kernel(SkArgs a) {
-    __shared__ __align__(128) Stage S;
-    init_stage(S);
-    uint32_t parity[2] = {0u, 0u};
-    DustPtrs D = dust_ptrs(a.dust, a.T);
-    const int n_tiles = a.ctrl[CTRL_N_ROW_TILES];
-    const Srcs src{{a.modX, a.modY, a.modZ, a.modW}, 4};
-    float my_err = 0.0f;
-    while (true) {
-        int tile = next_tile(S, a.ctrl + CTRL_HRV_NEXT, n_tiles);
-        if (tile < 0) break;
-        int4 td = a.row_tiles[tile];
-        int t = td.x;
-        int q = td.y + threadIdx.x;
-        bool valid = (int)threadIdx.x < td.z;
-        int ni = a.I_off[t + 1] - a.I_off[t];
-        int lrow = 2 * (q - a.I2_off[t]);
-        bool vb = valid && lrow + 1 < ni;
-        int jbase = a.J_off[t], j0 = a.J2_off[t], nj = a.J2_off[t + 1] - j0;
-        float dustv = a.mode == 2 ? kNegHuge : D.G0[a.mode ? t : 0] - a.kc;
-        float4 X = valid ? a.obsX[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 Y = valid ? a.obsY[q] : make_float4(0.f, 0.f, kPadFar, kPadFar);
-        f2 pxa = dup(X.x), pya = dup(X.z), pza = dup(Y.x), pxb = dup(X.y), pyb = dup(X.w), pzb = dup(Y.y);
-        Top2 A, B;
-        A.init();
-        B.init();
-        bool ok = stream_tile(S, parity, src, j0, nj, [&](int st, int n, int off) {
-            if (!valid) return;
-            for (int k = 0; k < n; ++k) {
-                ulonglong2 Xm = *(const ulonglong2*)&S.s[0][st][k];
-                ulonglong2 Ym = *(const ulonglong2*)&S.s[1][st][k];
-                ulonglong2 Zm = *(const ulonglong2*)&S.s[2][st][k];
-                ulonglong2 Wm = *(const ulonglong2*)&S.s[3][st][k];
-                f2 va = pair_v2(pxa, pya, pza, Xm.x, Xm.y, Ym.x, Zm.x, Zm.y, Wm.x, Wm.y, Ym.y);
-                f2 vv = pair_v2(pxb, pyb, pzb, Xm.x, Xm.y, Ym.x, Zm.x, Zm.y, Wm.x, Wm.y, Ym.y);
-                int j = jbase + 2 * (off + k);
-                A.add(lo(va), j, a.mod_perm);
-                A.add(hi(va), j + 1, a.mod_perm);  // padding slots have -3e38 and never win
-                B.add(lo(vv), j, a.mod_perm);
-                B.add(hi(vv), j + 1, a.mod_perm);
-            }
-        });
-        if (!ok) {
-            if (threadIdx.x == 0) set_status(a.ctrl, LAUE_ERR_TIMEOUT);
-            break;
-        }
-        if (valid) {
-            int i = a.I_off[t] + lrow;
-            for (int lane = 0; lane < 2; ++lane) {
-                if (lane == 1 && !vb) break;
-                Top2& P = lane ? B : A;
-                float F = lane ? Y.w : Y.z;
-                if (dustv > P.b1) {  // outlier column last, only when strictly larger
-                    P.b2 = P.b1;
-                    P.b1 = dustv;
-                    P.arg = -1;
-                } else if (dustv > P.b2) {
-                    P.b2 = dustv;
-                }
-                Lse2 L;
-                L.m = P.m;
-                L.s = P.s;
-                L.merge(dustv, 1.0f);
-                float rs = ex2(F + L.value());
-                my_err = fmaxf(my_err, fabsf(rs - 1.0f));
-                // unbalanced plan: a spot that keeps most of its mass is an outlier
-                if (a.mode == 2 && !(rs >= 0.5f)) P.arg = -1;
-                int ic = a.obs_perm[i + lane];  // the caller's index of this observed spot
-                if (a.assign) a.assign[ic] = P.arg >= 0 ? a.mod_perm[P.arg] : -1;
-                if (a.margin) a.margin[ic] = ex2(F + P.b1) - (P.b2 > kNegHuge ? ex2(F + P.b2) : 0.0f);
-            }
-        }
-    }
-    float e = block_max(S, my_err);
-    if (threadIdx.x == 0) atomicMax((int*)(D.err + 2), __float_as_int(e));  // non-negative floats
-    if (!last_cta(S, a.ctrl + CTRL_HRV_DONE)) return;
-    if (threadIdx.x == 0) {
-        float err = __int_as_float(*(int*)(D.err + 2));
-        int nd = a.mode == 2 ? 0 : (a.mode ? a.T : 1);
-        for (int d = 0; d < nd; ++d) {
-            if (D.log2U[d] > kNegHuge) err = fmaxf(err, fabsf(ex2(D.F0[d] - D.F0n[d]) - 1.0f));
-        }
-        D.err[0] = err;
-        a.ctrl[CTRL_HRV_NEXT] = 0;
-        a.ctrl[CTRL_HRV_DONE] = 0;
-    }
-}
-
-// --------------------------------------------------------- column harvest
-// Column mass q_j = sum_i Q_ij over observed rows and the column-marginal
-// error with the final potentials.
-__global__ void __launch_bounds__(kTPB) sk_harvest_col_kernel(SkArgs a) {
-    __shared__ __align__(128) Stage S;
-    init_stage(S);
-    uint32_t parity[2] = {0u, 0u};
-    DustPtrs D = dust_ptrs(a.dust, a.T);
-    const int n_tiles = a.ctrl[CTRL_N_COL_TILES];
-    const Srcs src{{a.obsX, a.obsY, nullptr, nullptr}, 2};
-    float my_err = 0.0f;
-    while (true) {
-        int tile = next_tile(S, a.ctrl + CTRL_HCOL_NEXT, n_tiles);
-        if (tile < 0) break;
-        int4 td = a.col_tiles[tile];
-        int t = td.x;
-        int q = td.y + threadIdx.x;
-        bool valid = (int)threadIdx.x < td.z;
-        int nj = a.J_off[t + 1] - a.J_off[t];
-        int lcol = 2 * (q - a.J2_off[t]);
-        bool vb = valid && lcol + 1 < nj;
-        int i0 = a.I2_off[t], ni = a.I2_off[t + 1] - i0;
-        ColPair C;
-        if (valid) load_col_pair(a, q, C);
-        C.A.init(kNegHuge);
-        C.B.init(kNegHuge);
-        C.A.S = pk(0.0f, 0.0f);
-        C.B.S = pk(0.0f, 0.0f);
-        bool ok = stream_tile(S, parity, src, i0, ni, [&](int st, int n, int) {
-            if (valid) col_chunk(C, S.s[0][st], S.s[1][st], n);
-        });
-        if (!ok) {
-            if (threadIdx.x == 0) set_status(a.ctrl, LAUE_ERR_TIMEOUT);
-            break;
-        }
-        if (valid) {
-            float4 Ym = a.modY[q];
-            float F0 = a.mode == 2 ? kNegHuge : D.F0[a.mode ? t : 0];
-            for (int lane = 0; lane < 2; ++lane) {
-                if (lane == 1 && !vb) break;
-                RowLse& L = lane ? C.B : C.A;
-                float G = lane ? Ym.w : Ym.z;
-                float ssum = lo(L.S) + hi(L.S);
-                float qj = ssum > 0.0f ? ex2(G + L.m + lg2(ssum)) : 0.0f;
-                if (a.q) a.q[a.mod_perm[a.J_off[t] + lcol + lane]] = qj;
-                my_err = fmaxf(my_err, fabsf(qj + ex2(G + F0) - 1.0f));
-            }
-        }
-    }
-    float e = block_max(S, my_err);
-    if (threadIdx.x == 0) atomicMax((int*)(D.err + 3), __float_as_int(e));
-    if (!last_cta(S, a.ctrl + CTRL_HCOL_DONE)) return;
-    if (threadIdx.x == 0) {
-        D.err[1] = __int_as_float(*(int*)(D.err + 3));
-        a.ctrl[CTRL_HCOL_NEXT] = 0;
-        a.ctrl[CTRL_HCOL_DONE] = 0;
-    }
-}
-
 // ---------------------------------------------------------------- finish
 __global__ void sk_finish_kernel(SkArgs a, int have_rows, int have_cols) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -994,14 +490,14 @@ __global__ void sk_finish_kernel(SkArgs a, int have_rows, int have_cols) {
     if (k < a.n_obs) {
         int t = block_of(a.I_off, a.T, k);
         int l = a.obs_pos[k];
-        float v = ((const float*)&a.obsY[a.I2_off[t] + (l >> 1)])[2 + (l & 1)];
+        float v = a.Fc[2 * a.I2_off[t] + l];
         bad |= !isfinite(v);
         a.f[k] = v * a.to_user;
     }
     if (k < a.n_model) {
         int t = block_of(a.J_off, a.T, k);
         int l = a.mod_pos[k];
-        float v = ((const float*)&a.modY[a.J2_off[t] + (l >> 1)])[2 + (l & 1)];
+        float v = a.Gc[2 * a.J2_off[t] + l];
         bad |= !isfinite(v);
         a.g[k] = v * a.to_user;
     }
@@ -1077,64 +573,39 @@ cudaError_t sinkhorn_prepare(const SkArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// Launch shapes of the pair passes the autotuner chooses from:
-// {threads per CTA (= pairs per tile), minimum resident CTAs per SM}.
-typedef void (*SkKernel)(SkArgs);
-static const SkKernel kRowKernels[kSkVariants] = {sk_row_kernel<256, 1>, sk_row_kernel<128, 1>, sk_row_kernel<128, 4>,
-                                                  sk_row_kernel<64, 8>};
-static const SkKernel kColKernels[kSkVariants] = {sk_col_kernel<256, 1>, sk_col_kernel<128, 1>, sk_col_kernel<128, 4>,
-                                                  sk_col_kernel<64, 8>};
-
-int sk_variant_threads(int v) { return v == 0 ? 256 : (v == 3 ? 64 : 128); }
-
-void sinkhorn_row_pass(const SkArgs& a, const SkLaunch& l, cudaStream_t s) {
-    kRowKernels[l.row_variant]<<<l.row_grid, sk_variant_threads(l.row_variant), 0, s>>>(a);
-}
-
-void sinkhorn_col_pass(const SkArgs& a, const SkLaunch& l, cudaStream_t s) {
-    kColKernels[l.col_variant]<<<l.col_grid, sk_variant_threads(l.col_variant), 0, s>>>(a);
-}
-
 cudaError_t sinkhorn_iterate(const SkArgs& a, const SkLaunch& l, int n_iter, cudaStream_t s) {
     for (int it = 0; it < n_iter; ++it) {
-        sinkhorn_row_pass(a, l, s);
-        sinkhorn_col_pass(a, l, s);
+        cudaError_t e = sinkhorn_row_pass(a, l, it, s);
+        if (e == cudaSuccess) e = sinkhorn_col_pass(a, l, it, s);
+        if (e != cudaSuccess) return e;
     }
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
-cudaError_t sinkhorn_finish(const SkArgs& a, const SkLaunch& l, bool want_rows, bool want_cols, cudaStream_t s) {
+cudaError_t sinkhorn_finish(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols,
+                            cudaStream_t s) {
     int nmax = a.n_obs > a.n_model ? a.n_obs : a.n_model;
     int blocks = (nmax + 255) / 256;
     if (blocks < 1) blocks = 1;
     if (want_rows || want_cols) sk_clear_err_kernel<<<1, 1, 0, s>>>(a);
-    // one thread per row (column) pair of the pass's tiles
-    if (want_rows) sk_harvest_row_kernel<<<l.hrv_grid, sk_variant_threads(l.row_variant), 0, s>>>(a);
-    if (want_cols) sk_harvest_col_kernel<<<l.hcol_grid, sk_variant_threads(l.col_variant), 0, s>>>(a);
+    cudaError_t e = sinkhorn_harvest(a, l, n_iter, want_rows, want_cols, s);
+    if (e != cudaSuccess) return e;
     sk_finish_kernel<<<blocks, 256, 0, s>>>(a, want_rows ? 1 : 0, want_cols ? 1 : 0);
     return cudaGetLastError();
 }
 
-cudaError_t sinkhorn_run(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols,
+cudaError_t sinkhorn_run(const SkArgs& a0, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols,
                          cudaStream_t s) {
+    SkArgs a = a0;
+    // listing the pairs costs about as much as one sweep of each side
+    if (n_iter < 2) a.pool_chunks = 0;
     cudaError_t e = sinkhorn_prepare(a, s);
+    if (e != cudaSuccess) return e;
+    e = sinkhorn_build_lists(a, l, s);
     if (e != cudaSuccess) return e;
     e = sinkhorn_iterate(a, l, n_iter, s);
     if (e != cudaSuccess) return e;
-    return sinkhorn_finish(a, l, want_rows, want_cols, s);
-}
-
-int sinkhorn_occupancy(int* row_blocks_per_sm, int* col_blocks_per_sm) {
-    for (int v = 0; v < kSkVariants; ++v) {
-        int r = 0, c = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, kRowKernels[v], sk_variant_threads(v), 0) != cudaSuccess)
-            return -1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, kColKernels[v], sk_variant_threads(v), 0) != cudaSuccess)
-            return -1;
-        row_blocks_per_sm[v] = r > 0 ? r : 1;
-        col_blocks_per_sm[v] = c > 0 ? c : 1;
-    }
-    return 0;
+    return sinkhorn_finish(a, l, n_iter, want_rows, want_cols, s);
 }
 
 }  // namespace laue

@@ -1,0 +1,105 @@
+"""The forms of the pair passes against each other: listed slices, slices left
+to the sweep for want of scratch, and every pair evaluated.
+
+All three add the same nonzero terms in the same order, so potentials,
+dustbins and read-outs are equal bit for bit; the parity with the oracle is
+checked elsewhere on the default form."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import synthgen as sg
+from _cases import GEOM, make_case, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    from paper_2404_06478_gb300 import api, build
+    build.build()
+    torch.cuda.set_device(0)
+    return dict(torch=torch, api=api, dev=torch.device("cuda", 0))
+
+
+def _blocks(sizes, seed, geom):
+    """Observed and model spots of len(sizes) angle blocks, the first m model
+    spots and about half as many noisy copies and half random ones observed."""
+    rng = np.random.default_rng(seed)
+    case = make_case(sg.CONFIGS["medium"], seed=seed, n_grains=60, T=4, geom=geom)
+    pool = case.fw
+    n = len(pool["t"])
+    ob, mod = [], []
+    for ni, nj in sizes:
+        j = rng.choice(n, nj, replace=nj > n)
+        s = pool["spot"][rng.choice(n, ni)] + rng.normal(size=(ni, 3)) * np.array([1.0, 1.0, 0.0])
+        far = rng.random(ni) < 0.3
+        s[far, :2] = rng.uniform(-128, 128, (int(far.sum()), 2))
+        ob.append(s)
+        mod.append(j)
+    j = np.concatenate(mod)
+    I_off = np.r_[0, np.cumsum([a for a, _ in sizes])]
+    J_off = np.r_[0, np.cumsum([b for _, b in sizes])]
+    return np.concatenate(ob), I_off, {k: pool[k][j] for k in ("grain", "plane", "ray", "center", "spot", "det")}, J_off
+
+
+def _smallest_workspace(h, torch, call, most):
+    """The fewest workspace bytes (to 4 KB) with which call() is accepted."""
+    from paper_2404_06478_gb300 import _native as N
+    from paper_2404_06478_gb300.api import LaueError
+    ws = torch.empty(most, dtype=torch.uint8, device="cuda")
+
+    def accepted(nbytes):
+        assert h.L.laue_set_workspace(h.h, ctypes.c_void_p(ws.data_ptr()), nbytes, None) == 0
+        try:
+            call()
+            return True
+        except LaueError as e:
+            assert e.code == N.LAUE_ERR_WORKSPACE
+            return False
+
+    lo, hi = 4096, most
+    while hi - lo > 4096:
+        mid = (lo + hi) // 2 // 256 * 256
+        lo, hi = (lo, mid) if accepted(mid) else (mid, hi)
+    assert accepted(hi)
+    return ws
+
+
+# blocks at the edges of slices (64 spots), sub-granules (16) and tiles (128); empty blocks; a block beyond the
+# lists' 16-bit slots
+EDGES = [(1, 1), (0, 5), (5, 0), (63, 64), (64, 63), (65, 129), (127, 15), (128, 16), (129, 17), (700, 311), (1, 700),
+         (900, 1)]
+
+
+@pytest.mark.parametrize("geom", [GEOM, sg.tilted_geometry()], ids=["flat", "tilted"])
+@pytest.mark.parametrize("eps,mode,sizes", [(1.0, 0, EDGES), (6.0, 1, EDGES), (300.0, 0, EDGES), (2.0, 2, EDGES),
+                                            (1.0, 0, [(70001, 33), (40, 20)]), (1.0, 1, [(33, 70001), (40, 20)])])
+def test_lists_sweeps_and_every_pair_agree(env, geom, eps, mode, sizes):
+    api, torch, dev = env["api"], env["torch"], env["dev"]
+    p, I_off, m, J_off = _blocks(sizes, 21, geom)
+    ob = api.ObsSpots.from_numpy(p, I_off, device=dev)
+    ms = api.ModelSpots.from_numpy(J_off, m["grain"], m["plane"], m["ray"], m["center"], m["spot"], m["det"], device=dev)
+    h = api.Handle(dev)
+
+    def call():
+        out = api.cost_sinkhorn(h, geom, ob, ms, eps, 2.25, 25, dust_mode=mode, harvest=True, col_harvest=True,
+                                kappa=30.0, lam=20.0)
+        torch.cuda.synchronize()
+        h.device_status()  # an isolated spot of the unbalanced mode may be reported; the bits are compared below
+        return out
+
+    listed = call()
+    h.set_pair_skipping(False)
+    every = call()
+    h.set_pair_skipping(True)
+    size = h.ws.numel()
+    h.reserve = lambda *a, **k: None
+    keep = _smallest_workspace(h, torch, call, size)
+    swept = call()
+    for k in listed:
+        assert torch.equal(listed[k].nan_to_num(9e9), every[k].nan_to_num(9e9)), ("every pair", k)
+        assert torch.equal(listed[k].nan_to_num(9e9), swept[k].nan_to_num(9e9)), ("swept", k)
+    del keep
