@@ -136,15 +136,6 @@ extern "C" int laue_create(laue_handle** h, int device) {
         free(H);
         return LAUE_ERR_CUDA;
     }
-    int prev = 0;
-    cudaGetDevice(&prev);
-    cudaSetDevice(device);
-    const cudaError_t e = sinkhorn_setup();
-    cudaSetDevice(prev);
-    if (e != cudaSuccess) {
-        free(H);
-        return LAUE_ERR_CUDA;
-    }
     H->row_variant = H->col_variant = kSkDefaultVariant;
     H->skip = 1;
     H->err[0] = 0;
@@ -549,13 +540,6 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
     a.warm = prm->warm_start ? 1 : 0;
     lc->row_variant = h->row_variant;
     lc->col_variant = h->col_variant;
-    // as many tiles to a CTA as it takes to have two CTAs per SM
-    auto ctas = [&](int tiles, int tile, int* per_cta) {
-        *per_cta = std::min(kPassThreads / tile, (tiles + 2 * h->sm_count - 1) / (2 * h->sm_count));
-        return std::max(1, (tiles + *per_cta - 1) / *per_cta);
-    };
-    lc->row_ctas = ctas(a.T + a.n_obs / 2 / a.tile_rows + 1, a.tile_rows, &lc->row_per_cta);
-    lc->col_ctas = ctas(a.T + a.n_model / 2 / a.tile_cols + 1, a.tile_cols, &lc->col_per_cta);
     lc->row_slices = (int)list_slices(a.T, a.n_obs, a.tile_rows);
     lc->col_slices = (int)list_slices(a.T, a.n_model, a.tile_cols);
     // the M-step pair kernel runs one thread per column pair of the column

@@ -187,12 +187,9 @@ void sparse_carve(SpArgs& a, char* base, int T, int n_obs, int n_model, int rho)
 cudaError_t sparse_sinkhorn_run(const SpArgs& a, int n_iter, bool rows, bool cols, cudaStream_t s);
 
 constexpr int kSkVariants = 4;       // launch shapes of the pair passes (see sinkhorn.cu)
-constexpr int kPassThreads = 512;     // CTA of the pair passes: at most kPassThreads / tile tiles
 constexpr int kSkDefaultVariant = 3;  // 64-pair tiles: the autotuner's usual pick
 
 struct SkLaunch {
-    int row_ctas, col_ctas;        // CTAs of the pair passes
-    int row_per_cta, col_per_cta;  // tiles of a CTA
     int row_slices, col_slices;  // bound on the slices of each side
     int col_grid;                // CTAs of the M-step's pair kernel
     int row_variant, col_variant;
@@ -205,7 +202,6 @@ cudaError_t sinkhorn_iterate(const SkArgs& a, const SkLaunch& l, int n_iter, cud
 cudaError_t sinkhorn_finish(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols, cudaStream_t s);
 cudaError_t sinkhorn_harvest(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols,
                              cudaStream_t s);
-cudaError_t sinkhorn_setup();
 cudaError_t sinkhorn_build_lists(const SkArgs& a, const SkLaunch& l, cudaStream_t s);
 int sk_variant_threads(int v);
 cudaError_t sinkhorn_row_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s);

@@ -12,15 +12,21 @@
 // the other side, even and odd slots in two accumulators), and every term
 // they leave out is exactly 0, so a potential has the same bits either way.
 //
-// CTAs are kPassThreads wide: the last one of a pass merges the tiles' partial
-// sums into the dustbin potentials, and needs the threads.  Where there are few
-// tiles a CTA takes fewer of them than it has warps for, so that they spread
-// over the SMs.
+// A pass has no serial end: the tiles' partial sums are merged into the dustbin
+// potentials by CTAs of the NEXT pass (see finish_pass), which does not need
+// them yet: the row update takes G_0 of the column pass before the last row
+// update, the column update F_0 of the column update before.  So CTAs are
+// small (four slices), and end as soon as their longest slice does.
 #include <type_traits>
 
 #include "pairs.cuh"
 
 namespace laue {
+
+// CTA of a pass over tiles of `tile` pairs that finishes a pass over tiles of `other`
+constexpr __host__ __device__ int pass_threads(int tile, int other = 0) {
+    return tile > 128 || other > 128 ? 256 : 128;
+}
 
 constexpr float kListLog2 = 127.0f;   // K e2 beyond which ex2.approx.ftz gives exactly 0 (potentials <= shift)
 constexpr float kTinySum = 1.0e-30f;  // below ~2^-100 the fast sum is recomputed exactly
@@ -160,12 +166,12 @@ struct Slice {
 };
 
 template <int TILE>
-__device__ __forceinline__ Slice slice_of(const int4* tiles, int n_tiles, int per_cta) {
+__device__ __forceinline__ Slice slice_of(const int4* tiles, int n_tiles, int block) {
     constexpr int kW = TILE / 32;
     Slice s;
     const int warp = threadIdx.x >> 5;
     s.lane = threadIdx.x & 31;
-    s.tile = warp / kW < per_cta ? blockIdx.x * per_cta + warp / kW : n_tiles;
+    s.tile = block * ((int)blockDim.x / TILE) + warp / kW;
     s.w = warp % kW;
     s.id = s.tile * kW + s.w;
     s.t = 0;
@@ -623,9 +629,8 @@ __device__ __noinline__ void exact_lse(const SkArgs& a, WarpStage& S, const Slic
 // ----------------------------------------------------- ends of the passes
 // Largest potential of each angle block, kept by the passes as the maximum of
 // the tile partials in an order-preserving code (0: none yet).  Rows and
-// columns have two sets each: pass `it` fills set it & 1, and the last CTA of
-// the pass clears the other side's set that the next pass fills, whose readers
-// are done.
+// columns have two sets each: pass `it` fills set it & 1, and clears the other
+// side's set that the next pass fills, whose readers are done.
 __device__ __forceinline__ unsigned max_code(float v) {
     const unsigned b = __float_as_uint(v);
     return b & 0x80000000u ? ~b : b | 0x80000000u;
@@ -648,24 +653,23 @@ __device__ __forceinline__ float final_col_max(const SkArgs& a, const DustPtrs& 
 // Lanes' partial log-sum-exps of a CTA's tiles into part[tile] and the angle
 // maxima: the warps of a tile in order.
 template <int TILE>
-__device__ __forceinline__ void store_parts(float m, float s, int per_cta, int n_tiles, int my_angle, float2* part,
-                                            unsigned* maxima, float* sm, float* ss) {
+__device__ __forceinline__ void store_parts(float m, float s, const Slice& sl, int n_tiles, float2* part, unsigned* maxima,
+                                            float* sm, float* ss) {
     constexpr int kW = TILE / 32;
     const int warp = threadIdx.x >> 5;
     warp_lse_reduce(m, s);
-    if ((threadIdx.x & 31) == 0) {
+    if (sl.lane == 0) {
         sm[warp] = m;
         ss[warp] = s;
     }
     __syncthreads();
-    const int tile = blockIdx.x * per_cta + threadIdx.x;
-    if ((int)threadIdx.x < per_cta && tile < n_tiles) {
+    if (sl.lane == 0 && sl.w == 0 && sl.tile < n_tiles) {
         Lse2 L;
         L.m = kNegHuge;
         L.s = 0.0f;
-        for (int k = 0; k < kW; ++k) L.merge(sm[threadIdx.x * kW + k], ss[threadIdx.x * kW + k]);
-        part[tile] = make_float2(L.m, L.s);
-        if (L.m > kNegHuge) atomicMax(maxima + my_angle, max_code(L.m));
+        for (int k = 0; k < kW; ++k) L.merge(sm[warp + k], ss[warp + k]);
+        part[sl.tile] = make_float2(L.m, L.s);
+        if (L.m > kNegHuge) atomicMax(maxima + sl.t, max_code(L.m));
     }
 }
 
@@ -682,16 +686,16 @@ __device__ __forceinline__ bool last_block(int* done, int* flag) {
     return last;
 }
 
-// Log-sum-exp of the n tile partials by the last CTA: TILE chains (chain c
+// Log-sum-exp of the n tile partials by one CTA: TILE chains (chain c
 // takes the tiles c, c + TILE, ... in order), then the chains by warp and the
 // warps in order.  A chain's running maxima are known before its sum (a prefix
 // maximum), so every exponential is taken in parallel and only the sum's
-// multiply-adds are serial: kPassThreads / TILE segments of a chain hold their
+// multiply-adds are serial: the CTA's segments of a chain hold their
 // elements in registers and hand the sum on.  Thread 0 gets (m, s).
-template <int TILE>
+template <int TILE, int THREADS>
 __device__ void merge_parts(const float2* part, int n, float& m_out, float& s_out, float* sm, float* ss,
                             float (*segmax)[TILE], float* cm, float* cs) {
-    constexpr int kSeg = kPassThreads / TILE, kR = 8;
+    constexpr int kSeg = THREADS / TILE, kR = 16;
     const int c = threadIdx.x % TILE, seg = threadIdx.x / TILE;
     if (seg == 0) {
         cm[c] = kNegHuge;
@@ -780,14 +784,79 @@ __device__ __forceinline__ void warp_merge_parts(const float2* part, int first, 
 }
 
 
-template <int TILE>
+template <int TILE, int THREADS = pass_threads(TILE)>
 struct PassShared {
-    WarpStage stage[kPassThreads / 32];
-    float sm[kPassThreads / 32], ss[kPassThreads / 32];
-    float segmax[kPassThreads / TILE][TILE];
+    WarpStage stage[THREADS / 32];
+    float sm[THREADS / 32], ss[THREADS / 32];
+    float segmax[THREADS / TILE][TILE];
     float cm[TILE], cs[TILE];
     int last;
 };
+
+// Dustbin potentials from the partials of a pass: rows (of iteration it): F_0
+// of the iteration and G_0 from it and the new F; columns: the next F_0 from
+// the new G and the current G_0.  Block `block` of `blocks`; also clears the
+// maxima set `clear` and counts the pass's pairs.
+template <int TILE, int THREADS, bool ROWS>
+__device__ void finish_pass(const SkArgs& a, PassShared<TILE, THREADS>& H, int block, int blocks, unsigned* clear) {
+    const DustPtrs D = dust_ptrs(a.dust, a.T);
+    const int lane = threadIdx.x & 31;
+    const float2* part = ROWS ? a.row_part : a.col_part;
+    if (a.mode == 1) {
+        const int warps = blockDim.x >> 5;
+        for (int u = block * warps + (threadIdx.x >> 5); u < a.T; u += blocks * warps) {
+            const int4 at = a.ang_tiles[u];
+            const float v0 = __ldcg((ROWS ? D.F0n : D.G0) + u);
+            float m = v0 - a.kc, s = 1.0f;
+            warp_merge_parts(part, ROWS ? at.x : at.z, ROWS ? at.y : at.w, m, s);
+            if (lane == 0) {
+                const float v = (ROWS ? D.log2O : D.log2U)[u] - (m + lg2(s));
+                if (ROWS) {
+                    D.F0[u] = v0;
+                    D.G0[u] = v;
+                } else {
+                    D.F0n[u] = v;
+                }
+            }
+        }
+    } else if (a.mode == 0 && block == 0) {
+        float m, s;
+        const float v0 = threadIdx.x == 0 ? __ldcg(ROWS ? D.F0n : D.G0) : 0.0f;
+        merge_parts<TILE, THREADS>(part, __ldcg(a.ctrl + (ROWS ? CTRL_N_ROW_TILES : CTRL_N_COL_TILES)), m, s, H.sm, H.ss,
+                          H.segmax, H.cm, H.cs);
+        if (threadIdx.x == 0) {
+            Lse2 L;
+            L.init(v0 - a.kc);
+            L.merge(m, s);
+            const float v = (ROWS ? D.log2O[0] : D.log2U[0]) - L.value();
+            if (ROWS) {
+                D.F0[0] = v0;
+                D.G0[0] = v;
+            } else {
+                D.F0n[0] = v;
+            }
+        }
+    }
+    if (block == 0) {
+        if (clear)
+            for (int u = threadIdx.x; u < a.T; u += blockDim.x) clear[u] = 0u;
+        if (threadIdx.x == 0)
+            *(unsigned long long*)(a.ctrl + CTRL_SK_PAIRS) +=
+                __ldcg((const unsigned long long*)(a.ctrl + (ROWS ? CTRL_ROW_EVAL : CTRL_COL_EVAL)));
+    }
+}
+
+// Blocks that finish the pass before: a warp per angle for per-angle dustbins.
+__host__ __device__ inline int finish_blocks(int mode, int T, int threads) {
+    return mode == 1 ? (T + threads / 32 - 1) / (threads / 32) : 1;
+}
+
+// The last column pass.
+template <int TILE>
+__global__ void __launch_bounds__(pass_threads(TILE)) sk_finish_pass_kernel(SkArgs a) {
+    extern __shared__ __align__(128) char pass_smem[];
+    finish_pass<TILE, pass_threads(TILE), false>(a, *(PassShared<TILE>*)pass_smem, blockIdx.x, gridDim.x, nullptr);
+}
 
 // Programmatic dependent launch: a pass starts while the one before it ends.
 // What it reads before pass_wait is what the list kernels and the scheduler
@@ -798,17 +867,28 @@ __device__ __forceinline__ void pass_release() { asm volatile("griddepcontrol.la
 
 // --------------------------------------------------- row and column passes
 // Iteration `it` of the row (ROWS) or column update.  What bounds it: at the
-// 1000-grain density the lists (HBM), below that the chain of a pass: the
-// potentials' gathers, the tickets and the merge of the tiles.
-template <int TILE, bool ROWS>
-__global__ void __launch_bounds__(kPassThreads, 2) sk_pass_kernel(SkArgs a, int it, int per_cta) {
+// 1000-grain density the lists (HBM), below that the chain of a pass: launch,
+// gathers of the potentials, partial sums.  The other side's tile width, for
+// the partials that the first blocks merge, is OTHER.
+template <int TILE, int OTHER, bool ROWS>
+__global__ void __launch_bounds__(pass_threads(TILE, OTHER), 1024 / pass_threads(TILE, OTHER))
+    sk_pass_kernel(SkArgs a, int it, int finishers) {
     extern __shared__ __align__(128) char pass_smem[];
-    PassShared<TILE>& H = *(PassShared<TILE>*)pass_smem;
+    constexpr int kThreads = pass_threads(TILE, OTHER);
+    PassShared<TILE, kThreads>& H = *(PassShared<TILE, kThreads>*)pass_smem;
     if (ROWS && it == 0) pass_wait();  // the first pass follows the kernels that write the lists
+    if ((int)blockIdx.x < finishers) {
+        if (!(ROWS && it == 0)) pass_wait();
+        pass_release();
+        unsigned* clear = ROWS ? col_max(a, it) : row_max(a, it + 1);
+        if (!ROWS || it > 0)
+            finish_pass<OTHER, kThreads, !ROWS>(a, *(PassShared<OTHER, kThreads>*)pass_smem, blockIdx.x, finishers, clear);
+        return;
+    }
     DustPtrs D = dust_ptrs(a.dust, a.T);
     const int n_tiles = __ldcg(a.ctrl + (ROWS ? CTRL_N_ROW_TILES : CTRL_N_COL_TILES));
     const int4* tiles = ROWS ? a.row_tiles : a.col_tiles;
-    const Slice sl = slice_of<TILE>(tiles, n_tiles, per_cta);
+    const Slice sl = slice_of<TILE>(tiles, n_tiles, blockIdx.x - finishers);
     const int t = sl.t, lane = sl.lane;
     const int* tab = ROWS ? a.row_tab : a.col_tab;
     ListHead h;
@@ -822,11 +902,6 @@ __global__ void __launch_bounds__(kPassThreads, 2) sk_pass_kernel(SkArgs a, int 
     float2 K = make_float2(a.negKD2, a.negKD2);  // -K of the lane's own spots (columns)
     if (!ROWS && sl.valid) K = *((const float2*)&a.modW[sl.q] + 1);
     if (!vb) K.y = -1.0f;
-    int my_angle = 0;
-    {
-        const int tile = blockIdx.x * per_cta + threadIdx.x;
-        if ((int)threadIdx.x < per_cta && tile < n_tiles) my_angle = tiles[tile].x;
-    }
     const float* pot = ROWS ? a.Gc : a.Fc;
     float* out = ROWS ? a.Fc : a.Gc;
     if (!(ROWS && it == 0)) pass_wait();
@@ -836,7 +911,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) sk_pass_kernel(SkArgs a, int 
     float pm = kNegHuge, ps = 0.0f;
     if (sl.n_own > 0) {
         // the dustbin's term: the outlier column (rows), the unmatched-model row with C_0j = 0 (columns)
-        const float dust = ub ? kNegHuge : ROWS ? __ldcg(D.G0 + d) - a.kc : __ldcg(D.F0 + d);
+        const float dust = ub ? kNegHuge : ROWS ? __ldcg(D.G0 + d) - a.kc : __ldcg(D.F0n + d);
         const float top = ROWS ? (it > 0 ? angle_max(col_max(a, it - 1), t, 0.0f) : D.Gmax[t])
                                : angle_max(row_max(a, it), t, a.kc);
         const float shift = ub ? top : fmaxf(top, dust);
@@ -875,51 +950,8 @@ __global__ void __launch_bounds__(kPassThreads, 2) sk_pass_kernel(SkArgs a, int 
             if (vb) lse_merge_into(pm, ps, vv - off, 1.0f);
         }
     }
-    float2* part = ROWS ? a.row_part : a.col_part;
-    store_parts<TILE>(pm, ps, per_cta, n_tiles, my_angle, part, ROWS ? row_max(a, it) : col_max(a, it), H.sm, H.ss);
-    if (!last_block(a.ctrl + (ROWS ? CTRL_ROW_DONE : CTRL_COL_DONE), &H.last)) return;
-    // rows: promote F_0, then G_0 from the new F; columns: next F_0 from the new G and the current G_0
-    if (a.mode == 1) {
-        for (int u = threadIdx.x >> 5; u < a.T; u += kPassThreads / 32) {
-            const int4 at = a.ang_tiles[u];
-            const float F0 = ROWS ? __ldcg(D.F0n + u) : 0.0f;
-            float m = (ROWS ? F0 : __ldcg(D.G0 + u)) - a.kc, s = 1.0f;
-            warp_merge_parts(part, ROWS ? at.x : at.z, ROWS ? at.y : at.w, m, s);
-            if (lane == 0) {
-                const float v = (ROWS ? D.log2O[u] : D.log2U[u]) - (m + lg2(s));
-                if (ROWS) {
-                    D.F0[u] = F0;
-                    D.G0[u] = v;
-                } else {
-                    D.F0n[u] = v;
-                }
-            }
-        }
-    } else if (a.mode == 0) {
-        float m, s;
-        const float at = threadIdx.x == 0 ? __ldcg(ROWS ? D.F0n : D.G0) : 0.0f;
-        merge_parts<TILE>(part, n_tiles, m, s, H.sm, H.ss, H.segmax, H.cm, H.cs);
-        if (threadIdx.x == 0) {
-            Lse2 L;
-            L.init(at - a.kc);
-            L.merge(m, s);
-            const float v = (ROWS ? D.log2O[0] : D.log2U[0]) - L.value();
-            if (ROWS) {
-                D.F0[0] = at;
-                D.G0[0] = v;
-            } else {
-                D.F0n[0] = v;
-            }
-        }
-    }
-    // the set of maxima that the other side's next pass fills
-    unsigned* clear = ROWS ? col_max(a, it) : row_max(a, it + 1);
-    for (int u = threadIdx.x; u < a.T; u += kPassThreads) clear[u] = 0u;
-    if (threadIdx.x == 0) {
-        a.ctrl[ROWS ? CTRL_ROW_DONE : CTRL_COL_DONE] = 0;
-        *(unsigned long long*)(a.ctrl + CTRL_SK_PAIRS) +=
-            *(const unsigned long long*)(a.ctrl + (ROWS ? CTRL_ROW_EVAL : CTRL_COL_EVAL));
-    }
+    store_parts<TILE>(pm, ps, sl, n_tiles, ROWS ? a.row_part : a.col_part, ROWS ? row_max(a, it) : col_max(a, it), H.sm,
+                      H.ss);
 }
 
 // ------------------------------------------------------------- read-out
@@ -930,7 +962,7 @@ __device__ __forceinline__ void block_err(float v, float* red, int* out) {
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int k = 1; k < kPassThreads / 32; ++k) v = fmaxf(v, red[k]);
+        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) v = fmaxf(v, red[k]);
         atomicMax(out, __float_as_int(v));
     }
 }
@@ -1036,11 +1068,12 @@ __device__ __noinline__ Lse2 whole_col(const SkArgs& a, int t, int q, int odd) {
 __device__ __forceinline__ bool is_entry(float e2) { return !(e2 > 2.0e38f); }
 
 template <int TILE>
-__global__ void __launch_bounds__(kPassThreads, 2) sk_harvest_row_kernel(SkArgs a, int n_iter, int per_cta) {
+__global__ void __launch_bounds__(pass_threads(TILE), 1024 / pass_threads(TILE)) sk_harvest_row_kernel(SkArgs a,
+                                                                                                     int n_iter) {
     extern __shared__ __align__(128) char pass_smem[];
     PassShared<TILE>& H = *(PassShared<TILE>*)pass_smem;
     DustPtrs D = dust_ptrs(a.dust, a.T);
-    const Slice sl = slice_of<TILE>(a.row_tiles, a.ctrl[CTRL_N_ROW_TILES], per_cta);
+    const Slice sl = slice_of<TILE>(a.row_tiles, a.ctrl[CTRL_N_ROW_TILES], blockIdx.x);
     const int t = sl.t, lane = sl.lane;
     float my_err = 0.0f;
     if (sl.n_own > 0) {
@@ -1143,11 +1176,12 @@ __global__ void __launch_bounds__(kPassThreads, 2) sk_harvest_row_kernel(SkArgs 
 // error with the final potentials, in base 2 with a running maximum.  Pairs
 // are left out, and columns read again, as for the rows.
 template <int TILE>
-__global__ void __launch_bounds__(kPassThreads, 2) sk_harvest_col_kernel(SkArgs a, int n_iter, int per_cta) {
+__global__ void __launch_bounds__(pass_threads(TILE), 1024 / pass_threads(TILE)) sk_harvest_col_kernel(SkArgs a,
+                                                                                                     int n_iter) {
     extern __shared__ __align__(128) char pass_smem[];
     PassShared<TILE>& H = *(PassShared<TILE>*)pass_smem;
     DustPtrs D = dust_ptrs(a.dust, a.T);
-    const Slice sl = slice_of<TILE>(a.col_tiles, a.ctrl[CTRL_N_COL_TILES], per_cta);
+    const Slice sl = slice_of<TILE>(a.col_tiles, a.ctrl[CTRL_N_COL_TILES], blockIdx.x);
     const int t = sl.t, lane = sl.lane;
     float my_err = 0.0f;
     if (sl.n_own > 0) {
@@ -1238,11 +1272,18 @@ cudaError_t with_tile(int v, Fn fn) {
     return fn(std::integral_constant<int, 128>{});
 }
 
-template <class Kernel, class... Args>
-cudaError_t launch_pass(Kernel k, int ctas, size_t smem, bool overlap, cudaStream_t s, Args... args) {
+// Both tile widths as integral constants.
+template <class Fn>
+cudaError_t with_tiles(const SkLaunch& l, Fn fn) {
+    return with_tile(l.row_variant, [&](auto row) { return with_tile(l.col_variant, [&](auto col) { return fn(row, col); }); });
+}
+
+template <class... Params, class... Args>
+cudaError_t launch_pass(void (*k)(Params...), int ctas, int threads, size_t smem, bool overlap, cudaStream_t s,
+                        Args... args) {
     cudaLaunchConfig_t c{};
     c.gridDim = dim3(ctas);
-    c.blockDim = dim3(kPassThreads);
+    c.blockDim = dim3(threads);
     c.dynamicSmemBytes = smem;
     c.stream = s;
     cudaLaunchAttribute at{};
@@ -1253,38 +1294,49 @@ cudaError_t launch_pass(Kernel k, int ctas, size_t smem, bool overlap, cudaStrea
     return cudaLaunchKernelEx(&c, k, args...);
 }
 
-template <int TILE>
-cudaError_t allow_smem() {
-    const int n = (int)sizeof(PassShared<TILE>);
-    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(sk_pass_kernel<TILE, true>, at, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_pass_kernel<TILE, false>, at, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_harvest_row_kernel<TILE>, at, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_harvest_col_kernel<TILE>, at, n);
-    return e;
+// CTAs that hold a side's tiles.
+int tile_ctas(int T, int n_spots, int tile, int threads) {
+    const int per = threads / tile, tiles = T + n_spots / 2 / tile + 1;
+    return (tiles + per - 1) / per;
+}
+
+template <int TILE, int OTHER, bool ROWS>
+cudaError_t run_pass(const SkArgs& a, int it, cudaStream_t s) {
+    constexpr int thr = pass_threads(TILE, OTHER);
+    constexpr size_t own = sizeof(PassShared<TILE, thr>), other = sizeof(PassShared<OTHER, thr>);
+    constexpr size_t smem = own > other ? own : other;
+    static_assert(smem <= 48 * 1024, "beyond the shared memory of a plain launch");
+    const int fin = finish_blocks(a.mode, a.T, thr);
+    return launch_pass(sk_pass_kernel<TILE, OTHER, ROWS>, fin + tile_ctas(a.T, ROWS ? a.n_obs : a.n_model, TILE, thr), thr,
+                       smem, true, s, a, it, fin);
 }
 
 }  // namespace
 
-// Once per device (the current one), before the first launch.
-cudaError_t sinkhorn_setup() {
-    cudaError_t e = allow_smem<64>();
-    if (e == cudaSuccess) e = allow_smem<128>();
-    if (e == cudaSuccess) e = allow_smem<256>();
-    return e;
-}
-
 cudaError_t sinkhorn_row_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s) {
-    return with_tile(l.row_variant, [&](auto tile) {
-        constexpr int t = decltype(tile)::value;
-        return launch_pass(sk_pass_kernel<t, true>, l.row_ctas, sizeof(PassShared<t>), true, s, a, it, l.row_per_cta);
+    return with_tiles(l, [&](auto row, auto col) {
+        return run_pass<decltype(row)::value, decltype(col)::value, true>(a, it, s);
     });
 }
 
 cudaError_t sinkhorn_col_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s) {
+    return with_tiles(l, [&](auto row, auto col) {
+        return run_pass<decltype(col)::value, decltype(row)::value, false>(a, it, s);
+    });
+}
+
+cudaError_t sinkhorn_iterate(const SkArgs& a, const SkLaunch& l, int n_iter, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    for (int it = 0; it < n_iter && e == cudaSuccess; ++it) {
+        e = sinkhorn_row_pass(a, l, it, s);
+        if (e == cudaSuccess) e = sinkhorn_col_pass(a, l, it, s);
+    }
+    if (e != cudaSuccess || n_iter == 0) return e;
     return with_tile(l.col_variant, [&](auto tile) {
         constexpr int t = decltype(tile)::value;
-        return launch_pass(sk_pass_kernel<t, false>, l.col_ctas, sizeof(PassShared<t>), true, s, a, it, l.col_per_cta);
+        sk_finish_pass_kernel<t><<<finish_blocks(a.mode, a.T, pass_threads(t)), pass_threads(t), sizeof(PassShared<t>), s>>>(
+            a);
+        return cudaGetLastError();
     });
 }
 
@@ -1307,14 +1359,14 @@ cudaError_t sinkhorn_harvest(const SkArgs& a, const SkLaunch& l, int n_iter, boo
     if (want_rows)
         e = with_tile(l.row_variant, [&](auto tile) {
             constexpr int t = decltype(tile)::value;
-            return launch_pass(sk_harvest_row_kernel<t>, l.row_ctas, sizeof(PassShared<t>), false, s, a, n_iter,
-                               l.row_per_cta);
+            return launch_pass(sk_harvest_row_kernel<t>, tile_ctas(a.T, a.n_obs, t, pass_threads(t)), pass_threads(t),
+                               sizeof(PassShared<t>), false, s, a, n_iter);
         });
     if (e == cudaSuccess && want_cols)
         e = with_tile(l.col_variant, [&](auto tile) {
             constexpr int t = decltype(tile)::value;
-            return launch_pass(sk_harvest_col_kernel<t>, l.col_ctas, sizeof(PassShared<t>), false, s, a, n_iter,
-                               l.col_per_cta);
+            return launch_pass(sk_harvest_col_kernel<t>, tile_ctas(a.T, a.n_model, t, pass_threads(t)), pass_threads(t),
+                               sizeof(PassShared<t>), false, s, a, n_iter);
         });
     return e;
 }

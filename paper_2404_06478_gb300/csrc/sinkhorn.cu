@@ -573,15 +573,6 @@ cudaError_t sinkhorn_prepare(const SkArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t sinkhorn_iterate(const SkArgs& a, const SkLaunch& l, int n_iter, cudaStream_t s) {
-    for (int it = 0; it < n_iter; ++it) {
-        cudaError_t e = sinkhorn_row_pass(a, l, it, s);
-        if (e == cudaSuccess) e = sinkhorn_col_pass(a, l, it, s);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
 cudaError_t sinkhorn_finish(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols,
                             cudaStream_t s) {
     int nmax = a.n_obs > a.n_model ? a.n_obs : a.n_model;
