@@ -136,6 +136,15 @@ extern "C" int laue_create(laue_handle** h, int device) {
         free(H);
         return LAUE_ERR_CUDA;
     }
+    int prev = 0;
+    cudaGetDevice(&prev);
+    cudaSetDevice(device);
+    const cudaError_t e = sinkhorn_setup();
+    cudaSetDevice(prev);
+    if (e != cudaSuccess) {
+        free(H);
+        return LAUE_ERR_CUDA;
+    }
     H->row_variant = H->col_variant = kSkDefaultVariant;
     H->skip = 1;
     H->err[0] = 0;
@@ -495,15 +504,34 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
         a.obs_ext = (float*)(a.mod_cone + L.max_mod_gran);
         a.mod_ext = a.obs_ext + L.max_obs_gran;
         a.skip = h->skip;
-        // the sort buffers, once the sort is done: compact potentials, sub-granule cones
+    }
+    a.tile_rows = sk_variant_threads(h->row_variant);
+    a.tile_cols = sk_variant_threads(h->col_variant);
+    lc->row_slices = (int)list_slices(a.T, a.n_obs, a.tile_rows);
+    lc->col_slices = (int)list_slices(a.T, a.n_model, a.tile_cols);
+    {
+        // the sort buffers, once the sort is done: slices, sub-granule cones, compact potentials
+        size_t rs = lc->row_slices, cs = lc->col_slices;
         char* b = ws + L.sortbuf;
-        a.obs_sub = (float4*)b;
-        a.mod_sub = a.obs_sub + (size_t)kSubs * L.max_obs_gran;
-        a.obs_subext = (float*)(a.mod_sub + (size_t)kSubs * L.max_mod_gran);
-        a.mod_subext = a.obs_subext + (size_t)kSubs * L.max_obs_gran;
-        a.Gc = (float*)(((uintptr_t)(a.mod_subext + (size_t)kSubs * L.max_mod_gran) + 15) / 16 * 16);
-        a.Fc = a.Gc + 2 * (size_t)L.max_mod_pairs;
-        a.pmax = (unsigned*)(a.Fc + 2 * (size_t)L.max_obs_pairs);
+        auto take = [&](size_t bytes) {
+            char* p = b;
+            b += align_up(bytes, 16);
+            return p;
+        };
+        a.row_desc = take(kSliceDescBytes * rs);
+        a.col_desc = take(kSliceDescBytes * cs);
+        a.obs_sub = (float4*)take(sizeof(float4) * kSubs * L.max_obs_gran);
+        a.mod_sub = (float4*)take(sizeof(float4) * kSubs * L.max_mod_gran);
+        a.obs_subext = (float*)take(sizeof(float) * kSubs * L.max_obs_gran);
+        a.mod_subext = (float*)take(sizeof(float) * kSubs * L.max_mod_gran);
+        a.Gc = (float*)take(sizeof(float) * 2 * L.max_mod_pairs);
+        a.Fc = (float*)take(sizeof(float) * 2 * L.max_obs_pairs);
+        a.row_order = (int*)take(sizeof(int) * rs);
+        a.col_order = (int*)take(sizeof(int) * cs);
+        a.pmax = (unsigned*)take(sizeof(unsigned) * 4 * a.T);
+        // a pass that holds all its slices at once needs no order
+        if (rs <= (size_t)kSlicesPerSm * h->sm_count && cs <= (size_t)kSlicesPerSm * h->sm_count)
+            a.row_order = a.col_order = nullptr;
     }
     a.row_tiles = (int4*)(ws + L.row_tiles);
     a.col_tiles = (int4*)(ws + L.col_tiles);
@@ -514,8 +542,6 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
     a.ctrl = (int*)(ws + L.ctrl);
     a.max_row_tiles = L.max_row_tiles;
     a.max_col_tiles = L.max_col_tiles;
-    a.tile_rows = sk_variant_threads(h->row_variant);  // row pairs per tile (one per thread)
-    a.tile_cols = sk_variant_threads(h->col_variant);
     double eps = prm->eps;
     a.negKD2 = (float)(-(double)geom->D * geom->D * 1.4426950408889634 / eps);
     {
@@ -540,8 +566,6 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
     a.warm = prm->warm_start ? 1 : 0;
     lc->row_variant = h->row_variant;
     lc->col_variant = h->col_variant;
-    lc->row_slices = (int)list_slices(a.T, a.n_obs, a.tile_rows);
-    lc->col_slices = (int)list_slices(a.T, a.n_model, a.tile_cols);
     // the M-step pair kernel runs one thread per column pair of the column
     // pass's tiles (narrow tiles skip more), about 768 threads per SM
     lc->col_grid = std::max(1, std::min(h->sm_count * (768 / a.tile_cols), L.max_col_tiles));
@@ -549,9 +573,7 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
     size_t from = align_up(std::max(L.total, list_from), 256);
     size_t fixed = list_fixed_bytes(a.T, a.n_obs, a.n_model, a.tile_rows, a.tile_cols);
     if (a.skip && a.skipK > 0.0f && from + fixed + kListChunkBytes <= h->ws_bytes) {
-        a.row_hdr = (int*)(ws + from);
-        a.col_hdr = a.row_hdr + lc->row_slices;
-        a.row_tab = a.col_hdr + lc->col_slices;
+        a.row_tab = (int*)(ws + from);
         a.col_tab = a.row_tab + (size_t)kListChunks * lc->row_slices;
         a.pool = ws + from + fixed;
         size_t chunks = (h->ws_bytes - from - fixed) / kListChunkBytes;

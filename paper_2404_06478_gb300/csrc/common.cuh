@@ -68,6 +68,12 @@ constexpr int kSubs = kConeGran / kSubGran;
 constexpr int kListDepth = 8;
 constexpr int kListChunks = 128;  // chunks a slice can hold (1024 entries per spot)
 constexpr size_t kListChunkBytes = (size_t)kListDepth * 64 * 6;
+constexpr size_t kSliceDescBytes = 32;
+constexpr int kMaxTile = 256;      // largest tile (in spot pairs) of a launch shape
+// Slices of one side of a problem (a bound), for tiles of `tile` pairs.
+inline size_t list_slices(int T, int n_spots, int tile) {
+    return (size_t)T * (tile / 32 + 1) + (size_t)n_spots / 64 + 2;
+}
 constexpr size_t kCtrlBytes = 4096;  // status + counters + small scalars
 
 // ---------------------------------------------------------------------------
@@ -83,8 +89,8 @@ struct Layout {
     size_t modX, modY, modZ, modW;// pair-interleaved model spots
     size_t pairoff;               // int: I2_off[T+1], J2_off[T+1] (pair offsets), granule bases (2 x (T+1))
     size_t perm;                  // int: observed and model sort permutations (order -> caller, caller -> order)
-    size_t sortbuf;               // sort keys and indices (two buffers each); after the sort the compact
-                                  // potentials and the sub-granule cones
+    size_t sortbuf;               // sort keys and indices (two buffers each); after the sort the slices, the
+                                  // compact potentials and the sub-granule cones
     size_t cone;                  // float4 + float per granule of 32 pairs, observed then model
     size_t fwd_blocks;            // int per forward block (count, then offset)
     size_t jsum;                  // float per model spot x 12 (M-step sums)
@@ -139,7 +145,9 @@ inline Layout make_layout(const LaueProblemDims& d, int sm_count) {
     L.max_mod_gran = (int)((jp + kConeGran - 1) / kConeGran) + T + 1;
     {
         size_t sort_bytes = sizeof(int) * 4 * nsp;
-        size_t reuse = sizeof(float) * 2 * (ip + jp) + sizeof(unsigned) * 4 * T + 64 +
+        size_t slices = list_slices(T, d.n_obs, kMaxTile) + list_slices(T, d.n_model, kMaxTile);
+        size_t reuse = slices * (kSliceDescBytes + sizeof(int)) + sizeof(float) * 2 * (ip + jp) +
+                       sizeof(unsigned) * 4 * T + 128 +
                        (sizeof(float4) + sizeof(float)) * kSubs * (size_t)(L.max_obs_gran + L.max_mod_gran);
         L.sortbuf = take(sort_bytes > reuse ? sort_bytes : reuse);
     }
@@ -161,14 +169,10 @@ inline Layout make_layout(const LaueProblemDims& d, int sm_count) {
 
 // Pair lists: they take whatever the workspace holds beyond the layout (and
 // stay off where that is too little), so a workspace of the layout's size
-// still runs every call.  Slices of one side of a problem, for tiles of `tile`
-// pairs:
-inline size_t list_slices(int T, int n_spots, int tile) {
-    return (size_t)T * (tile / 32 + 1) + (size_t)n_spots / 64 + 2;
-}
+// still runs every call.
 inline size_t list_fixed_bytes(int T, int n_obs, int n_model, int tile_rows, int tile_cols) {
     size_t s = list_slices(T, n_obs, tile_rows) + list_slices(T, n_model, tile_cols);
-    return align_up(s * sizeof(int) * (1 + (size_t)kListChunks), 256);
+    return align_up(s * sizeof(int) * (size_t)kListChunks, 256);
 }
 // Bytes the lists can use: room for every same-angle pair of both sides with a
 // quarter more for padding, and at most kListPoolMax chunks (3 GB; 400 million

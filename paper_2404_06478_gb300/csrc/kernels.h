@@ -95,9 +95,12 @@ struct SkArgs {
     // potentials of the passes by ordered slot: pair offset of the block x 2 + rank
     float *Fc, *Gc;
     unsigned* pmax;        // 4T: maxima per angle of the last passes (passes.cu)
-    // pair lists (pool_chunks = 0: none): chunks per slice (-1: the slice is not
-    // listed), chunk numbers of each slice, the pool
-    int *row_hdr, *col_hdr, *row_tab, *col_tab;
+    // slices of the passes (passes.cu): descriptors; tiles by descending weight
+    // (null: in their own order)
+    void *row_desc, *col_desc;
+    int *row_order, *col_order;
+    // pair lists (pool_chunks = 0: none): chunk numbers of each slice, the pool
+    int *row_tab, *col_tab;
     char* pool;
     int pool_chunks;
     int uniK;              // every detector has the same cost length: K_j = -negKD2
@@ -187,6 +190,7 @@ void sparse_carve(SpArgs& a, char* base, int T, int n_obs, int n_model, int rho)
 cudaError_t sparse_sinkhorn_run(const SpArgs& a, int n_iter, bool rows, bool cols, cudaStream_t s);
 
 constexpr int kSkVariants = 4;       // launch shapes of the pair passes (see sinkhorn.cu)
+constexpr int kSlicesPerSm = 20;      // slices of a pass that an SM holds at once
 constexpr int kSkDefaultVariant = 3;  // 64-pair tiles: the autotuner's usual pick
 
 struct SkLaunch {
@@ -202,6 +206,7 @@ cudaError_t sinkhorn_iterate(const SkArgs& a, const SkLaunch& l, int n_iter, cud
 cudaError_t sinkhorn_finish(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols, cudaStream_t s);
 cudaError_t sinkhorn_harvest(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols,
                              cudaStream_t s);
+cudaError_t sinkhorn_setup();  // once per device, the current one
 cudaError_t sinkhorn_build_lists(const SkArgs& a, const SkLaunch& l, cudaStream_t s);
 int sk_variant_threads(int v);
 cudaError_t sinkhorn_row_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s);

@@ -48,6 +48,7 @@ int static_device(StaticDevice** out) {
         if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || p == nullptr) return LAUE_ERR_CUDA;
         int sm = 0;
         if (cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return LAUE_ERR_CUDA;
+        if (sinkhorn_setup() != cudaSuccess) return LAUE_ERR_CUDA;
         d.device = dev;
         d.scratch = p;
         d.sm_count = sm;

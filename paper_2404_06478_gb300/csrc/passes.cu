@@ -17,6 +17,7 @@
 // them yet: the row update takes G_0 of the column pass before the last row
 // update, the column update F_0 of the column update before.  So CTAs are
 // small (four slices), and end as soon as their longest slice does.
+#include <algorithm>
 #include <type_traits>
 
 #include "pairs.cuh"
@@ -156,35 +157,45 @@ __device__ __forceinline__ f2 pair_e2(f2 px, f2 py, f2 pz, f2 ncx, f2 ncy, f2 nc
     return fma2(ez, ez, e2);
 }
 
-// A slice's place in its pass.
+// What a pass needs to know of a slice, written with the lists and kept for
+// the iterations.
+struct __align__(32) SliceDesc {
+    int t, q, nspot;  // angle, first pair of its own, its spots (0: no slice)
+    int nch;          // chunks of its lists, -1: swept
+    int s0, ns;       // first pair and pairs of the streamed block
+    int weight;       // about how long it takes
+    int unused;
+};
+static_assert(sizeof(SliceDesc) == kSliceDescBytes, "laid out by the host");
+
+// A warp's slice; the lanes' own pairs.
 struct Slice {
-    int tile, w;     // tile, and which slice of the tile
-    int id;          // slice number (header and chunk table)
-    int t, q, lane;  // angle, the lane's own pair, lane
-    bool valid;
-    int n_own;       // pairs of the slice
+    int id, t, q, lane, nch;
+    int s0, ns;
+    bool valid, vb;  // the lane's spots a and b exist
+    bool any;
 };
 
-template <int TILE>
-__device__ __forceinline__ Slice slice_of(const int4* tiles, int n_tiles, int block) {
-    constexpr int kW = TILE / 32;
+__device__ __forceinline__ Slice load_slice(const SliceDesc* desc, int id) {
     Slice s;
-    const int warp = threadIdx.x >> 5;
+    s.id = id;
     s.lane = threadIdx.x & 31;
-    s.tile = block * ((int)blockDim.x / TILE) + warp / kW;
-    s.w = warp % kW;
-    s.id = s.tile * kW + s.w;
-    s.t = 0;
-    s.q = 0;
-    s.n_own = 0;
-    if (s.tile < n_tiles) {
-        const int4 td = tiles[s.tile];
-        s.t = td.x;
-        s.q = td.y + 32 * s.w + s.lane;
-        s.n_own = min(32, max(0, td.z - 32 * s.w));
-    }
-    s.valid = s.lane < s.n_own;
+    const int4 d0 = __ldcg((const int4*)&desc[id]), d1 = __ldcg((const int4*)&desc[id] + 1);
+    s.t = d0.x;
+    s.q = d0.y + s.lane;
+    s.nch = d0.z > 0 ? d0.w : 0;
+    s.s0 = d1.x;
+    s.ns = d1.y;
+    s.any = d0.z > 0;
+    s.valid = 2 * s.lane < d0.z;
+    s.vb = 2 * s.lane + 1 < d0.z;
     return s;
+}
+
+// Number of slices of a side: kW per tile.
+template <int TILE>
+__device__ __forceinline__ int slice_count(const SkArgs& a, bool rows) {
+    return __ldcg(a.ctrl + (rows ? CTRL_N_ROW_TILES : CTRL_N_COL_TILES)) * (TILE / 32);
 }
 
 // Observed pair of a lane, duplicated for the packed arithmetic.
@@ -243,9 +254,9 @@ __global__ void __launch_bounds__(32 * kListWarps) sk_list_kernel(SkArgs a) {
     ListStage& L = stage[threadIdx.x >> 5];
     const int4 td = (ROWS ? a.row_tiles : a.col_tiles)[tile];
     const int t = td.x, first = td.y + 32 * w, n_own = min(32, max(0, td.z - 32 * w));
-    int* hdr = (ROWS ? a.row_hdr : a.col_hdr) + id;
+    SliceDesc& desc = ((SliceDesc*)(ROWS ? a.row_desc : a.col_desc))[id];
     if (n_own == 0) {
-        if (lane == 0 && a.pool_chunks > 0) *hdr = 0;
+        if (lane < 8) ((int*)&desc)[lane] = 0;  // no spots, no chunks
         return;
     }
     const int q = first + lane;
@@ -412,63 +423,110 @@ __global__ void __launch_bounds__(32 * kListWarps) sk_list_kernel(SkArgs a) {
             }
     }
     if (lane == 0) {
-        if (a.pool_chunks > 0) *hdr = fail ? -1 : nch;
+        desc.t = t;
+        desc.q = first;
+        desc.nspot = min(64, own_off[t + 1] - own_off[t] - 2 * (first - o0));
+        desc.nch = fail ? -1 : nch;
+        desc.s0 = b0;
+        desc.ns = np;
+        desc.weight = fail ? evaluated / 4 : nch;  // a chunk takes about as long as four swept pairs
         const long long n = fail ? 4LL * n_own * evaluated : 64LL * kListDepth * nch;
         atomicAdd((unsigned long long*)(a.ctrl + (ROWS ? CTRL_ROW_EVAL : CTRL_COL_EVAL)), (unsigned long long)n);
     }
 }
 
-// ---------------------------------------------------- entries of a listed slice
-// Half a chunk (four entries of each of the lane's spots) in registers; the
-// next half is loaded while one is used.  The lists are read once per pass:
-// they stay out of L1.
-constexpr int kHalf = kListDepth / 2;
-struct Entries {
-    float2 e2[kHalf];     // costs of the lane's spots a and b
-    unsigned slot[kHalf];  // slots: a in the low half, b in the high half
-};
-
-__device__ __forceinline__ void load_entries(Entries& E, const char* chunk, int half, int lane) {
-#pragma unroll
-    for (int k = 0; k < kHalf; ++k) {
-        E.e2[k] = __ldcg((const float2*)chunk + 32 * (kHalf * half + k) + lane);
-        E.slot[k] = __ldcg((const unsigned*)(chunk + kListDepth * 64 * 4) + 32 * (kHalf * half + k) + lane);
-    }
-}
-
-// A listed slice: its number of chunks (-1: swept), the lane's share of the
-// first 32 chunk numbers and the first half chunk, which a pass loads before
-// it waits for the pass before it.
-struct ListHead {
-    int nch, mine;
-    Entries E;
-};
-
-__device__ __forceinline__ ListHead list_head(const SkArgs& a, const int* hdr, const int* tab, int id, int lane) {
-    ListHead h;
-    h.nch = a.pool_chunks > 0 ? __ldcg(hdr + id) : -1;
-    h.mine = lane < h.nch ? __ldcg(tab + (size_t)kListChunks * id + lane) : 0;
-    if (h.nch > 0)
-        load_entries(h.E, a.pool + (size_t)__shfl_sync(0xffffffffu, h.mine, 0) * kListChunkBytes, 0, lane);
-    return h;
-}
-
-// fn(entries) for every half chunk of the slice, in order.
-template <class Fn>
-__device__ __forceinline__ void for_each_half(const SkArgs& a, ListHead& h, const int* tab, int id, int lane, Fn fn) {
-    Entries N;
-    const char* p = a.pool + (size_t)__shfl_sync(0xffffffffu, h.mine, 0) * kListChunkBytes;
-    for (int c = 0; c < h.nch; ++c) {
-        load_entries(N, p, 1, lane);
-        fn(h.E);
-        if (c + 1 < h.nch) {
-            if (((c + 1) & 31) == 0)
-                h.mine = c + 1 + lane < h.nch ? __ldcg(tab + (size_t)kListChunks * id + c + 1 + lane) : 0;
-            p = a.pool + (size_t)__shfl_sync(0xffffffffu, h.mine, (c + 1) & 31) * kListChunkBytes;
-            load_entries(h.E, p, 0, lane);
+// Tiles of one side (block 0: rows, 1: columns) by descending weight of their
+// longest slice, so that a pass that does not hold them all at once starts its
+// longest ones first: a counting sort by one CTA.
+template <int ROW_TILE, int COL_TILE>
+__global__ void __launch_bounds__(1024) sk_order_kernel(SkArgs a) {
+    __shared__ int count[257];
+    const bool rows = blockIdx.x == 0;
+    const int n = a.ctrl[rows ? CTRL_N_ROW_TILES : CTRL_N_COL_TILES], per = (rows ? ROW_TILE : COL_TILE) / 32;
+    const SliceDesc* desc = (const SliceDesc*)(rows ? a.row_desc : a.col_desc);
+    int* order = rows ? a.row_order : a.col_order;
+    auto bucket = [&](int k) {
+        int w = 0;
+        for (int q = 0; q < per; ++q) w = max(w, desc[k * per + q].weight);
+        return 256 - min(255, w);
+    };
+    for (int k = threadIdx.x; k < 257; k += blockDim.x) count[k] = 0;
+    __syncthreads();
+    for (int k = threadIdx.x; k < n; k += blockDim.x) atomicAdd(&count[bucket(k)], 1);
+    __syncthreads();
+    if (threadIdx.x < 32) {  // exclusive prefix, eight buckets to a lane
+        int c[8], sum = 0;
+        for (int k = 0; k < 8; ++k) {
+            c[k] = count[1 + 8 * threadIdx.x + k];
+            sum += c[k];
         }
-        fn(N);
+        int incl = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if ((int)threadIdx.x >= o) incl += y;
+        }
+        int at = incl - sum;
+        for (int k = 0; k < 8; ++k) {
+            count[1 + 8 * threadIdx.x + k] = at;
+            at += c[k];
+        }
     }
+    __syncthreads();
+    for (int k = threadIdx.x; k < n; k += blockDim.x) order[atomicAdd(&count[bucket(k)], 1)] = k;
+}
+
+// ---------------------------------------------------- entries of a listed slice
+// A chunk in memory: the costs of 8 entries of each of the 64 spots, then their slots.
+struct Chunk {
+    float2 e2[kListDepth][32];      // of the lane's spots a and b
+    unsigned slot[kListDepth][32];  // a in the low half, b in the high half
+};
+static_assert(sizeof(Chunk) == kListChunkBytes, "laid out by the host");
+
+// A warp's ring of chunks in shared memory, filled by cp.async: the lists are
+// read once per pass, from HBM at the 1000-grain density, so the next chunks
+// are in flight while one is used.  The first ones are asked for before the
+// pass waits for the one before it.
+constexpr int kRing = 3;
+struct Ring {
+    Chunk c[kRing];
+};
+
+// The lane's share of a slice's chunk numbers [32 k, 32 k + 32).
+__device__ __forceinline__ int chunk_numbers(const SkArgs& a, const int* tab, int id, int lane, int k) {
+    return a.pool_chunks > 0 ? __ldcg(tab + (size_t)kListChunks * id + 32 * k + lane) : 0;
+}
+
+__device__ __forceinline__ void ring_fill(const SkArgs& a, Ring& R, int c, int nch, int number, int lane) {
+    if (c < nch) {
+        const char* src = a.pool + (size_t)number * kListChunkBytes + 16 * lane;
+        char* dst = (char*)&R.c[c % kRing] + 16 * lane;
+#pragma unroll
+        for (int k = 0; k < (int)kListChunkBytes / 512; ++k) cp16(dst + 512 * k, src + 512 * k);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// numbers: the lane's share of the first 32 chunk numbers
+__device__ __forceinline__ void ring_start(const SkArgs& a, Ring& R, const Slice& sl, int numbers) {
+#pragma unroll
+    for (int c = 0; c < kRing - 1; ++c) ring_fill(a, R, c, sl.nch, __shfl_sync(0xffffffffu, numbers, c), sl.lane);
+}
+
+// fn(chunk) for every chunk of the slice, in order.
+template <class Fn>
+__device__ __forceinline__ void for_each_chunk(const SkArgs& a, Ring& R, const int* tab, const Slice& sl, int numbers,
+                                               Fn fn) {
+    for (int c = 0; c < sl.nch; ++c) {
+        const int ahead = c + kRing - 1;
+        if ((ahead & 31) == 0 && ahead < sl.nch) numbers = chunk_numbers(a, tab, sl.id, sl.lane, ahead >> 5);
+        ring_fill(a, R, ahead, sl.nch, __shfl_sync(0xffffffffu, numbers, ahead & 31), sl.lane);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 1) : "memory");
+        __syncwarp();
+        fn(R.c[c % kRing]);
+        __syncwarp();
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
 // Sums of 2^(pot_slot - shift - K e2) over a listed slice's entries for the
@@ -479,25 +537,29 @@ struct ListSum {
 };
 
 template <bool GATHER_K>
-__device__ __forceinline__ void list_sum(const SkArgs& a, ListHead& h, const int* tab, int id, int lane, const float* pot,
-                                         float shift, float ka, float kb, const float4* modW, ListSum& S) {
-    for_each_half(a, h, tab, id, lane, [&](const Entries& E) {
-        float pa[kHalf], pb[kHalf];
+__device__ __forceinline__ void list_sum(const SkArgs& a, Ring& R, const int* tab, const Slice& sl, int numbers,
+                                         const float* pot, float shift, float ka, float kb, const float4* modW,
+                                         ListSum& S) {
+    for_each_chunk(a, R, tab, sl, numbers, [&](const Chunk& C) {
+        float pa[kListDepth], pb[kListDepth];
 #pragma unroll
-        for (int k = 0; k < kHalf; ++k) {
-            pa[k] = pot[E.slot[k] & 0xffffu];
-            pb[k] = pot[E.slot[k] >> 16];
+        for (int k = 0; k < kListDepth; ++k) {
+            const unsigned s = C.slot[k][sl.lane];
+            pa[k] = pot[s & 0xffffu];
+            pb[k] = pot[s >> 16];
         }
 #pragma unroll
-        for (int k = 0; k < kHalf; ++k) {
+        for (int k = 0; k < kListDepth; ++k) {
+            const unsigned s = C.slot[k][sl.lane];
+            const float2 e2 = C.e2[k][sl.lane];
             if (GATHER_K) {
-                const unsigned ja = E.slot[k] & 0xffffu, jb = E.slot[k] >> 16;
+                const unsigned ja = s & 0xffffu, jb = s >> 16;
                 const float2 wa = *((const float2*)&modW[ja >> 1] + 1), wb = *((const float2*)&modW[jb >> 1] + 1);
                 ka = ja & 1u ? wa.y : wa.x;
                 kb = jb & 1u ? wb.y : wb.x;
             }
-            const float ta = ex2(fmaf(E.e2[k].x, ka, pa[k] - shift)), tb = ex2(fmaf(E.e2[k].y, kb, pb[k] - shift));
-            const bool oa = E.slot[k] & 1u, ob = E.slot[k] & 0x10000u;
+            const float ta = ex2(fmaf(e2.x, ka, pa[k] - shift)), tb = ex2(fmaf(e2.y, kb, pb[k] - shift));
+            const bool oa = s & 1u, ob = s & 0x10000u;
             S.ea += oa ? 0.0f : ta;
             S.oa += oa ? ta : 0.0f;
             S.eb += ob ? 0.0f : tb;
@@ -538,15 +600,13 @@ __device__ __forceinline__ Sweep sweep_of(const SkArgs& a, const Slice& sl) {
         w.own = load_cone(a.obs_cone, a.obs_ext, a.obs_gbase[t] + (first - a.I2_off[t]) / kGran);
         w.sub = a.mod_sub + (size_t)kSubs * a.mod_gbase[t];
         w.ext = a.mod_subext + (size_t)kSubs * a.mod_gbase[t];
-        w.b0 = a.J2_off[t];
-        w.n = a.J2_off[t + 1] - w.b0;
     } else {
         w.own = load_cone(a.mod_cone, a.mod_ext, a.mod_gbase[t] + (first - a.J2_off[t]) / kGran);
         w.sub = a.obs_sub + (size_t)kSubs * a.obs_gbase[t];
         w.ext = a.obs_subext + (size_t)kSubs * a.obs_gbase[t];
-        w.b0 = a.I2_off[t];
-        w.n = a.I2_off[t + 1] - w.b0;
     }
+    w.b0 = sl.s0;
+    w.n = sl.ns;
     return w;
 }
 
@@ -650,26 +710,26 @@ __device__ __forceinline__ float final_col_max(const SkArgs& a, const DustPtrs& 
     return n_iter > 0 ? angle_max(col_max(a, n_iter - 1), t, 0.0f) : D.Gmax[t];
 }
 
-// Lanes' partial log-sum-exps of a CTA's tiles into part[tile] and the angle
-// maxima: the warps of a tile in order.
+// Lanes' partial log-sum-exps of a tile into part[tile], its warps in order,
+// and the angle's maximum.  Only the tile's own warps meet here.
 template <int TILE>
-__device__ __forceinline__ void store_parts(float m, float s, const Slice& sl, int n_tiles, float2* part, unsigned* maxima,
-                                            float* sm, float* ss) {
+__device__ __forceinline__ void store_part(float m, float s, int tile, int t, float2* part, unsigned* maxima, float* sm,
+                                           float* ss) {
     constexpr int kW = TILE / 32;
     const int warp = threadIdx.x >> 5;
     warp_lse_reduce(m, s);
-    if (sl.lane == 0) {
+    if ((threadIdx.x & 31) == 0) {
         sm[warp] = m;
         ss[warp] = s;
     }
-    __syncthreads();
-    if (sl.lane == 0 && sl.w == 0 && sl.tile < n_tiles) {
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + warp / kW), "n"(TILE) : "memory");
+    if ((int)threadIdx.x % TILE == 0) {
         Lse2 L;
         L.m = kNegHuge;
         L.s = 0.0f;
         for (int k = 0; k < kW; ++k) L.merge(sm[warp + k], ss[warp + k]);
-        part[sl.tile] = make_float2(L.m, L.s);
-        if (L.m > kNegHuge) atomicMax(maxima + sl.t, max_code(L.m));
+        part[tile] = make_float2(L.m, L.s);
+        if (L.m > kNegHuge) atomicMax(maxima + t, max_code(L.m));
     }
 }
 
@@ -695,7 +755,7 @@ __device__ __forceinline__ bool last_block(int* done, int* flag) {
 template <int TILE, int THREADS>
 __device__ void merge_parts(const float2* part, int n, float& m_out, float& s_out, float* sm, float* ss,
                             float (*segmax)[TILE], float* cm, float* cs) {
-    constexpr int kSeg = THREADS / TILE, kR = 16;
+    constexpr int kSeg = THREADS / TILE, kR = 8;
     const int c = threadIdx.x % TILE, seg = threadIdx.x / TILE;
     if (seg == 0) {
         cm[c] = kNegHuge;
@@ -786,7 +846,11 @@ __device__ __forceinline__ void warp_merge_parts(const float2* part, int first, 
 
 template <int TILE, int THREADS = pass_threads(TILE)>
 struct PassShared {
-    WarpStage stage[THREADS / 32];
+    union Warp {
+        WarpStage stage;
+        Ring ring;
+    };
+    Warp w[THREADS / 32];
     float sm[THREADS / 32], ss[THREADS / 32];
     float segmax[THREADS / TILE][TILE];
     float cm[TILE], cs[TILE];
@@ -885,23 +949,22 @@ __global__ void __launch_bounds__(pass_threads(TILE, OTHER), 1024 / pass_threads
             finish_pass<OTHER, kThreads, !ROWS>(a, *(PassShared<OTHER, kThreads>*)pass_smem, blockIdx.x, finishers, clear);
         return;
     }
-    DustPtrs D = dust_ptrs(a.dust, a.T);
-    const int n_tiles = __ldcg(a.ctrl + (ROWS ? CTRL_N_ROW_TILES : CTRL_N_COL_TILES));
-    const int4* tiles = ROWS ? a.row_tiles : a.col_tiles;
-    const Slice sl = slice_of<TILE>(tiles, n_tiles, blockIdx.x - finishers);
-    const int t = sl.t, lane = sl.lane;
+    const SliceDesc* desc = (const SliceDesc*)(ROWS ? a.row_desc : a.col_desc);
     const int* tab = ROWS ? a.row_tab : a.col_tab;
-    ListHead h;
-    h.nch = 0;
-    if (sl.n_own > 0) h = list_head(a, ROWS ? a.row_hdr : a.col_hdr, tab, sl.id, lane);
-    const int* own_off = ROWS ? a.I_off : a.J_off;
-    const int* own2 = ROWS ? a.I2_off : a.J2_off;
-    const int* str2 = ROWS ? a.J2_off : a.I2_off;
-    const bool vb = sl.valid && 2 * (sl.q - own2[t]) + 1 < own_off[t + 1] - own_off[t];
-    const int s0 = str2[t], ns = str2[t + 1] - s0;
+    constexpr int kW = TILE / 32;
+    const int at = (blockIdx.x - finishers) * (kThreads / TILE) + (int)threadIdx.x / TILE;
+    if (at >= __ldcg(a.ctrl + (ROWS ? CTRL_N_ROW_TILES : CTRL_N_COL_TILES))) return;
+    typename PassShared<TILE, kThreads>::Warp& M = H.w[threadIdx.x >> 5];
+    const int* order = ROWS ? a.row_order : a.col_order;
+    const int tile = order ? __ldcg(order + at) : at, id = tile * kW + (threadIdx.x >> 5) % kW;
+    const int numbers = chunk_numbers(a, tab, id, threadIdx.x & 31, 0);
+    const Slice sl = load_slice(desc, id);
+    ring_start(a, M.ring, sl, numbers);
+    const int t = sl.t, lane = sl.lane;
     float2 K = make_float2(a.negKD2, a.negKD2);  // -K of the lane's own spots (columns)
     if (!ROWS && sl.valid) K = *((const float2*)&a.modW[sl.q] + 1);
-    if (!vb) K.y = -1.0f;
+    if (!sl.vb) K.y = -1.0f;
+    const DustPtrs D = dust_ptrs(a.dust, a.T);
     const float* pot = ROWS ? a.Gc : a.Fc;
     float* out = ROWS ? a.Fc : a.Gc;
     if (!(ROWS && it == 0)) pass_wait();
@@ -909,7 +972,7 @@ __global__ void __launch_bounds__(pass_threads(TILE, OTHER), 1024 / pass_threads
     const bool ub = a.mode == 2;  // unbalanced OT: no dustbins, scaled update
     const int d = a.mode ? t : 0;
     float pm = kNegHuge, ps = 0.0f;
-    if (sl.n_own > 0) {
+    if (sl.any) {
         // the dustbin's term: the outlier column (rows), the unmatched-model row with C_0j = 0 (columns)
         const float dust = ub ? kNegHuge : ROWS ? __ldcg(D.G0 + d) - a.kc : __ldcg(D.F0n + d);
         const float top = ROWS ? (it > 0 ? angle_max(col_max(a, it - 1), t, 0.0f) : D.Gmax[t])
@@ -917,19 +980,19 @@ __global__ void __launch_bounds__(pass_threads(TILE, OTHER), 1024 / pass_threads
         const float shift = ub ? top : fmaxf(top, dust);
         const float e0 = ub ? 0.0f : ex2(dust - shift);
         ListSum S{e0, 0.0f, e0, 0.0f};
-        if (h.nch < 0)
-            swept_sum<ROWS>(a, H.stage[threadIdx.x >> 5], sl, shift, S);
+        if (sl.nch < 0)
+            swept_sum<ROWS>(a, M.stage, sl, shift, S);
         else if (!ROWS || a.uniK)
-            list_sum<false>(a, h, tab, sl.id, lane, pot + 2 * s0, shift, K.x, ROWS ? a.negKD2 : K.y, nullptr, S);
+            list_sum<false>(a, M.ring, tab, sl, numbers, pot + 2 * sl.s0, shift, K.x, ROWS ? a.negKD2 : K.y, nullptr, S);
         else
-            list_sum<ROWS>(a, h, tab, sl.id, lane, pot + 2 * s0, shift, 0.0f, 0.0f, a.modW + s0, S);
+            list_sum<ROWS>(a, M.ring, tab, sl, numbers, pot + 2 * sl.s0, shift, 0.0f, 0.0f, a.modW + sl.s0, S);
         const float sa = S.ea + S.oa, sb = S.eb + S.ob;
-        float va = -(shift + lg2(sa)), vv = vb ? -(shift + lg2(sb)) : 0.0f;
+        float va = -(shift + lg2(sa)), vv = sl.vb ? -(shift + lg2(sb)) : 0.0f;
         const unsigned low_a = __ballot_sync(0xffffffffu, sl.valid && !(sa > kTinySum));
-        const unsigned low_b = __ballot_sync(0xffffffffu, vb && !(sb > kTinySum));
+        const unsigned low_b = __ballot_sync(0xffffffffu, sl.vb && !(sb > kTinySum));
         if (low_a | low_b) {
             float xa, xb;
-            exact_lse<ROWS>(a, H.stage[threadIdx.x >> 5], sl, dust, xa, xb);
+            exact_lse<ROWS>(a, M.stage, sl, dust, xa, xb);
             if ((low_a >> lane) & 1u) va = -xa;
             if ((low_b >> lane) & 1u) vv = -xb;
             if (lane == 0)
@@ -939,19 +1002,19 @@ __global__ void __launch_bounds__(pass_threads(TILE, OTHER), 1024 / pass_threads
         if (sl.valid) {
             if (ub) {  // Algorithm UnbalancedOT: the balanced update raised to kappa / (kappa + eps)
                 const float tau = ROWS ? a.tau_row : a.tau_col;
-                va = ns > 0 ? tau * va : 0.0f;
-                vv = ns > 0 ? tau * vv : 0.0f;
+                va = sl.ns > 0 ? tau * va : 0.0f;
+                vv = sl.ns > 0 ? tau * vv : 0.0f;
             }
-            *(float2*)&out[2 * (size_t)sl.q] = make_float2(va, vb ? vv : kNegHuge);
+            *(float2*)&out[2 * (size_t)sl.q] = make_float2(va, sl.vb ? vv : kNegHuge);
             // tile partial of LSE2(F_i - kc) for the outlier column, of LSE2(G_j) for the unmatched row
             const float off = ROWS ? a.kc : 0.0f;
             pm = va - off;
             ps = 1.0f;
-            if (vb) lse_merge_into(pm, ps, vv - off, 1.0f);
+            if (sl.vb) lse_merge_into(pm, ps, vv - off, 1.0f);
         }
     }
-    store_parts<TILE>(pm, ps, sl, n_tiles, ROWS ? a.row_part : a.col_part, ROWS ? row_max(a, it) : col_max(a, it), H.sm,
-                      H.ss);
+    // the tile's first slice is never empty: its angle is the tile's
+    store_part<TILE>(pm, ps, tile, t, ROWS ? a.row_part : a.col_part, ROWS ? row_max(a, it) : col_max(a, it), H.sm, H.ss);
 }
 
 // ------------------------------------------------------------- read-out
@@ -1073,13 +1136,16 @@ __global__ void __launch_bounds__(pass_threads(TILE), 1024 / pass_threads(TILE))
     extern __shared__ __align__(128) char pass_smem[];
     PassShared<TILE>& H = *(PassShared<TILE>*)pass_smem;
     DustPtrs D = dust_ptrs(a.dust, a.T);
-    const Slice sl = slice_of<TILE>(a.row_tiles, a.ctrl[CTRL_N_ROW_TILES], blockIdx.x);
+    const SliceDesc* desc = (const SliceDesc*)a.row_desc;
+    const int at = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+    Slice sl{};
+    if (at < slice_count<TILE>(a, true)) sl = load_slice(desc, at);
     const int t = sl.t, lane = sl.lane;
     float my_err = 0.0f;
-    if (sl.n_own > 0) {
-        WarpStage& S = H.stage[threadIdx.x >> 5];
+    if (sl.any) {
+        typename PassShared<TILE>::Warp& M = H.w[threadIdx.x >> 5];
         const int lrow = 2 * (sl.q - a.I2_off[t]);
-        const bool vb = sl.valid && lrow + 1 < a.I_off[t + 1] - a.I_off[t];
+        const bool vb = sl.vb;
         const int jbase = a.J_off[t], j0 = a.J2_off[t];
         const float dustv = a.mode == 2 ? kNegHuge : D.G0[a.mode ? t : 0] - a.kc;
         Top2 A, B;
@@ -1087,9 +1153,9 @@ __global__ void __launch_bounds__(pass_threads(TILE), 1024 / pass_threads(TILE))
         B.init();
         const RowPair R = load_row_pair(a, sl.q, sl.valid);
         auto sweep_all = [&](int skip) {
-            for_each_swept<true>(a, S, sl, skip, [&](int st, int j, float2 P, int k) {
+            for_each_swept<true>(a, M.stage, sl, skip, [&](int st, int j, float2 P, int k) {
                 f2 va, vv;
-                row_pair_v(R, S, st, j, pk(P.x, P.y), va, vv);
+                row_pair_v(R, M.stage, st, j, pk(P.x, P.y), va, vv);
                 const int at = jbase + 2 * k;
                 if (!sl.valid) return;
                 A.add(lo(va), at, a.mod_perm);
@@ -1098,20 +1164,21 @@ __global__ void __launch_bounds__(pass_threads(TILE), 1024 / pass_threads(TILE))
                 B.add(hi(vv), at + 1, a.mod_perm);
             });
         };
-        ListHead h = list_head(a, a.row_hdr, a.row_tab, sl.id, lane);
-        if (h.nch >= 0) {
+        if (sl.nch >= 0) {
             const float* pot = a.Gc + 2 * j0;
-            for_each_half(a, h, a.row_tab, sl.id, lane, [&](const Entries& E) {
-#pragma unroll
-                for (int k = 0; k < kHalf; ++k) {
-                    const int ja = E.slot[k] & 0xffffu, jb = E.slot[k] >> 16;
+            const int numbers = chunk_numbers(a, a.row_tab, sl.id, lane, 0);
+            ring_start(a, M.ring, sl, numbers);
+            for_each_chunk(a, M.ring, a.row_tab, sl, numbers, [&](const Chunk& E) {
+                for (int k = 0; k < kListDepth; ++k) {
+                    const int ja = E.slot[k][lane] & 0xffffu, jb = E.slot[k][lane] >> 16;
+                    const float2 e2 = E.e2[k][lane];
                     float ka = a.negKD2, kb = a.negKD2;
                     if (!a.uniK) {
                         ka = ((const float*)&a.modW[j0 + (ja >> 1)])[2 + (ja & 1)];
                         kb = ((const float*)&a.modW[j0 + (jb >> 1)])[2 + (jb & 1)];
                     }
-                    if (is_entry(E.e2[k].x)) A.add(fmaf(E.e2[k].x, ka, pot[ja]), jbase + ja, a.mod_perm);
-                    if (is_entry(E.e2[k].y)) B.add(fmaf(E.e2[k].y, kb, pot[jb]), jbase + jb, a.mod_perm);
+                    if (is_entry(e2.x)) A.add(fmaf(e2.x, ka, pot[ja]), jbase + ja, a.mod_perm);
+                    if (is_entry(e2.y)) B.add(fmaf(e2.y, kb, pot[jb]), jbase + jb, a.mod_perm);
                 }
             });
         } else {
@@ -1181,13 +1248,16 @@ __global__ void __launch_bounds__(pass_threads(TILE), 1024 / pass_threads(TILE))
     extern __shared__ __align__(128) char pass_smem[];
     PassShared<TILE>& H = *(PassShared<TILE>*)pass_smem;
     DustPtrs D = dust_ptrs(a.dust, a.T);
-    const Slice sl = slice_of<TILE>(a.col_tiles, a.ctrl[CTRL_N_COL_TILES], blockIdx.x);
+    const SliceDesc* desc = (const SliceDesc*)a.col_desc;
+    const int at = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+    Slice sl{};
+    if (at < slice_count<TILE>(a, false)) sl = load_slice(desc, at);
     const int t = sl.t, lane = sl.lane;
     float my_err = 0.0f;
-    if (sl.n_own > 0) {
-        WarpStage& S = H.stage[threadIdx.x >> 5];
+    if (sl.any) {
+        typename PassShared<TILE>::Warp& M = H.w[threadIdx.x >> 5];
         const int lcol = 2 * (sl.q - a.J2_off[t]);
-        const bool vb = sl.valid && lcol + 1 < a.J_off[t + 1] - a.J_off[t];
+        const bool vb = sl.vb;
         const int i0 = a.I2_off[t];
         const float F0 = a.mode == 2 ? kNegHuge : D.F0[a.mode ? t : 0];
         Lse2 A, B;
@@ -1204,24 +1274,26 @@ __global__ void __launch_bounds__(pass_threads(TILE), 1024 / pass_threads(TILE))
         ColPair C;
         load_col_pair(a, sl.valid ? sl.q : sl.q - lane, C);
         auto sweep_all = [&](int skip) {
-            for_each_swept<false>(a, S, sl, skip, [&](int st, int j, float2 P, int) {
+            for_each_swept<false>(a, M.stage, sl, skip, [&](int st, int j, float2 P, int) {
                 f2 va, vv;
-                col_pair_v(C, S, st, j, pk(P.x, P.y), va, vv);
+                col_pair_v(C, M.stage, st, j, pk(P.x, P.y), va, vv);
                 add(A, lo(va));
                 add(A, hi(va));
                 add(B, lo(vv));
                 add(B, hi(vv));
             });
         };
-        ListHead h = list_head(a, a.col_hdr, a.col_tab, sl.id, lane);
-        if (h.nch >= 0) {
+        if (sl.nch >= 0) {
             const float* pot = a.Fc + 2 * i0;
             const float ka = lo(C.ka), kb = lo(C.kb);
-            for_each_half(a, h, a.col_tab, sl.id, lane, [&](const Entries& E) {
-#pragma unroll
-                for (int k = 0; k < kHalf; ++k) {
-                    if (is_entry(E.e2[k].x)) add(A, fmaf(E.e2[k].x, ka, pot[E.slot[k] & 0xffffu]));
-                    if (is_entry(E.e2[k].y)) add(B, fmaf(E.e2[k].y, kb, pot[E.slot[k] >> 16]));
+            const int numbers = chunk_numbers(a, a.col_tab, sl.id, lane, 0);
+            ring_start(a, M.ring, sl, numbers);
+            for_each_chunk(a, M.ring, a.col_tab, sl, numbers, [&](const Chunk& E) {
+                for (int k = 0; k < kListDepth; ++k) {
+                    const unsigned s = E.slot[k][lane];
+                    const float2 e2 = E.e2[k][lane];
+                    if (is_entry(e2.x)) add(A, fmaf(e2.x, ka, pot[s & 0xffffu]));
+                    if (is_entry(e2.y)) add(B, fmaf(e2.y, kb, pot[s >> 16]));
                 }
             });
         } else {
@@ -1278,6 +1350,21 @@ cudaError_t with_tiles(const SkLaunch& l, Fn fn) {
     return with_tile(l.row_variant, [&](auto row) { return with_tile(l.col_variant, [&](auto col) { return fn(row, col); }); });
 }
 
+// Once per device (the current one), before the first launch.
+template <int A, int B>
+cudaError_t allow_smem() {
+    constexpr int thr = pass_threads(A, B);
+    const int n = (int)std::max(sizeof(PassShared<A, thr>), sizeof(PassShared<B, thr>));
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(sk_pass_kernel<A, B, true>, at, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_pass_kernel<A, B, false>, at, n);
+    if (A != B || e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(sk_harvest_row_kernel<A>, at, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_harvest_col_kernel<A>, at, n);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_finish_pass_kernel<A>, at, n);
+    return e;
+}
+
 template <class... Params, class... Args>
 cudaError_t launch_pass(void (*k)(Params...), int ctas, int threads, size_t smem, bool overlap, cudaStream_t s,
                         Args... args) {
@@ -1294,10 +1381,10 @@ cudaError_t launch_pass(void (*k)(Params...), int ctas, int threads, size_t smem
     return cudaLaunchKernelEx(&c, k, args...);
 }
 
-// CTAs that hold a side's tiles.
-int tile_ctas(int T, int n_spots, int tile, int threads) {
-    const int per = threads / tile, tiles = T + n_spots / 2 / tile + 1;
-    return (tiles + per - 1) / per;
+// CTAs that hold a side's slices.
+int slice_ctas(int T, int n_spots, int tile, int threads) {
+    const int per = threads / 32;
+    return ((int)list_slices(T, n_spots, tile) + per - 1) / per;
 }
 
 template <int TILE, int OTHER, bool ROWS>
@@ -1305,13 +1392,22 @@ cudaError_t run_pass(const SkArgs& a, int it, cudaStream_t s) {
     constexpr int thr = pass_threads(TILE, OTHER);
     constexpr size_t own = sizeof(PassShared<TILE, thr>), other = sizeof(PassShared<OTHER, thr>);
     constexpr size_t smem = own > other ? own : other;
-    static_assert(smem <= 48 * 1024, "beyond the shared memory of a plain launch");
     const int fin = finish_blocks(a.mode, a.T, thr);
-    return launch_pass(sk_pass_kernel<TILE, OTHER, ROWS>, fin + tile_ctas(a.T, ROWS ? a.n_obs : a.n_model, TILE, thr), thr,
+    return launch_pass(sk_pass_kernel<TILE, OTHER, ROWS>, fin + slice_ctas(a.T, ROWS ? a.n_obs : a.n_model, TILE, thr), thr,
                        smem, true, s, a, it, fin);
 }
 
 }  // namespace
+
+cudaError_t sinkhorn_setup() {
+    cudaError_t e = cudaSuccess;
+    for (int r = 0; r < kSkVariants && e == cudaSuccess; ++r)
+        for (int c = 0; c < kSkVariants && e == cudaSuccess; ++c)
+            e = with_tile(r, [&](auto row) {
+                return with_tile(c, [&](auto col) { return allow_smem<decltype(row)::value, decltype(col)::value>(); });
+            });
+    return e;
+}
 
 cudaError_t sinkhorn_row_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s) {
     return with_tiles(l, [&](auto row, auto col) {
@@ -1342,13 +1438,11 @@ cudaError_t sinkhorn_iterate(const SkArgs& a, const SkLaunch& l, int n_iter, cud
 
 cudaError_t sinkhorn_build_lists(const SkArgs& a, const SkLaunch& l, cudaStream_t s) {
     const int rg = (l.row_slices + kListWarps - 1) / kListWarps, cg = (l.col_slices + kListWarps - 1) / kListWarps;
-    cudaError_t e = with_tile(l.row_variant, [&](auto tile) {
-        sk_list_kernel<decltype(tile)::value, true><<<rg, 32 * kListWarps, 0, s>>>(a);
-        return cudaGetLastError();
-    });
-    if (e != cudaSuccess) return e;
-    return with_tile(l.col_variant, [&](auto tile) {
-        sk_list_kernel<decltype(tile)::value, false><<<cg, 32 * kListWarps, 0, s>>>(a);
+    return with_tiles(l, [&](auto row, auto col) {
+        constexpr int rt = decltype(row)::value, ct = decltype(col)::value;
+        sk_list_kernel<rt, true><<<rg, 32 * kListWarps, 0, s>>>(a);
+        sk_list_kernel<ct, false><<<cg, 32 * kListWarps, 0, s>>>(a);
+        if (a.row_order) sk_order_kernel<rt, ct><<<2, 1024, 0, s>>>(a);
         return cudaGetLastError();
     });
 }
@@ -1359,13 +1453,13 @@ cudaError_t sinkhorn_harvest(const SkArgs& a, const SkLaunch& l, int n_iter, boo
     if (want_rows)
         e = with_tile(l.row_variant, [&](auto tile) {
             constexpr int t = decltype(tile)::value;
-            return launch_pass(sk_harvest_row_kernel<t>, tile_ctas(a.T, a.n_obs, t, pass_threads(t)), pass_threads(t),
+            return launch_pass(sk_harvest_row_kernel<t>, slice_ctas(a.T, a.n_obs, t, pass_threads(t)), pass_threads(t),
                                sizeof(PassShared<t>), false, s, a, n_iter);
         });
     if (e == cudaSuccess && want_cols)
         e = with_tile(l.col_variant, [&](auto tile) {
             constexpr int t = decltype(tile)::value;
-            return launch_pass(sk_harvest_col_kernel<t>, tile_ctas(a.T, a.n_model, t, pass_threads(t)), pass_threads(t),
+            return launch_pass(sk_harvest_col_kernel<t>, slice_ctas(a.T, a.n_model, t, pass_threads(t)), pass_threads(t),
                                sizeof(PassShared<t>), false, s, a, n_iter);
         });
     return e;

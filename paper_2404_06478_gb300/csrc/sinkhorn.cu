@@ -128,7 +128,6 @@ __global__ void __launch_bounds__(1024) sk_schedule_kernel(SkArgs a) {
                 a.col_tiles[idx] = make_int4(t, j0 + k * a.tile_cols, min(a.tile_cols, nj - k * a.tile_cols), 0);
         }
     }
-    for (int u = threadIdx.x; u < 4 * T; u += blockDim.x) a.pmax[u] = 0u;
     // dustbin masses (paper: T_a = T_b - b^T 1 + a^T 1), in double precision
     DustPtrs D = dust_ptrs(a.dust, T);
     int nd = a.mode ? T : 1;
@@ -382,6 +381,7 @@ __global__ void __launch_bounds__(256) sk_cone_kernel(SkArgs a) {
 __global__ void sk_pack_kernel(SkArgs a) {
     const float s = 1.0f / a.to_user;  // mm^2 -> base-2 internal units
     int k = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int u = k; u < 4 * a.T; u += gridDim.x * blockDim.x) a.pmax[u] = 0u;
     if (k < a.n_obs) {
         int t = block_of(a.I_off, a.T, k);
         int l = a.obs_pos[k];  // rank of the spot in its block's spatial order
