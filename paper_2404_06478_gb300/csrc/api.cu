@@ -566,9 +566,6 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
     a.warm = prm->warm_start ? 1 : 0;
     lc->row_variant = h->row_variant;
     lc->col_variant = h->col_variant;
-    // the M-step pair kernel runs one thread per column pair of the column
-    // pass's tiles (narrow tiles skip more), about 768 threads per SM
-    lc->col_grid = std::max(1, std::min(h->sm_count * (768 / a.tile_cols), L.max_col_tiles));
     // pair lists in the workspace beyond the layout (skipping off: every pair is evaluated)
     size_t from = align_up(std::max(L.total, list_from), 256);
     size_t fixed = list_fixed_bytes(a.T, a.n_obs, a.n_model, a.tile_rows, a.tile_cols);
@@ -814,9 +811,9 @@ extern "C" int laue_autotune(laue_handle* h, const LaueGeometry* geom, const Lau
 
 // ------------------------------------------------------------- not yet built
 
-static int mstep_entry(laue_handle* h, const LaueGeometry* geom, const LaueLattice* lat, const LaueObsSpots* obs,
+int laue_mstep_any(laue_handle* h, const LaueGeometry* geom, const LaueLattice* lat, const LaueObsSpots* obs,
                        const LaueModelSpots* model, const float* f, const float* g, const LaueMParams* prm,
-                       const float* omega, float* R, float* x, int N, float* step_norms, void* stream, bool adjoint) {
+                       const float* omega, float* R, float* x, int N, float* step_norms, void* stream, bool adjoint, bool sorted) {
     if (!h) return LAUE_ERR_INVALID_ARG;
     int rc;
     if ((rc = laue_check_geom(h, geom))) return rc;
@@ -825,6 +822,7 @@ static int mstep_entry(laue_handle* h, const LaueGeometry* geom, const LaueLatti
     if (obs->T != model->T) return laue_fail(h, LAUE_ERR_INVALID_ARG, "observed and model T differ");
     if (!prm || !(prm->eps > 0.0f) || prm->n_newton < 0 || prm->n_mm < 0)
         return laue_fail(h, LAUE_ERR_INVALID_ARG, "M-step params: eps > 0, n_newton >= 0, n_mm >= 0");
+    if (adjoint && !(prm->hreg >= 0.0f)) return laue_fail(h, LAUE_ERR_INVALID_ARG, "mstep_adjoint: hreg >= 0");
     if (!lat || lat->M < 1 || !lat->w_d0 || !aligned16(lat->w_d0))
         return laue_fail(h, LAUE_ERR_INVALID_ARG, "lattice: M >= 1 and aligned w_d0");
     if (N < 0 || (N > 0 && (!R || !x)) || !omega || (obs->n > 0 && !f) || (model->n > 0 && !g))
@@ -870,23 +868,22 @@ static int mstep_entry(laue_handle* h, const LaueGeometry* geom, const LaueLatti
         for (int k = 0; k < 4; ++k) m.D2det[k] = k < G.n_det ? G.Dd[k] * G.Dd[k] : m.D2;
     }
     if (adjoint)
-        return laue_cuda_check(h, mstep_adjoint_run(m, lc, prm->n_newton, (cudaStream_t)stream),
+        return laue_cuda_check(h, mstep_adjoint_run(m, lc, prm->n_newton, sorted, (cudaStream_t)stream),
                                "mstep_adjoint launch");
-    return laue_cuda_check(h, mstep_run(m, lc, (cudaStream_t)stream), "mstep launch");
+    return laue_cuda_check(h, mstep_run(m, lc, sorted, (cudaStream_t)stream), "mstep launch");
 }
 
 extern "C" int laue_mstep(laue_handle* h, const LaueGeometry* geom, const LaueLattice* lat, const LaueObsSpots* obs,
                           const LaueModelSpots* model, const float* f, const float* g, const LaueMParams* prm,
                           const float* omega, float* R, float* x, int N, float* step_norms, void* stream) {
-    return mstep_entry(h, geom, lat, obs, model, f, g, prm, omega, R, x, N, step_norms, stream, false);
+    return laue_mstep_any(h, geom, lat, obs, model, f, g, prm, omega, R, x, N, step_norms, stream, false, false);
 }
 
 extern "C" int laue_mstep_adjoint(laue_handle* h, const LaueGeometry* geom, const LaueLattice* lat,
                                   const LaueObsSpots* obs, const LaueModelSpots* model, const float* f,
                                   const float* g, const LaueMParams* prm, const float* omega, float* R, float* x,
                                   int N, float* step_norms, void* stream) {
-    if (prm && !(prm->hreg >= 0.0f)) return laue_fail(h, LAUE_ERR_INVALID_ARG, "mstep_adjoint: hreg >= 0");
-    return mstep_entry(h, geom, lat, obs, model, f, g, prm, omega, R, x, N, step_norms, stream, true);
+    return laue_mstep_any(h, geom, lat, obs, model, f, g, prm, omega, R, x, N, step_norms, stream, true, false);
 }
 
 extern "C" int laue_objective_grad(laue_handle* h, const LaueGeometry* geom, const LaueLattice* lat,

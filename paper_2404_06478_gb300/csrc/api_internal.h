@@ -27,3 +27,9 @@ int laue_need_ws(laue_handle* h, const LaueProblemDims& d, laue::Layout* L);
 int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* obs, const LaueModelSpots* model,
                  const LaueOTParams* prm, const laue::Layout& L, laue::SkArgs* out, laue::SkLaunch* lc,
                  size_t list_from = 0);
+// The M-steps of the ABI.  sorted: the call before on the handle and stream was
+// an E-step on the same spots, whose order, tiles and cones the workspace holds.
+int laue_mstep_any(laue_handle* h, const LaueGeometry* geom, const LaueLattice* lat, const LaueObsSpots* obs,
+                   const LaueModelSpots* model, const float* f, const float* g, const LaueMParams* prm,
+                   const float* omega, float* R, float* x, int N, float* step_norms, void* stream, bool adjoint,
+                   bool sorted);

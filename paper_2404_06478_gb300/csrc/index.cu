@@ -225,9 +225,8 @@ extern "C" int laue_em(laue_handle* h, const LaueGeometry* geom, const LaueLatti
         if (k == prm->n_em) break;  // the final E-step
         LaueMParams mp = prm->mstep;
         mp.eps = (float)eps;
-        rc = prm->mstep_kind == 1
-                 ? laue_mstep_adjoint(h, geom, lat, obs, model, f, g, &mp, omega, R, x, N, nullptr, stream)
-                 : laue_mstep(h, geom, lat, obs, model, f, g, &mp, omega, R, x, N, nullptr, stream);
+        rc = laue_mstep_any(h, geom, lat, obs, model, f, g, &mp, omega, R, x, N, nullptr, stream, prm->mstep_kind == 1,
+                            true);
         if (rc) return rc;
     }
     return LAUE_OK;

@@ -195,15 +195,17 @@ constexpr int kSkDefaultVariant = 3;  // 64-pair tiles: the autotuner's usual pi
 
 struct SkLaunch {
     int row_slices, col_slices;  // bound on the slices of each side
-    int col_grid;                // CTAs of the M-step's pair kernel
     int row_variant, col_variant;
 };
 
 cudaError_t sinkhorn_run(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols,
                          cudaStream_t s);
-cudaError_t sinkhorn_prepare(const SkArgs& a, cudaStream_t s);
+// Tiles, spatial order, pair copies, cones and starting dustbins (dustbins);
+// sorted: the workspace holds the order, tiles and cones of the same spots.
+cudaError_t sinkhorn_prepare(const SkArgs& a, cudaStream_t s, bool dustbins = true, bool sorted = false);
 cudaError_t sinkhorn_iterate(const SkArgs& a, const SkLaunch& l, int n_iter, cudaStream_t s);
 cudaError_t sinkhorn_finish(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols, cudaStream_t s);
+cudaError_t sinkhorn_list_plan(const SkArgs& a, const SkLaunch& l, cudaStream_t s);
 cudaError_t sinkhorn_harvest(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols,
                              cudaStream_t s);
 cudaError_t sinkhorn_setup();  // once per device, the current one
@@ -238,8 +240,9 @@ struct MsArgs {
     float* value;           // N (adjoint, optional)
 };
 
-cudaError_t mstep_run(const MsArgs& m, const SkLaunch& l, cudaStream_t s);
-cudaError_t mstep_adjoint_run(const MsArgs& m, const SkLaunch& l, int n_steps, cudaStream_t s);
+// sorted: straight after an E-step on the same spots and workspace
+cudaError_t mstep_run(const MsArgs& m, const SkLaunch& l, bool sorted, cudaStream_t s);
+cudaError_t mstep_adjoint_run(const MsArgs& m, const SkLaunch& l, int n_steps, bool sorted, cudaStream_t s);
 
 // ------------------------------------------------------- single-grain fits
 constexpr int kSfMaxT = 1024;       // angles a fit supports

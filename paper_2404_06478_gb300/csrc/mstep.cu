@@ -2,10 +2,11 @@
 // Appendix "M-steps for grain position and rotation", Algorithms
 // LauePosNewton, LaueRotMM and Wahba).
 //
-// The plan is never stored: Q_ij = 2^(F_i + G_j - K e2_ij) is recomputed from
-// the E-step potentials and the E-step rays/centres of the model list (the
-// pair-interleaved workspace copies made by the Sinkhorn pack kernel), pairs
-// with Q_ij < 2^-40 are skipped, and the geometric terms use the current
+// The plan Q_ij = 2^(F_i + G_j - K e2_ij) is that of the E-step's potentials
+// and rays/centres (the pair-interleaved workspace copies made by the Sinkhorn
+// pack kernel) for the whole M-step, so its entries of at least 2^-40 are
+// listed once per call (sk_list_kernel in passes.cu); slices without a list
+// recompute them in every pass.  The geometric terms use the current
 // positions.  Per model spot a pass over its angle block accumulates, in
 // registers:
 //   Newton  g_c = sum_i Q (-(r - (rhat.r) rhat) / tau)
@@ -19,12 +20,10 @@
 // M_m = M0_m + max(0, -lmin(M0_m)) I and R <- Wahba(M_m R w_m, w_m): the Wahba
 // step maximises tr(R^T B), B = sum a b^T, through the top eigenvector of
 // Horn's 4x4 symmetric matrix (a unit quaternion).
-#include "pairs.cuh"
+#include "slices.cuh"
 #include "mstep_common.cuh"
 
 namespace laue {
-
-constexpr float kQSkip = -40.0f;  // log2 of the smallest plan entry kept
 
 // ------------------------------------------------------- segment table
 // seg[t (N+1) + n] = first model spot of grain n at angle t (the list is sorted
@@ -35,17 +34,21 @@ __global__ void ms_seg_count_kernel(MsArgs m) {
     atomicAdd(&m.seg[m.angle[j] * (m.N + 1) + m.grain[j]], 1);
 }
 
-__global__ void ms_seg_scan_kernel(MsArgs m) {
-    int t = blockIdx.x;
-    if (threadIdx.x != 0) return;
+__global__ void ms_seg_scan_kernel(MsArgs m) {  // one warp per angle
+    const int t = blockIdx.x, lane = threadIdx.x;
     int* s = m.seg + t * (m.N + 1);
     int acc = m.J_off[t];
-    for (int n = 0; n < m.N; ++n) {
-        int c = s[n];
-        s[n] = acc;
-        acc += c;
+    for (int n0 = 0; n0 < m.N; n0 += 32) {
+        const int c = n0 + lane < m.N ? s[n0 + lane] : 0;
+        int incl = c;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (n0 + lane < m.N) s[n0 + lane] = acc + incl - c;
+        acc += __shfl_sync(0xffffffffu, incl, 31);
     }
-    s[m.N] = acc;
+    if (lane == 0) s[m.N] = acc;
 }
 
 __global__ void ms_init_kernel(MsArgs m) {
@@ -72,9 +75,7 @@ struct MsCol {
     float acc[10];
 };
 
-__device__ __forceinline__ void ms_pair(MsCol& C, int mode, float px, float py, float pz, float v) {
-    if (!C.ok || v < kQSkip) return;
-    float Q = ex2(v);
+__device__ __forceinline__ void ms_pair(MsCol& C, int mode, float px, float py, float pz, float Q) {
     float d0 = px - C.c[0], d1 = py - C.c[1], d2 = pz - C.c[2];
     float is = rsqrtf(fmaf(d0, d0, fmaf(d1, d1, d2 * d2)));
     float h0 = d0 * is, h1 = d1 * is, h2 = d2 * is;
@@ -118,188 +119,164 @@ __device__ __forceinline__ void ms_pair(MsCol& C, int mode, float px, float py, 
         }
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(kTPB) ms_pair_kernel(MsArgs m) {
+// One warp per slice of 32 model spot pairs, each lane summing over two of
+// them.  Bound by the gathers of the listed entries' positions.  At 300 grains
+// x 90 angles, 1 mm^2, a pass took 447 us when it evaluated every pair that
+// the cones let through; listing the plan takes 279 us once and a pass 27 us.
+constexpr int kMsThreads = 128;
+
+template <int TILE, int MODE>
+__global__ void __launch_bounds__(kMsThreads) ms_pair_kernel(MsArgs m) {
     const SkArgs& a = m.sk;
-    __shared__ __align__(128) Stage S;
-    init_stage(S);
-    uint32_t parity[2] = {0u, 0u};
-    const int n_tiles = a.ctrl[CTRL_N_COL_TILES];
-    const Srcs src{{a.obsX, a.obsY, nullptr, nullptr}, 2};
-    while (true) {
-        int tile = next_tile(S, a.ctrl + CTRL_GEN_NEXT, n_tiles);
-        if (tile < 0) break;
-        int4 td = a.col_tiles[tile];
-        int t = td.x;
-        int q = td.y + threadIdx.x;
-        bool valid = (int)threadIdx.x < td.z;
-        int nj = a.J_off[t + 1] - a.J_off[t];
-        int lcol = 2 * (q - a.J2_off[t]);
-        int i0 = a.I2_off[t], ni = a.I2_off[t + 1] - i0;
-        float cg, sg;
-        gamma_t(m.omega[t], cg, sg);
-        ColPair P;
-        MsCol A, B;
-        float Ga = kNegHuge, Gb = kNegHuge;
-        A.ok = B.ok = false;
-        if (valid) {
-            load_col_pair(a, q, P);
-            float4 Y = a.modY[q];
-            float4 Z = a.modZ[q];
-            float4 W = a.modW[q];
-            Ga = Y.z;
-            Gb = Y.w;
-            for (int lane = 0; lane < 2; ++lane) {
-                MsCol& C = lane ? B : A;
-                C.ok = lcol + lane < nj;
-                if (!C.ok) continue;
-                C.j = a.mod_perm[a.J_off[t] + lcol + lane];  // the caller's index
-                C.n = m.grain[C.j];
-                C.t = t;
-                if (MODE == 0 && m.gstate[4 * C.n] == 0.0f) C.ok = false;  // converged grain
-                gam_apply(cg, sg, m.x + 3 * C.n, C.c);
-                C.r[0] = -(lane ? Z.y : Z.x);
-                C.r[1] = -(lane ? Z.w : Z.z);
-                C.r[2] = -(lane ? W.y : W.x);
-                if (MODE == 3) {  // the ray of the current orientation
-                    const float* Rn = m.R + 9 * C.n;
-                    float4 wd = m.w_d0[m.plane[C.j]];
-                    float v[3], u[3];
-                    for (int r = 0; r < 3; ++r) v[r] = Rn[3 * r] * wd.x + Rn[3 * r + 1] * wd.y + Rn[3 * r + 2] * wd.z;
-                    gam_apply(cg, sg, v, u);
-                    float ue = u[0] * m.e[0] + u[1] * m.e[1] + u[2] * m.e[2];
-                    for (int r = 0; r < 3; ++r) C.r[r] = m.e[r] - 2.0f * ue * u[r];
-                }
-                for (int k = 0; k < 10; ++k) C.acc[k] = 0.0f;
+    __shared__ __align__(16) WarpBuffer buffer[kMsThreads / 32];
+    WarpBuffer& M = buffer[threadIdx.x >> 5];
+    const int id = blockIdx.x * (kMsThreads / 32) + (threadIdx.x >> 5);
+    if (id >= a.ctrl[CTRL_N_COL_TILES] * (TILE / 32)) return;
+    if (id == 0 && (threadIdx.x & 31) == 0)
+        atomicAdd((unsigned long long*)(a.ctrl + CTRL_MS_PAIRS), *(const unsigned long long*)(a.ctrl + CTRL_COL_EVAL));
+    const int numbers = chunk_numbers(a, a.col_tab, id, threadIdx.x & 31, 0);
+    const Slice sl = load_slice((const SliceDesc*)a.col_desc, id);
+    if (!sl.any) return;
+    ring_start(a, M.ring, sl, numbers);
+    const int t = sl.t, q = sl.q, lcol = 2 * (q - a.J2_off[t]);
+    float cg, sg;
+    gamma_t(m.omega[t], cg, sg);
+    ColPair P;
+    load_col_pair(a, sl.valid ? q : q - sl.lane, P);
+    MsCol A, B;
+    A.ok = B.ok = false;
+    float Ga = kNegHuge, Gb = kNegHuge;
+    if (sl.valid) {
+        const float4 Z = a.modZ[q], W = a.modW[q];
+        const float2 G = *(const float2*)&a.Gc[2 * (size_t)q];
+        Ga = G.x;
+        Gb = G.y;
+#pragma unroll
+        for (int lane = 0; lane < 2; ++lane) {
+            MsCol& C = lane ? B : A;
+            C.ok = lane ? sl.vb : true;
+            if (!C.ok) continue;
+            C.j = a.mod_perm[a.J_off[t] + lcol + lane];  // the caller's index
+            C.n = m.grain[C.j];
+            C.t = t;
+            if (MODE == 0 && m.gstate[4 * C.n] == 0.0f) C.ok = false;  // converged grain
+            gam_apply(cg, sg, m.x + 3 * C.n, C.c);
+            C.r[0] = -(lane ? Z.y : Z.x);
+            C.r[1] = -(lane ? Z.w : Z.z);
+            C.r[2] = -(lane ? W.y : W.x);
+            if (MODE == 3) {  // the ray of the current orientation
+                const float* Rn = m.R + 9 * C.n;
+                float4 wd = m.w_d0[m.plane[C.j]];
+                float v[3], u[3];
+                for (int r = 0; r < 3; ++r) v[r] = Rn[3 * r] * wd.x + Rn[3 * r + 1] * wd.y + Rn[3 * r + 2] * wd.z;
+                gam_apply(cg, sg, v, u);
+                float ue = u[0] * m.e[0] + u[1] * m.e[1] + u[2] * m.e[2];
+                for (int r = 0; r < 3; ++r) C.r[r] = m.e[r] - 2.0f * ue * u[r];
             }
-        }
-        const f2 Gpa = dup(Ga), Gpb = dup(Gb);
-        // staged observed pairs [h, h + m) of stage st
-        auto run = [&](int st, int h, int m) {
-            const float4* sX = S.s[0][st];
-            const float4* sY = S.s[1][st];
-            for (int k = h; k < h + m; ++k) {
-                ulonglong2 X = *(const ulonglong2*)&sX[k];
-                ulonglong2 Y = *(const ulonglong2*)&sY[k];
-                // E-step plan exponents of the 2 x 2 pairs: F_i + G_j - K e2
-                f2 va = add2(pair_v2(X.x, X.y, Y.x, P.ncxa, P.ncya, P.ncza, P.nrxa, P.nrya, P.nrza, P.ka, Y.y), Gpa);
-                f2 vb = add2(pair_v2(X.x, X.y, Y.x, P.ncxb, P.ncyb, P.nczb, P.nrxb, P.nryb, P.nrzb, P.kb, Y.y), Gpb);
-                float m4 = fmaxf(fmaxf(lo(va), hi(va)), fmaxf(lo(vb), hi(vb)));
-                if (m4 < kQSkip) continue;
-                float4 x4 = sX[k], y4 = sY[k];
-                ms_pair(A, MODE, x4.x, x4.z, y4.x, lo(va));
-                ms_pair(A, MODE, x4.y, x4.w, y4.y, hi(va));
-                ms_pair(B, MODE, x4.x, x4.z, y4.x, lo(vb));
-                ms_pair(B, MODE, x4.y, x4.w, y4.y, hi(vb));
-            }
-        };
-        auto body = [&](int st, int n, int, int mask = (1 << kParts) - 1) {
-            if (!valid) return;
-            for_each_run(mask, n, [&](int h, int m) { run(st, h, m); });
-        };
-        // the observed granules that can hold a plan entry >= 2^kQSkip for this
-        // tile: log2 Q_ij = F_i + G_j - |K_j| e2 <= max_t F + max_tile G - the
-        // cones' cost bound, so a granule whose bound exceeds
-        // max F + max G - kQSkip holds only pairs the sums skip (exact)
-        const float gtile = block_max(S, fmaxf(Ga, Gb));
-        const int nch = (ni + kChunk - 1) / kChunk;
-        const bool use_list = a.skip && nch > 0 && nch <= kMaxList;
-        int n_list = nch;
-        if (use_list) {
-            const DustPtrs D = dust_ptrs(a.dust, a.T);
-            const Cone M = tile_cone(a.mod_cone, a.mod_ext, a.mod_gbase[t], a.J2_off[t], td.y, td.z, false);
-            const float K = a.skipK;  // the smallest cost factor of any spot
-            const float lim = D.Fmax[t] + gtile - kQSkip + 1.0f;
-            const int og = a.obs_gbase[t], ng = (ni + kGran - 1) / kGran;
-            n_list = build_chunk_list(S, nch, [&](int c) {
-                int msk = 0;
-                for (int hh = 0; hh < kParts; ++hh)
-                    if (kParts * c + hh < ng &&
-                        min_scaled_cost(load_cone(a.obs_cone, a.obs_ext, og + kParts * c + hh), M, K) <= lim)
-                        msk |= 1 << hh;
-                return msk;
-            });
-        }
-        auto no_prep = [](int, int) {};
-        bool ok = use_list ? stream_list_prep(S, parity, src, i0, ni, n_list, no_prep, body)
-                           : stream_tile(S, parity, src, i0, ni, [&](int st, int n, int) { body(st, n, 0); });
-        if (threadIdx.x == 0) {
-            long long np = 0;
-            if (use_list)
-                for (int c = 0; c < n_list; ++c)
-                    np += list_pairs(S.list[c] & 0xffffff, (int)((unsigned)S.list[c] >> 24), ni);
-            else
-                np = ni;
-            atomicAdd((unsigned long long*)(a.ctrl + CTRL_MS_PAIRS), (unsigned long long)(4LL * td.z * np));
-        }
-        if (!ok) {
-            if (threadIdx.x == 0) set_status(a.ctrl, LAUE_ERR_TIMEOUT);
-            break;
-        }
-        if (valid) {
-            for (int lane = 0; lane < 2; ++lane) {
-                MsCol& C = lane ? B : A;
-                if (lcol + lane >= nj) continue;
-                const int jc = a.mod_perm[a.J_off[t] + lcol + lane];
-                float* o = m.jsum + 12 * (size_t)jc;
-                // cost length of the spot's detector: C_ij = D_j^2 |rhat - r|^2, so the
-                // Newton and MM sums carry the weight (D_j / D)^2
-                const int det = a.mod_s ? (int)a.mod_s[jc].w : -1;
-                const float D2j = (det >= 0 && det < a.n_det) ? m.D2det[det] : m.D2;
-                const float kd = D2j / m.D2;
-                if (MODE >= 2) {
-                    // per-spot gradient: x part Gamma^T dC/dc, rotation part
-                    // v x (Gamma^T y), y = -2 ((gr.u) e + (u.e) gr), u = Gamma R w_m
-                    float D2x2 = 2.0f * D2j;
-                    float gc[3] = {D2x2 * C.acc[0], D2x2 * C.acc[1], D2x2 * C.acc[2]};
-                    float gr[3] = {D2x2 * C.acc[3], D2x2 * C.acc[4], D2x2 * C.acc[5]};
-                    float gx[3];
-                    gamT_apply(cg, sg, gc, gx);
-                    const float* Rn = m.R + 9 * C.n;
-                    float4 wd = m.w_d0[m.plane[C.j]];
-                    float v[3], u[3];
-                    for (int r = 0; r < 3; ++r) v[r] = Rn[3 * r] * wd.x + Rn[3 * r + 1] * wd.y + Rn[3 * r + 2] * wd.z;
-                    gam_apply(cg, sg, v, u);
-                    float gu = gr[0] * u[0] + gr[1] * u[1] + gr[2] * u[2];
-                    float ue = u[0] * m.e[0] + u[1] * m.e[1] + u[2] * m.e[2];
-                    float y[3], Gy[3];
-                    for (int r = 0; r < 3; ++r) y[r] = -2.0f * (gu * m.e[r] + ue * gr[r]);
-                    gamT_apply(cg, sg, y, Gy);
-                    o[0] = v[1] * Gy[2] - v[2] * Gy[1];
-                    o[1] = v[2] * Gy[0] - v[0] * Gy[2];
-                    o[2] = v[0] * Gy[1] - v[1] * Gy[0];
-                    o[3] = gx[0];
-                    o[4] = gx[1];
-                    o[5] = gx[2];
-                    o[6] = D2j * C.acc[6];
-                    if (MODE == 3) {  // the Gauss-Newton sums, weighted (the grain kernel applies 2 D^2)
-                        o[7] = kd * C.acc[7];
-                        o[8] = kd * C.acc[8];
-                        o[9] = kd * C.acc[9];
-                    }
-                    if (!C.ok)
-                        for (int k = 0; k < (MODE == 3 ? 10 : 7); ++k) o[k] = 0.0f;
-                } else if (MODE == 1) {
-                    o[9] = C.ok ? kd * C.acc[0] : 0.0f;
-                    o[10] = C.ok ? kd * C.acc[1] : 0.0f;
-                    o[11] = C.ok ? kd * C.acc[2] : 0.0f;
-                } else if (C.ok) {
-                    float gx[3];
-                    gamT_apply(cg, sg, C.acc, gx);
-                    float hx[6];
-                    sym_gamT_gam(cg, sg, C.acc + 3, hx);
-                    for (int k = 0; k < 3; ++k) o[k] = kd * gx[k];
-                    for (int k = 0; k < 6; ++k) o[3 + k] = kd * hx[k];
-                } else {
-                    for (int k = 0; k < 9; ++k) o[k] = 0.0f;
-                }
-            }
+            for (int k = 0; k < 10; ++k) C.acc[k] = 0.0f;
         }
     }
-    if (!last_cta(S, a.ctrl + CTRL_GEN_DONE)) return;
-    if (threadIdx.x == 0) {
-        a.ctrl[CTRL_GEN_NEXT] = 0;
-        a.ctrl[CTRL_GEN_DONE] = 0;
+    if (sl.nch >= 0) {
+        for_each_chunk(a, M.ring, a.col_tab, sl, numbers, [&](const Chunk& E) {
+#pragma unroll 4
+            for (int k = 0; k < kListDepth; ++k) {
+                const unsigned s = E.slot[k][sl.lane];
+                const float2 Q = E.e2[k][sl.lane];  // plan entries, 0: padding
+                auto one = [&](MsCol& C, int slot, float Qij) {
+                    const float* X = (const float*)&a.obsX[sl.s0 + (slot >> 1)];
+                    const float* Y = (const float*)&a.obsY[sl.s0 + (slot >> 1)];
+                    const int odd = slot & 1;
+                    const float px = X[odd], py = X[2 + odd], pz = Y[odd];
+                    if (C.ok && Qij != 0.0f) ms_pair(C, MODE, px, py, pz, Qij);
+                };
+                one(A, s & 0xffffu, Q.x);
+                one(B, s >> 16, Q.y);
+            }
+        });
+    } else {
+        const Cone own = load_cone(a.mod_cone, a.mod_ext, a.mod_gbase[t] + (q - sl.lane - a.J2_off[t]) / kGran);
+        const f2 Gpa = dup(Ga), Gpb = dup(Gb);
+        sweep<false>(a, M.stage, own, a.obs_sub + (size_t)kSubs * a.obs_gbase[t],
+                     a.obs_subext + (size_t)kSubs * a.obs_gbase[t], sl.s0, sl.ns, a.skip, sl.cut, a.Fc,
+                     [&](int st, int n, const int4&) {
+                         for (int j = 0; j < n; ++j) {
+                             // E-step plan exponents of the 2 x 2 pairs: F_i + G_j - K e2
+                             f2 va, vb;
+                             col_pair_v(P, M.stage, st, j, *(const f2*)&M.stage.P[st][j], va, vb);
+                             va = add2(va, Gpa);
+                             vb = add2(vb, Gpb);
+                             const float m4 = fmaxf(fmaxf(lo(va), hi(va)), fmaxf(lo(vb), hi(vb)));
+                             if (m4 < kQSkip) continue;
+                             const float4 x4 = M.stage.X[st][j];
+                             const float2 z2 = M.stage.Y[st][j];
+                             auto one = [&](MsCol& C, float px, float py, float pz, float v) {
+                                 if (C.ok && !(v < kQSkip)) ms_pair(C, MODE, px, py, pz, ex2(v));
+                             };
+                             one(A, x4.x, x4.z, z2.x, lo(va));
+                             one(A, x4.y, x4.w, z2.y, hi(va));
+                             one(B, x4.x, x4.z, z2.x, lo(vb));
+                             one(B, x4.y, x4.w, z2.y, hi(vb));
+                         }
+                     });
+    }
+    if (sl.valid) {
+        for (int lane = 0; lane < 2; ++lane) {
+            MsCol& C = lane ? B : A;
+            if (!(lane ? sl.vb : sl.valid)) continue;
+            const int jc = a.mod_perm[a.J_off[t] + lcol + lane];
+            float* o = m.jsum + 12 * (size_t)jc;
+            // cost length of the spot's detector: C_ij = D_j^2 |rhat - r|^2, so the
+            // Newton and MM sums carry the weight (D_j / D)^2
+            const int det = a.mod_s ? (int)a.mod_s[jc].w : -1;
+            const float D2j = (det >= 0 && det < a.n_det) ? m.D2det[det] : m.D2;
+            const float kd = D2j / m.D2;
+            if (MODE >= 2) {
+                // per-spot gradient: x part Gamma^T dC/dc, rotation part
+                // v x (Gamma^T y), y = -2 ((gr.u) e + (u.e) gr), u = Gamma R w_m
+                float D2x2 = 2.0f * D2j;
+                float gc[3] = {D2x2 * C.acc[0], D2x2 * C.acc[1], D2x2 * C.acc[2]};
+                float gr[3] = {D2x2 * C.acc[3], D2x2 * C.acc[4], D2x2 * C.acc[5]};
+                float gx[3];
+                gamT_apply(cg, sg, gc, gx);
+                const float* Rn = m.R + 9 * C.n;
+                float4 wd = m.w_d0[m.plane[C.j]];
+                float v[3], u[3];
+                for (int r = 0; r < 3; ++r) v[r] = Rn[3 * r] * wd.x + Rn[3 * r + 1] * wd.y + Rn[3 * r + 2] * wd.z;
+                gam_apply(cg, sg, v, u);
+                float gu = gr[0] * u[0] + gr[1] * u[1] + gr[2] * u[2];
+                float ue = u[0] * m.e[0] + u[1] * m.e[1] + u[2] * m.e[2];
+                float y[3], Gy[3];
+                for (int r = 0; r < 3; ++r) y[r] = -2.0f * (gu * m.e[r] + ue * gr[r]);
+                gamT_apply(cg, sg, y, Gy);
+                o[0] = v[1] * Gy[2] - v[2] * Gy[1];
+                o[1] = v[2] * Gy[0] - v[0] * Gy[2];
+                o[2] = v[0] * Gy[1] - v[1] * Gy[0];
+                o[3] = gx[0];
+                o[4] = gx[1];
+                o[5] = gx[2];
+                o[6] = D2j * C.acc[6];
+                if (MODE == 3) {  // the Gauss-Newton sums, weighted (the grain kernel applies 2 D^2)
+                    o[7] = kd * C.acc[7];
+                    o[8] = kd * C.acc[8];
+                    o[9] = kd * C.acc[9];
+                }
+                if (!C.ok)
+                    for (int k = 0; k < (MODE == 3 ? 10 : 7); ++k) o[k] = 0.0f;
+            } else if (MODE == 1) {
+                o[9] = C.ok ? kd * C.acc[0] : 0.0f;
+                o[10] = C.ok ? kd * C.acc[1] : 0.0f;
+                o[11] = C.ok ? kd * C.acc[2] : 0.0f;
+            } else if (C.ok) {
+                float gx[3];
+                gamT_apply(cg, sg, C.acc, gx);
+                float hx[6];
+                sym_gamT_gam(cg, sg, C.acc + 3, hx);
+                for (int k = 0; k < 3; ++k) o[k] = kd * gx[k];
+                for (int k = 0; k < 6; ++k) o[3 + k] = kd * hx[k];
+            } else {
+                for (int k = 0; k < 9; ++k) o[k] = 0.0f;
+            }
+        }
     }
 }
 
@@ -560,12 +537,29 @@ static cudaError_t seg_table(const MsArgs& m, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// The E-step's plan (schedule, pair copies with F and G, its entries) and the segment table.
+static cudaError_t prepare(const MsArgs& m, const SkLaunch& l, bool sorted, cudaStream_t s) {
+    cudaError_t e = sinkhorn_prepare(m.sk, s, false, sorted);
+    if (e == cudaSuccess) e = sinkhorn_list_plan(m.sk, l, s);
+    if (e == cudaSuccess) e = seg_table(m, s);
+    return e;
+}
+
+template <int MODE>
+static void pair_pass(const MsArgs& m, const SkLaunch& l, cudaStream_t s) {
+    const int ctas = (l.col_slices + kMsThreads / 32 - 1) / (kMsThreads / 32);
+    switch (m.sk.tile_cols) {
+        case 64: ms_pair_kernel<64, MODE><<<ctas, kMsThreads, 0, s>>>(m); break;
+        case 128: ms_pair_kernel<128, MODE><<<ctas, kMsThreads, 0, s>>>(m); break;
+        default: ms_pair_kernel<256, MODE><<<ctas, kMsThreads, 0, s>>>(m);
+    }
+}
+
 cudaError_t grad_run(const MsArgs& m, const SkLaunch& l, cudaStream_t s) {
-    cudaError_t e = sinkhorn_prepare(m.sk, s);
+    cudaError_t e = prepare(m, l, false, s);
     if (e != cudaSuccess) return e;
-    if ((e = seg_table(m, s)) != cudaSuccess) return e;
     if (m.N > 0) ms_init_kernel<<<(m.N + 255) / 256, 256, 0, s>>>(m);
-    ms_pair_kernel<2><<<l.col_grid, m.sk.tile_cols, 0, s>>>(m);
+    pair_pass<2>(m, l, s);
     if (m.N > 0) ms_grad_grain_kernel<<<(m.N * 32 + 127) / 128, 128, 0, s>>>(m);
     return cudaGetLastError();
 }
@@ -650,13 +644,12 @@ cudaError_t axis_angle_vjp_run(const float* w, const float* grad, const float* g
     return cudaGetLastError();
 }
 
-cudaError_t mstep_adjoint_run(const MsArgs& m, const SkLaunch& l, int n_steps, cudaStream_t s) {
-    cudaError_t e = sinkhorn_prepare(m.sk, s);  // the E-step plan: pair copies with F, G
+cudaError_t mstep_adjoint_run(const MsArgs& m, const SkLaunch& l, int n_steps, bool sorted, cudaStream_t s) {
+    cudaError_t e = prepare(m, l, sorted, s);
     if (e != cudaSuccess) return e;
-    if ((e = seg_table(m, s)) != cudaSuccess) return e;
     if (m.N > 0) ms_init_kernel<<<(m.N + 255) / 256, 256, 0, s>>>(m);
     for (int k = 0; k < n_steps; ++k) {
-        ms_pair_kernel<3><<<l.col_grid, m.sk.tile_cols, 0, s>>>(m);
+        pair_pass<3>(m, l, s);
         if (m.N > 0) ms_adj_grain_kernel<<<(m.N * 32 + 127) / 128, 128, 0, s>>>(m);
     }
     if (m.N > 0) ms_norms_kernel<<<(m.N + 255) / 256, 256, 0, s>>>(m);
@@ -668,17 +661,16 @@ cudaError_t axis_angle_run(const float* w, const float* R0, float* R, float* JlT
     return cudaGetLastError();
 }
 
-cudaError_t mstep_run(const MsArgs& m, const SkLaunch& l, cudaStream_t s) {
-    cudaError_t e = sinkhorn_prepare(m.sk, s);  // schedule + pair-interleaved copies with F, G
+cudaError_t mstep_run(const MsArgs& m, const SkLaunch& l, bool sorted, cudaStream_t s) {
+    cudaError_t e = prepare(m, l, sorted, s);
     if (e != cudaSuccess) return e;
-    if ((e = seg_table(m, s)) != cudaSuccess) return e;
     if (m.N > 0) ms_init_kernel<<<(m.N + 255) / 256, 256, 0, s>>>(m);
     for (int k = 0; k < m.n_newton; ++k) {
-        ms_pair_kernel<0><<<l.col_grid, m.sk.tile_cols, 0, s>>>(m);
+        pair_pass<0>(m, l, s);
         if (m.N > 0) ms_newton_grain_kernel<<<(m.N * 32 + 127) / 128, 128, 0, s>>>(m);
     }
     if (m.n_mm > 0 && m.N > 0) {
-        ms_pair_kernel<1><<<l.col_grid, m.sk.tile_cols, 0, s>>>(m);
+        pair_pass<1>(m, l, s);
         size_t shm = sizeof(float) * (6 * (size_t)m.M + 9 * kMmThreads);
         if (shm > 48 * 1024) {
             e = cudaFuncSetAttribute(ms_mm_grain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);

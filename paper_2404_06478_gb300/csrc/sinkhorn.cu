@@ -25,16 +25,9 @@
 // rays are stored negated (d = p + (-c), e = d/|d| + (-r)).  Padding entries
 // carry a potential of -3e38, which makes their plan entries exactly 0.
 //
-// Passes.  Each pass is one persistent launch over all angle blocks: CTAs pull
-// tiles (angle t, first pair, count) from a queue the scheduler kernel built
-// on the device in longest-block-first order.  A thread keeps one PAIR of rows
-// (row pass) or columns (column pass) in registers and streams the other side
-// of its angle block, as pairs, through shared memory in chunks loaded by the
-// bulk-copy engine (cp.async.bulk) into a two-stage mbarrier pipeline: every
-// staged pair feeds 4 pair evaluations.  The log-sum-exps are online, in
-// groups of 4 staged pairs (8 values) per max/rescale step.  The last CTA to
-// finish a pass combines the per-tile partial log-sum-exps into the dustbin
-// potentials:
+// Passes (passes.cu).  Every pass is one launch over the tiles of all angle
+// blocks; its tiles' partial log-sum-exps become the dustbin potentials
+// beside the next pass:
 //   end of a row pass:    F_0 <- F_0(next), then G_0 from the new F and F_0
 //   end of a column pass: F_0(next) from the new G and G_0
 // which reproduces the sequential order of the algorithm exactly.
@@ -43,63 +36,102 @@
 namespace laue {
 
 // ---------------------------------------------------------------- scheduler
+// Exclusive prefix of get(i), i < n, by a CTA of 1024 threads: put(i, prefix);
+// returns the sum.
+template <class Get, class Put>
+__device__ int block_prefix(int n, int* warp_sum, Get get, Put put) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int base = 0;
+    for (int i0 = 0; i0 < n; i0 += 1024) {
+        const int i = i0 + threadIdx.x;
+        const int c = i < n ? get(i) : 0;
+        int incl = c;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) warp_sum[w] = incl;
+        __syncthreads();
+        if (w == 0) {
+            int v = warp_sum[lane];
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += y;
+            }
+            warp_sum[lane] = v;
+        }
+        __syncthreads();
+        if (i < n) put(i, base + (w ? warp_sum[w - 1] : 0) + incl - c);
+        base += warp_sum[31];
+        __syncthreads();
+    }
+    return base;
+}
+
+// Slots among the pairs [0, n) that warp w of 1024 threads reads (pair q is
+// thread q % 1024's).
+__device__ __forceinline__ int warp_share(int n, int w) {
+    return 2 * (n / 1024 * 32 + min(32, max(0, n % 1024 - 32 * w)));
+}
+
 // One CTA.  Pair offsets of the padded blocks, row and column tile queues
 // (angles by descending work, tiles of one angle contiguous), per-angle tile
-// ranges, log2 masses of the dustbins; clears the queue counters.
-__global__ void __launch_bounds__(1024) sk_schedule_kernel(SkArgs a) {
+// ranges, log2 masses of the dustbins; clears the counters.  A cold start's
+// potentials are all 0, so its maxima and first F_0 need no pass over them:
+// the sums of sk_init_dust_kernel are then counts of spots.
+constexpr int kSchedAngles = 1024;  // angles whose offsets fit in shared memory
+__global__ void __launch_bounds__(1024) sk_schedule_kernel(SkArgs a, int dustbins) {
+    __shared__ int sI[kSchedAngles + 1], sJ[kSchedAngles + 1], warp_sum[32], pads[32];
     const int T = a.T;
+    const int *I = a.I_off, *J = a.J_off;
+    if (T <= kSchedAngles) {
+        for (int t = threadIdx.x; t <= T; t += blockDim.x) {
+            sI[t] = I[t];
+            sJ[t] = J[t];
+        }
+        __syncthreads();
+        I = sI;
+        J = sJ;
+    }
     int* order_r = (int*)a.row_part;  // scratch until the passes run
     int* order_c = (int*)a.col_part;
     for (int t = threadIdx.x; t < T; t += blockDim.x) {
-        int wr = a.J_off[t + 1] - a.J_off[t];
-        int wc = a.I_off[t + 1] - a.I_off[t];
+        const int wr = J[t + 1] - J[t], wc = I[t + 1] - I[t];
         int rr = 0, rc = 0;
         for (int u = 0; u < T; ++u) {
-            int ur = a.J_off[u + 1] - a.J_off[u];
-            int uc = a.I_off[u + 1] - a.I_off[u];
+            const int ur = J[u + 1] - J[u], uc = I[u + 1] - I[u];
             rr += (ur > wr) || (ur == wr && u < t);
             rc += (uc > wc) || (uc == wc && u < t);
         }
         order_r[rr] = t;
         order_c[rc] = t;
     }
-    __syncthreads();
+    auto pairs_i = [&](int t) { return (I[t + 1] - I[t] + 1) / 2; };
+    auto pairs_j = [&](int t) { return (J[t + 1] - J[t] + 1) / 2; };
+    auto granules = [](int n) { return (n + kGran - 1) / kGran; };
+    const int ni2 = block_prefix(T, warp_sum, pairs_i, [&](int t, int v) { a.I2_off[t] = v; });
+    const int nj2 = block_prefix(T, warp_sum, pairs_j, [&](int t, int v) { a.J2_off[t] = v; });
+    const int ngi = block_prefix(T, warp_sum, [&](int t) { return granules(pairs_i(t)); },
+                                 [&](int t, int v) { a.obs_gbase[t] = v; });
+    const int ngj = block_prefix(T, warp_sum, [&](int t) { return granules(pairs_j(t)); },
+                                 [&](int t, int v) { a.mod_gbase[t] = v; });
+    auto tiles_r = [&](int k) { return (pairs_i(order_r[k]) + a.tile_rows - 1) / a.tile_rows; };
+    auto tiles_c = [&](int k) { return (pairs_j(order_c[k]) + a.tile_cols - 1) / a.tile_cols; };
+    int nr = block_prefix(T, warp_sum, tiles_r, [&](int k, int v) {
+        int4& at = a.ang_tiles[order_r[k]];
+        at.x = v;
+        at.y = tiles_r(k);
+    });
+    int nc = block_prefix(T, warp_sum, tiles_c, [&](int k, int v) {
+        int4& at = a.ang_tiles[order_c[k]];
+        at.z = v;
+        at.w = tiles_c(k);
+    });
     if (threadIdx.x == 0) {
-        int ip = 0, jp = 0;
-        for (int t = 0; t < T; ++t) {
-            a.I2_off[t] = ip;
-            a.J2_off[t] = jp;
-            ip += (a.I_off[t + 1] - a.I_off[t] + 1) / 2;
-            jp += (a.J_off[t + 1] - a.J_off[t] + 1) / 2;
-        }
-        a.I2_off[T] = ip;
-        a.J2_off[T] = jp;
-        int go = 0, gm = 0;
-        for (int t = 0; t < T; ++t) {
-            a.obs_gbase[t] = go;
-            a.mod_gbase[t] = gm;
-            go += (a.I2_off[t + 1] - a.I2_off[t] + kGran - 1) / kGran;
-            gm += (a.J2_off[t + 1] - a.J2_off[t] + kGran - 1) / kGran;
-        }
-        a.obs_gbase[T] = go;
-        a.mod_gbase[T] = gm;
-        int nr = 0, nc = 0;
-        for (int k = 0; k < T; ++k) {
-            int t = order_r[k];
-            int np = (a.I_off[t + 1] - a.I_off[t] + 1) / 2;
-            int cnt = (np + a.tile_rows - 1) / a.tile_rows;
-            a.ang_tiles[t].x = nr;
-            a.ang_tiles[t].y = cnt;
-            nr += cnt;
-        }
-        for (int k = 0; k < T; ++k) {
-            int t = order_c[k];
-            int np = (a.J_off[t + 1] - a.J_off[t] + 1) / 2;
-            int cnt = (np + a.tile_cols - 1) / a.tile_cols;
-            a.ang_tiles[t].z = nc;
-            a.ang_tiles[t].w = cnt;
-            nc += cnt;
-        }
+        a.I2_off[T] = ni2;
+        a.J2_off[T] = nj2;
+        a.obs_gbase[T] = ngi;
+        a.mod_gbase[T] = ngj;
         if (nr > a.max_row_tiles || nc > a.max_col_tiles) {
             set_status(a.ctrl, LAUE_ERR_CAPACITY);
             nr = min(nr, a.max_row_tiles);
@@ -109,8 +141,6 @@ __global__ void __launch_bounds__(1024) sk_schedule_kernel(SkArgs a) {
         a.ctrl[CTRL_N_COL_TILES] = nc;
         for (int k = CTRL_ROW_NEXT; k <= CTRL_GEN_DONE; ++k)
             if (k != CTRL_N_ROW_TILES && k != CTRL_N_COL_TILES && k != CTRL_FWD_TOTAL) a.ctrl[k] = 0;
-        a.ctrl[CTRL_POOL_NEXT] = 0;
-        for (int k = CTRL_ROW_EVAL; k < CTRL_COL_EVAL + 2; ++k) a.ctrl[k] = 0;
     }
     __syncthreads();
     for (int t = threadIdx.x; t < T; t += blockDim.x) {
@@ -128,20 +158,47 @@ __global__ void __launch_bounds__(1024) sk_schedule_kernel(SkArgs a) {
                 a.col_tiles[idx] = make_int4(t, j0 + k * a.tile_cols, min(a.tile_cols, nj - k * a.tile_cols), 0);
         }
     }
+    if (!a.warm)
+        for (int t = threadIdx.x; t < T; t += blockDim.x) {
+            DustPtrs D = dust_ptrs(a.dust, T);
+            D.Gmax[t] = J[t + 1] > J[t] ? 0.0f : kNegHuge;
+            D.Fmax[t] = I[t + 1] > I[t] ? 0.0f : kNegHuge;
+        }
+    if (!dustbins) return;
     // dustbin masses (paper: T_a = T_b - b^T 1 + a^T 1), in double precision
     DustPtrs D = dust_ptrs(a.dust, T);
-    int nd = a.mode ? T : 1;
+    const int nd = a.mode ? T : 1;
+    if (threadIdx.x < 32) pads[threadIdx.x] = 0;
+    __syncthreads();
+    if (!a.mode)
+        for (int t = threadIdx.x; t < T; t += blockDim.x)
+            if ((J[t + 1] - J[t]) & 1) atomicAdd(&pads[(a.J2_off[t] + pairs_j(t) - 1) % 1024 / 32], 1);
+    __syncthreads();
     for (int d = threadIdx.x; d < nd; d += blockDim.x) {
-        long long nI = a.mode ? (a.I_off[d + 1] - a.I_off[d]) : a.I_off[T];
-        long long nJ = a.mode ? (a.J_off[d + 1] - a.J_off[d]) : a.J_off[T];
+        long long nI = a.mode ? (I[d + 1] - I[d]) : I[T];
+        long long nJ = a.mode ? (J[d + 1] - J[d]) : J[T];
         double u = ceil(a.frac * (double)nJ - 1e-9);
         double o = u + (double)nI - (double)nJ;
         if (o < 0) {
             u = (double)(nJ - nI);
             o = 0;
         }
-        D.log2U[d] = u > 0 ? (float)log2(u) : kNegHuge;
+        const float log2U = u > 0 ? (float)log2(u) : kNegHuge;
+        D.log2U[d] = log2U;
         D.log2O[d] = o > 0 ? (float)log2(o) : kNegHuge;
+        if (!a.warm && a.mode != 2) {
+            // F_0(next) = log2 U - LSE2({0}_j u {-kc}), in the order of sk_init_dust_kernel
+            const int n = a.mode ? pairs_j(d) : nj2;
+            Lse2 L;
+            L.init(0.0f - a.kc);
+            for (int w = 0; w < 32; ++w) {
+                int c = warp_share(n, w);
+                if (!a.mode) c -= pads[w];
+                else if ((nJ & 1) && (n - 1) % 1024 / 32 == w) --c;
+                L.merge(c > 0 ? 0.0f : kNegHuge, (float)c);
+            }
+            D.F0n[d] = log2U - L.value();
+        }
     }
 }
 
@@ -188,6 +245,7 @@ __device__ __forceinline__ unsigned direction_key(float x, float y, float z) {
 }
 
 constexpr int kSortThreads = 1024;
+constexpr int kRankSort = 512;
 
 // Blocks 0..T-1 sort the observed blocks, T..2T-1 the model blocks.
 __global__ void __launch_bounds__(kSortThreads) sk_sort_kernel(SkArgs a) {
@@ -204,6 +262,37 @@ __global__ void __launch_bounds__(kSortThreads) sk_sort_kernel(SkArgs a) {
     int* perm = (mod ? a.mod_perm : a.obs_perm) + b0;
     int* pos = (mod ? a.mod_pos : a.obs_pos) + b0;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (n <= kRankSort) {
+        // a small block: every thread counts the keys before its own, n / 4 steps of the warps that hold keys
+        // against six passes of five barriers
+        __shared__ __align__(16) unsigned key[kRankSort];
+        const int l = threadIdx.x;
+        unsigned mine = 0xffffffffu;
+        if (l < n) {
+            float4 v = mod ? a.mod_r[b0 + l] : a.obs_p[b0 + l];
+            mine = direction_key(v.x, v.y, v.z);
+        }
+        if (l < kRankSort) key[l] = mine;
+        __syncthreads();
+        if (32 * w >= n) return;
+        int before = 0;
+        const int before_own = l / 4 * 4;  // whole groups of four keys before the own one
+        for (int u = 0; u < n; u += 4) {
+            const uint4 k = *(const uint4*)&key[u];
+            if (u < before_own)
+                before += (k.x <= mine) + (k.y <= mine) + (k.z <= mine) + (k.w <= mine);
+            else if (u > before_own)
+                before += (k.x < mine) + (k.y < mine) + (k.z < mine) + (k.w < mine);
+            else
+                before += (k.x < mine || (k.x == mine && u < l)) + (k.y < mine || (k.y == mine && u + 1 < l)) +
+                          (k.z < mine || (k.z == mine && u + 2 < l)) + (k.w < mine);
+        }
+        if (l < n) {
+            perm[before] = b0 + l;
+            pos[l] = before;
+        }
+        return;
+    }
     for (int l = threadIdx.x; l < n; l += kSortThreads) {
         float4 v = mod ? a.mod_r[b0 + l] : a.obs_p[b0 + l];
         kbuf[0][l] = direction_key(v.x, v.y, v.z);
@@ -382,6 +471,10 @@ __global__ void sk_pack_kernel(SkArgs a) {
     const float s = 1.0f / a.to_user;  // mm^2 -> base-2 internal units
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     for (int u = k; u < 4 * a.T; u += gridDim.x * blockDim.x) a.pmax[u] = 0u;
+    if (k == 0) {  // the lists are built next
+        a.ctrl[CTRL_POOL_NEXT] = 0;
+        for (int u = CTRL_ROW_EVAL; u < CTRL_COL_EVAL + 2; ++u) a.ctrl[u] = 0;
+    }
     if (k < a.n_obs) {
         int t = block_of(a.I_off, a.T, k);
         int l = a.obs_pos[k];  // rank of the spot in its block's spatial order
@@ -446,7 +539,8 @@ __global__ void sk_pack_kernel(SkArgs a) {
     }
 }
 
-// One CTA: F_0(next) = log2 U - LSE2({G_j} u {G_0 - kc}) for the starting G.
+// One CTA: F_0(next) = log2 U - LSE2({G_j} u {G_0 - kc}) for the starting G of a
+// warm start.
 __global__ void __launch_bounds__(1024) sk_init_dust_kernel(SkArgs a) {
     __shared__ float sm[32], ss[32];
     DustPtrs D = dust_ptrs(a.dust, a.T);
@@ -557,19 +651,23 @@ __global__ void __launch_bounds__(256) sk_init_gmax_kernel(SkArgs a) {
     }
 }
 
-cudaError_t sinkhorn_prepare(const SkArgs& a, cudaStream_t s) {
+cudaError_t sinkhorn_prepare(const SkArgs& a, cudaStream_t s, bool dustbins, bool sorted) {
     int nmax = a.n_obs > a.n_model ? a.n_obs : a.n_model;
     int blocks = (nmax + 255) / 256;
     if (blocks < 1) blocks = 1;
-    sk_schedule_kernel<<<1, 1024, 0, s>>>(a);
-    if (a.T > 0) sk_sort_kernel<<<2 * a.T, kSortThreads, 0, s>>>(a);
+    if (!sorted) {
+        sk_schedule_kernel<<<1, 1024, 0, s>>>(a, dustbins ? 1 : 0);
+        sk_sort_kernel<<<2 * a.T, kSortThreads, 0, s>>>(a);
+    }
     sk_pack_kernel<<<blocks, 256, 0, s>>>(a);
-    {
+    if (!sorted) {
         int max_gran = (a.n_obs + a.n_model) / (2 * kGran) + 2 * a.T + 2;  // bound on the granule count
         sk_cone_kernel<<<(max_gran * 32 + 255) / 256, 256, 0, s>>>(a);
     }
-    if (a.mode != 2) sk_init_dust_kernel<<<1, 1024, 0, s>>>(a);
-    if (a.T > 0) sk_init_gmax_kernel<<<a.T, 256, 0, s>>>(a);
+    if (a.warm) {
+        if (a.mode != 2 && dustbins) sk_init_dust_kernel<<<1, 1024, 0, s>>>(a);
+        sk_init_gmax_kernel<<<a.T, 256, 0, s>>>(a);
+    }
     return cudaGetLastError();
 }
 
