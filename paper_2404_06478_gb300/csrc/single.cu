@@ -132,9 +132,23 @@ __device__ void sf_cut(const SfArgs& a, SfShared& S, const SfScratch& Z) {
     __syncthreads();
     const int nr = a.T * a.M;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // largest stretch of the pose (1 for a rotation), with a margin: planes whose
+    // 2 d0 |R w| |e| stays below the band have no harmonic in it at any angle
+    // (two thirds of the |hkl| <= 6 planes)
+    float stretch = 0.0f;
+    for (int r = 0; r < 3; ++r) {
+        float row = 0.0f;
+        for (int c = 0; c < 3; ++c)
+            row += fabsf(S.R[r] * S.R[c] + S.R[3 + r] * S.R[3 + c] + S.R[6 + r] * S.R[6 + c]);
+        stretch = fmaxf(stretch, row);
+    }
+    const float e2 = a.G.e[0] * a.G.e[0] + a.G.e[1] * a.G.e[1] + a.G.e[2] * a.G.e[2];
+    const float lam2 = a.G.lam_min * a.G.lam_min, reach = 4.0f * 1.001f * stretch * e2;
     auto detector_of = [&](int id, int& t, int& m) {
         t = id / a.M;
         m = id - t * a.M;
+        const float4 wd = a.w_d0[m];
+        if (reach * wd.w * wd.w * (wd.x * wd.x + wd.y * wd.y + wd.z * wd.z) < lam2) return -1;
         float r[3], c[3], lam0;
         int nh;
         sf_ray(a, S.cs, S.R, S.x, t, m, r, c, &lam0, &nh);
@@ -602,64 +616,77 @@ __device__ __forceinline__ void sf_column_sums(const SfScratch& Z, int j, int n,
 __device__ void sf_columns(const SfArgs& a, SfShared& S, const SfScratch& Z, float negK, float dust, bool massonly,
                            unsigned long long& npair) {
     int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto centre = [&](int t, float* c) {
+        const float cg = S.cs[t].x, sg = S.cs[t].y;
+        c[0] = cg * S.x[0] + sg * S.x[2];
+        c[1] = S.x[1];
+        c[2] = -sg * S.x[0] + cg * S.x[2];
+    };
+    auto finish = [&](int j, float s0, float s1, float s2) {
+        for (int o = 16; o > 0; o >>= 1) {
+            s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+            s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        }
+        if (lane == 0) {
+            const float w = massonly ? 1.0f : Z.kd[j];  // MM weight (D_j / D)^2
+            Z.v[3 * j] = s0 * w;
+            Z.v[3 * j + 1] = s1 * w;
+            Z.v[3 * j + 2] = s2 * w;
+        }
+    };
+    for (int j = warp; j < S.n_spots; j += kSfThreads / 32) {
+        const int t = Z.tm[j] >> 16, off = S.near_off[t];
+        if (off < 0) continue;
+        float c[3], s0 = 0.f, s1 = 0.f, s2 = 0.f;
+        centre(t, c);
+        sf_column_sums(Z, j, S.near_end[t] - off, massonly, c,
+                       [&](int k, float4& p, float& l) {
+                           p = Z.near[off + k];
+                           l = p.w;
+                       },
+                       s0, s1, s2, npair);
+        finish(j, s0, s1, s2);
+    }
+    // angles whose near rows did not fit the list
     for (int t = 0; t < a.T; ++t) {
         int j0 = S.t_off[t], j1 = S.t_off[t + 1];
-        if (j0 == j1) continue;
-        const int off = S.near_off[t];
+        if (j0 == j1 || S.near_off[t] >= 0) continue;
         int i0 = a.I_off[t], ni = a.I_off[t + 1] - i0;
         int nl = min(ni, a.icap);
-        if (off < 0) {
-            for (int k = threadIdx.x; k < nl; k += blockDim.x) {
-                float vmax;
-                Z.lse[k] = sf_row_lse(a, S, Z, t, a.p[i0 + k], dust, npair, vmax);
-            }
-            __syncthreads();
+        for (int k = threadIdx.x; k < nl; k += blockDim.x) {
+            float vmax;
+            Z.lse[k] = sf_row_lse(a, S, Z, t, a.p[i0 + k], dust, npair, vmax);
         }
-        const float cg = S.cs[t].x, sg = S.cs[t].y;
-        float c[3] = {cg * S.x[0] + sg * S.x[2], S.x[1], -sg * S.x[0] + cg * S.x[2]};
+        __syncthreads();
+        float c[3];
+        centre(t, c);
         for (int j = j0 + warp; j < j1; j += blockDim.x / 32) {
             float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-            if (off >= 0) {
-                sf_column_sums(Z, j, S.near_end[t] - off, massonly, c,
-                               [&](int k, float4& p, float& l) {
-                                   p = Z.near[off + k];
-                                   l = p.w;
-                               },
-                               s0, s1, s2, npair);
-            } else {
-                sf_column_sums(Z, j, ni, massonly, c,
-                               [&](int k, float4& p, float& l) {
-                                   p = a.p[i0 + k];
-                                   float vmax;
-                                   l = k < nl ? Z.lse[k] : sf_row_lse(a, S, Z, t, p, dust, npair, vmax);
-                               },
-                               s0, s1, s2, npair);
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-                s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-                s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-            }
-            if (lane == 0) {
-                const float w = massonly ? 1.0f : Z.kd[j];  // MM weight (D_j / D)^2
-                Z.v[3 * j] = s0 * w;
-                Z.v[3 * j + 1] = s1 * w;
-                Z.v[3 * j + 2] = s2 * w;
-            }
+            sf_column_sums(Z, j, ni, massonly, c,
+                           [&](int k, float4& p, float& l) {
+                               p = a.p[i0 + k];
+                               float vmax;
+                               l = k < nl ? Z.lse[k] : sf_row_lse(a, S, Z, t, p, dust, npair, vmax);
+                           },
+                           s0, s1, s2, npair);
+            finish(j, s0, s1, s2);
         }
         __syncthreads();
     }
+    __syncthreads();
 }
 
 // MM on R (majorisation-minimisation with Wahba steps); planes in smem.
 __device__ void sf_mm(const SfArgs& a, SfShared& S, const SfScratch& Z, float* M6) {
     for (int k = threadIdx.x; k < 6 * a.M; k += blockDim.x) M6[k] = 0.0f;
     __syncthreads();
-    for (int t = 0; t < a.T; ++t) {
+    // angle by angle (the planes of one angle are distinct), by the first warp
+    for (int t = threadIdx.x < 32 ? 0 : a.T; t < a.T; ++t) {
         int j0 = S.t_off[t], j1 = S.t_off[t + 1];
         if (j0 == j1) continue;
         const float cg = S.cs[t].x, sg = S.cs[t].y;
-        for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {  // distinct planes within one angle
+        for (int j = j0 + threadIdx.x; j < j1; j += 32) {
             const float* v = Z.v + 3 * j;
             const float* e = a.G.e;
             float A[6] = {2 * v[0] * e[0], v[0] * e[1] + e[0] * v[1], v[0] * e[2] + e[0] * v[2],
@@ -669,8 +696,9 @@ __device__ void sf_mm(const SfArgs& a, SfShared& S, const SfScratch& Z, float* M
             float* dst = M6 + 6 * (Z.tm[j] & 0xffff);
             for (int k = 0; k < 6; ++k) dst[k] -= Gm[k];
         }
-        __syncthreads();
+        __syncwarp();
     }
+    __syncthreads();
     for (int p = threadIdx.x; p < a.M; p += blockDim.x) psd_shift(M6 + 6 * p);
     if (threadIdx.x == 0) S.stop = 0;
     __syncthreads();
