@@ -412,8 +412,10 @@ int laue_set_pair_skipping(laue_handle* h, int enable);
  * support); dust_mode 0 or 1 (the unbalanced mode is not offered here);
  * rho 1..64.  nbr (optional, device, model->n x rho ints): N(j) in order of
  * increasing cost, -1 past its end.  Needs a workspace of
- * laue_sparse_workspace_size bytes (16 rho |J| + 16 (|I| + |J|) bytes plus
- * small tables).  Asynchronous. */
+ * 16 rho |J| + 16 (|I| + |J|) bytes plus small tables; laue_sparse_workspace_size
+ * adds room for the direction order of the spots, with which the neighbours are
+ * searched near each ray only (without it among every pair, with the same
+ * result).  Asynchronous. */
 int laue_sparse_workspace_size(int T, int n_obs, int n_model, int rho, size_t* bytes);
 int laue_cost_sinkhorn_sparse(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* obs,
                               const LaueModelSpots* model, const LaueOTParams* prm, int rho, float* f,

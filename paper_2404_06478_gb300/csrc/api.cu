@@ -622,7 +622,8 @@ extern "C" int laue_cost_sinkhorn(laue_handle* h, const LaueGeometry* geom, cons
 
 extern "C" int laue_sparse_workspace_size(int T, int n_obs, int n_model, int rho, size_t* bytes) {
     if (!bytes || T < 1 || n_obs < 0 || n_model < 0 || rho < 1 || rho > kSparseMaxRho) return LAUE_ERR_INVALID_ARG;
-    *bytes = kCtrlBytes + sparse_workspace_bytes(T, n_obs, n_model, rho);
+    LaueProblemDims d{T, n_obs, n_model, 0, 0, 0, 0};
+    *bytes = align_up(kCtrlBytes + sparse_workspace_bytes(T, n_obs, n_model, rho), 256) + make_layout(d, 1).total;
     return LAUE_OK;
 }
 
@@ -687,8 +688,25 @@ extern "C" int laue_cost_sinkhorn_sparse(laue_handle* h, const LaueGeometry* geo
     a.nbr_out = nbr;
     bool rows = assign || margin || marg_err;
     bool cols = q || marg_err;
-    return laue_cuda_check(h, sparse_sinkhorn_run(a, prm->n_iter, rows, cols, (cudaStream_t)stream),
-                           "sparse sinkhorn launch");
+    // the neighbours' search takes the direction order and the cones of the dense passes where the workspace has
+    // room for them behind the sparse arrays
+    SkArgs sk;
+    SkLaunch lc;
+    const size_t behind = align_up(need, 256);
+    const LaueProblemDims d{obs->T, obs->n, model->n, 0, 0, 0, 0};
+    const Layout L = make_layout(d, h->sm_count);
+    const bool ordered = behind + L.total <= h->ws_bytes;
+    if (ordered) {
+        laue_handle view = *h;  // a handle on the rest of the workspace
+        view.ws = (char*)h->ws + behind;
+        view.ws_bytes = h->ws_bytes - behind;
+        LaueOTParams op = *prm;
+        op.warm_start = 0;
+        laue_fill_sk(&view, geom, obs, model, &op, L, &sk, &lc);
+    }
+    return laue_cuda_check(
+        h, sparse_sinkhorn_run(a, ordered ? &sk : nullptr, prm->n_iter, rows, cols, (cudaStream_t)stream),
+        "sparse sinkhorn launch");
 }
 
 // ------------------------------------------------------------- autotuner

@@ -187,7 +187,10 @@ struct SpArgs {
 constexpr int kSparseMaxRho = 64;  // neighbour lists live in shared memory while they are built
 size_t sparse_workspace_bytes(int T, int n_obs, int n_model, int rho);
 void sparse_carve(SpArgs& a, char* base, int T, int n_obs, int n_model, int rho);
-cudaError_t sparse_sinkhorn_run(const SpArgs& a, int n_iter, bool rows, bool cols, cudaStream_t s);
+// order: workspace of the direction order and cones of the same spots (null: the
+// neighbours are searched among every pair)
+cudaError_t sparse_sinkhorn_run(const SpArgs& a, const SkArgs* order, int n_iter, bool rows, bool cols,
+                                cudaStream_t s);
 
 constexpr int kSkVariants = 4;       // launch shapes of the pair passes (see sinkhorn.cu)
 constexpr int kSlicesPerSm = 20;      // slices of a pass that an SM holds at once

@@ -18,14 +18,15 @@
 // and the dustbin updates in the same order as the dense passes.
 //
 // Work split: the spots of each angle block are cut into tiles of kSpTile;
-// one CTA per tile, one warp per spot, the lanes over the spot's entries
-// (8-byte {index, e2} records read coalesced), a warp log-sum-exp with the
-// running maximum (no shifted fast sum, so no underflow fallback is needed).
-// The last CTA of a pass (completion ticket) merges the per-tile partial
-// log-sum-exps into the dustbin potentials, one warp per dustbin.
+// one CTA per tile, eight lanes per spot (8-byte {index, e2} records read
+// coalesced), sums shifted by the angle block's largest potential.  The
+// per-tile partial log-sum-exps of a pass are merged into the dustbin
+// potentials by the first blocks of the pass after it, which does not need
+// them yet (as for the dense passes), and passes overlap their launches.
 #include <algorithm>
 
 #include "api_internal.h"
+#include "slices.cuh"
 
 namespace laue {
 
@@ -68,19 +69,49 @@ __device__ __forceinline__ float sp_e2(float4 p, float4 c, float4 r) {
 }
 
 // ---------------------------------------------------------------- schedule
-__global__ void sp_schedule_kernel(SpArgs a) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    int nr = 0, nc = 0;
-    for (int t = 0; t < a.T; ++t) {
-        a.rt_base[t] = nr;
-        for (int s = a.I_off[t]; s < a.I_off[t + 1]; s += kSpTile)
-            a.rtile[nr++] = make_int4(t, s, min(s + kSpTile, a.I_off[t + 1]), 0);
-        a.ct_base[t] = nc;
-        for (int s = a.J_off[t]; s < a.J_off[t + 1]; s += kSpTile)
-            a.ctile[nc++] = make_int4(t, s, min(s + kSpTile, a.J_off[t + 1]), 0);
+// One CTA: tiles of every angle (rt_base / ct_base their prefix).
+__global__ void __launch_bounds__(1024) sp_schedule_kernel(SpArgs a) {
+    __shared__ int warp_sum[2][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int base[2] = {0, 0};
+    for (int t0 = 0; t0 < a.T; t0 += 1024) {
+        const int t = t0 + threadIdx.x;
+        int incl[2], c[2];
+        for (int k = 0; k < 2; ++k) {
+            const int* off = k ? a.J_off : a.I_off;
+            c[k] = t < a.T ? (off[t + 1] - off[t] + kSpTile - 1) / kSpTile : 0;
+            incl[k] = c[k];
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl[k], o);
+                if (lane >= o) incl[k] += y;
+            }
+            if (lane == 31) warp_sum[k][w] = incl[k];
+        }
+        __syncthreads();
+        for (int k = 0; k < 2; ++k) {
+            int before = base[k], all = 0;
+            for (int u = 0; u < 32; ++u) {
+                if (u < w) before += warp_sum[k][u];
+                all += warp_sum[k][u];
+            }
+            if (t < a.T) (k ? a.ct_base : a.rt_base)[t] = before + incl[k] - c[k];
+            base[k] += all;
+        }
+        __syncthreads();
     }
-    a.rt_base[a.T] = nr;
-    a.ct_base[a.T] = nc;
+    if (threadIdx.x == 0) {
+        a.rt_base[a.T] = base[0];
+        a.ct_base[a.T] = base[1];
+    }
+    __syncthreads();
+    for (int k = 0; k < 2; ++k) {
+        const int *off = k ? a.J_off : a.I_off, *tb = k ? a.ct_base : a.rt_base;
+        int4* tile = k ? a.ctile : a.rtile;
+        for (int q = threadIdx.x; q < base[k]; q += 1024) {
+            const int t = block_of(tb, a.T, q), s = off[t] + (q - tb[t]) * kSpTile;
+            tile[q] = make_int4(t, s, min(s + kSpTile, off[t + 1]), 0);
+        }
+    }
 }
 
 // ------------------------------------------------------------- neighbours
@@ -132,6 +163,106 @@ __global__ void __launch_bounds__(kKnnThreads) sp_knn_kernel(SpArgs a) {
     }
 }
 
+// The same lists where the workspace has room for the direction order and the
+// cones of the dense passes (k: a warp's 32 model spots of one granule): only
+// the observed sub-granules that the granule can see within an angle are
+// searched, an angle that should hold about twice rho spots at the block's
+// density; a warp with a spot that has fewer than rho neighbours inside it
+// searches again with a wider one.  The pairs come in the order of directions,
+// so an insertion compares (e2, index) and the lists are those of the search
+// over every pair.
+struct KnnStage {
+    float4 p[2][32];  // observed spots of a batch: x, y, z, caller's index
+};
+
+__global__ void __launch_bounds__(128) sp_knn_cone_kernel(SpArgs a, SkArgs k) {
+    extern __shared__ __align__(16) char knn_smem[];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    KnnStage& S = ((KnnStage*)knn_smem)[w];
+    int2* L = (int2*)(knn_smem + 4 * sizeof(KnnStage)) + (size_t)w * 32 * a.rho + lane;  // entry q at L[32 q]
+    const int half = blockIdx.x * 4 + w, g = half >> 1;
+    if (g >= k.mod_gbase[a.T]) return;
+    const int t = block_of(k.mod_gbase, a.T, g);
+    const int rank = 64 * (g - k.mod_gbase[t]) + 32 * (half & 1) + lane;
+    const int nj = a.J_off[t + 1] - a.J_off[t], i0 = a.I_off[t], ni = a.I_off[t + 1] - i0;
+    const bool valid = rank < nj;
+    if (!__any_sync(0xffffffffu, valid)) return;
+    const int j = valid ? k.mod_perm[a.J_off[t] + rank] : k.mod_perm[a.J_off[t]];
+    const float4 c = a.c[j], r = a.r[j];
+    const Cone own = load_cone(k.mod_cone, k.mod_ext, g);
+    const float4* sub = k.obs_sub + (size_t)kSubs * k.obs_gbase[t];
+    const float* ext = k.obs_subext + (size_t)kSubs * k.obs_gbase[t];
+    const int np = k.I2_off[t + 1] - k.I2_off[t];
+    const int want = min(a.rho, ni);
+    // two detectors see about 2 sr
+    float th = sqrtf(2.0f * 2.0f * (float)a.rho / (3.14159f * (float)max(ni, 1)));
+    int n = 0;
+    while (true) {
+        const bool everything = !(th < 1.5f);
+        const float sh = sinf(0.5f * fminf(th, 3.14f));
+        const float limit = everything ? 3.0e38f : 4.0f * sh * sh;
+        float worst = everything ? 3.0e38f : limit * 0.9999f;  // costs within it are all met
+        int worst_i = 0x7fffffff;
+        n = 0;
+        SubWalk walk;
+        walk.init(sub, ext, np);
+        auto fetch = [&](int st) {  // two sub-granules of 16 spots
+            const int s0 = walk.next(own, false, everything ? 0 : 1, 1.0f, limit);
+            const int s1 = s0 < 0 ? -1 : walk.next(own, false, everything ? 0 : 1, 1.0f, limit);
+            const int s = lane < 16 ? s0 : s1, q = 16 * s + (lane & 15);
+            float4 v = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(-1));
+            if (s >= 0 && q < ni) {
+                const int i = k.obs_perm[i0 + q];
+                v = a.p[i];
+                v.w = __int_as_float(i);
+            }
+            S.p[st][lane] = v;
+            return s0 >= 0;
+        };
+        int st = 0;
+        bool more = fetch(0);
+        while (more) {
+            __syncwarp();
+            const bool next = fetch(st ^ 1);
+#pragma unroll 4
+            for (int q = 0; q < 32; ++q) {
+                const float4 p = S.p[st][q];
+                const int i = __float_as_int(p.w);
+                const float v = sp_e2(p, c, r);
+                if (i < 0 || !(v < worst || (v == worst && i < worst_i))) continue;
+                int at = n < want ? n++ : want - 1;
+                while (at > 0) {
+                    const int2 b = L[32 * (at - 1)];
+                    const float bv = __int_as_float(b.y);
+                    if (!(bv > v || (bv == v && b.x > i))) break;
+                    L[32 * at] = b;
+                    --at;
+                }
+                L[32 * at] = make_int2(i, __float_as_int(v));
+                if (n == want) {
+                    const int2 b = L[32 * (want - 1)];
+                    worst = __int_as_float(b.y);
+                    worst_i = b.x;
+                }
+            }
+            st ^= 1;
+            more = next;
+        }
+        if (everything || !__any_sync(0xffffffffu, valid && n < want)) break;
+        th *= 1.6f;
+        __syncwarp();
+    }
+    if (!valid) return;
+    const int det = a.s ? (int)a.s[j].w : -1;
+    const float kd = (det >= 0 && det < a.n_det) ? a.kdet[det] : 1.0f;
+    int2* out = a.cent + (size_t)j * a.rho;
+    for (int q = 0; q < a.rho; ++q) {
+        const int2 b = q < n ? L[32 * q] : make_int2(-1, 0);
+        out[q] = q < n ? make_int2(b.x, __float_as_int(__int_as_float(b.y) * kd)) : b;
+        if (a.nbr_out) a.nbr_out[(size_t)j * a.rho + q] = b.x;
+    }
+}
+
 __global__ void sp_count_kernel(SpArgs a) {
     size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (size_t)a.n_model * a.rho) return;
@@ -139,29 +270,60 @@ __global__ void sp_count_kernel(SpArgs a) {
     if (i >= 0) atomicAdd(&a.rptr[i + 1], 1);
 }
 
-// inclusive prefix sum of rptr[1..n_obs] by one CTA (rptr[0] = 0)
-__global__ void __launch_bounds__(1024) sp_scan_kernel(SpArgs a) {
-    __shared__ int part[1024];
-    const int n = a.n_obs;
-    const int per = (n + 1023) / 1024;
-    const int b0 = 1 + (int)threadIdx.x * per, b1 = min(n + 1, b0 + per);
+// Inclusive prefix sum of rptr[1..n_obs] (rptr[0] = 0): sums of blocks of
+// kScan rows, then each block adds the sums before it.  The sums sit in the
+// fill counters, which are cleared after.
+constexpr int kScan = 8192;
+__global__ void __launch_bounds__(1024) sp_scan_sums_kernel(SpArgs a) {
+    __shared__ int warp_sum[32];
     int s = 0;
-    for (int b = b0; b < b1; ++b) s += a.rptr[b];
-    part[threadIdx.x] = s;
+    for (int k = threadIdx.x; k < kScan; k += 1024) {
+        const long long i = (long long)blockIdx.x * kScan + k;
+        if (i < a.n_obs) s += a.rptr[1 + i];
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) warp_sum[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
-        int acc = 0;
-        for (int k = 0; k < 1024; ++k) {
-            int v = part[k];
-            part[k] = acc;
-            acc += v;
-        }
+        for (int w = 1; w < 32; ++w) s += warp_sum[w];
+        a.rfill[blockIdx.x] = s;
     }
+}
+
+__global__ void __launch_bounds__(1024) sp_scan_kernel(SpArgs a) {
+    __shared__ int warp_sum[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    auto block_sum = [&](int s) {
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) warp_sum[w] = s;
+        __syncthreads();
+        int all = 0;
+        for (int u = 0; u < 32; ++u) all += warp_sum[u];
+        __syncthreads();
+        return all;
+    };
+    int before = 0;
+    for (int k = threadIdx.x; k < (int)blockIdx.x; k += 1024) before += a.rfill[k];
+    before = block_sum(before);
+    constexpr int kPer = kScan / 1024;
+    const long long i0 = (long long)blockIdx.x * kScan + kPer * threadIdx.x;
+    int v[kPer], s = 0;
+    for (int q = 0; q < kPer; ++q) {
+        v[q] = i0 + q < a.n_obs ? a.rptr[1 + i0 + q] : 0;
+        s += v[q];
+    }
+    int incl = s;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) warp_sum[w] = incl;
     __syncthreads();
-    int acc = part[threadIdx.x];
-    for (int b = b0; b < b1; ++b) {
-        acc += a.rptr[b];
-        a.rptr[b] = acc;
+    int at = before + incl - s;
+    for (int u = 0; u < w; ++u) at += warp_sum[u];
+    for (int q = 0; q < kPer; ++q) {
+        at += v[q];
+        if (i0 + q < a.n_obs) a.rptr[1 + i0 + q] = at;
     }
 }
 
@@ -258,31 +420,21 @@ __device__ __forceinline__ void sp_block_lse(float& m, float& s, float* red_m, f
     }
 }
 
-// True in the last CTA of the grid to arrive; that CTA resets the ticket.
-__device__ __forceinline__ bool sp_last(int* ticket, int* flag) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        int last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
-        if (last) *ticket = 0;
-        *flag = last;
-    }
-    __syncthreads();
-    bool last = *flag != 0;
-    if (last) __threadfence();
-    return last;
-}
-
 // Warp-level LSE of the partials of tiles [k0, k1) (valid in every lane).
 __device__ __forceinline__ void sp_merge_parts(const float2* part, int k0, int k1, float& m, float& s) {
     m = kNegHuge;
     s = 0.0f;
-    for (int k = k0 + (int)(threadIdx.x & 31); k < k1; k += 32) {
-        float2 v = part[k];
-        Lse2 L{m, s};
-        L.merge(v.x, v.y);
-        m = L.m;
-        s = L.s;
+    for (int k = k0 + (int)(threadIdx.x & 31); k < k1; k += 32 * 8) {
+        float2 v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = k + 32 * q < k1 ? __ldcg(&part[k + 32 * q]) : make_float2(kNegHuge, 0.0f);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            Lse2 L{m, s};
+            L.merge(v[q].x, v[q].y);
+            m = L.m;
+            s = L.s;
+        }
     }
     warp_lse_reduce(m, s);
 }
@@ -333,119 +485,134 @@ __global__ void __launch_bounds__(256) sp_gmax_kernel(SpArgs a) {
     }
 }
 
-__global__ void __launch_bounds__(kSpThreads) sp_row_kernel(SpArgs a) {
-    __shared__ float red_m[kSpWarps], red_s[kSpWarps];
-    __shared__ int flag;
+// Dustbin potentials from the tile partials of a pass.  Rows: F_0 of the
+// iteration and G_0 from it and the new F; columns: the next F_0 from the new G
+// and the current G_0.  A warp per dustbin.
+template <bool ROWS>
+__device__ __forceinline__ void sp_finish_pass(const SpArgs& a, int block, int blocks) {
     const int nd = a.mode ? a.T : 1;
-    SpDust D = sp_dust(a.dust, nd);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int grp = lane / kSpLanes, gl = lane % kSpLanes;
-    const int n_tiles = a.rt_base[a.T];
-    float pm = kNegHuge, ps = 0.0f;  // LSE of F_i - kc over this lane's rows
-    if ((int)blockIdx.x < n_tiles) {
-        const int4 td = a.rtile[blockIdx.x];
-        const float dustv = D.G0[a.mode ? td.x : 0] - a.kc;
-        const float shift = fmaxf(a.gmax[td.x], dustv);
-        const float dterm = ex2(dustv - shift);
-        for (int ib = td.y + w * (32 / kSpLanes); ib < td.z; ib += kSpWarps * (32 / kSpLanes)) {
-            const int i = ib + grp;
-            const bool vr = i < td.z;
-            float sum = 0.0f;
-            if (vr)
-                for (int e = a.rptr[i] + gl; e < a.rptr[i + 1]; e += kSpLanes) {
-                    int2 v = a.rent[e];
-                    sum += ex2(a.G[v.x] + a.negK * __int_as_float(v.y) - shift);
-                }
-#pragma unroll
-            for (int o = kSpLanes / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            if (vr && gl == 0) {
-                sum += dterm;
-                float F = -(sum > kSpTiny ? shift + lg2(sum) : sp_row_exact(a, i, dustv, false));
-                a.F[i] = F;
-                acc_lse(pm, ps, F - a.kc);
+    const SpDust D = sp_dust(a.dust, nd);
+    const int *base = ROWS ? a.rt_base : a.ct_base;
+    for (int d = block * kSpWarps + (int)(threadIdx.x >> 5); d < nd; d += blocks * kSpWarps) {
+        float m, s;
+        sp_merge_parts(ROWS ? a.rpart : a.cpart, a.mode ? base[d] : 0, a.mode ? base[d + 1] : base[a.T], m, s);
+        if ((threadIdx.x & 31) == 0) {
+            Lse2 L{m, s};
+            if (ROWS) {
+                const float F0 = __ldcg(D.F0n + d);
+                D.F0[d] = F0;
+                L.merge(F0 - a.kc, 1.0f);
+                D.G0[d] = D.log2O[d] - L.value();
+            } else {
+                L.merge(__ldcg(D.G0 + d) - a.kc, 1.0f);
+                D.F0n[d] = D.log2U[d] - L.value();
             }
         }
-    }
-    sp_block_lse(pm, ps, red_m, red_s);
-    if (threadIdx.x == 0 && (int)blockIdx.x < n_tiles) a.rpart[blockIdx.x] = make_float2(pm, ps);
-    if (!sp_last(a.ctrl + CTRL_SP_DONE, &flag)) return;
-    // promote F_0 and compute G_0 from the new F (as after a dense row pass)
-    for (int d = w; d < nd; d += kSpWarps) {
-        float m, s;
-        sp_merge_parts(a.rpart, a.mode ? a.rt_base[d] : 0, a.mode ? a.rt_base[d + 1] : n_tiles, m, s);
-        if (lane == 0) {
-            float F0 = D.F0n[d];
-            D.F0[d] = F0;
-            Lse2 L{m, s};
-            L.merge(F0 - a.kc, 1.0f);
-            D.G0[d] = D.log2O[d] - L.value();
-        }
-    }
-    // per-angle largest F for the column pass's shift (the tile partials keep max(F - kc))
-    for (int t = w; t < a.T; t += kSpWarps) {
-        float m = kNegHuge;
-        for (int k = a.rt_base[t] + lane; k < a.rt_base[t + 1]; k += 32) m = fmaxf(m, a.rpart[k].x);
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (lane == 0) a.fmax[t] = m > kNegHuge ? m + a.kc : kNegHuge;
     }
 }
 
-// ------------------------------------------------------------ column pass
-__global__ void __launch_bounds__(kSpThreads) sp_col_kernel(SpArgs a) {
+__global__ void __launch_bounds__(kSpThreads) sp_finish_pass_kernel(SpArgs a) {
+    sp_finish_pass<false>(a, blockIdx.x, gridDim.x);
+}
+
+// Row (ROWS) or column update of iteration it; the first blocks finish the
+// pass before.  Eight lanes per spot stride over its records, four records of
+// a lane and the records of two spots loaded together: bound by the latency of
+// record -> potential -> exponential.
+constexpr int kSpBatch = 4;
+
+template <bool ROWS>
+__global__ void __launch_bounds__(kSpThreads) sp_pass_kernel(SpArgs a, int it, int finishers) {
     __shared__ float red_m[kSpWarps], red_s[kSpWarps];
-    __shared__ int flag;
+    // programmatic dependent launch: everything read here was complete before the pass before waited
+    if (ROWS && it == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
     const int nd = a.mode ? a.T : 1;
-    SpDust D = sp_dust(a.dust, nd);
+    const SpDust D = sp_dust(a.dust, nd);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int grp = lane / kSpLanes, gl = lane % kSpLanes;
-    const int n_tiles = a.ct_base[a.T];
-    float pm = kNegHuge, ps = 0.0f;  // LSE of G_j over this lane's columns
-    if ((int)blockIdx.x < n_tiles) {
-        const int4 td = a.ctile[blockIdx.x];
-        const float F0 = D.F0[a.mode ? td.x : 0];
-        const float shift = fmaxf(a.fmax[td.x], F0);
-        const float dterm = ex2(F0 - shift);
-        for (int jb = td.y + w * (32 / kSpLanes); jb < td.z; jb += kSpWarps * (32 / kSpLanes)) {
-            const int j = jb + grp;
-            const bool vc = j < td.z;
-            float sum = 0.0f;
-            if (vc) {
-                const int2* ce = a.cent + (size_t)j * a.rho;
-                for (int k = gl; k < a.rho; k += kSpLanes) {
-                    int2 v = ce[k];
-                    if (v.x >= 0) sum += ex2(a.F[v.x] + a.negK * __int_as_float(v.y) - shift);
-                }
-            }
+    const int *base = ROWS ? a.rt_base : a.ct_base, *other = ROWS ? a.ct_base : a.rt_base;
+    const int tile = (int)blockIdx.x - finishers;
+    const bool live = tile >= 0 && tile < base[a.T];
+    const int4 td = live ? (ROWS ? a.rtile : a.ctile)[tile] : make_int4(0, 0, 0, 0);
+    const int o0 = other[td.x], o1 = other[td.x + 1];
+    if (!(ROWS && it == 0)) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (tile < 0) {
+        if (!ROWS || it > 0) sp_finish_pass<!ROWS>(a, blockIdx.x, finishers);
+        return;
+    }
+    if (!live) return;
+    const int2* rec = ROWS ? a.rent : a.cent;
+    const float* pot = ROWS ? a.G : a.F;
+    float* out = ROWS ? a.F : a.G;
+    const float off = ROWS ? a.kc : 0.0f;
+    // the dustbin's term; the other side's largest potential of the angle, from its tiles' partials (they keep
+    // max(F - kc) and max G)
+    const float dust = ROWS ? __ldcg(D.G0 + (a.mode ? td.x : 0)) - a.kc : __ldcg(D.F0n + (a.mode ? td.x : 0));
+    float top = kNegHuge;
+    if (ROWS && it == 0) {
+        top = a.gmax[td.x];
+    } else {
+        const float2* part = ROWS ? a.cpart : a.rpart;
+        for (int k = o0 + lane; k < o1; k += 32) top = fmaxf(top, __ldcg(&part[k].x));
 #pragma unroll
-            for (int o = kSpLanes / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            if (vc && gl == 0) {
-                sum += dterm;
-                float G = -(sum > kSpTiny ? shift + lg2(sum) : sp_col_exact(a, j, F0, false));
-                a.G[j] = G;
-                acc_lse(pm, ps, G);
+        for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+        if (!ROWS) top = top > kNegHuge ? top + a.kc : kNegHuge;
+    }
+    const float shift = fmaxf(top, dust);
+    const float dterm = ex2(dust - shift);
+    float pm = kNegHuge, ps = 0.0f;  // LSE of the new potentials (less kc) over this lane's spots
+    constexpr int kStep = kSpWarps * (32 / kSpLanes);
+    for (int ib = td.y + w * (32 / kSpLanes); ib < td.z; ib += 2 * kStep) {
+        int e0[2], e1[2];
+        float sum[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int i = ib + u * kStep + grp;
+            const bool v = i < td.z;
+            e0[u] = v ? (ROWS ? a.rptr[i] : i * a.rho) + gl : 0;
+            e1[u] = v ? (ROWS ? a.rptr[i + 1] : (i + 1) * a.rho) : 0;
+            sum[u] = 0.0f;
+        }
+        while (true) {
+            int2 v[2][kSpBatch];
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int q = 0; q < kSpBatch; ++q) {
+                    const int e = e0[u] + q * kSpLanes;
+                    v[u][q] = e < e1[u] ? __ldcg(&rec[e]) : make_int2(-1, 0);
+                }
+            float g[2][kSpBatch];
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int q = 0; q < kSpBatch; ++q) g[u][q] = v[u][q].x >= 0 ? pot[v[u][q].x] : 0.0f;
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int q = 0; q < kSpBatch; ++q)
+                    if (v[u][q].x >= 0) sum[u] += ex2(g[u][q] + a.negK * __int_as_float(v[u][q].y) - shift);
+            e0[0] += kSpBatch * kSpLanes;
+            e0[1] += kSpBatch * kSpLanes;
+            if (!__any_sync(0xffffffffu, e0[0] < e1[0] || e0[1] < e1[1])) break;
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int i = ib + u * kStep + grp;
+#pragma unroll
+            for (int o = kSpLanes / 2; o > 0; o >>= 1) sum[u] += __shfl_xor_sync(0xffffffffu, sum[u], o);
+            if (i < td.z && gl == 0) {
+                sum[u] += dterm;
+                const float lse = sum[u] > kSpTiny ? shift + lg2(sum[u])
+                                                   : (ROWS ? sp_row_exact(a, i, dust, false) : sp_col_exact(a, i, dust, false));
+                out[i] = -lse;
+                acc_lse(pm, ps, -lse - off);
             }
         }
     }
     sp_block_lse(pm, ps, red_m, red_s);
-    if (threadIdx.x == 0 && (int)blockIdx.x < n_tiles) a.cpart[blockIdx.x] = make_float2(pm, ps);
-    if (!sp_last(a.ctrl + CTRL_SP_DONE, &flag)) return;
-    // F_0 of the next row pass from the new G and the current G_0
-    for (int d = w; d < nd; d += kSpWarps) {
-        float m, s;
-        sp_merge_parts(a.cpart, a.mode ? a.ct_base[d] : 0, a.mode ? a.ct_base[d + 1] : n_tiles, m, s);
-        if (lane == 0) {
-            Lse2 L{m, s};
-            L.merge(D.G0[d] - a.kc, 1.0f);
-            D.F0n[d] = D.log2U[d] - L.value();
-        }
-    }
-    // per-angle largest G for the next row pass's shift (the tile partials keep max G)
-    for (int t = w; t < a.T; t += kSpWarps) {
-        float m = kNegHuge;
-        for (int k = a.ct_base[t] + lane; k < a.ct_base[t + 1]; k += 32) m = fmaxf(m, a.cpart[k].x);
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (lane == 0) a.gmax[t] = m;
-    }
+    if (threadIdx.x == 0) (ROWS ? a.rpart : a.cpart)[tile] = make_float2(pm, ps);
 }
 
 // ------------------------------------------------------------- read-out
@@ -642,22 +809,52 @@ void sparse_carve(SpArgs& a, char* base, int T, int n_obs, int n_model, int rho)
 
 size_t sparse_knn_smem(int rho) { return (size_t)kKnnThreads * rho * sizeof(int2); }
 
-cudaError_t sparse_sinkhorn_run(const SpArgs& a, int n_iter, bool rows, bool cols, cudaStream_t s) {
+template <bool ROWS>
+static cudaError_t sp_pass(const SpArgs& a, int it, cudaStream_t s) {
+    const int finishers = a.mode ? (a.T + kSpWarps - 1) / kSpWarps : 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(finishers + (ROWS ? a.max_rt : a.max_ct));
+    c.blockDim = dim3(kSpThreads);
+    c.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, sp_pass_kernel<ROWS>, a, it, finishers);
+}
+
+cudaError_t sparse_sinkhorn_run(const SpArgs& a, const SkArgs* order, int n_iter, bool rows, bool cols,
+                                cudaStream_t s) {
     cudaError_t e;
     const size_t nnz = (size_t)a.n_model * a.rho;
     const int nd = a.mode ? a.T : 1;
-    sp_schedule_kernel<<<1, 32, 0, s>>>(a);
+    sp_schedule_kernel<<<1, 1024, 0, s>>>(a);
     // neighbour lists and their transpose
-    const size_t shm = sparse_knn_smem(a.rho);
-    if ((e = cudaFuncSetAttribute(sp_knn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm)) !=
-        cudaSuccess)
-        return e;
-    sp_knn_kernel<<<a.max_ct, kKnnThreads, shm, s>>>(a);
+    if (order && a.n_obs > 0 && a.n_model > 0) {
+        if ((e = sinkhorn_prepare(*order, s, false)) != cudaSuccess) return e;
+        const size_t shm = 4 * sizeof(KnnStage) + (size_t)128 * a.rho * sizeof(int2);
+        if ((e = cudaFuncSetAttribute(sp_knn_cone_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm)) !=
+            cudaSuccess)
+            return e;
+        const int halves = 2 * (a.n_model / 64 + a.T + 1);  // bound on the granules' halves
+        sp_knn_cone_kernel<<<(halves + 3) / 4, 128, shm, s>>>(a, *order);
+    } else {
+        const size_t shm = sparse_knn_smem(a.rho);
+        if ((e = cudaFuncSetAttribute(sp_knn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm)) !=
+            cudaSuccess)
+            return e;
+        sp_knn_kernel<<<a.max_ct, kKnnThreads, shm, s>>>(a);
+    }
     if ((e = cudaMemsetAsync(a.rptr, 0, sizeof(int) * ((size_t)a.n_obs + 2), s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(a.rfill, 0, sizeof(int) * ((size_t)a.n_obs + 1), s)) != cudaSuccess) return e;
     const unsigned nb = (unsigned)((nnz + 255) / 256);
     if (nnz > 0) sp_count_kernel<<<nb, 256, 0, s>>>(a);
-    sp_scan_kernel<<<1, 1024, 0, s>>>(a);
+    if (a.n_obs > 0) {
+        const int blocks = (a.n_obs + kScan - 1) / kScan;
+        sp_scan_sums_kernel<<<blocks, 1024, 0, s>>>(a);
+        sp_scan_kernel<<<blocks, 1024, 0, s>>>(a);
+    }
+    if ((e = cudaMemsetAsync(a.rfill, 0, sizeof(int) * ((size_t)a.n_obs + 1), s)) != cudaSuccess) return e;
     if (nnz > 0) sp_fill_kernel<<<nb, 256, 0, s>>>(a);
     if (a.n_obs > 0) sp_sort_rows_kernel<<<(a.n_obs + 255) / 256, 256, 0, s>>>(a);
     const int blocks = std::max(1, (std::max(a.n_obs, a.n_model) + 255) / 256);
@@ -665,9 +862,10 @@ cudaError_t sparse_sinkhorn_run(const SpArgs& a, int n_iter, bool rows, bool col
     sp_init_dust_kernel<<<nd, 1024, 0, s>>>(a);
     if (a.T > 0) sp_gmax_kernel<<<a.T, 256, 0, s>>>(a);
     for (int it = 0; it < n_iter; ++it) {
-        sp_row_kernel<<<a.max_rt, kSpThreads, 0, s>>>(a);
-        sp_col_kernel<<<a.max_ct, kSpThreads, 0, s>>>(a);
+        if ((e = sp_pass<true>(a, it, s)) != cudaSuccess) return e;
+        if ((e = sp_pass<false>(a, it, s)) != cudaSuccess) return e;
     }
+    if (n_iter > 0) sp_finish_pass_kernel<<<a.mode ? (a.T + kSpWarps - 1) / kSpWarps : 1, kSpThreads, 0, s>>>(a);
     if (rows || cols) sp_clear_err_kernel<<<1, 1, 0, s>>>(a);
     if (rows) sp_harvest_row_kernel<<<a.max_rt, kSpThreads, 0, s>>>(a);
     if (cols) sp_harvest_col_kernel<<<a.max_ct, kSpThreads, 0, s>>>(a);

@@ -103,3 +103,31 @@ def test_lists_sweeps_and_every_pair_agree(env, geom, eps, mode, sizes):
         assert torch.equal(listed[k].nan_to_num(9e9), every[k].nan_to_num(9e9)), ("every pair", k)
         assert torch.equal(listed[k].nan_to_num(9e9), swept[k].nan_to_num(9e9)), ("swept", k)
     del keep
+
+
+@pytest.mark.parametrize("rho", [1, 8, 64])
+@pytest.mark.parametrize("sizes", [EDGES, [(5000, 40), (3, 900), (64, 64)]], ids=["edges", "uneven"])
+def test_sparse_neighbour_searches_agree(env, rho, sizes):
+    """The neighbour search over the cones against the one over every pair
+    (which a workspace without room for the order takes): lists, potentials
+    and read-out equal bit for bit."""
+    api, torch, dev = env["api"], env["torch"], env["dev"]
+    p, I_off, m, J_off = _blocks(sizes, 22, GEOM)
+    ob = api.ObsSpots.from_numpy(p, I_off, device=dev)
+    ms = api.ModelSpots.from_numpy(J_off, m["grain"], m["plane"], m["ray"], m["center"], m["spot"], m["det"], device=dev)
+    h = api.Handle(dev)
+
+    def call():
+        out = api.cost_sinkhorn_sparse(h, GEOM, ob, ms, 2.0, 2.25, 15, rho=rho, dust_mode=1, col_harvest=True,
+                                       neighbours=True)
+        torch.cuda.synchronize()
+        return out
+
+    cones = call()
+    size = h.ws.numel()
+    h.reserve_bytes = lambda *a, **k: None
+    keep = _smallest_workspace(h, torch, call, size)
+    pairs = call()
+    for k in cones:
+        assert torch.equal(cones[k].nan_to_num(9e9), pairs[k].nan_to_num(9e9)), k
+    del keep
