@@ -317,6 +317,7 @@ __device__ __forceinline__ uint32_t dist_key(float4 n, float3 n0) {
 }
 
 constexpr int kSetThreads = 256;
+static_assert(kSetThreads == 2 * KSET, "the sort takes a thread per pair of the two KSETs");
 
 // Finds, among the keys of [lo, hi) minus i0 that match `prefix` on the
 // bits of `pmask`, the bin of bits [sh, sh + nbits) that holds the k-th
@@ -354,13 +355,177 @@ __device__ void radix_round(const SetsArgs& a, int lo, int hi, int i0, float3 n0
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kSetThreads) sets_kernel(SetsArgs a) {
-    __shared__ int hist[2048];
-    __shared__ int part[kSetThreads];
-    __shared__ unsigned long long sel[KSET];
-    __shared__ int wcnt[kSetThreads / 32];
-    __shared__ int nsel_s, ties_s;
+// The k-th smallest key (1-based) of the n candidates in shared memory, eight
+// bits at a time.
+__device__ uint32_t select_key(const unsigned long long* cand, int n, int k, int* hist, int* found) {
+    uint32_t prefix = 0, pmask = 0;
+    for (int sh = 24; sh >= 0; sh -= 8) {
+        if (threadIdx.x < 256) hist[threadIdx.x] = 0;
+        __syncthreads();
+        for (int q = threadIdx.x; q < n; q += kSetThreads) {
+            const uint32_t key = (uint32_t)(cand[q] >> 32);
+            if ((key & pmask) == prefix) atomicAdd(&hist[(key >> sh) & 255u], 1);
+        }
+        __syncthreads();
+        if (threadIdx.x < 32) {  // the bin that holds it: eight bins to a lane
+            int c[8], sum = 0;
+            for (int q = 0; q < 8; ++q) sum += c[q] = hist[8 * threadIdx.x + q];
+            int incl = sum;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if ((int)threadIdx.x >= o) incl += y;
+            }
+            int at = incl - sum;
+            if (at < k && k <= incl)
+                for (int q = 0; q < 8; ++q) {
+                    if (at + c[q] >= k) {
+                        found[0] = 8 * threadIdx.x + q;
+                        found[1] = k - at;
+                        break;
+                    }
+                    at += c[q];
+                }
+        }
+        __syncthreads();
+        prefix |= (uint32_t)found[0] << sh;
+        pmask |= 255u << sh;
+        k = found[1];
+        __syncthreads();
+    }
+    return prefix;
+}
+
+// The KSET - 1 smallest (key, index) of the spots [lo, hi) without i0, count of
+// them, into sel: any order, at most 2 KSET with the ties of the last key.  A
+// fraction d of the axes lies within distance d of a direction if they are
+// spread evenly, so the spots nearer than a few times the distance that should
+// hold KSET are collected in one pass over the axes, and the rest of the work
+// is on them (about a thousand) in shared memory; a window whose axes are
+// spread otherwise is read again with another distance.  Returns the number
+// collected, -1 when that does not succeed (select_wide then takes over).
+constexpr int kCand = 4096;
+__device__ int select_near(const SetsArgs& a, int lo, int hi, int i0, float3 n0, int count, unsigned long long* cand,
+                           int* hist, int* found, unsigned long long* sel) {
+    const int lane = threadIdx.x & 31;
+    const int K = min(KSET - 1, count);
+    float cut = count <= kCand ? 2.0f : 8.0f * (float)KSET / (float)count;
+    int n = 0;
+    for (int attempt = 0;; ++attempt) {
+        if (attempt == 4) return -1;
+        if (threadIdx.x == 0) found[2] = 0;
+        __syncthreads();
+        const uint32_t most = __float_as_uint(cut);
+        for (int base = lo; base < hi; base += 4 * kSetThreads) {
+            float4 x[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = base + q * kSetThreads + threadIdx.x;
+                if (i < hi) x[q] = a.axes[i];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = base + q * kSetThreads + threadIdx.x;
+                const uint32_t key = i < hi && i != i0 ? dist_key(x[q], n0) : 0xFFFFFFFFu;
+                const bool in = key <= most;
+                const unsigned b = __ballot_sync(0xffffffffu, in);
+                int at = 0;
+                if (lane == 0 && b) at = atomicAdd(&found[2], __popc(b));
+                at = __shfl_sync(0xffffffffu, at, 0) + __popc(b & ((1u << lane) - 1u));
+                if (in && at < kCand) cand[at] = ((unsigned long long)key << 32) | (uint32_t)i;
+            }
+        }
+        __syncthreads();
+        n = found[2];
+        __syncthreads();
+        if (n > kCand) cut *= 0.25f;
+        else if (n < K) cut = fminf(2.0f, 4.0f * cut);
+        else break;
+    }
+    if (n <= 2 * KSET) {
+        for (int q = threadIdx.x; q < n; q += kSetThreads) sel[q] = cand[q];
+        __syncthreads();
+        return n;
+    }
+    const uint32_t tau = select_key(cand, n, K, hist, found);
+    if (threadIdx.x == 0) found[2] = 0;
+    __syncthreads();
+    for (int q = threadIdx.x; q < n; q += kSetThreads)
+        if ((uint32_t)(cand[q] >> 32) <= tau) {
+            const int at = atomicAdd(&found[2], 1);
+            if (at < 2 * KSET) sel[at] = cand[q];
+        }
+    __syncthreads();
+    n = found[2];
+    __syncthreads();
+    return n <= 2 * KSET ? n : -1;
+}
+
+// The same by radix rounds over the axes and an ordered collection.
+__device__ __noinline__ void select_wide(const SetsArgs& a, int lo, int hi, int i0, float3 n0, int count, int* hist,
+                                         int* part, int* wcnt, int* nsel, int* ties, unsigned long long* sel) {
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    int &nsel_s = *nsel, &ties_s = *ties;
+    uint32_t tau = 0xFFFFFFFFu;
+    int k_tie = 0x7FFFFFFF;
+    if (count > KSET - 1) {
+        uint32_t prefix = 0, pmask = 0;
+        int k = KSET - 1;
+        radix_round(a, lo, hi, i0, n0, 21, 11, prefix, pmask, k, hist, part);
+        radix_round(a, lo, hi, i0, n0, 10, 11, prefix, pmask, k, hist, part);
+        radix_round(a, lo, hi, i0, n0, 0, 10, prefix, pmask, k, hist, part);
+        tau = prefix;
+        k_tie = k;
+    }
+    // ordered collection: keys < tau, then the first k_tie keys == tau by index
+    if (threadIdx.x == 0) {
+        nsel_s = 0;
+        ties_s = 0;
+    }
+    for (int e = threadIdx.x; e < 2 * KSET; e += blockDim.x) sel[e] = ~0ull;
+    __syncthreads();
+    for (int base = lo; base < hi; base += blockDim.x) {
+        int i = base + threadIdx.x;
+        uint32_t key = 0;
+        bool in = i < hi && i != i0;
+        if (in) key = dist_key(a.axes[i], n0);
+        bool lt = in && (count <= KSET - 1 || key < tau);
+        bool eq = in && count > KSET - 1 && key == tau;
+        unsigned beq = __ballot_sync(0xffffffffu, eq);
+        if (lane == 0) wcnt[wp] = __popc(beq);
+        __syncthreads();
+        int before = 0, tot = 0;
+        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
+            if (q < wp) before += wcnt[q];
+            tot += wcnt[q];
+        }
+        int tie_rank = ties_s + before + __popc(beq & ((1u << lane) - 1u));
+        bool take = lt || (eq && tie_rank < k_tie);
+        __syncthreads();
+        unsigned bt = __ballot_sync(0xffffffffu, take);
+        if (lane == 0) wcnt[wp] = __popc(bt);
+        __syncthreads();
+        int bt_before = 0, bt_tot = 0;
+        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
+            if (q < wp) bt_before += wcnt[q];
+            bt_tot += wcnt[q];
+        }
+        int pos = nsel_s + bt_before + __popc(bt & ((1u << lane) - 1u));
+        if (take && pos < KSET - 1) sel[pos] = ((unsigned long long)key << 32) | (uint32_t)i;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            nsel_s += bt_tot;
+            ties_s += tot;
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kSetThreads) sets_kernel(SetsArgs a) {
+    __shared__ unsigned long long cand[kCand];
+    __shared__ int part[kSetThreads];
+    __shared__ unsigned long long sel[2 * KSET];
+    __shared__ int wcnt[kSetThreads / 32], hist[256], found[3];
+    __shared__ int nsel_s, ties_s;
     const int n_total = a.I_off[a.n_angles];
     for (int b = blockIdx.x; b < a.B; b += gridDim.x) {
         int i0 = a.seeds[b];
@@ -390,75 +555,29 @@ __global__ void __launch_bounds__(kSetThreads) sets_kernel(SetsArgs a) {
         const int lo = a.I_off[wl], hi = a.I_off[wh];
         const int count = hi - lo - ((i0 >= lo && i0 < hi) ? 1 : 0);
         const int K = min(KSET - 1, count);
-        uint32_t tau = 0xFFFFFFFFu;
-        int k_tie = 0x7FFFFFFF;
-        if (count > KSET - 1) {
-            uint32_t prefix = 0, pmask = 0;
-            int k = KSET - 1;
-            radix_round(a, lo, hi, i0, n0, 21, 11, prefix, pmask, k, hist, part);
-            radix_round(a, lo, hi, i0, n0, 10, 11, prefix, pmask, k, hist, part);
-            radix_round(a, lo, hi, i0, n0, 0, 10, prefix, pmask, k, hist, part);
-            tau = prefix;
-            k_tie = k;
-        }
-        // ordered collection: keys < tau, then the first k_tie keys == tau by index
-        if (threadIdx.x == 0) {
-            nsel_s = 0;
-            ties_s = 0;
-        }
-        for (int e = threadIdx.x; e < KSET; e += blockDim.x) sel[e] = ~0ull;
-        __syncthreads();
-        for (int base = lo; base < hi; base += blockDim.x) {
-            int i = base + threadIdx.x;
-            uint32_t key = 0;
-            bool in = i < hi && i != i0;
-            if (in) key = dist_key(a.axes[i], n0);
-            bool lt = in && (count <= KSET - 1 || key < tau);
-            bool eq = in && count > KSET - 1 && key == tau;
-            unsigned beq = __ballot_sync(0xffffffffu, eq);
-            if (lane == 0) wcnt[wp] = __popc(beq);
-            __syncthreads();
-            int before = 0, tot = 0;
-            for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
-                if (q < wp) before += wcnt[q];
-                tot += wcnt[q];
-            }
-            int tie_rank = ties_s + before + __popc(beq & ((1u << lane) - 1u));
-            bool take = lt || (eq && tie_rank < k_tie);
-            __syncthreads();
-            unsigned bt = __ballot_sync(0xffffffffu, take);
-            if (lane == 0) wcnt[wp] = __popc(bt);
-            __syncthreads();
-            int bt_before = 0, bt_tot = 0;
-            for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
-                if (q < wp) bt_before += wcnt[q];
-                bt_tot += wcnt[q];
-            }
-            int pos = nsel_s + bt_before + __popc(bt & ((1u << lane) - 1u));
-            if (take && pos < KSET - 1) sel[pos] = ((unsigned long long)key << 32) | (uint32_t)i;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                nsel_s += bt_tot;
-                ties_s += tot;
-            }
+        const int n_sel = select_near(a, lo, hi, i0, n0, count, cand, hist, found, sel);
+        if (n_sel < 0) {
+            select_wide(a, lo, hi, i0, n0, count, (int*)cand, part, wcnt, &nsel_s, &ties_s, sel);
+        } else {
+            for (int e = n_sel + threadIdx.x; e < 2 * KSET; e += kSetThreads) sel[e] = ~0ull;
             __syncthreads();
         }
         // bitonic sort of the (key, index) pairs, ascending
-        for (int size = 2; size <= KSET; size <<= 1) {
+        for (int size = 2; size <= 2 * KSET; size <<= 1) {
             for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                for (int e = threadIdx.x; e < KSET; e += blockDim.x) {
-                    int partner = e ^ stride;
-                    if (partner > e) {
-                        bool up = (e & size) == 0;
-                        unsigned long long x = sel[e], y = sel[partner];
-                        if ((x > y) == up) {
-                            sel[e] = y;
-                            sel[partner] = x;
-                        }
+                const int e = threadIdx.x, partner = e ^ stride;
+                if (partner > e) {
+                    bool up = (e & size) == 0;
+                    unsigned long long x = sel[e], y = sel[partner];
+                    if ((x > y) == up) {
+                        sel[e] = y;
+                        sel[partner] = x;
                     }
                 }
-                __syncthreads();
+                if (stride > 16) __syncthreads();
+                else __syncwarp();
             }
+            __syncthreads();
         }
         // seed frame
         float a1x = -n0.y * n0.x, a1y = 1.0f - n0.y * n0.y, a1z = -n0.y * n0.z;
