@@ -36,7 +36,10 @@ constexpr float kFarLog2 = 60.0f;     // see the read-out kernels
 // passes would recompute: 0.44 % of the 9.2e9 same-angle pairs of the
 // 1000-grain configuration at 1 mm^2, where the passes used to evaluate
 // 28.9 %.  A pass then streams 6 bytes per entry (HBM) instead of spending 13
-// packed instructions and two MUFU per evaluated pair.
+// packed instructions and two MUFU per evaluated pair.  Measured at that size:
+// listing 1.72 + 1.50 ms once, a pass 1.57 / 1.50 ms before and 0.069 ms now.
+// A single iteration is not worth listing for: one sweep of both sides takes
+// about as long (sinkhorn_run).
 //
 // One warp lists one slice; chunks come from the pool as the longest of the
 // slice's 64 lists grows (a chunk's place in the pool is not reproducible, its
@@ -383,12 +386,12 @@ __device__ __forceinline__ void swept_sum(const SkArgs& a, WarpStage& S, const S
     out = ListSum{lo(Sa), hi(Sa), lo(Sb), hi(Sb)};
 }
 
-// Exact log-sum-exps (running maximum) of the lanes' two spots over the whole
-// block, where a shifted sum underflowed: four streamed pairs to a group.
-template <bool ROWS>
-__device__ __noinline__ void exact_lse(const SkArgs& a, WarpStage& S, const Slice& sl, float dust, float& va_out,
-                                       float& vb_out) {
-    RowLse A, B;
+// Exact log-sum-exps (running maximum) of the lanes' two spots over part
+// `part` of PARTS of the block (dust: the starting value), where a shifted sum
+// underflowed: four streamed pairs to a group.
+template <bool ROWS, int PARTS>
+__device__ __forceinline__ void exact_sums(const SkArgs& a, WarpStage& S, const Slice& sl, float dust, int part,
+                                           RowLse& A, RowLse& B) {
     A.init(dust);
     B.init(dust);
     RowPair R{};
@@ -396,7 +399,14 @@ __device__ __noinline__ void exact_lse(const SkArgs& a, WarpStage& S, const Slic
     if (ROWS) R = load_row_pair(a, sl.q, sl.valid);
     else load_col_pair(a, sl.valid ? sl.q : sl.q - sl.lane, C);
     const Sweep w = sweep_of<ROWS>(a, sl);
-    sweep<ROWS>(a, S, w.own, w.sub, w.ext, w.b0, w.n, 0, kSkipLog2, ROWS ? a.Gc : a.Fc, [&](int st, int n, const int4&) {
+    int from = 0, to = w.n;
+    if (PARTS > 1) {
+        const int subs = (w.n + kSubGran - 1) / kSubGran;
+        from = subs * part / PARTS * kSubGran;
+        to = min(subs * (part + 1) / PARTS * kSubGran, w.n);
+    }
+    sweep<ROWS>(a, S, w.own, w.sub, w.ext, w.b0 + from, to - from, 0, kSkipLog2, ROWS ? a.Gc : a.Fc,
+                [&](int st, int n, const int4&) {
         auto pair = [&](int j, f2& va, f2& vb) {
             const f2 base = *(const f2*)&S.P[st][j];
             if (ROWS) row_pair_v(R, S, st, j, base, va, vb);
@@ -417,8 +427,23 @@ __device__ __noinline__ void exact_lse(const SkArgs& a, WarpStage& S, const Slic
             B.add1(vb);
         }
     });
+}
+
+template <bool ROWS>
+__device__ __noinline__ void exact_lse(const SkArgs& a, WarpStage& S, const Slice& sl, float dust, float& va_out,
+                                       float& vb_out) {
+    RowLse A, B;
+    exact_sums<ROWS, 1>(a, S, sl, dust, 0, A, B);
     va_out = A.value();
     vb_out = B.value();
+}
+
+// One of several parts: {max a, sum a, max b, sum b}.
+template <bool ROWS, int PARTS>
+__device__ __noinline__ float4 exact_part(const SkArgs& a, WarpStage& S, const Slice& sl, float dust, int part) {
+    RowLse A, B;
+    exact_sums<ROWS, PARTS>(a, S, sl, dust, part, A, B);
+    return make_float4(A.m, lo(A.S) + hi(A.S), B.m, lo(B.S) + hi(B.S));
 }
 
 // ----------------------------------------------------- ends of the passes
@@ -588,6 +613,26 @@ struct PassShared {
     int last;
 };
 
+// A split pass (see sk_pass_kernel): for each slice kExactParts - 1 more warps,
+// that read their parts of the block when its sums underflowed.
+constexpr int kExactParts = 4;
+template <int THREADS>
+struct ExactShared {
+    WarpStage stage[kExactParts - 1][THREADS / 32];
+    float4 lse[kExactParts - 1][THREADS];
+    unsigned low[THREADS / 32];
+};
+template <int TILE, int OTHER>
+constexpr __host__ __device__ size_t pass_smem_bytes() {
+    constexpr int thr = pass_threads(TILE, OTHER);
+    constexpr size_t own = sizeof(PassShared<TILE, thr>), other = sizeof(PassShared<OTHER, thr>);
+    return ((own > other ? own : other) + 127) / 128 * 128;
+}
+// The warps of a slice.
+__device__ __forceinline__ void slice_barrier(int warp) {
+    asm volatile("bar.sync %0, %1;" ::"r"(5 + warp), "n"(32 * kExactParts) : "memory");
+}
+
 // Dustbin potentials from the partials of a pass: rows (of iteration it): F_0
 // of the iteration and G_0 from it and the new F; columns: the next F_0 from
 // the new G and the current G_0.  Block `block` of `blocks`; also clears the
@@ -598,7 +643,7 @@ __device__ void finish_pass(const SkArgs& a, PassShared<TILE, THREADS>& H, int b
     const int lane = threadIdx.x & 31;
     const float2* part = ROWS ? a.row_part : a.col_part;
     if (a.mode == 1) {
-        const int warps = blockDim.x >> 5;
+        constexpr int warps = THREADS / 32;
         for (int u = block * warps + (threadIdx.x >> 5); u < a.T; u += blocks * warps) {
             const int4 at = a.ang_tiles[u];
             const float v0 = __ldcg((ROWS ? D.F0n : D.G0) + u);
@@ -634,7 +679,7 @@ __device__ void finish_pass(const SkArgs& a, PassShared<TILE, THREADS>& H, int b
     }
     if (block == 0) {
         if (clear)
-            for (int u = threadIdx.x; u < a.T; u += blockDim.x) clear[u] = 0u;
+            for (int u = threadIdx.x; u < a.T; u += THREADS) clear[u] = 0u;
         if (threadIdx.x == 0)
             *(unsigned long long*)(a.ctrl + CTRL_SK_PAIRS) +=
                 __ldcg((const unsigned long long*)(a.ctrl + (ROWS ? CTRL_ROW_EVAL : CTRL_COL_EVAL)));
@@ -662,17 +707,31 @@ __device__ __forceinline__ void pass_release() { asm volatile("griddepcontrol.la
 
 // --------------------------------------------------- row and column passes
 // Iteration `it` of the row (ROWS) or column update.  What bounds it: at the
-// 1000-grain density the lists (HBM), below that the chain of a pass: launch,
-// gathers of the potentials, partial sums.  The other side's tile width, for
-// the partials that the first blocks merge, is OTHER.
-template <int TILE, int OTHER, bool ROWS>
-__global__ void __launch_bounds__(pass_threads(TILE, OTHER), 1024 / pass_threads(TILE, OTHER))
+// 1000-grain density the lists (324 MB a pass, 48 us at the copy rate, 69 us
+// measured: 4.7 TB/s), below that the chain of a pass: launch, gathers of the
+// potentials, partial sums (100 grains: 53 / 43 us a pass when it evaluated
+// pairs, 4.1 us now; 5 grains: 11 and 3.0 us).  The other side's tile width,
+// for the partials that the first blocks merge, is OTHER.
+//
+// Without dustbins (unbalanced OT) a shifted sum underflows for most spots:
+// the potentials of spots far from any partner are the largest, and shift all
+// the others.  Their slices read the whole block with a running maximum, a
+// serial chain of about 0.1 us per 4 pairs, so a pass over few slices has
+// PARTS warps to a slice that read a part of the block each; part 0's warp
+// merges.  23 grains x 17 angles at 4 mm^2: 23 us a pass with one warp, 14 us
+// with four.
+template <int TILE, int OTHER, bool ROWS, int PARTS>
+__global__ void __launch_bounds__(PARTS* pass_threads(TILE, OTHER), 1024 / pass_threads(TILE, OTHER) / PARTS)
     sk_pass_kernel(SkArgs a, int it, int finishers) {
     extern __shared__ __align__(128) char pass_smem[];
     constexpr int kThreads = pass_threads(TILE, OTHER);
     PassShared<TILE, kThreads>& H = *(PassShared<TILE, kThreads>*)pass_smem;
+    ExactShared<kThreads>& X = *(ExactShared<kThreads>*)(pass_smem + pass_smem_bytes<TILE, OTHER>());
+    const int part = PARTS > 1 ? threadIdx.x / kThreads : 0, own = threadIdx.x - part * kThreads;
+    const int warp = own >> 5;
     if (ROWS && it == 0) pass_wait();  // the first pass follows the kernels that write the lists
     if ((int)blockIdx.x < finishers) {
+        if (PARTS > 1 && part > 0) return;
         if (!(ROWS && it == 0)) pass_wait();
         pass_release();
         unsigned* clear = ROWS ? col_max(a, it) : row_max(a, it + 1);
@@ -683,13 +742,24 @@ __global__ void __launch_bounds__(pass_threads(TILE, OTHER), 1024 / pass_threads
     const SliceDesc* desc = (const SliceDesc*)(ROWS ? a.row_desc : a.col_desc);
     const int* tab = ROWS ? a.row_tab : a.col_tab;
     constexpr int kW = TILE / 32;
-    const int at = (blockIdx.x - finishers) * (kThreads / TILE) + (int)threadIdx.x / TILE;
+    const int at = (blockIdx.x - finishers) * (kThreads / TILE) + own / TILE;
     if (at >= __ldcg(a.ctrl + (ROWS ? CTRL_N_ROW_TILES : CTRL_N_COL_TILES))) return;
-    WarpBuffer& M = H.w[threadIdx.x >> 5];
     const int* order = ROWS ? a.row_order : a.col_order;
-    const int tile = order ? __ldcg(order + at) : at, id = tile * kW + (threadIdx.x >> 5) % kW;
-    const int numbers = chunk_numbers(a, tab, id, threadIdx.x & 31, 0);
+    const int tile = order ? __ldcg(order + at) : at, id = tile * kW + warp % kW;
+    int numbers = 0;
+    if (part == 0) numbers = chunk_numbers(a, tab, id, threadIdx.x & 31, 0);
     const Slice sl = load_slice(desc, id);
+    if (PARTS > 1 && part > 0) {
+        if (!(ROWS && it == 0)) pass_wait();
+        pass_release();
+        if (!sl.any) return;
+        slice_barrier(warp);
+        if (!X.low[warp]) return;
+        X.lse[part - 1][own] = exact_part<ROWS, PARTS>(a, X.stage[part - 1][warp], sl, kNegHuge, part);
+        slice_barrier(warp);
+        return;
+    }
+    WarpBuffer& M = H.w[warp];
     ring_start(a, M.ring, sl, numbers);
     const int t = sl.t, lane = sl.lane;
     float2 K = make_float2(a.negKD2, a.negKD2);  // -K of the lane's own spots (columns)
@@ -721,9 +791,25 @@ __global__ void __launch_bounds__(pass_threads(TILE, OTHER), 1024 / pass_threads
         float va = -(shift + lg2(sa)), vv = sl.vb ? -(shift + lg2(sb)) : 0.0f;
         const unsigned low_a = __ballot_sync(0xffffffffu, sl.valid && !(sa > kTinySum));
         const unsigned low_b = __ballot_sync(0xffffffffu, sl.vb && !(sb > kTinySum));
+        if (PARTS > 1) {
+            if (lane == 0) X.low[warp] = low_a | low_b;
+            slice_barrier(warp);
+        }
         if (low_a | low_b) {
             float xa, xb;
-            exact_lse<ROWS>(a, M.stage, sl, dust, xa, xb);
+            if (PARTS == 1) {
+                exact_lse<ROWS>(a, M.stage, sl, dust, xa, xb);
+            } else {
+                float4 x = exact_part<ROWS, PARTS>(a, M.stage, sl, dust, 0);
+                slice_barrier(warp);
+                for (int p = 0; p < PARTS - 1; ++p) {
+                    const float4 y = X.lse[p][own];
+                    lse_merge_into(x.x, x.y, y.x, y.y);
+                    lse_merge_into(x.z, x.w, y.z, y.w);
+                }
+                xa = x.x + lg2(x.y);
+                xb = x.z + lg2(x.w);
+            }
             if ((low_a >> lane) & 1u) va = -xa;
             if ((low_b >> lane) & 1u) vv = -xb;
             if (lane == 0)
@@ -1085,14 +1171,16 @@ cudaError_t with_tiles(const SkLaunch& l, Fn fn) {
 template <int A, int B>
 cudaError_t allow_smem() {
     constexpr int thr = pass_threads(A, B);
-    const int n = (int)std::max(sizeof(PassShared<A, thr>), sizeof(PassShared<B, thr>));
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(sk_pass_kernel<A, B, true>, at, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_pass_kernel<A, B, false>, at, n);
+    const int n1 = (int)pass_smem_bytes<A, B>(), n4 = n1 + (int)sizeof(ExactShared<thr>);
+    cudaError_t e = cudaFuncSetAttribute(sk_pass_kernel<A, B, true, 1>, at, n1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_pass_kernel<A, B, false, 1>, at, n1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_pass_kernel<A, B, true, kExactParts>, at, n4);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_pass_kernel<A, B, false, kExactParts>, at, n4);
     if (A != B || e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(sk_harvest_row_kernel<A>, at, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_harvest_col_kernel<A>, at, n);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_finish_pass_kernel<A>, at, n);
+    e = cudaFuncSetAttribute(sk_harvest_row_kernel<A>, at, n1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_harvest_col_kernel<A>, at, n1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sk_finish_pass_kernel<A>, at, n1);
     return e;
 }
 
@@ -1119,13 +1207,15 @@ int slice_ctas(int T, int n_spots, int tile, int threads) {
 }
 
 template <int TILE, int OTHER, bool ROWS>
-cudaError_t run_pass(const SkArgs& a, int it, cudaStream_t s) {
+cudaError_t run_pass(const SkArgs& a, int it, bool split, cudaStream_t s) {
     constexpr int thr = pass_threads(TILE, OTHER);
-    constexpr size_t own = sizeof(PassShared<TILE, thr>), other = sizeof(PassShared<OTHER, thr>);
-    constexpr size_t smem = own > other ? own : other;
+    constexpr size_t smem = pass_smem_bytes<TILE, OTHER>();
     const int fin = finish_blocks(a.mode, a.T, thr);
-    return launch_pass(sk_pass_kernel<TILE, OTHER, ROWS>, fin + slice_ctas(a.T, ROWS ? a.n_obs : a.n_model, TILE, thr), thr,
-                       smem, true, s, a, it, fin);
+    const int ctas = fin + slice_ctas(a.T, ROWS ? a.n_obs : a.n_model, TILE, thr);
+    if (split)
+        return launch_pass(sk_pass_kernel<TILE, OTHER, ROWS, kExactParts>, ctas, kExactParts * thr,
+                           smem + sizeof(ExactShared<thr>), true, s, a, it, fin);
+    return launch_pass(sk_pass_kernel<TILE, OTHER, ROWS, 1>, ctas, thr, smem, true, s, a, it, fin);
 }
 
 }  // namespace
@@ -1142,13 +1232,13 @@ cudaError_t sinkhorn_setup() {
 
 cudaError_t sinkhorn_row_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s) {
     return with_tiles(l, [&](auto row, auto col) {
-        return run_pass<decltype(row)::value, decltype(col)::value, true>(a, it, s);
+        return run_pass<decltype(row)::value, decltype(col)::value, true>(a, it, l.row_split, s);
     });
 }
 
 cudaError_t sinkhorn_col_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s) {
     return with_tiles(l, [&](auto row, auto col) {
-        return run_pass<decltype(col)::value, decltype(row)::value, false>(a, it, s);
+        return run_pass<decltype(col)::value, decltype(row)::value, false>(a, it, l.col_split, s);
     });
 }
 

@@ -105,6 +105,41 @@ def test_lists_sweeps_and_every_pair_agree(env, geom, eps, mode, sizes):
     del keep
 
 
+@pytest.mark.parametrize("eps,sizes", [(2.0, EDGES), (8.0, EDGES), (2.0, [(9, 31), (33, 7), (8, 8), (260, 257)])])
+def test_split_exact_sums_agree(env, eps, sizes):
+    """The unbalanced update, few slices (several warps share a slice's exact
+    sums) against the same blocks many times over (one warp each); blocks are
+    independent without dustbins.  A sum merged from four parts has at most
+    twelve roundings of 2^-22 more, so a potential at most 6e-6 (base 2) more
+    error per update, and the rounding of an exponent at most 4 ulp of the
+    largest potential; an iteration contracts by tau_row tau_col."""
+    api, torch, dev = env["api"], env["torch"], env["dev"]
+    p, I_off, m, J_off = _blocks(sizes, 23, GEOM)
+    kappa, lam, copies = 30.0, 20.0, 120
+
+    def solve(k):
+        h = api.Handle(dev)
+        off = lambda o: np.concatenate([[0]] + [o[1:] + c * o[-1] for c in range(k)])
+        tile = lambda v: np.concatenate([v] * k)
+        ob = api.ObsSpots.from_numpy(tile(p), off(I_off), device=dev)
+        ms = api.ModelSpots.from_numpy(off(J_off), *(tile(m[n]) for n in ("grain", "plane", "ray", "center", "spot", "det")),
+                                       device=dev)
+        out = api.cost_sinkhorn(h, GEOM, ob, ms, eps, 2.25, 25, dust_mode=2, harvest=False, kappa=kappa, lam=lam)
+        torch.cuda.synchronize()
+        c = h.counters()
+        return [out[n].double().cpu().numpy() for n in ("f", "g")], c
+
+    one, c_one = solve(1)
+    many, c_many = solve(copies)
+    assert c_one["exact_rows"] > 0 and c_one["exact_cols"] > 0
+    top = max(np.abs(v).max() for v in one) / (eps * np.log(2.0))
+    assert top < 1e6
+    tau = kappa / (kappa + eps) * lam / (lam + eps)
+    tol = 2 * (6e-6 + 4 * 2.0 ** -23 * top) / (1.0 - tau) * eps * np.log(2.0)
+    for a, b in zip(one, many):
+        assert np.abs(np.tile(a, copies) - b).max() <= tol
+
+
 @pytest.mark.parametrize("rho", [1, 8, 64])
 @pytest.mark.parametrize("sizes", [EDGES, [(5000, 40), (3, 900), (64, 64)]], ids=["edges", "uneven"])
 def test_sparse_neighbour_searches_agree(env, rho, sizes):
