@@ -528,12 +528,7 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
         a.mod_subext = (float*)take(sizeof(float) * kSubs * L.max_mod_gran);
         a.Gc = (float*)take(sizeof(float) * 2 * L.max_mod_pairs);
         a.Fc = (float*)take(sizeof(float) * 2 * L.max_obs_pairs);
-        a.row_order = (int*)take(sizeof(int) * rs);
-        a.col_order = (int*)take(sizeof(int) * cs);
         a.pmax = (unsigned*)take(sizeof(unsigned) * 4 * a.T);
-        // a pass that holds all its slices at once needs no order
-        if (rs <= (size_t)kSlicesPerSm * h->sm_count && cs <= (size_t)kSlicesPerSm * h->sm_count)
-            a.row_order = a.col_order = nullptr;
     }
     a.row_tiles = (int4*)(ws + L.row_tiles);
     a.col_tiles = (int4*)(ws + L.col_tiles);

@@ -145,7 +145,7 @@ inline Layout make_layout(const LaueProblemDims& d, int sm_count) {
     {
         size_t sort_bytes = sizeof(int) * 4 * nsp;
         size_t slices = list_slices(T, d.n_obs, kMaxTile) + list_slices(T, d.n_model, kMaxTile);
-        size_t reuse = slices * (kSliceDescBytes + sizeof(int)) + sizeof(float) * 2 * (ip + jp) +
+        size_t reuse = slices * kSliceDescBytes + sizeof(float) * 2 * (ip + jp) +
                        sizeof(unsigned) * 4 * T + 128 +
                        (sizeof(float4) + sizeof(float)) * kSubs * (size_t)(L.max_obs_gran + L.max_mod_gran);
         L.sortbuf = take(sort_bytes > reuse ? sort_bytes : reuse);

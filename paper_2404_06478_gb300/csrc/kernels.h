@@ -95,10 +95,7 @@ struct SkArgs {
     // potentials of the passes by ordered slot: pair offset of the block x 2 + rank
     float *Fc, *Gc;
     unsigned* pmax;        // 4T: maxima per angle of the last passes (passes.cu)
-    // slices of the passes (passes.cu): descriptors; tiles by descending weight
-    // (null: in their own order)
-    void *row_desc, *col_desc;
-    int *row_order, *col_order;
+    void *row_desc, *col_desc;  // descriptors of the slices of the passes (passes.cu)
     // pair lists (pool_chunks = 0: none): chunk numbers of each slice, the pool
     int *row_tab, *col_tab;
     char* pool;
@@ -193,7 +190,6 @@ cudaError_t sparse_sinkhorn_run(const SpArgs& a, const SkArgs* order, int n_iter
                                 cudaStream_t s);
 
 constexpr int kSkVariants = 4;       // launch shapes of the pair passes (see sinkhorn.cu)
-constexpr int kSlicesPerSm = 20;      // slices of a pass that an SM holds at once
 // Unbalanced passes of at most this many slices per SM are split (four warps a
 // slice): an SM holds 8 such slices at once, so warps that find nothing to do
 // cost nothing.  Measured (50 iterations, 60 angles, split against not): 7
