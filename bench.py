@@ -4,7 +4,7 @@ Workload: 1000 grains, |hkl| <= 6 bcc (a = 2.87 A), 90 rotations over 360 deg,
 0.5 mm spot noise, 70% outliers with uneven per-angle Poisson counts, eps =
 1 mm^2, 200 Sinkhorn iterations per EM step (synthetic, seeded).  One step =
 one EM iteration: refresh of the frozen model list at the current poses, the
-fused cost + Sinkhorn E-step (all angle blocks in each persistent launch), the
+fused cost + Sinkhorn E-step (all angle blocks in each launch), the
 plan read-out, and the M-step (Newton on positions, MM on orientations).
 
 Metric: cost-pair evaluations per second in Sinkhorn (2 * sum_t |I_t| |J_t| per
@@ -32,7 +32,10 @@ UNIT = "pairs/s"
 # DRAM bytes of one row-pass launch on the 1000-grain workload, counted by ncu
 # (dram__bytes_read.sum + dram__bytes_write.sum) for the current kernels; None
 # after a kernel change until it is captured again
-SK_PASS_DRAM_BYTES = 42244608
+SK_PASS_DRAM_BYTES = 351607296
+# bytes of a listed pair as the passes stream it: squared ray distance (float)
+# and slot of the other side's spot (16 bits)
+SK_ENTRY_BYTES = 6
 
 
 def max_over_ranks(value, world, device):
@@ -753,23 +756,18 @@ def main():
                   note="paper Section 'Working with sparse assignment matrices'; agreement over rows whose dense "
                        "top-two margin exceeds 1e-3")
 
-    # refresh 1; Sinkhorn: schedule, pack, dust init, G maxima, 2 per iteration, clear, harvest,
-    # finish; M-step: schedule, pack, dust init, G maxima, segment count + scan, init, 2 per Newton step,
-    # MM pair + MM grain, norms
-    launches_per_step = 1 + (4 + 2 * cfg.n_sinkhorn + 3) + (4 + 2 + 1 + 2 * 4 + 2 + 1)
-    # roofline: the algorithmic pair evaluation is 13 FP32 lane-ops (3 sub,
-    # 3 for |d|^2, 3 for d.r, 1 for the cosine, 1 fold with the potential, 1
-    # running-maximum update, 1 accumulate), 1 MUFU rsqrt and 1 MUFU ex2; the
-    # peak is the slowest of the three pipes, each measured on this device by
-    # laue_alu_peaks.  The kernel itself spends 14 (it forms |rhat - r|^2 from
-    # the difference vector, which keeps the small costs of matched pairs free
-    # of cancellation, and needs no running maximum): frac_kernel_ops.
+    # refresh 1; Sinkhorn: schedule, sort, pack, cones, two lists, 2 per iteration,
+    # dustbins of the last pass, clear, harvest, finish; M-step: pack, G maxima, plan list, segment
+    # count + scan, init, 2 per Newton step, MM pair + MM grain, norms
+    launches_per_step = 1 + (6 + 2 * cfg.n_sinkhorn + 4) + (2 + 1 + 2 + 1 + 2 * 4 + 2 + 1)
+    # roofline: a pass streams its side's list of the pairs whose plan entries
+    # can differ from 0 (a squared ray distance and a 16-bit slot each), reads
+    # the other side's potentials and its own side's cost factors, and writes
+    # its own potentials; at this size hardly any slice is swept instead
+    achieved = SK_ENTRY_BYTES * evaluated_per_launch + 6.0 * (W["nI"] + W["nJ"])
+    achieved *= 1e-9 / (per_launch_ms / 1e3)
+    peak = hbm_peak
     pk_ = W["h"].alu_peaks()
-    fp32 = max(pk_["ffma"], pk_["ffma2"])
-    peak = min(fp32 / 13.0, pk_["ex2"], pk_["rsqrt"])
-    peak14 = min(fp32 / 14.0, pk_["ex2"], pk_["rsqrt"])
-    bound_by = min((fp32 / 13.0, "fp32"), (pk_["ex2"], "mufu_ex2"), (pk_["rsqrt"], "mufu_rsqrt"))[1]
-    achieved = evaluated_per_launch / (per_launch_ms / 1e3)
     line = dict(
         metric=METRIC, value=value, unit=UNIT, n_gpus=world, steps=args.steps, warmup=args.warmup,
         ms_per_step=ms, higher_is_better=True, scaling="weak", vs_baseline=None, dtype="f32",
@@ -784,15 +782,15 @@ def main():
                     l2="256 MB buffer written between timed steps", parallelism="replicas" if world > 1 else "1 GPU",
                     autotuned_shapes={"row": tuned[0], "col": tuned[1],
                                       "ms_per_pass": [[round(r, 3), round(c, 3)] for r, c in tuned[2]]}),
-        roofline=dict(bound="alu", achieved=achieved, peak=peak, unit="pairs/s", frac=achieved / peak,
-                      frac_kernel_ops=achieved / peak14,
+        roofline=dict(bound="hbm", achieved=achieved, peak=peak, unit="GB/s", frac=(achieved / peak) if peak else None,
+                      ms_per_launch=per_launch_ms, entries_per_launch=evaluated_per_launch,
                       traffic=SK_PASS_DRAM_BYTES if (cfg.n_grains == 1000 and SK_PASS_DRAM_BYTES) else None,
                       traffic_unit="bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum of one row-pass "
-                                   "launch, ncu capture of this workload; profiles/sk_row_kernel_dram_1000grains_"
+                                   "launch, ncu capture of this workload; profiles/sk_pass_kernel_dram_1000grains_"
                                    "90angles.md)",
-                      kernel="sk_row_kernel+sk_col_kernel (per launch; evaluated pairs after the exact skipping)",
-                      peak_basis="min(FP32 lane-ops/s / 13, MUFU ex2/s, MUFU rsqrt/s), measured by "
-                                 "laue_alu_peaks; binding pipe: %s" % bound_by,
+                      kernel="sk_pass_kernel (per launch, mean of row and column passes)",
+                      peak_basis="copy bandwidth measured on this device type; algorithmic bytes: %d per listed entry "
+                                 "plus the potentials and cost factors" % SK_ENTRY_BYTES,
                       pipes={k: v for k, v in pk_.items()}),
         clocks=clk,
         e2e=dict(value=pairs_step / (e2e_ms / 1e3), unit=UNIT, h2d_bytes_per_step=int(h2d),
@@ -802,8 +800,9 @@ def main():
         pairs=dict(dense_equivalent_per_s=value, evaluated_per_s=value * evaluated_per_launch / W["pairs_half"],
                    evaluated_fraction=evaluated_per_launch / W["pairs_half"],
                    note="value counts 2 sum_t |I_t||J_t| pair evaluations per Sinkhorn iteration (the dense "
-                        "plan); the passes skip (tile, chunk) combinations whose plan entries all underflow to "
-                        "exactly 0 in FP32 (potentials bit-identical), and evaluate the fraction shown"),
+                        "plan); the passes leave out pairs whose plan entries underflow to exactly 0 in FP32 "
+                        "(potentials bit-identical), list the others once per E-step and evaluate the "
+                        "fraction shown (list padding included)"),
         adjoint=adjoint,
         sparse_estep=sparse,
     )
