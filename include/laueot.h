@@ -444,7 +444,7 @@ int laue_mstep(laue_handle* h, const LaueGeometry* geom, const LaueLattice* lat,
  * the plan Q held at the E-step (potentials f, g and the model list's rays and
  * centres, which must be those of the E-step), over theta = (phi, x) with
  * R <- exp([phi]x) R.  Each step runs the adjoint pair pass at the current
- * pose (the gradient of laue_objective_grad, costs recomputed, never stored)
+ * pose (the gradient of laue_objective_grad, no cost matrix stored)
  * together with the sums q_j = sum_i Q_ij, s1_j = sum_i Q_ij / tau_ij and
  * s2_j = sum_i Q_ij / tau_ij^2; the Gauss-Newton matrix takes each spot's
  * model-ray projector P_j = I - r_j r_j^T:

@@ -11,7 +11,8 @@
 //   column G_j = -LSE2({F_i - K e2_ij}_{i in I_t} u {F_0})
 //   dust   G_0 = log2 O - LSE2({F_i - kc}_i u {F_0 - kc})
 // with e2_ij = |rhat_ij - r_j|^2 and kc = c_out log2(e)/eps.  The cost matrix
-// is never stored: every pass recomputes e2 from the spot coordinates.
+// is never stored: the passes keep e2 of the pairs whose plan entry can be
+// nonzero for one E-step, and recompute it from the spot coordinates elsewhere.
 //
 // Unbalanced mode (Appendix "Optimal transport variants", Algorithm
 // UnbalancedOT): no dustbins, and each balanced update is scaled by

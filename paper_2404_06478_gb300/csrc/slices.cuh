@@ -148,7 +148,7 @@ struct __align__(32) SliceDesc {
     int t, q, nspot;  // angle, first pair of its own, its spots (0: no slice)
     int nch;          // chunks of its lists, -1: swept
     int s0, ns;       // first pair and pairs of the streamed block
-    int pad;
+    int pad;          // 0
     float cut;        // cost bound beyond which the M-step's sweep skips
 };
 static_assert(sizeof(SliceDesc) == kSliceDescBytes, "laid out by the host");
