@@ -757,9 +757,9 @@ def main():
                        "top-two margin exceeds 1e-3")
 
     # refresh 1; Sinkhorn: schedule, sort, pack, cones, two lists, 2 per iteration,
-    # dustbins of the last pass, clear, harvest, finish; M-step: pack, G maxima, plan list, segment
-    # count + scan, init, 2 per Newton step, MM pair + MM grain, norms
-    launches_per_step = 1 + (6 + 2 * cfg.n_sinkhorn + 4) + (2 + 1 + 2 + 1 + 2 * 4 + 2 + 1)
+    # dustbins of the last pass, clear, harvest, finish; M-step: pack, G maxima, plan list,
+    # segment table, 2 per Newton step, MM pair + MM grain, norms
+    launches_per_step = 1 + (6 + 2 * cfg.n_sinkhorn + 4) + (2 + 1 + 1 + 2 * 4 + 2 + 1)
     # roofline: a pass streams its side's list of the pairs whose plan entries
     # can differ from 0 (a squared ray distance and a 16-bit slot each), reads
     # the other side's potentials and its own side's cost factors, and writes

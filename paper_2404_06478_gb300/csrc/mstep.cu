@@ -28,18 +28,27 @@ namespace laue {
 // ------------------------------------------------------- segment table
 // seg[t (N+1) + n] = first model spot of grain n at angle t (the list is sorted
 // by (t, n, m)); seg[t (N+1) + N] = J_off[t+1].
-__global__ void ms_seg_count_kernel(MsArgs m) {
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= m.n_model) return;
-    atomicAdd(&m.seg[m.angle[j] * (m.N + 1) + m.grain[j]], 1);
-}
-
-__global__ void ms_seg_scan_kernel(MsArgs m) {  // one warp per angle
-    const int t = blockIdx.x, lane = threadIdx.x;
+// One CTA per angle counts its spots by grain and takes the prefix; the grains'
+// states are set beside it.  (A clear, a count, a scan and the states were four
+// launches, which a small problem's call waits for.)
+constexpr int kSegThreads = 512;
+__global__ void __launch_bounds__(kSegThreads) ms_start_kernel(MsArgs m) {
+    const int t = blockIdx.x, lane = threadIdx.x & 31;
+    for (int n = t * kSegThreads + threadIdx.x; n < m.N; n += gridDim.x * kSegThreads) {
+        m.gstate[4 * n + 0] = 1.0f;  // Newton still active
+        m.gstate[4 * n + 1] = 0.0f;  // last |dx|
+        m.gstate[4 * n + 2] = 0.0f;  // last |dR|_F
+    }
     int* s = m.seg + t * (m.N + 1);
-    int acc = m.J_off[t];
+    const int j0 = m.J_off[t], j1 = m.J_off[t + 1];
+    for (int n = threadIdx.x; n <= m.N; n += kSegThreads) s[n] = 0;
+    __syncthreads();
+    for (int j = j0 + threadIdx.x; j < j1; j += kSegThreads) atomicAdd(&s[m.grain[j]], 1);
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    int acc = j0;
     for (int n0 = 0; n0 < m.N; n0 += 32) {
-        const int c = n0 + lane < m.N ? s[n0 + lane] : 0;
+        const int c = n0 + lane < m.N ? __ldcg(s + n0 + lane) : 0;
         int incl = c;
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, incl, o);
@@ -49,14 +58,6 @@ __global__ void ms_seg_scan_kernel(MsArgs m) {  // one warp per angle
         acc += __shfl_sync(0xffffffffu, incl, 31);
     }
     if (lane == 0) s[m.N] = acc;
-}
-
-__global__ void ms_init_kernel(MsArgs m) {
-    int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= m.N) return;
-    m.gstate[4 * n + 0] = 1.0f;  // Newton still active
-    m.gstate[4 * n + 1] = 0.0f;  // last |dx|
-    m.gstate[4 * n + 2] = 0.0f;  // last |dR|_F
 }
 
 // ------------------------------------------------------------ pair pass
@@ -529,20 +530,13 @@ __global__ void ms_adj_grain_kernel(MsArgs m) {
     m.gstate[4 * n + 2] = th;
 }
 
-static cudaError_t seg_table(const MsArgs& m, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(m.seg, 0, sizeof(int) * (size_t)m.T * (m.N + 1), s);
-    if (e != cudaSuccess) return e;
-    if (m.n_model > 0) ms_seg_count_kernel<<<(m.n_model + 255) / 256, 256, 0, s>>>(m);
-    ms_seg_scan_kernel<<<m.T, 32, 0, s>>>(m);
-    return cudaGetLastError();
-}
-
-// The E-step's plan (schedule, pair copies with F and G, its entries) and the segment table.
+// The E-step's plan (schedule, pair copies with F and G, its entries), the segment table and the grains' states.
 static cudaError_t prepare(const MsArgs& m, const SkLaunch& l, bool sorted, cudaStream_t s) {
     cudaError_t e = sinkhorn_prepare(m.sk, s, false, sorted);
     if (e == cudaSuccess) e = sinkhorn_list_plan(m.sk, l, s);
-    if (e == cudaSuccess) e = seg_table(m, s);
-    return e;
+    if (e != cudaSuccess) return e;
+    ms_start_kernel<<<m.T, kSegThreads, 0, s>>>(m);
+    return cudaGetLastError();
 }
 
 template <int MODE>
@@ -558,7 +552,6 @@ static void pair_pass(const MsArgs& m, const SkLaunch& l, cudaStream_t s) {
 cudaError_t grad_run(const MsArgs& m, const SkLaunch& l, cudaStream_t s) {
     cudaError_t e = prepare(m, l, false, s);
     if (e != cudaSuccess) return e;
-    if (m.N > 0) ms_init_kernel<<<(m.N + 255) / 256, 256, 0, s>>>(m);
     pair_pass<2>(m, l, s);
     if (m.N > 0) ms_grad_grain_kernel<<<(m.N * 32 + 127) / 128, 128, 0, s>>>(m);
     return cudaGetLastError();
@@ -647,7 +640,6 @@ cudaError_t axis_angle_vjp_run(const float* w, const float* grad, const float* g
 cudaError_t mstep_adjoint_run(const MsArgs& m, const SkLaunch& l, int n_steps, bool sorted, cudaStream_t s) {
     cudaError_t e = prepare(m, l, sorted, s);
     if (e != cudaSuccess) return e;
-    if (m.N > 0) ms_init_kernel<<<(m.N + 255) / 256, 256, 0, s>>>(m);
     for (int k = 0; k < n_steps; ++k) {
         pair_pass<3>(m, l, s);
         if (m.N > 0) ms_adj_grain_kernel<<<(m.N * 32 + 127) / 128, 128, 0, s>>>(m);
@@ -664,7 +656,6 @@ cudaError_t axis_angle_run(const float* w, const float* R0, float* R, float* JlT
 cudaError_t mstep_run(const MsArgs& m, const SkLaunch& l, bool sorted, cudaStream_t s) {
     cudaError_t e = prepare(m, l, sorted, s);
     if (e != cudaSuccess) return e;
-    if (m.N > 0) ms_init_kernel<<<(m.N + 255) / 256, 256, 0, s>>>(m);
     for (int k = 0; k < m.n_newton; ++k) {
         pair_pass<0>(m, l, s);
         if (m.N > 0) ms_newton_grain_kernel<<<(m.N * 32 + 127) / 128, 128, 0, s>>>(m);
