@@ -680,8 +680,17 @@ __device__ __forceinline__ void pass_release() { asm volatile("griddepcontrol.la
 // PARTS warps to a slice that read a part of the block each; part 0's warp
 // merges.  23 grains x 17 angles at 4 mm^2: 23 us a pass with one warp, 14 us
 // with four.
+//
+// Registers: 128 a thread, 512 threads to an SM.  No more are resident anyway:
+// a named barrier whose id is not a constant takes all 16 of a CTA, four CTAs to
+// an SM.  With 64 registers the sums over swept pairs spilled: 90 angles of
+// 13300 x 7744 spots at 100 mm^2 without lists 5.8 ms an iteration, now 4.8; one
+// block of 200000 x 8000 spots 11.1 ms, now 7.0.  (The split passes keep 64:
+// four times the warps.)
+constexpr int kPassThreadsPerSm = 512;
 template <int TILE, int OTHER, bool ROWS, int PARTS>
-__global__ void __launch_bounds__(PARTS* pass_threads(TILE, OTHER), 1024 / pass_threads(TILE, OTHER) / PARTS)
+__global__ void __launch_bounds__(PARTS* pass_threads(TILE, OTHER),
+                                  (PARTS > 1 ? 1024 : kPassThreadsPerSm) / pass_threads(TILE, OTHER) / PARTS)
     sk_pass_kernel(SkArgs a, int it, int finishers) {
     extern __shared__ __align__(128) char pass_smem[];
     constexpr int kThreads = pass_threads(TILE, OTHER);
@@ -909,8 +918,8 @@ __device__ __noinline__ Lse2 whole_col(const SkArgs& a, int t, int q, int odd) {
 __device__ __forceinline__ bool is_entry(float e2) { return !(e2 > 2.0e38f); }
 
 template <int TILE>
-__global__ void __launch_bounds__(pass_threads(TILE), 1024 / pass_threads(TILE)) sk_harvest_row_kernel(SkArgs a,
-                                                                                                     int n_iter) {
+__global__ void __launch_bounds__(pass_threads(TILE), kPassThreadsPerSm / pass_threads(TILE))
+    sk_harvest_row_kernel(SkArgs a, int n_iter) {
     extern __shared__ __align__(128) char pass_smem[];
     PassShared<TILE>& H = *(PassShared<TILE>*)pass_smem;
     DustPtrs D = dust_ptrs(a.dust, a.T);
@@ -1021,8 +1030,8 @@ __global__ void __launch_bounds__(pass_threads(TILE), 1024 / pass_threads(TILE))
 // error with the final potentials, in base 2 with a running maximum.  Pairs
 // are left out, and columns read again, as for the rows.
 template <int TILE>
-__global__ void __launch_bounds__(pass_threads(TILE), 1024 / pass_threads(TILE)) sk_harvest_col_kernel(SkArgs a,
-                                                                                                     int n_iter) {
+__global__ void __launch_bounds__(pass_threads(TILE), kPassThreadsPerSm / pass_threads(TILE))
+    sk_harvest_col_kernel(SkArgs a, int n_iter) {
     extern __shared__ __align__(128) char pass_smem[];
     PassShared<TILE>& H = *(PassShared<TILE>*)pass_smem;
     DustPtrs D = dust_ptrs(a.dust, a.T);
