@@ -543,17 +543,20 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
     a.negKD2 = (float)(-(double)geom->D * geom->D * 1.4426950408889634 / eps);
     {
         GeomDev G = laue_geom_dev(*geom);
-        double dmin = geom->D;
+        double dmin = geom->D, dmax = geom->D;
         a.n_det = G.n_det;
         for (int k = 0; k < 4; ++k) {
             double Dk = k < G.n_det ? (double)G.Dd[k] : (double)geom->D;
             a.negK_det[k] = (float)(-Dk * Dk * 1.4426950408889634 / eps);
             if (k < G.n_det && Dk < dmin) dmin = Dk;
+            if (k < G.n_det && Dk > dmax) dmax = Dk;
         }
         a.skipK = (float)(dmin * dmin * 1.4426950408889634 / eps);
+        a.listK = (float)(dmax * dmax * 1.4426950408889634 / eps);
         a.uniK = 1;
         for (int k = 0; k < G.n_det; ++k) a.uniK &= a.negK_det[k] == a.negKD2;
     }
+    a.list_share = 1.0f;
     a.kc = (float)((double)prm->c_out * 1.4426950408889634 / eps);
     a.frac = prm->unmatched_frac;
     a.to_user = (float)(eps * 0.6931471805599453);

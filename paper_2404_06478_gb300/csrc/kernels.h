@@ -100,6 +100,8 @@ struct SkArgs {
     int *row_tab, *col_tab;
     char* pool;
     int pool_chunks;
+    float list_share;      // entries a spot may have per swept pair of its slice for listing to pay (passes.cu)
+    float listK;           // largest K of any cost length (skipK: the smallest)
     int uniK;              // every detector has the same cost length: K_j = -negKD2
     int4* row_tiles;
     int4* col_tiles;
@@ -218,6 +220,8 @@ cudaError_t sinkhorn_harvest(const SkArgs& a, const SkLaunch& l, int n_iter, boo
 cudaError_t sinkhorn_setup();  // once per device, the current one
 cudaError_t sinkhorn_build_lists(const SkArgs& a, const SkLaunch& l, cudaStream_t s);
 int sk_variant_threads(int v);
+float list_share_of(int n_iter);
+float plan_share_of(const SkArgs& a, int n_pass);
 cudaError_t sinkhorn_row_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s);
 cudaError_t sinkhorn_col_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s);
 

@@ -530,10 +530,14 @@ __global__ void ms_adj_grain_kernel(MsArgs m) {
     m.gstate[4 * n + 2] = th;
 }
 
-// The E-step's plan (schedule, pair copies with F and G, its entries), the segment table and the grains' states.
-static cudaError_t prepare(const MsArgs& m, const SkLaunch& l, bool sorted, cudaStream_t s) {
-    cudaError_t e = sinkhorn_prepare(m.sk, s, false, sorted);
-    if (e == cudaSuccess) e = sinkhorn_list_plan(m.sk, l, s);
+// The E-step's plan (schedule, pair copies with F and G, its entries for `passes` passes), the segment table and the
+// grains' states.
+static cudaError_t prepare(const MsArgs& m, const SkLaunch& l, int passes, bool sorted, cudaStream_t s) {
+    SkArgs a = m.sk;
+    a.list_share = plan_share_of(a, passes);
+    if (a.list_share == 0.0f) a.pool_chunks = 0;
+    cudaError_t e = sinkhorn_prepare(a, s, false, sorted);
+    if (e == cudaSuccess) e = sinkhorn_list_plan(a, l, s);
     if (e != cudaSuccess) return e;
     ms_start_kernel<<<m.T, kSegThreads, 0, s>>>(m);
     return cudaGetLastError();
@@ -550,7 +554,7 @@ static void pair_pass(const MsArgs& m, const SkLaunch& l, cudaStream_t s) {
 }
 
 cudaError_t grad_run(const MsArgs& m, const SkLaunch& l, cudaStream_t s) {
-    cudaError_t e = prepare(m, l, false, s);
+    cudaError_t e = prepare(m, l, 1, false, s);
     if (e != cudaSuccess) return e;
     pair_pass<2>(m, l, s);
     if (m.N > 0) ms_grad_grain_kernel<<<(m.N * 32 + 127) / 128, 128, 0, s>>>(m);
@@ -638,7 +642,7 @@ cudaError_t axis_angle_vjp_run(const float* w, const float* grad, const float* g
 }
 
 cudaError_t mstep_adjoint_run(const MsArgs& m, const SkLaunch& l, int n_steps, bool sorted, cudaStream_t s) {
-    cudaError_t e = prepare(m, l, sorted, s);
+    cudaError_t e = prepare(m, l, n_steps, sorted, s);
     if (e != cudaSuccess) return e;
     for (int k = 0; k < n_steps; ++k) {
         pair_pass<3>(m, l, s);
@@ -654,7 +658,7 @@ cudaError_t axis_angle_run(const float* w, const float* R0, float* R, float* JlT
 }
 
 cudaError_t mstep_run(const MsArgs& m, const SkLaunch& l, bool sorted, cudaStream_t s) {
-    cudaError_t e = prepare(m, l, sorted, s);
+    cudaError_t e = prepare(m, l, m.n_newton + (m.n_mm > 0 ? 1 : 0), sorted, s);
     if (e != cudaSuccess) return e;
     for (int k = 0; k < m.n_newton; ++k) {
         pair_pass<0>(m, l, s);

@@ -48,6 +48,18 @@ constexpr float kFarLog2 = 60.0f;     // see the read-out kernels
 // the pairs it evaluates would be listed: a listed entry costs about as much
 // as two swept pairs.
 //
+// A list that is given up halfway is lost time (up to fifteen swept passes of
+// the slice), so a slice first estimates its entries: how many of the streamed
+// spots' sub-granules lie, by their axes, within the listed angle of its own
+// spots.  It is left to the sweep if they exceed a list, or list_share of its
+// evaluated pairs.  Measured as the cost of listing in swept iterations, 1.4 at
+// an entry per 30 pairs, 3 at one in 6, 4 to 11 at one in 3: so the share
+// grows with the iterations that a list is used for.  90 angles of 13300 x 7744
+// spots, 20 iterations at 100 mm^2: 91.6 ms when every slice tried, 77.7 now (at
+// 21 mm^2, where the pool holds a part of the entries: 48.0 and 46); 60 angles
+// of 1020 x 776 spots, 2 and 5 iterations at 100 mm^2: 0.90 and 1.06 ms, now 0.52
+// and 0.78; at 1 mm^2 the same slices are listed.
+//
 // Most of the pairs that the cones let through are still too far apart, so a
 // cheap test comes first: the angle between p (seen from the origin) and r is
 // at most the angle of the cost bound plus the parallax asin(|c| / |p|), three
@@ -105,33 +117,47 @@ __global__ void __launch_bounds__(32 * kListWarps) sk_list_kernel(SkArgs a) {
         for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
         cut = cone_cut = dust_ptrs(a.dust, a.T).Fmax[t] + top - kQSkip + 1.0f;
     }
-    const int evaluated = count_pairs(own, ROWS, sub, subext, np, a.skip, a.skipK, cone_cut);
+    RowPair R{};
+    ColPair C;
+    if (ROWS) R = load_row_pair(a, q, valid);
+    else load_col_pair(a, valid ? q : first, C);
+    // unit directions of the lane's spots
+    float da[3], db[3];
+    if (ROWS) {
+        const float x[6] = {lo(R.pxa), lo(R.pya), lo(R.pza), lo(R.pxb), lo(R.pyb), lo(R.pzb)};
+        const float ra = rsqrtf(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]);
+        const float rb = rsqrtf(x[3] * x[3] + x[4] * x[4] + x[5] * x[5]);
+        for (int k = 0; k < 3; ++k) {
+            da[k] = x[k] * ra;
+            db[k] = x[3 + k] * rb;
+        }
+    } else {
+        da[0] = -lo(C.nrxa), da[1] = -lo(C.nrya), da[2] = -lo(C.nrza);
+        db[0] = -lo(C.nrxb), db[1] = -lo(C.nryb), db[2] = -lo(C.nrzb);
+    }
+    // the angle of a cost of `most` in units of 1 / K, K 4 sin^2(th / 2) = most
+    auto angle_of = [](float most, float K) {
+        const float h = fmaxf(most, 0.0f) / (4.0f * K);
+        return h < 1.0f ? 2.0f * asinf(sqrtf(h)) : 7.0f;
+    };
     bool fail = a.pool_chunks == 0 || n_str > 65536;
+    int evaluated;
+    if (fail) {
+        evaluated = count_pairs<false>(own, ROWS, sub, subext, np, n_str, a.skip, a.skipK, cone_cut, da, 2.0f).pairs;
+    } else {
+        // the entries that the lanes' first spots will have, on average: too many to list, or to be worth it?
+        const float far = angle_of(PLAN ? dust_ptrs(a.dust, a.T).Fmax[t] + G.x - kQSkip : cut, a.listK);
+        const SliceCount n = count_pairs<true>(own, ROWS, sub, subext, np, n_str, a.skip, a.skipK, cone_cut, da,
+                                               !valid ? 2.0f : far < 3.1f ? cosf(far) : -3.0f);
+        evaluated = n.pairs;
+        const float mean = (float)n.near / (float)n_own;
+        fail = mean > (float)(kListDepth * kListChunks) || mean > a.list_share * (float)evaluated;
+    }
     int ca = 0, cb = 0, nch = 0;
     if (!fail) {
-        RowPair R{};
-        ColPair C;
-        if (ROWS) R = load_row_pair(a, q, valid);
-        else load_col_pair(a, valid ? q : first, C);
-        // unit directions of the lane's spots, and the parallax of its pairs
-        float da[3], db[3];
-        if (ROWS) {
-            const float x[6] = {lo(R.pxa), lo(R.pya), lo(R.pza), lo(R.pxb), lo(R.pyb), lo(R.pzb)};
-            const float ra = rsqrtf(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]);
-            const float rb = rsqrtf(x[3] * x[3] + x[4] * x[4] + x[5] * x[5]);
-            for (int k = 0; k < 3; ++k) {
-                da[k] = x[k] * ra;
-                db[k] = x[3 + k] * rb;
-            }
-        } else {
-            da[0] = -lo(C.nrxa), da[1] = -lo(C.nrya), da[2] = -lo(C.nrza);
-            db[0] = -lo(C.nrxb), db[1] = -lo(C.nryb), db[2] = -lo(C.nrzb);
-        }
+        const float th = angle_of(cut, a.skipK);  // of the largest listed cost of any spot
         const f2 dax = dup(da[0]), day = dup(da[1]), daz = dup(da[2]);
         const f2 dbx = dup(db[0]), dby = dup(db[1]), dbz = dup(db[2]);
-        // the angle of the largest listed cost of any spot, K 4 sin^2(th / 2) = cut
-        const float h = fmaxf(cut, 0.0f) / (4.0f * a.skipK);
-        const float th = h < 1.0f ? 2.0f * asinf(sqrtf(h)) : 7.0f;
         auto put = [&](int& cnt, int ab, float e2, int slot) {
             char* p = a.pool + (size_t)L.tab[cnt / kListDepth] * kListChunkBytes;
             const int at = (cnt % kListDepth) * 64 + 2 * lane + ab;
@@ -1120,6 +1146,23 @@ __global__ void __launch_bounds__(pass_threads(TILE), kPassThreadsPerSm / pass_t
 // Launch shapes of the pair passes the autotuner chooses from: the pairs of a
 // tile.  (Shapes 1 and 2 are the same kernels.)
 int sk_variant_threads(int v) { return v == 0 ? 256 : (v == 3 ? 64 : 128); }
+
+// Largest entries per spot, as a share of the slice's swept pairs, that are
+// worth listing for n_iter iterations: where the cost of listing (see above) is
+// made up by passes over lists (0.03 to 0.5 of a swept one).
+float list_share_of(int n_iter) { return (n_iter - 1.0f) / (n_iter + 14.0f); }
+
+// The same for n_pass passes of an M-step.  A single pass is listed for, whole,
+// or swept, whole: listed slices beside swept ones only add up.  The line lies at
+// 20 entries of a spot (two detectors see about 2 sr; 2^-40 at the usual
+// potentials).  Gradients, listed against swept: 1 mm^2, 1020 observed spots an
+// angle (1 entry) 0.171 and 0.183 ms, 13300 (16) 1.84 and 1.96; 21 mm^2, 1020 (26)
+// 0.224 and 0.198, 3700 (95) 0.75 and 0.57; 100 mm^2, 13300: 19.2 and 3.8.
+float plan_share_of(const SkArgs& a, int n_pass) {
+    if (n_pass > 1) return n_pass / (n_pass + 4.0f);
+    const float th2 = (4.0f - kQSkip) / a.skipK;
+    return (float)a.n_obs / (float)a.T * 3.14159f * th2 / 2.0f > 20.0f ? 0.0f : 1.0f;
+}
 
 namespace {
 

@@ -48,14 +48,38 @@ struct SubWalk {
     }
 };
 
-// Pairs of the sub-granules a slice can see: those whose cost bound is at most limit.
-__device__ __forceinline__ int count_pairs(const Cone& own, bool own_obs, const float4* sub, const float* ext,
-                                           int n_pairs, int skip, float K, float limit) {
-    SubWalk w;
-    w.init(sub, ext, n_pairs);
-    int n = 0;
-    for (int s = w.next(own, own_obs, skip, K, limit); s >= 0; s = w.next(own, own_obs, skip, K, limit))
-        n += min(kSubGran, n_pairs - s * kSubGran);
+// What a slice has to do.  pairs: those of the sub-granules that it can see
+// (whose cost bound is at most limit).  near (if asked for): about how many
+// streamed spots lie within a lane's own angle of its direction d (least: the
+// angle's cosine), summed over the lanes, from the axes of the sub-granules.
+struct SliceCount {
+    int pairs, near;
+};
+template <bool NEAR>
+__device__ __forceinline__ SliceCount count_pairs(const Cone& own, bool own_obs, const float4* sub, const float* ext,
+                                                  int n_pairs, int n_spots, int skip, float K, float limit,
+                                                  const float (&d)[3], float least) {
+    SliceCount n{0, 0};
+    const int nsub = (n_pairs + kSubGran - 1) / kSubGran;
+    for (int s0 = 0; s0 < nsub; s0 += 32) {
+        const int s = s0 + (threadIdx.x & 31);
+        Cone c{0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        bool need = s < nsub;
+        if (need) {
+            c = load_cone(sub, ext, s);
+            if (skip) need = (own_obs ? min_scaled_cost(own, c, K) : min_scaled_cost(c, own, K)) <= limit;
+        }
+        if (need) n.pairs += min(kSubGran, n_pairs - s * kSubGran);
+        if (!NEAR) continue;
+        for (unsigned m = __ballot_sync(0xffffffffu, need); m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            const float dot = __shfl_sync(0xffffffffu, c.ax, l) * d[0] + __shfl_sync(0xffffffffu, c.ay, l) * d[1] +
+                              __shfl_sync(0xffffffffu, c.az, l) * d[2];
+            if (dot >= least) n.near += min(2 * kSubGran, n_spots - 2 * (s0 + l) * kSubGran);
+        }
+    }
+    n.pairs = __reduce_add_sync(0xffffffffu, n.pairs);
+    if (NEAR) n.near = __reduce_add_sync(0xffffffffu, n.near);
     return n;
 }
 
