@@ -28,25 +28,19 @@ namespace laue {
 // ------------------------------------------------------- segment table
 // seg[t (N+1) + n] = first model spot of grain n at angle t (the list is sorted
 // by (t, n, m)); seg[t (N+1) + N] = J_off[t+1].
-// One CTA per angle counts its spots by grain and takes the prefix; the grains'
-// states are set beside it.  (A clear, a count, a scan and the states were four
-// launches, which a small problem's call waits for.)
-constexpr int kSegThreads = 512;
-__global__ void __launch_bounds__(kSegThreads) ms_start_kernel(MsArgs m) {
-    const int t = blockIdx.x, lane = threadIdx.x & 31;
-    for (int n = t * kSegThreads + threadIdx.x; n < m.N; n += gridDim.x * kSegThreads) {
+__device__ __forceinline__ void grain_states(const MsArgs& m, int first, int stride) {
+    for (int n = first; n < m.N; n += stride) {
         m.gstate[4 * n + 0] = 1.0f;  // Newton still active
         m.gstate[4 * n + 1] = 0.0f;  // last |dx|
         m.gstate[4 * n + 2] = 0.0f;  // last |dR|_F
     }
+}
+
+// The counts of angle t by grain become first spots; by one warp.
+__device__ __forceinline__ void seg_prefix(const MsArgs& m, int t) {
+    const int lane = threadIdx.x & 31;
     int* s = m.seg + t * (m.N + 1);
-    const int j0 = m.J_off[t], j1 = m.J_off[t + 1];
-    for (int n = threadIdx.x; n <= m.N; n += kSegThreads) s[n] = 0;
-    __syncthreads();
-    for (int j = j0 + threadIdx.x; j < j1; j += kSegThreads) atomicAdd(&s[m.grain[j]], 1);
-    __syncthreads();
-    if (threadIdx.x >= 32) return;
-    int acc = j0;
+    int acc = m.J_off[t];
     for (int n0 = 0; n0 < m.N; n0 += 32) {
         const int c = n0 + lane < m.N ? __ldcg(s + n0 + lane) : 0;
         int incl = c;
@@ -59,6 +53,37 @@ __global__ void __launch_bounds__(kSegThreads) ms_start_kernel(MsArgs m) {
     }
     if (lane == 0) s[m.N] = acc;
 }
+
+// One CTA per angle counts its spots by grain and takes the prefix; the grains'
+// states are set beside it.  (A clear, a count, a scan and the states were four
+// launches, which a small problem's call waits for.)
+constexpr int kSegThreads = 512;
+__global__ void __launch_bounds__(kSegThreads) ms_start_kernel(MsArgs m) {
+    const int t = blockIdx.x;
+    grain_states(m, t * kSegThreads + threadIdx.x, gridDim.x * kSegThreads);
+    int* s = m.seg + t * (m.N + 1);
+    const int j0 = m.J_off[t], j1 = m.J_off[t + 1];
+    for (int n = threadIdx.x; n <= m.N; n += kSegThreads) s[n] = 0;
+    __syncthreads();
+    for (int j = j0 + threadIdx.x; j < j1; j += kSegThreads) atomicAdd(&s[m.grain[j]], 1);
+    __syncthreads();
+    if (threadIdx.x < 32) seg_prefix(m, t);
+}
+
+// The same where an angle has too many spots for one CTA (kSegSpots): the count
+// spreads over the spots, behind a clear of the table.
+__global__ void __launch_bounds__(256) ms_seg_count_kernel(MsArgs m) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    grain_states(m, j, gridDim.x * blockDim.x);
+    if (j < m.n_model) atomicAdd(&m.seg[block_of(m.J_off, m.T, j) * (m.N + 1) + m.grain[j]], 1);
+}
+__global__ void __launch_bounds__(32) ms_seg_prefix_kernel(MsArgs m) { seg_prefix(m, blockIdx.x); }
+
+// Mean spots of an angle above which the count leaves its CTA, which takes 0.7 us
+// per 512 of them.  Gradients of one angle, one CTA against the spread count: 100000
+// spots of 1000 grains 1.36 and 1.32 ms, 500000 of 5000 6.49 and 6.08; at 8000
+// spots the two more launches cost what the CTA does (about 10 us).
+constexpr int kSegSpots = 8192;
 
 // ------------------------------------------------------------ pair pass
 // mode 0: Newton sums (9 floats in the x frame), mode 1: v_j (3 floats, lab),
@@ -124,7 +149,9 @@ __device__ __forceinline__ void ms_pair(MsCol& C, int mode, float px, float py, 
 // them.  Bound by the gathers of the listed entries' positions.  At 300 grains
 // x 90 angles, 1 mm^2, a pass took 447 us when it evaluated every pair that
 // the cones let through; listing the plan takes 279 us once and a pass 27 us.
-constexpr int kMsThreads = 128;
+// Two slices to a CTA: swept slices are few and uneven where there are no lists
+// (a block of 80000 x 80000 spots: gradient 6.3 ms with four, 5.4 with two).
+constexpr int kMsThreads = 64;
 
 template <int TILE, int MODE>
 __global__ void __launch_bounds__(kMsThreads) ms_pair_kernel(MsArgs m) {
@@ -539,7 +566,14 @@ static cudaError_t prepare(const MsArgs& m, const SkLaunch& l, int passes, bool 
     cudaError_t e = sinkhorn_prepare(a, s, false, sorted);
     if (e == cudaSuccess) e = sinkhorn_list_plan(a, l, s);
     if (e != cudaSuccess) return e;
-    ms_start_kernel<<<m.T, kSegThreads, 0, s>>>(m);
+    if (m.n_model / m.T <= kSegSpots) {
+        ms_start_kernel<<<m.T, kSegThreads, 0, s>>>(m);
+    } else {
+        e = cudaMemsetAsync(m.seg, 0, sizeof(int) * (size_t)m.T * (m.N + 1), s);
+        if (e != cudaSuccess) return e;
+        ms_seg_count_kernel<<<(m.n_model + 255) / 256, 256, 0, s>>>(m);
+        ms_seg_prefix_kernel<<<m.T, 32, 0, s>>>(m);
+    }
     return cudaGetLastError();
 }
 
