@@ -151,8 +151,8 @@ struct SpArgs {
     // workspace
     int2* cent;            // n_model x rho: {observed index or -1, e2 (D_j / D)^2 bits}, by increasing e2
     int2* rent;            // CSR rows: {model index, e2 bits}, ascending model index
-    int* rptr;             // n_obs + 1 row starts
-    int* rfill;            // n_obs fill counters
+    long long* rptr;       // n_obs + 1 row starts (n_model x rho may pass 2^31)
+    int* rfill;            // n_obs counters: entries of each row, then those filled
     float* F;              // n_obs
     float* G;              // n_model
     float* dust;           // F0, F0n, G0, log2U, log2O (nd each), errors (4)

@@ -267,60 +267,62 @@ __global__ void sp_count_kernel(SpArgs a) {
     size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (size_t)a.n_model * a.rho) return;
     int i = a.cent[e].x;
-    if (i >= 0) atomicAdd(&a.rptr[i + 1], 1);
+    if (i >= 0) atomicAdd(&a.rfill[i], 1);
 }
 
-// Inclusive prefix sum of rptr[1..n_obs] (rptr[0] = 0): sums of blocks of
-// kScan rows, then each block adds the sums before it.  The sums sit in the
-// fill counters, which are cleared after.
+// Row starts from the entries of each row: sums of blocks of kScan rows, then
+// each block adds the sums before it.  The sums sit where the tile partials of
+// the row passes will.
 constexpr int kScan = 8192;
 __global__ void __launch_bounds__(1024) sp_scan_sums_kernel(SpArgs a) {
-    __shared__ int warp_sum[32];
-    int s = 0;
+    __shared__ long long warp_sum[32];
+    long long s = 0;
     for (int k = threadIdx.x; k < kScan; k += 1024) {
         const long long i = (long long)blockIdx.x * kScan + k;
-        if (i < a.n_obs) s += a.rptr[1 + i];
+        if (i < a.n_obs) s += a.rfill[i];
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) warp_sum[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int w = 1; w < 32; ++w) s += warp_sum[w];
-        a.rfill[blockIdx.x] = s;
+        ((long long*)a.rpart)[blockIdx.x] = s;
     }
 }
 
 __global__ void __launch_bounds__(1024) sp_scan_kernel(SpArgs a) {
-    __shared__ int warp_sum[32];
+    __shared__ long long warp_sum[32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    auto block_sum = [&](int s) {
+    auto block_sum = [&](long long s) {
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) warp_sum[w] = s;
         __syncthreads();
-        int all = 0;
+        long long all = 0;
         for (int u = 0; u < 32; ++u) all += warp_sum[u];
         __syncthreads();
         return all;
     };
-    int before = 0;
-    for (int k = threadIdx.x; k < (int)blockIdx.x; k += 1024) before += a.rfill[k];
+    long long before = 0;
+    for (int k = threadIdx.x; k < (int)blockIdx.x; k += 1024) before += ((const long long*)a.rpart)[k];
     before = block_sum(before);
     constexpr int kPer = kScan / 1024;
     const long long i0 = (long long)blockIdx.x * kScan + kPer * threadIdx.x;
-    int v[kPer], s = 0;
+    int v[kPer];
+    long long s = 0;
     for (int q = 0; q < kPer; ++q) {
-        v[q] = i0 + q < a.n_obs ? a.rptr[1 + i0 + q] : 0;
+        v[q] = i0 + q < a.n_obs ? a.rfill[i0 + q] : 0;
         s += v[q];
     }
-    int incl = s;
+    long long incl = s;
     for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        const long long y = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += y;
     }
     if (lane == 31) warp_sum[w] = incl;
     __syncthreads();
-    int at = before + incl - s;
+    long long at = before + incl - s;
     for (int u = 0; u < w; ++u) at += warp_sum[u];
+    if (i0 == 0) a.rptr[0] = 0;
     for (int q = 0; q < kPer; ++q) {
         at += v[q];
         if (i0 + q < a.n_obs) a.rptr[1 + i0 + q] = at;
@@ -332,7 +334,7 @@ __global__ void sp_fill_kernel(SpArgs a) {
     if (e >= (size_t)a.n_model * a.rho) return;
     int2 v = a.cent[e];
     if (v.x < 0) return;
-    int slot = a.rptr[v.x] + atomicAdd(&a.rfill[v.x], 1);
+    const long long slot = a.rptr[v.x] + atomicAdd(&a.rfill[v.x], 1);
     a.rent[slot] = make_int2((int)(e / a.rho), v.y);
 }
 
@@ -340,15 +342,16 @@ __global__ void sp_fill_kernel(SpArgs a) {
 __global__ void sp_sort_rows_kernel(SpArgs a) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.n_obs) return;
-    const int s0 = a.rptr[i], s1 = a.rptr[i + 1];
-    for (int k = s0 + 1; k < s1; ++k) {
-        int2 v = a.rent[k];
+    int2* row = a.rent + a.rptr[i];
+    const int n = (int)(a.rptr[i + 1] - a.rptr[i]);
+    for (int k = 1; k < n; ++k) {
+        int2 v = row[k];
         int q = k - 1;
-        while (q >= s0 && a.rent[q].x > v.x) {
-            a.rent[q + 1] = a.rent[q];
+        while (q >= 0 && row[q].x > v.x) {
+            row[q + 1] = row[q];
             --q;
         }
-        a.rent[q + 1] = v;
+        row[q + 1] = v;
     }
 }
 
@@ -452,7 +455,7 @@ constexpr int kSpLanes = 8;  // lanes per spot
 __device__ float sp_row_exact(const SpArgs& a, int i, float dustv, bool ub) {
     float m = kNegHuge, s = 0.0f;
     if (!ub) acc_lse(m, s, dustv);
-    for (int e = a.rptr[i]; e < a.rptr[i + 1]; ++e) {
+    for (long long e = a.rptr[i]; e < a.rptr[i + 1]; ++e) {
         int2 v = a.rent[e];
         acc_lse(m, s, a.G[v.x] + a.negK * __int_as_float(v.y));
     }
@@ -564,24 +567,27 @@ __global__ void __launch_bounds__(kSpThreads) sp_pass_kernel(SpArgs a, int it, i
     float pm = kNegHuge, ps = 0.0f;  // LSE of the new potentials (less kc) over this lane's spots
     constexpr int kStep = kSpWarps * (32 / kSpLanes);
     for (int ib = td.y + w * (32 / kSpLanes); ib < td.z; ib += 2 * kStep) {
-        int e0[2], e1[2];
+        const int2* r[2];  // the lane's records of the spot: every kSpLanes-th of n
+        int n[2];
         float sum[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int i = ib + u * kStep + grp;
             const bool v = i < td.z;
-            e0[u] = v ? (ROWS ? a.rptr[i] : i * a.rho) + gl : 0;
-            e1[u] = v ? (ROWS ? a.rptr[i + 1] : (i + 1) * a.rho) : 0;
+            const long long e = v ? (ROWS ? a.rptr[i] : (long long)i * a.rho) : 0;
+            n[u] = v ? (ROWS ? (int)(a.rptr[i + 1] - e) : a.rho) : 0;
+            r[u] = rec + e;
             sum[u] = 0.0f;
         }
+        int at = gl;
         while (true) {
             int2 v[2][kSpBatch];
 #pragma unroll
             for (int u = 0; u < 2; ++u)
 #pragma unroll
                 for (int q = 0; q < kSpBatch; ++q) {
-                    const int e = e0[u] + q * kSpLanes;
-                    v[u][q] = e < e1[u] ? __ldcg(&rec[e]) : make_int2(-1, 0);
+                    const int e = at + q * kSpLanes;
+                    v[u][q] = e < n[u] ? __ldcg(r[u] + e) : make_int2(-1, 0);
                 }
             float g[2][kSpBatch];
 #pragma unroll
@@ -593,9 +599,8 @@ __global__ void __launch_bounds__(kSpThreads) sp_pass_kernel(SpArgs a, int it, i
 #pragma unroll
                 for (int q = 0; q < kSpBatch; ++q)
                     if (v[u][q].x >= 0) sum[u] += ex2(g[u][q] + a.negK * __int_as_float(v[u][q].y) - shift);
-            e0[0] += kSpBatch * kSpLanes;
-            e0[1] += kSpBatch * kSpLanes;
-            if (!__any_sync(0xffffffffu, e0[0] < e1[0] || e0[1] < e1[1])) break;
+            at += kSpBatch * kSpLanes;
+            if (!__any_sync(0xffffffffu, at < n[0] || at < n[1])) break;
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
@@ -641,7 +646,7 @@ __global__ void __launch_bounds__(kSpThreads) sp_harvest_row_kernel(SpArgs a) {
         for (int i = td.y + w; i < td.z; i += kSpWarps) {
             float m = kNegHuge, s = 0.0f;
             SpTop2 T2{kNegHuge, kNegHuge, -1};
-            for (int e = a.rptr[i] + lane; e < a.rptr[i + 1]; e += 32) {
+            for (long long e = a.rptr[i] + lane; e < a.rptr[i + 1]; e += 32) {
                 int2 v = a.rent[e];
                 float x = a.G[v.x] + a.negK * __int_as_float(v.y);
                 acc_lse(m, s, x);
@@ -766,7 +771,7 @@ size_t sparse_workspace_bytes(int T, int n_obs, int n_model, int rho) {
     auto add = [&](size_t bytes) { b += align_up(bytes > 0 ? bytes : 1, 256); };
     add(sizeof(int2) * nnz);                         // cent
     add(sizeof(int2) * nnz);                         // rent
-    add(sizeof(int) * ((size_t)n_obs + 2));          // rptr
+    add(sizeof(long long) * ((size_t)n_obs + 2));    // rptr
     add(sizeof(int) * ((size_t)n_obs + 1));          // rfill
     add(sizeof(float) * ((size_t)n_obs + 1));        // F
     add(sizeof(float) * ((size_t)n_model + 1));      // G
@@ -790,7 +795,7 @@ void sparse_carve(SpArgs& a, char* base, int T, int n_obs, int n_model, int rho)
     };
     a.cent = (int2*)take(sizeof(int2) * nnz);
     a.rent = (int2*)take(sizeof(int2) * nnz);
-    a.rptr = (int*)take(sizeof(int) * ((size_t)n_obs + 2));
+    a.rptr = (long long*)take(sizeof(long long) * ((size_t)n_obs + 2));
     a.rfill = (int*)take(sizeof(int) * ((size_t)n_obs + 1));
     a.F = (float*)take(sizeof(float) * ((size_t)n_obs + 1));
     a.G = (float*)take(sizeof(float) * ((size_t)n_model + 1));
@@ -846,7 +851,7 @@ cudaError_t sparse_sinkhorn_run(const SpArgs& a, const SkArgs* order, int n_iter
             return e;
         sp_knn_kernel<<<a.max_ct, kKnnThreads, shm, s>>>(a);
     }
-    if ((e = cudaMemsetAsync(a.rptr, 0, sizeof(int) * ((size_t)a.n_obs + 2), s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(a.rfill, 0, sizeof(int) * ((size_t)a.n_obs + 1), s)) != cudaSuccess) return e;
     const unsigned nb = (unsigned)((nnz + 255) / 256);
     if (nnz > 0) sp_count_kernel<<<nb, 256, 0, s>>>(a);
     if (a.n_obs > 0) {
