@@ -334,13 +334,13 @@ int laue_cost_sinkhorn(laue_handle* h, const LaueGeometry* geom, const LaueObsSp
  * hosted by a framework that owns every device allocation.  This entry point
  * has no counterpart in the paper.
  *
- * Scratch: a fixed 64 MiB array in device memory owned by this library
+ * Scratch: a fixed 128 MiB array in device memory owned by this library
  * module, reserved on every GPU where the module is loaded and held there
  * until the process exits; the call allocates nothing (no cudaMalloc,
- * cudaFree or allocating library routine).  It fits problems whose E-step
- * layout (laue_workspace_size with only T, n_obs, n_model set, up to the
- * E-step regions) is at most 64 MiB, about 1.5 million observed plus 1 million
- * model spots; larger problems return LAUE_ERR_CAPACITY before any launch.
+ * cudaFree or allocating library routine).  It takes problems whose spots,
+ * order and tables need at most 64 MiB (40 bytes an observed and 56 a model
+ * spot, about 200 an angle: 800000 observed plus 560000 model spots over 8000
+ * angles); larger problems return LAUE_ERR_CAPACITY before any launch.
  * The first call on a device looks the array's device address up (with that
  * device current) and caches it: make that first call before any stream
  * capture begins.  Every call on a device shares the one array, which keeps

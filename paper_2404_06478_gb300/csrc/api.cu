@@ -513,19 +513,18 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
     lc->col_split = prm->dust_mode == 2 && lc->col_slices <= kSplitSlicesPerSm * h->sm_count;
     {
         // the sort buffers, once the sort is done: slices, sub-granule cones, compact potentials
-        size_t rs = lc->row_slices, cs = lc->col_slices;
         char* b = ws + L.sortbuf;
         auto take = [&](size_t bytes) {
             char* p = b;
             b += align_up(bytes, 16);
             return p;
         };
-        a.row_desc = take(kSliceDescBytes * rs);
-        a.col_desc = take(kSliceDescBytes * cs);
-        a.obs_sub = (float4*)take(sizeof(float4) * kSubs * L.max_obs_gran);
-        a.mod_sub = (float4*)take(sizeof(float4) * kSubs * L.max_mod_gran);
-        a.obs_subext = (float*)take(sizeof(float) * kSubs * L.max_obs_gran);
-        a.mod_subext = (float*)take(sizeof(float) * kSubs * L.max_mod_gran);
+        a.row_desc = take(kSliceDescBytes * held_slices(a.T, a.n_obs, a.tile_rows));
+        a.col_desc = take(kSliceDescBytes * held_slices(a.T, a.n_model, a.tile_cols));
+        a.obs_sub = (float4*)take(sizeof(float4) * kSubs * L.obs_sub_gran);
+        a.mod_sub = (float4*)take(sizeof(float4) * kSubs * L.mod_sub_gran);
+        a.obs_subext = (float*)take(sizeof(float) * kSubs * L.obs_sub_gran);
+        a.mod_subext = (float*)take(sizeof(float) * kSubs * L.mod_sub_gran);
         a.Gc = (float*)take(sizeof(float) * 2 * L.max_mod_pairs);
         a.Fc = (float*)take(sizeof(float) * 2 * L.max_obs_pairs);
         a.pmax = (unsigned*)take(sizeof(unsigned) * 4 * a.T);
@@ -537,8 +536,8 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
     a.col_part = (float2*)(ws + L.col_part);
     a.dust = (float*)(ws + L.dust);
     a.ctrl = (int*)(ws + L.ctrl);
-    a.max_row_tiles = L.max_row_tiles;
-    a.max_col_tiles = L.max_col_tiles;
+    a.max_row_tiles = (int)std::min<size_t>(L.max_row_tiles, block_groups(a.T, a.n_obs, a.tile_rows));
+    a.max_col_tiles = (int)std::min<size_t>(L.max_col_tiles, block_groups(a.T, a.n_model, a.tile_cols));
     double eps = prm->eps;
     a.negKD2 = (float)(-(double)geom->D * geom->D * 1.4426950408889634 / eps);
     {

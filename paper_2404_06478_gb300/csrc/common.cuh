@@ -73,6 +73,14 @@ constexpr int kMaxTile = 256;      // largest tile (in spot pairs) of a launch s
 inline size_t list_slices(int T, int n_spots, int tile) {
     return (size_t)T * (tile / 32 + 1) + (size_t)n_spots / 64 + 2;
 }
+// The same without room for angles that have no spots: b = min(T, n_spots)
+// blocks hold at most (n_spots + b) / 2 pairs, in full groups of `width` pairs
+// and one more to a block.
+inline size_t block_groups(int T, int n_spots, int width) {
+    const size_t b = n_spots < T ? (n_spots > 0 ? n_spots : 0) : T;
+    return ((size_t)n_spots + b) / 2 / width + b + 1;
+}
+inline size_t held_slices(int T, int n_spots, int tile) { return block_groups(T, n_spots, tile) * (tile / 32); }
 constexpr size_t kCtrlBytes = 4096;  // status + counters + small scalars
 
 // ---------------------------------------------------------------------------
@@ -101,6 +109,8 @@ struct Layout {
     int max_row_tiles, max_col_tiles, max_fwd_blocks;
     int max_obs_pairs, max_mod_pairs;
     int max_obs_gran, max_mod_gran;
+    int obs_sub_gran, mod_sub_gran;  // granules that have sub-granule cones
+    size_t sort_more;                // bytes by which sortbuf outgrows the sort's own
 };
 
 constexpr int kMinTile = 64;      // smallest tile (in spot pairs) any launch shape uses
@@ -108,7 +118,8 @@ constexpr int kFwdBlock = 256;    // rays per forward block
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-inline Layout make_layout(const LaueProblemDims& d, int sm_count) {
+// tile: the largest tile whose slices have to fit
+inline Layout make_layout(const LaueProblemDims& d, int sm_count, int tile = kMaxTile) {
     Layout L{};
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -144,10 +155,13 @@ inline Layout make_layout(const LaueProblemDims& d, int sm_count) {
     L.max_mod_gran = (int)((jp + kConeGran - 1) / kConeGran) + T + 1;
     {
         size_t sort_bytes = sizeof(int) * 4 * nsp;
-        size_t slices = list_slices(T, d.n_obs, kMaxTile) + list_slices(T, d.n_model, kMaxTile);
+        size_t slices = held_slices(T, d.n_obs, tile) + held_slices(T, d.n_model, tile);
+        L.obs_sub_gran = (int)block_groups(T, d.n_obs, kConeGran);
+        L.mod_sub_gran = (int)block_groups(T, d.n_model, kConeGran);
         size_t reuse = slices * kSliceDescBytes + sizeof(float) * 2 * (ip + jp) +
                        sizeof(unsigned) * 4 * T + 128 +
-                       (sizeof(float4) + sizeof(float)) * kSubs * (size_t)(L.max_obs_gran + L.max_mod_gran);
+                       (sizeof(float4) + sizeof(float)) * kSubs * (size_t)(L.obs_sub_gran + L.mod_sub_gran);
+        if (reuse > sort_bytes) L.sort_more = align_up(reuse, 256) - align_up(sort_bytes, 256);
         L.sortbuf = take(sort_bytes > reuse ? sort_bytes : reuse);
     }
     L.cone = take((sizeof(float4) + sizeof(float)) * (size_t)(L.max_obs_gran + L.max_mod_gran) + 64);

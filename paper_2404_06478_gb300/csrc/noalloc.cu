@@ -14,7 +14,12 @@
 
 namespace laue {
 
-constexpr size_t kStaticScratchBytes = (size_t)64 << 20;  // 64 MiB
+// Problems are taken whose E-step fits kNoAllocBytes with the sort's buffers
+// counted for the sort alone.  What the passes keep there afterwards (slices,
+// cones, potentials) outgrows them where angles hold few spots, to 127.4 MiB in
+// all at one observed and one model spot for each of 225456 angles.
+constexpr size_t kNoAllocBytes = (size_t)64 << 20;
+constexpr size_t kStaticScratchBytes = (size_t)128 << 20;
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 
@@ -78,12 +83,13 @@ extern "C" int laue_cost_sinkhorn_noalloc(const LaueGeometry* geom, const LaueOb
     if ((rc = static_device(&d))) return rc;
     // the E-step uses the layout regions in front of the forward-model scratch
     LaueProblemDims dims{obs->T, obs->n, model->n, 0, 0, 0, 0};
-    Layout L = make_layout(dims, d->sm_count);
-    if (L.fwd_blocks > kStaticScratchBytes) return LAUE_ERR_CAPACITY;
+    const int variant = kSkDefaultVariant;
+    Layout L = make_layout(dims, d->sm_count, sk_variant_threads(variant));
+    if (L.fwd_blocks - L.sort_more > kNoAllocBytes || L.fwd_blocks > kStaticScratchBytes) return LAUE_ERR_CAPACITY;
     laue_handle h{};  // a view of the static scratch; nothing is allocated
     h.device = d->device;
     h.sm_count = d->sm_count;
-    h.row_variant = h.col_variant = kSkDefaultVariant;
+    h.row_variant = h.col_variant = variant;
     h.skip = 1;
     h.ws = d->scratch;
     h.ws_bytes = kStaticScratchBytes;
