@@ -208,9 +208,11 @@ const char* laue_last_error(const laue_handle* h);
 /* Workspace bytes for problems bounded by *dims.  The Sinkhorn passes list the
  * pairs whose plan entry can be nonzero in what the workspace holds beyond
  * the calls' own needs; the size includes room for those lists (at most 3 GB).
- * A smaller workspace, down to the calls' own needs, is accepted: the passes
- * then evaluate those pairs anew in every iteration, with the same results. */
+ * A smaller workspace, down to the calls' own needs (laue_workspace_min_size),
+ * is accepted: the passes then evaluate those pairs anew in every iteration,
+ * with the same results. */
 int laue_workspace_size(laue_handle* h, const LaueProblemDims* dims, size_t* bytes);
+int laue_workspace_min_size(laue_handle* h, const LaueProblemDims* dims, size_t* bytes);
 
 /* Hands the library a device buffer of `bytes` bytes (256-byte aligned) to
  * use as scratch; it must stay valid while calls that use it are in flight.
@@ -414,9 +416,10 @@ int laue_set_pair_skipping(laue_handle* h, int enable);
  * increasing cost, -1 past its end.  Needs a workspace of
  * 16 rho |J| + 16 (|I| + |J|) bytes plus small tables; laue_sparse_workspace_size
  * adds room for the direction order of the spots, with which the neighbours are
- * searched near each ray only (without it among every pair, with the same
- * result).  Asynchronous. */
+ * searched near each ray only (without it, laue_sparse_workspace_min_size,
+ * among every pair, with the same result).  Asynchronous. */
 int laue_sparse_workspace_size(int T, int n_obs, int n_model, int rho, size_t* bytes);
+int laue_sparse_workspace_min_size(int T, int n_obs, int n_model, int rho, size_t* bytes);
 int laue_cost_sinkhorn_sparse(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* obs,
                               const LaueModelSpots* model, const LaueOTParams* prm, int rho, float* f,
                               float* g, float* dust, int* assign, float* margin, float* marg_err, float* q,

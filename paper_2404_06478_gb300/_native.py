@@ -88,6 +88,7 @@ SIGNATURES = {
     "laue_destroy": [_vp],
     "laue_last_error": [_vp],
     "laue_workspace_size": [_vp, _P(LaueProblemDims), _P(ctypes.c_size_t)],
+    "laue_workspace_min_size": [_vp, _P(LaueProblemDims), _P(ctypes.c_size_t)],
     "laue_set_workspace": [_vp, _vp, ctypes.c_size_t, _vp],
     "laue_device_status": [_vp, _vp, _pi],
     "laue_reflections": [_d, _i, _i, _i, _vp, _vp, _vp, _pi],
@@ -107,6 +108,7 @@ SIGNATURES = {
     "laue_em": [_vp, _P(LaueGeometry), _P(LaueLattice), _P(LaueObsSpots), _vp, _P(LaueModelSpots), _vp, _vp, _i,
                 _P(LaueEMParams), _vp, _vp, _vp, _vp, _vp, _vp],
     "laue_sparse_workspace_size": [_i, _i, _i, _i, _P(ctypes.c_size_t)],
+    "laue_sparse_workspace_min_size": [_i, _i, _i, _i, _P(ctypes.c_size_t)],
     "laue_cost_sinkhorn_sparse": [_vp, _P(LaueGeometry), _P(LaueObsSpots), _P(LaueModelSpots), _P(LaueOTParams),
                                   _i, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp],
     "laue_read_counters": [_vp, _vp, _P(ctypes.c_longlong), _i],

@@ -223,6 +223,7 @@ class Handle:
             raise LaueError(rc, "laue_create failed")
         self.h = h
         self.ws = None
+        self._denied = None  # the smallest workspace that could not be allocated
 
     def close(self):
         if self.h:
@@ -250,18 +251,32 @@ class Handle:
     def reserve(self, T, n_obs=0, n_model=0, n_grains=0, n_planes=0, n_starts=0, n_candidates=0, extra=0,
                 stream=None):
         need = self.workspace_size(T, n_obs, n_model, n_grains, n_planes, n_starts, n_candidates) + int(extra)
-        if self.ws is None or self.ws.numel() < need:
-            self.ws = torch.empty(need + 256, dtype=torch.uint8, device=self.device)
-            self.check(self.L.laue_set_workspace(self.h, _ptr(self.ws), self.ws.numel(), _stream(stream)),
-                       "set_workspace")
-        return self.ws
+        if self.ws is not None and self.ws.numel() >= need:
+            return self.ws
+        d = N.LaueProblemDims(T, n_obs, n_model, n_grains, n_planes, n_starts, n_candidates)
+        b = ctypes.c_size_t()
+        self.check(self.L.laue_workspace_min_size(self.h, ctypes.byref(d), ctypes.byref(b)), "workspace_min_size")
+        return self.reserve_bytes(need, stream=stream, least=b.value + int(extra))
 
-    def reserve_bytes(self, need, stream=None):
-        """Grow the workspace to at least `need` bytes (keeps a larger one)."""
-        if self.ws is None or self.ws.numel() < need:
-            self.ws = torch.empty(int(need) + 256, dtype=torch.uint8, device=self.device)
-            self.check(self.L.laue_set_workspace(self.h, _ptr(self.ws), self.ws.numel(), _stream(stream)),
-                       "set_workspace")
+    def reserve_bytes(self, need, stream=None, least=None):
+        """Grow the workspace to at least `need` bytes (keeps a larger one), or
+        to `least` where the device has no room for them; a size that it had no
+        room for is not asked for again."""
+        need = int(need)
+        if least is not None and self._denied is not None and need >= self._denied:
+            need = int(least)
+        if self.ws is not None and self.ws.numel() >= need:
+            return self.ws
+        try:
+            ws = torch.empty(need + 256, dtype=torch.uint8, device=self.device)
+        except torch.cuda.OutOfMemoryError:
+            if least is None or need <= least:
+                raise
+            self._denied = need
+            return self.reserve_bytes(least, stream=stream)
+        self.ws = ws
+        self.check(self.L.laue_set_workspace(self.h, _ptr(self.ws), self.ws.numel(), _stream(stream)),
+                   "set_workspace")
         return self.ws
 
     def alu_peaks(self, stream=None) -> dict:
@@ -385,7 +400,11 @@ def cost_sinkhorn_sparse(h: Handle, geom, obs: ObsSpots, model: ModelSpots, eps,
     nI, nJ = int(obs.p.shape[0]), model.n
     b = ctypes.c_size_t()
     h.check(h.L.laue_sparse_workspace_size(T, nI, nJ, int(rho), ctypes.byref(b)), "sparse_workspace_size")
-    h.reserve_bytes(b.value, stream=stream)
+    if h.ws is None or h.ws.numel() < b.value:
+        least = ctypes.c_size_t()
+        h.check(h.L.laue_sparse_workspace_min_size(T, nI, nJ, int(rho), ctypes.byref(least)),
+                "sparse_workspace_min_size")
+        h.reserve_bytes(b.value, stream=stream, least=least.value)
     nd = T if dust_mode else 1
     if init is not None:
         f, g, dust = (t.clone().float().contiguous() for t in init)

@@ -167,6 +167,12 @@ extern "C" int laue_workspace_size(laue_handle* h, const LaueProblemDims* dims, 
     return LAUE_OK;
 }
 
+extern "C" int laue_workspace_min_size(laue_handle* h, const LaueProblemDims* dims, size_t* bytes) {
+    const int rc = laue_workspace_size(h, dims, bytes);
+    if (rc == LAUE_OK) *bytes -= list_bytes(*dims);
+    return rc;
+}
+
 extern "C" int laue_set_workspace(laue_handle* h, void* dev_ptr, size_t bytes, void* stream) {
     if (!h) return LAUE_ERR_INVALID_ARG;
     if (dev_ptr && ((uintptr_t)dev_ptr & 255u))
@@ -624,6 +630,12 @@ extern "C" int laue_sparse_workspace_size(int T, int n_obs, int n_model, int rho
     LaueProblemDims d{T, n_obs, n_model, 0, 0, 0, 0};
     *bytes = align_up(kCtrlBytes + sparse_workspace_bytes(T, n_obs, n_model, rho), 256) + make_layout(d, 1).total;
     return LAUE_OK;
+}
+
+extern "C" int laue_sparse_workspace_min_size(int T, int n_obs, int n_model, int rho, size_t* bytes) {
+    const int rc = laue_sparse_workspace_size(T, n_obs, n_model, rho, bytes);
+    if (rc == LAUE_OK) *bytes = kCtrlBytes + sparse_workspace_bytes(T, n_obs, n_model, rho);
+    return rc;
 }
 
 extern "C" int laue_cost_sinkhorn_sparse(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* obs,

@@ -198,7 +198,9 @@ inline size_t list_bytes(const LaueProblemDims& d) {
     double slices = (double)list_slices(T, d.n_obs, 256) + (double)list_slices(T, d.n_model, 256);
     double chunks = 2.5 * pairs / (kListDepth * 64) + 2.0 * slices;
     size_t pool = chunks < (double)kListPoolMax ? (size_t)chunks + 1 : kListPoolMax;
-    return list_fixed_bytes(T, d.n_obs, d.n_model, 256, 256) + pool * kListChunkBytes;
+    const size_t all = list_fixed_bytes(T, d.n_obs, d.n_model, 256, 256) + pool * kListChunkBytes;
+    const size_t most = kListPoolMax * kListChunkBytes;  // also where many angles need large tables of chunk numbers
+    return all < most ? all : most;
 }
 
 // ---------------------------------------------------------------------------
