@@ -220,7 +220,7 @@ cudaError_t sinkhorn_harvest(const SkArgs& a, const SkLaunch& l, int n_iter, boo
 cudaError_t sinkhorn_setup();  // once per device, the current one
 cudaError_t sinkhorn_build_lists(const SkArgs& a, const SkLaunch& l, cudaStream_t s);
 int sk_variant_threads(int v);
-float list_share_of(int n_iter);
+float list_share_of(const SkArgs& a, int n_iter);
 float plan_share_of(const SkArgs& a, int n_pass);
 cudaError_t sinkhorn_row_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s);
 cudaError_t sinkhorn_col_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s);

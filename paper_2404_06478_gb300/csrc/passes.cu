@@ -26,6 +26,7 @@ namespace laue {
 
 constexpr float kTinySum = 1.0e-30f;  // below ~2^-100 the fast sum is recomputed exactly
 constexpr float kFarLog2 = 60.0f;     // see the read-out kernels
+constexpr float kListAlways = 1.0e30f;  // list_share of slices that need not look
 
 // ------------------------------------------------------------- pair lists
 // For fixed poses and temperature the pairs whose plan entry can be nonzero
@@ -52,13 +53,13 @@ constexpr float kFarLog2 = 60.0f;     // see the read-out kernels
 // the slice), so a slice first estimates its entries: how many of the streamed
 // spots' sub-granules lie, by their axes, within the listed angle of its own
 // spots.  It is left to the sweep if they exceed a list, or list_share of its
-// evaluated pairs.  Measured as the cost of listing in swept iterations, 1.4 at
-// an entry per 30 pairs, 3 at one in 6, 4 to 11 at one in 3: so the share
+// evaluated pairs (list_share_of).  The cost of listing is 1.4 swept iterations at
+// an entry per 30 evaluated pairs, 3 at one in 6, 4 to 11 at one in 3, so the share
 // grows with the iterations that a list is used for.  90 angles of 13300 x 7744
 // spots, 20 iterations at 100 mm^2: 91.6 ms when every slice tried, 77.7 now (at
-// 21 mm^2, where the pool holds a part of the entries: 48.0 and 46); 60 angles
+// 21 mm^2, where the pool holds a part of the entries: 48.0 and 46.4); 60 angles
 // of 1020 x 776 spots, 2 and 5 iterations at 100 mm^2: 0.90 and 1.06 ms, now 0.52
-// and 0.78; at 1 mm^2 the same slices are listed.
+// and 0.79; at 1 mm^2 the same slices are listed.
 //
 // Most of the pairs that the cones let through are still too far apart, so a
 // cheap test comes first: the angle between p (seen from the origin) and r is
@@ -142,7 +143,7 @@ __global__ void __launch_bounds__(32 * kListWarps) sk_list_kernel(SkArgs a) {
     };
     bool fail = a.pool_chunks == 0 || n_str > 65536;
     int evaluated;
-    if (fail) {
+    if (fail || a.list_share >= kListAlways) {
         evaluated = count_pairs<false>(own, ROWS, sub, subext, np, n_str, a.skip, a.skipK, cone_cut, da, 2.0f).pairs;
     } else {
         // the entries that the lanes' first spots will have, on average: too many to list, or to be worth it?
@@ -1147,21 +1148,33 @@ __global__ void __launch_bounds__(pass_threads(TILE), kPassThreadsPerSm / pass_t
 // tile.  (Shapes 1 and 2 are the same kernels.)
 int sk_variant_threads(int v) { return v == 0 ? 256 : (v == 3 ? 64 : 128); }
 
+// Entries that a spot can expect for costs of `most` in units of 1 / K (two
+// detectors see about 2 sr).
+static float expected_entries(const SkArgs& a, float most, int n_streamed) {
+    return (float)n_streamed / (float)a.T * 3.14159f * (most / a.skipK) / 2.0f;
+}
+
 // Largest entries per spot, as a share of the slice's swept pairs, that are
 // worth listing for n_iter iterations: where the cost of listing (see above) is
-// made up by passes over lists (0.03 to 0.5 of a swept one).
-float list_share_of(int n_iter) { return (n_iter - 1.0f) / (n_iter + 14.0f); }
+// made up by passes over lists (0.03 to 0.5 of a swept one).  From 40 iterations
+// on every list is that fits, and where the entries are few the slices need not
+// look (kListAlways).
+float list_share_of(const SkArgs& a, int n_iter) {
+    const float share = (n_iter - 1.0f) / (15.0f + 0.6f * n_iter);
+    if (share < 1.0f) return share;
+    return expected_entries(a, kListLog2, std::max(a.n_obs, a.n_model)) <= 128.0f ? kListAlways : 1.0f;
+}
 
-// The same for n_pass passes of an M-step.  A single pass is listed for, whole,
-// or swept, whole: listed slices beside swept ones only add up.  The line lies at
-// 20 entries of a spot (two detectors see about 2 sr; 2^-40 at the usual
-// potentials).  Gradients, listed against swept: 1 mm^2, 1020 observed spots an
-// angle (1 entry) 0.171 and 0.183 ms, 13300 (16) 1.84 and 1.96; 21 mm^2, 1020 (26)
-// 0.224 and 0.198, 3700 (95) 0.75 and 0.57; 100 mm^2, 13300: 19.2 and 3.8.
+// The same for n_pass passes of an M-step (entries of at least 2^-40 at the usual
+// potentials).  A single pass is listed for, whole, or swept, whole: listed slices
+// beside swept ones only add up.  The line lies at 20 entries of a spot.
+// Gradients, listed against swept: 1 mm^2, 1020 observed spots an angle (1 entry)
+// 0.171 and 0.183 ms, 13300 (16) 1.84 and 1.96; 21 mm^2, 1020 (26) 0.224 and 0.198,
+// 3700 (95) 0.75 and 0.57; 100 mm^2, 13300: 19.2 and 3.8.
 float plan_share_of(const SkArgs& a, int n_pass) {
-    if (n_pass > 1) return n_pass / (n_pass + 4.0f);
-    const float th2 = (4.0f - kQSkip) / a.skipK;
-    return (float)a.n_obs / (float)a.T * 3.14159f * th2 / 2.0f > 20.0f ? 0.0f : 1.0f;
+    const float entries = expected_entries(a, 4.0f - kQSkip, a.n_obs);
+    if (entries <= (n_pass > 1 ? 128.0f : 20.0f)) return kListAlways;
+    return n_pass > 1 ? n_pass / (n_pass + 4.0f) : 0.0f;
 }
 
 namespace {

@@ -689,7 +689,7 @@ cudaError_t sinkhorn_run(const SkArgs& a0, const SkLaunch& l, int n_iter, bool w
     SkArgs a = a0;
     // listing the pairs costs about as much as one sweep of each side
     if (n_iter < 2) a.pool_chunks = 0;
-    a.list_share = list_share_of(n_iter);
+    a.list_share = list_share_of(a, n_iter);
     cudaError_t e = sinkhorn_prepare(a, s);
     if (e != cudaSuccess) return e;
     e = sinkhorn_build_lists(a, l, s);
