@@ -791,6 +791,13 @@ extern "C" int laue_autotune(laue_handle* h, const LaueGeometry* geom, const Lau
     int row_v = 0, col_v = 0;
     int save_r = h->row_variant, save_c = h->col_variant;
     for (int v = 0; v < kSkVariants && rc == LAUE_OK; ++v) {
+        if (v > 0 && sk_variant_threads(v) == sk_variant_threads(v - 1)) {  // the same kernels
+            if (ms_host) {
+                ms_host[2 * v] = ms_host[2 * (v - 1)];
+                ms_host[2 * v + 1] = ms_host[2 * (v - 1) + 1];
+            }
+            continue;
+        }
         // each shape with its own tile size: rebuild the schedule, warm up, time the passes
         h->row_variant = v;
         h->col_variant = v;
@@ -838,7 +845,7 @@ extern "C" int laue_autotune(laue_handle* h, const LaueGeometry* geom, const Lau
     return LAUE_OK;
 }
 
-// ------------------------------------------------------------- not yet built
+// --------------------------------------------------------------- M-step
 
 int laue_mstep_any(laue_handle* h, const LaueGeometry* geom, const LaueLattice* lat, const LaueObsSpots* obs,
                        const LaueModelSpots* model, const float* f, const float* g, const LaueMParams* prm,
@@ -878,7 +885,6 @@ int laue_mstep_any(laue_handle* h, const LaueGeometry* geom, const LaueLattice* 
     m.J_off = model->J_off;
     m.grain = model->grain;
     m.plane = model->plane;
-    m.angle = model->angle;
     m.R = R;
     m.x = x;
     m.jsum = (float*)(ws + L.jsum);
@@ -951,7 +957,6 @@ extern "C" int laue_objective_grad(laue_handle* h, const LaueGeometry* geom, con
     m.J_off = model->J_off;
     m.grain = model->grain;
     m.plane = model->plane;
-    m.angle = model->angle;
     m.R = const_cast<float*>(R);
     m.x = const_cast<float*>(x);
     m.jsum = (float*)(ws + L.jsum);

@@ -14,21 +14,12 @@ namespace laue {
 // ---------------------------------------------------------------------------
 enum CtrlSlot {
     CTRL_STATUS = 0,      // first device-side error code (0 = none)
-    CTRL_ROW_NEXT = 1,    // tile queue head of the row pass
-    CTRL_ROW_DONE = 2,    // finished-CTA ticket of the row pass
-    CTRL_COL_NEXT = 3,
-    CTRL_COL_DONE = 4,
     CTRL_N_ROW_TILES = 5, // tiles built by the scheduler
     CTRL_N_COL_TILES = 6,
     CTRL_FWD_TOTAL = 7,   // visible spots found by the forward pass
-    CTRL_HRV_NEXT = 8,    // harvest passes
-    CTRL_HRV_DONE = 9,
-    CTRL_HCOL_NEXT = 10,
-    CTRL_HCOL_DONE = 11,
-    CTRL_GEN_NEXT = 12,   // generic queue / ticket pair for other passes
-    CTRL_GEN_DONE = 13,
-    CTRL_SF_NEXT = 14,    // single-grain fit start queue / ticket
-    CTRL_SF_DONE = 15,
+    CTRL_HRV_DONE = 9,    // finished CTAs of the read-outs of the rows
+    CTRL_HCOL_DONE = 11,  // and of the columns
+    CTRL_SF_NEXT = 14,    // single-grain fit start queue
     CTRL_EXACT_ROWS = 16, // row / column log-sum-exps recomputed on the exact path
     CTRL_EXACT_COLS = 17,
     CTRL_SF_PAIRS = 18,   // 64-bit count (slots 18-19) of single-fit pair evaluations
@@ -188,8 +179,9 @@ inline size_t list_fixed_bytes(int T, int n_obs, int n_model, int tile_rows, int
     return align_up(s * sizeof(int) * (size_t)kListChunks, 256);
 }
 // Bytes the lists can use: room for every same-angle pair of both sides with a
-// quarter more for padding, and at most kListPoolMax chunks (3 GB; 400 million
-// entries: the 1000-grain configuration's passes hold 81 million at 1 mm^2).
+// quarter more for padding, and at most kListPoolMax chunks (3 GB; 537 million
+// entries: the 1000-grain configuration's lists hold 108 million at 1 mm^2, both
+// sides and their padding included).
 constexpr size_t kListPoolMax = 1u << 20;
 inline size_t list_bytes(const LaueProblemDims& d) {
     if (d.n_obs <= 0 || d.n_model <= 0) return 0;
@@ -238,9 +230,7 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-// mbarrier + bulk async copy (TMA, non-tensor form).  Addresses and sizes of
-// cp.async.bulk must be multiples of 16 bytes: every staged array here is
-// float4 rows starting at 256-byte aligned bases.
+// mbarriers (the tiled copies that complete on them are in gemm_tc.cu).
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count)
                  : "memory");
@@ -253,13 +243,6 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
         "{\n\t.reg .b64 st;\n\t"
         "mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(smem_u32(bar)),
         "r"(bytes)
-        : "memory");
-}
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar))
         : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {

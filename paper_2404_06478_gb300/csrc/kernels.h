@@ -163,7 +163,6 @@ struct SpArgs {
     int* rt_base;          // T + 1 first row tile of each angle (entry T = row tile count)
     int* ct_base;          // T + 1
     float* gmax;           // T: largest G of each angle block (shift of the row pass)
-    float* fmax;           // T: largest F of each angle block (shift of the column pass)
     int max_rt, max_ct;
     int* ctrl;
     float negK;            // -D^2 log2(e) / eps
@@ -191,13 +190,14 @@ void sparse_carve(SpArgs& a, char* base, int T, int n_obs, int n_model, int rho)
 cudaError_t sparse_sinkhorn_run(const SpArgs& a, const SkArgs* order, int n_iter, bool rows, bool cols,
                                 cudaStream_t s);
 
-constexpr int kSkVariants = 4;       // launch shapes of the pair passes (see sinkhorn.cu)
+constexpr int kSkVariants = 4;       // launch shapes of the pair passes (see passes.cu)
 // Unbalanced passes of at most this many slices per SM are split (four warps a
-// slice): an SM holds 8 such slices at once, so warps that find nothing to do
-// cost nothing.  Measured (50 iterations, 60 angles, split against not): 7
-// slices per SM, 5.2 against 6.8 ms at 4 mm^2 where every column takes the exact
-// path, 6.9 against 6.9 at 100 mm^2 where none does; 23 per SM, 28.5 against
-// 40.7 and 49.5 against 44.1 ms.
+// slice).  It pays where slices take the exact path, which every column does at
+// 4 mm^2 and none of these at 100 mm^2, and there the split warps are in the way;
+// the host cannot know which.  Measured (50 iterations, 60 angles, split against
+// not, at 4 and 100 mm^2): 2 slices per SM 1.24 against 1.50 and 2.32 against 2.15
+// ms; 7 per SM 5.2 against 5.4 and 6.7 against 5.5; 23 per SM 23.4 against 28.2
+// and 39.7 against 28.1.
 constexpr int kSplitSlicesPerSm = 8;
 constexpr int kSkDefaultVariant = 3;  // 64-pair tiles: the autotuner's usual pick
 
@@ -235,7 +235,6 @@ struct MsArgs {
     const int* J_off;
     const int* grain;
     const int* plane;
-    const int* angle;
     float* R;               // N x 9, in/out
     float* x;               // N x 3, in/out
     float* jsum;            // 12 floats per model spot

@@ -151,7 +151,6 @@ struct ColPair {
     f2 ncxa, ncya, ncza, nrxa, nrya, nrza;
     f2 ncxb, ncyb, nczb, nrxb, nryb, nrzb;
     f2 ka, kb;  // {-K_a, -K_a}, {-K_b, -K_b}: cost factors of the two model spots
-    RowLse A, B;
 };
 
 __device__ __forceinline__ void load_col_pair(const SkArgs& a, int q, ColPair& C) {

@@ -703,10 +703,9 @@ __device__ __forceinline__ void pass_release() { asm volatile("griddepcontrol.la
 // Without dustbins (unbalanced OT) a shifted sum underflows for most spots:
 // the potentials of spots far from any partner are the largest, and shift all
 // the others.  Their slices read the whole block with a running maximum, a
-// serial chain of about 0.1 us per 4 pairs, so a pass over few slices has
-// PARTS warps to a slice that read a part of the block each; part 0's warp
-// merges.  23 grains x 17 angles at 4 mm^2: 23 us a pass with one warp, 14 us
-// with four.
+// serial chain, so a pass over few slices has PARTS warps to a slice that read a
+// part of the block each; part 0's warp merges.  23 grains x 17 angles at 4 mm^2:
+// 17 us a pass with one warp, 14 us with four.
 //
 // Registers: 128 a thread, 512 threads to an SM.  No more are resident anyway:
 // a named barrier whose id is not a constant takes all 16 of a CTA, four CTAs to

@@ -140,8 +140,7 @@ __global__ void __launch_bounds__(1024) sk_schedule_kernel(SkArgs a, int dustbin
         }
         a.ctrl[CTRL_N_ROW_TILES] = nr;
         a.ctrl[CTRL_N_COL_TILES] = nc;
-        for (int k = CTRL_ROW_NEXT; k <= CTRL_GEN_DONE; ++k)
-            if (k != CTRL_N_ROW_TILES && k != CTRL_N_COL_TILES && k != CTRL_FWD_TOTAL) a.ctrl[k] = 0;
+        a.ctrl[CTRL_HRV_DONE] = a.ctrl[CTRL_HCOL_DONE] = 0;
     }
     __syncthreads();
     for (int t = threadIdx.x; t < T; t += blockDim.x) {
@@ -648,7 +647,7 @@ __global__ void __launch_bounds__(256) sk_init_gmax_kernel(SkArgs a) {
         }
         DustPtrs D = dust_ptrs(a.dust, a.T);
         D.Gmax[t] = m;
-        D.Fmax[t] = f;  // the M-step's skipping bound; a row pass rewrites it
+        D.Fmax[t] = f;  // the M-step's skipping bound
     }
 }
 

@@ -452,9 +452,9 @@ __device__ __forceinline__ void sp_merge_parts(const float2* part, int k0, int k
 constexpr float kSpTiny = 1.0e-30f;
 constexpr int kSpLanes = 8;  // lanes per spot
 
-__device__ float sp_row_exact(const SpArgs& a, int i, float dustv, bool ub) {
+__device__ float sp_row_exact(const SpArgs& a, int i, float dustv) {
     float m = kNegHuge, s = 0.0f;
-    if (!ub) acc_lse(m, s, dustv);
+    acc_lse(m, s, dustv);
     for (long long e = a.rptr[i]; e < a.rptr[i + 1]; ++e) {
         int2 v = a.rent[e];
         acc_lse(m, s, a.G[v.x] + a.negK * __int_as_float(v.y));
@@ -462,9 +462,9 @@ __device__ float sp_row_exact(const SpArgs& a, int i, float dustv, bool ub) {
     return s > 0.0f ? m + lg2(s) : kNegHuge;
 }
 
-__device__ float sp_col_exact(const SpArgs& a, int j, float F0, bool ub) {
+__device__ float sp_col_exact(const SpArgs& a, int j, float F0) {
     float m = kNegHuge, s = 0.0f;
-    if (!ub) acc_lse(m, s, F0);
+    acc_lse(m, s, F0);
     const int2* ce = a.cent + (size_t)j * a.rho;
     for (int k = 0; k < a.rho; ++k) {
         int2 v = ce[k];
@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(kSpThreads) sp_pass_kernel(SpArgs a, int it, i
             if (i < td.z && gl == 0) {
                 sum[u] += dterm;
                 const float lse = sum[u] > kSpTiny ? shift + lg2(sum[u])
-                                                   : (ROWS ? sp_row_exact(a, i, dust, false) : sp_col_exact(a, i, dust, false));
+                                                   : (ROWS ? sp_row_exact(a, i, dust) : sp_col_exact(a, i, dust));
                 out[i] = -lse;
                 acc_lse(pm, ps, -lse - off);
             }
@@ -781,7 +781,7 @@ size_t sparse_workspace_bytes(int T, int n_obs, int n_model, int rho) {
     add(sizeof(int4) * sp_max_tiles(n_obs, T));      // rtile
     add(sizeof(int4) * sp_max_tiles(n_model, T));    // ctile
     add(sizeof(int) * 2 * ((size_t)T + 1));          // rt_base, ct_base
-    add(sizeof(float) * 2 * ((size_t)T + 1));        // gmax, fmax
+    add(sizeof(float) * ((size_t)T + 1));            // gmax
     return b;
 }
 
@@ -806,8 +806,7 @@ void sparse_carve(SpArgs& a, char* base, int T, int n_obs, int n_model, int rho)
     a.ctile = (int4*)take(sizeof(int4) * sp_max_tiles(n_model, T));
     a.rt_base = (int*)take(sizeof(int) * 2 * ((size_t)T + 1));
     a.ct_base = a.rt_base + T + 1;
-    a.gmax = (float*)take(sizeof(float) * 2 * ((size_t)T + 1));
-    a.fmax = a.gmax + T + 1;
+    a.gmax = (float*)take(sizeof(float) * ((size_t)T + 1));
     a.max_rt = (int)sp_max_tiles(n_obs, T);
     a.max_ct = (int)sp_max_tiles(n_model, T);
 }
