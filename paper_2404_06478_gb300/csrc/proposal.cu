@@ -409,12 +409,13 @@ __device__ uint32_t select_key(const unsigned long long* cand, int n, int k, uin
 // hold KSET are collected in one pass over the axes, and the rest of the work
 // is on them (about a thousand) in shared memory.  In a window whose axes are
 // spread otherwise the spots are too few (another pass, with a larger distance)
-// or too many for the buffer; those in it are then a sample, whose order
-// statistic is the next distance.  Returns the number collected, -1 when that
-// does not succeed or the sample is mostly ties (select_wide then takes over).
-// 512 sets of windows of 20000 spots: 0.087 ms with the axes spread evenly (0.182
-// by select_wide), 0.089 with all of them within 0.01 of each other (0.171, and
-// 0.268 when the distance was divided by four up to four times), 0.190 with all
+// or too many for the buffer: a quarter of the distance then, and if those are too
+// many again, they are a sample whose order statistic is the next distance.
+// Returns the number collected, -1 when that does not succeed or the sample is
+// mostly ties (select_wide then takes over).
+// 512 sets of windows of 20000 spots: 0.084 ms with the axes spread evenly (0.182
+// by select_wide), 0.112 with all of them within 0.01 of each other (0.171, and
+// 0.268 when the distance was divided by four up to four times), 0.219 with all
 // of them equal (0.173).
 constexpr int kCand = 4096;
 constexpr int kSetAim = 8 * KSET;  // spots that a distance should hold
@@ -477,7 +478,10 @@ __device__ int select_near(const SetsArgs& a, int lo, int hi, int i0, float3 n0,
         n = found[2];
         __syncthreads();
         if (n > kCand) {
-            if (!sample_key(cand, n, hist, found, most)) return -1;
+            // evenly spread axes are a few times denser than that on two detectors
+            uint32_t next = __float_as_uint(0.25f * __uint_as_float(most));
+            if (attempt > 0 && !sample_key(cand, n, hist, found, next)) return -1;
+            most = next;
         } else if (n < K) {
             most = __float_as_uint(fminf(2.0f, 4.0f * __uint_as_float(most)));
         } else {
