@@ -151,7 +151,8 @@ struct SpArgs {
     // workspace
     int2* cent;            // n_model x rho: {observed index or -1, e2 (D_j / D)^2 bits}, by increasing e2
     int2* rent;            // CSR rows: {model index, e2 bits}, ascending model index
-    long long* rptr;       // n_obs + 1 row starts (n_model x rho may pass 2^31)
+    int* rptr;             // n_obs + 1 row starts, or
+    long long* rptr64;     // (not null) where n_model x rho records may pass 2^31
     int* rfill;            // n_obs counters: entries of each row, then those filled
     float* F;              // n_obs
     float* G;              // n_model
