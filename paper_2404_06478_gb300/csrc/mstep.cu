@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kMsThreads) ms_pair_kernel(MsArgs m) {
     } else {
         const Cone own = load_cone(a.mod_cone, a.mod_ext, a.mod_gbase[t] + (q - sl.lane - a.J2_off[t]) / kGran);
         const f2 Gpa = dup(Ga), Gpb = dup(Gb);
-        sweep<false>(a, M.stage, own, a.obs_sub + (size_t)kSubs * a.obs_gbase[t],
+        sweep<false, false>(a, M.stage, own, a.obs_sub + (size_t)kSubs * a.obs_gbase[t],
                      a.obs_subext + (size_t)kSubs * a.obs_gbase[t], sl.s0, sl.ns, a.skip, sl.cut, a.Fc,
                      [&](int st, int n, const int4&) {
                          for (int j = 0; j < n; ++j) {

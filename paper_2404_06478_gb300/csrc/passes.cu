@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(32 * kListWarps) sk_list_kernel(SkArgs a) {
             ((unsigned short*)(p + kListDepth * 64 * 4))[at] = (unsigned short)slot;
             ++cnt;
         };
-        sweep<ROWS>(a, L.S, own, sub, subext, b0, np, a.skip, cone_cut, PLAN ? a.Fc : nullptr,
+        sweep<ROWS, false>(a, L.S, own, sub, subext, b0, np, a.skip, cone_cut, PLAN ? a.Fc : nullptr,
                     [&](int st, int n, const int4& f) {
             if (fail || kListDepth * nch > evaluated) {
                 fail = true;  // mostly nonzero: the sweep is as good
@@ -356,17 +356,17 @@ __device__ __forceinline__ void swept_sum(const SkArgs& a, WarpStage& S, const S
     };
     if (ROWS) {
         const RowPair R = load_row_pair(a, sl.q, sl.valid);
-        for_each_swept<ROWS>(a, S, sl, a.skip, [&](int st, int j, float2 P, int) {
+        for_each_swept<ROWS>(a, S, sl, a.skip, shift, [&](int st, int j, int) {
             f2 va, vb;
-            row_pair_v(R, S, st, j, pk(P.x - shift, P.y - shift), va, vb);
+            row_pair_v(R, S, st, j, *(const f2*)&S.P[st][j], va, vb);
             add(va, vb);
         });
     } else {
         ColPair C;
         load_col_pair(a, sl.valid ? sl.q : sl.q - sl.lane, C);
-        for_each_swept<ROWS>(a, S, sl, a.skip, [&](int st, int j, float2 P, int) {
+        for_each_swept<ROWS>(a, S, sl, a.skip, shift, [&](int st, int j, int) {
             f2 va, vb;
-            col_pair_v(C, S, st, j, pk(P.x - shift, P.y - shift), va, vb);
+            col_pair_v(C, S, st, j, *(const f2*)&S.P[st][j], va, vb);
             add(va, vb);
         });
     }
@@ -392,7 +392,7 @@ __device__ __forceinline__ void exact_sums(const SkArgs& a, WarpStage& S, const 
         from = subs * part / PARTS * kSubGran;
         to = min(subs * (part + 1) / PARTS * kSubGran, w.n);
     }
-    sweep<ROWS>(a, S, w.own, w.sub, w.ext, w.b0 + from, to - from, 0, kSkipLog2, ROWS ? a.Gc : a.Fc,
+    sweep<ROWS, true>(a, S, w.own, w.sub, w.ext, w.b0 + from, to - from, 0, kSkipLog2, ROWS ? a.Gc : a.Fc,
                 [&](int st, int n, const int4&) {
         auto pair = [&](int j, f2& va, f2& vb) {
             const f2 base = *(const f2*)&S.P[st][j];
@@ -710,8 +710,8 @@ __device__ __forceinline__ void pass_release() { asm volatile("griddepcontrol.la
 // Registers: 128 a thread, 512 threads to an SM.  No more are resident anyway:
 // a named barrier whose id is not a constant takes all 16 of a CTA, four CTAs to
 // an SM.  With 64 registers the sums over swept pairs spilled: 90 angles of
-// 13300 x 7744 spots at 100 mm^2 without lists 5.8 ms an iteration, now 4.8; one
-// block of 200000 x 8000 spots 11.1 ms, now 7.0.  (The split passes keep 64:
+// 13300 x 7744 spots at 100 mm^2 without lists 5.8 ms an iteration, now 4.6; one
+// block of 200000 x 8000 spots 11.1 ms, now 6.3.  (The split passes keep 64:
 // four times the warps.)
 constexpr int kPassThreadsPerSm = 512;
 template <int TILE, int OTHER, bool ROWS, int PARTS>
@@ -966,9 +966,9 @@ __global__ void __launch_bounds__(pass_threads(TILE), kPassThreadsPerSm / pass_t
         B.init();
         const RowPair R = load_row_pair(a, sl.q, sl.valid);
         auto sweep_all = [&](int skip) {
-            for_each_swept<true>(a, M.stage, sl, skip, [&](int st, int j, float2 P, int k) {
+            for_each_swept<true>(a, M.stage, sl, skip, 0.0f, [&](int st, int j, int k) {
                 f2 va, vv;
-                row_pair_v(R, M.stage, st, j, pk(P.x, P.y), va, vv);
+                row_pair_v(R, M.stage, st, j, *(const f2*)&M.stage.P[st][j], va, vv);
                 const int at = jbase + 2 * k;
                 if (!sl.valid) return;
                 A.add(lo(va), at, a.mod_perm);
@@ -1087,9 +1087,9 @@ __global__ void __launch_bounds__(pass_threads(TILE), kPassThreadsPerSm / pass_t
         ColPair C;
         load_col_pair(a, sl.valid ? sl.q : sl.q - lane, C);
         auto sweep_all = [&](int skip) {
-            for_each_swept<false>(a, M.stage, sl, skip, [&](int st, int j, float2 P, int) {
+            for_each_swept<false>(a, M.stage, sl, skip, 0.0f, [&](int st, int j, int) {
                 f2 va, vv;
-                col_pair_v(C, M.stage, st, j, pk(P.x, P.y), va, vv);
+                col_pair_v(C, M.stage, st, j, *(const f2*)&M.stage.P[st][j], va, vv);
                 add(A, lo(va));
                 add(A, hi(va));
                 add(B, lo(vv));

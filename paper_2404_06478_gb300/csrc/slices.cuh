@@ -106,7 +106,7 @@ __device__ __forceinline__ void cp8(void* dst, const void* src) {
 // first pair of each of its sub-granules).  The streamed block: n_pairs pairs
 // from pair b0 of the model spots (MODEL) or the observed spots; pot their
 // potentials (nullptr: not staged).
-template <bool MODEL, class Fn>
+template <bool MODEL, bool DENSE, class Fn>
 __device__ __forceinline__ void sweep(const SkArgs& a, WarpStage& S, const Cone& own, const float4* sub, const float* ext,
                                       int b0, int n_pairs, int skip, float limit, const float* pot, Fn fn) {
     const int lane = threadIdx.x & 31;
@@ -115,12 +115,23 @@ __device__ __forceinline__ void sweep(const SkArgs& a, WarpStage& S, const Cone&
     auto fetch = [&](int st, int4& first) {  // issues the copies of the next batch; its pairs
         int n = 0;
         int f[4] = {0, 0, 0, 0};
+        if (DENSE && __popc(walk.mask) >= 4) {  // without the search for more
+            unsigned m = walk.mask;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int s = walk.next(own, MODEL, skip, a.skipK, limit);
-            if (s < 0) break;
-            f[c] = s * kSubGran;
-            n = c * kSubGran + min(kSubGran, n_pairs - f[c]);
+            for (int c = 0; c < 4; ++c) {
+                f[c] = (walk.s0 + __ffs(m) - 1) * kSubGran;
+                m &= m - 1;
+            }
+            walk.mask = m;
+            n = 3 * kSubGran + min(kSubGran, n_pairs - f[3]);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int s = walk.next(own, MODEL, skip, a.skipK, limit);
+                if (s < 0) break;
+                f[c] = s * kSubGran;
+                n = c * kSubGran + min(kSubGran, n_pairs - f[c]);
+            }
         }
         first = make_int4(f[0], f[1], f[2], f[3]);
         if (lane < n) {
@@ -317,14 +328,19 @@ __device__ __forceinline__ Sweep sweep_of(const SkArgs& a, const Slice& sl) {
     return w;
 }
 
-// fn(stage, pair of the stage, base potentials' packed pair, pair of the block)
-// over the slice's sweep; skip = 0: over the whole block.
+// fn(stage, pair of the stage, pair of the block) over the slice's sweep, whose
+// staged potentials are less `shift`; skip = 0: over the whole block.
 template <bool ROWS, class Fn>
-__device__ __forceinline__ void for_each_swept(const SkArgs& a, WarpStage& S, const Slice& sl, int skip, Fn fn) {
+__device__ __forceinline__ void for_each_swept(const SkArgs& a, WarpStage& S, const Slice& sl, int skip, float shift,
+                                               Fn fn) {
     const Sweep w = sweep_of<ROWS>(a, sl);
-    sweep<ROWS>(a, S, w.own, w.sub, w.ext, w.b0, w.n, skip, kSkipLog2, ROWS ? a.Gc : a.Fc, [&](int st, int n, const int4& f) {
+    sweep<ROWS, true>(a, S, w.own, w.sub, w.ext, w.b0, w.n, skip, kSkipLog2, ROWS ? a.Gc : a.Fc,
+                      [&](int st, int n, const int4& f) {
+        float2& P = S.P[st][sl.lane];
+        if (sl.lane < n) P = make_float2(P.x - shift, P.y - shift);
+        __syncwarp();
 #pragma unroll 4
-        for (int j = 0; j < n; ++j) fn(st, j, S.P[st][j], nth(f, j / kSubGran) + j % kSubGran);
+        for (int j = 0; j < n; ++j) fn(st, j, nth(f, j / kSubGran) + j % kSubGran);
     });
 }
 
