@@ -515,8 +515,7 @@ int laue_fill_sk(laue_handle* h, const LaueGeometry* geom, const LaueObsSpots* o
     a.tile_cols = sk_variant_threads(h->col_variant);
     lc->row_slices = (int)list_slices(a.T, a.n_obs, a.tile_rows);
     lc->col_slices = (int)list_slices(a.T, a.n_model, a.tile_cols);
-    lc->row_split = prm->dust_mode == 2 && lc->row_slices <= kSplitSlicesPerSm * h->sm_count;
-    lc->col_split = prm->dust_mode == 2 && lc->col_slices <= kSplitSlicesPerSm * h->sm_count;
+    lc->split = prm->dust_mode == 2 && std::max(lc->row_slices, lc->col_slices) <= kSplitSlicesPerSm * h->sm_count;
     {
         // the sort buffers, once the sort is done: slices, sub-granule cones, compact potentials
         char* b = ws + L.sortbuf;

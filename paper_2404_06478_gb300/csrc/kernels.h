@@ -192,20 +192,21 @@ cudaError_t sparse_sinkhorn_run(const SpArgs& a, const SkArgs* order, int n_iter
                                 cudaStream_t s);
 
 constexpr int kSkVariants = 4;       // launch shapes of the pair passes (see passes.cu)
-// Unbalanced passes of at most this many slices per SM are split (four warps a
-// slice).  It pays where slices take the exact path, which every column does at
-// 4 mm^2 and none of these at 100 mm^2, and there the split warps are in the way;
-// the host cannot know which.  Measured (50 iterations, 60 angles, split against
-// not, at 4 and 100 mm^2): 2 slices per SM 1.24 against 1.50 and 2.32 against 2.15
-// ms; 7 per SM 5.2 against 5.4 and 6.7 against 5.5; 23 per SM 23.4 against 28.2
-// and 39.7 against 28.1.
+// Unbalanced passes of at most this many slices per SM on either side are split
+// (four warps a slice).  It pays where slices take the exact path, which every
+// column does at 4 mm^2 and none at 100 mm^2 here; the host cannot know which.
+// Measured (50 iterations, 60 angles, split against not, at 4 and 100 mm^2): 2
+// slices per SM 1.14 against 1.45 and 1.82 against 2.10 ms; 5 per SM 2.1 against
+// 3.0 and 3.1 against 2.9; 7 per SM 4.0 against 5.3 and 6.1 against 5.4; 23 per SM
+// 23.3 against 27.9 and 37.0 against 27.6.  One side split and the other not is
+// worse than either (5 per SM: 3.5 and 3.8): their CTAs do not share an SM.
 constexpr int kSplitSlicesPerSm = 8;
 constexpr int kSkDefaultVariant = 3;  // 64-pair tiles: the autotuner's usual pick
 
 struct SkLaunch {
     int row_slices, col_slices;  // bound on the slices of each side
     int row_variant, col_variant;
-    bool row_split, col_split;  // passes whose slices have several warps where their sums underflow
+    bool split;  // the passes' slices have several warps where their sums underflow
 };
 
 cudaError_t sinkhorn_run(const SkArgs& a, const SkLaunch& l, int n_iter, bool want_rows, bool want_cols,

@@ -705,18 +705,20 @@ __device__ __forceinline__ void pass_release() { asm volatile("griddepcontrol.la
 // the others.  Their slices read the whole block with a running maximum, a
 // serial chain, so a pass over few slices has PARTS warps to a slice that read a
 // part of the block each; part 0's warp merges.  23 grains x 17 angles at 4 mm^2:
-// 17 us a pass with one warp, 14 us with four.
+// 17 us a pass with one warp, 13 us with four.
 //
 // Registers: 128 a thread, 512 threads to an SM.  No more are resident anyway:
 // a named barrier whose id is not a constant takes all 16 of a CTA, four CTAs to
 // an SM.  With 64 registers the sums over swept pairs spilled: 90 angles of
 // 13300 x 7744 spots at 100 mm^2 without lists 5.8 ms an iteration, now 4.6; one
-// block of 200000 x 8000 spots 11.1 ms, now 6.3.  (The split passes keep 64:
-// four times the warps.)
+// block of 200000 x 8000 spots 11.1 ms, now 6.3; split, 23 grains x 60 angles at 4
+// and 100 mm^2, 50 iterations, 1.24 and 2.32 ms, now 1.14 and 1.82.
 constexpr int kPassThreadsPerSm = 512;
 template <int TILE, int OTHER, bool ROWS, int PARTS>
 __global__ void __launch_bounds__(PARTS* pass_threads(TILE, OTHER),
-                                  (PARTS > 1 ? 1024 : kPassThreadsPerSm) / pass_threads(TILE, OTHER) / PARTS)
+                                  kPassThreadsPerSm / pass_threads(TILE, OTHER) / PARTS > 0
+                                      ? kPassThreadsPerSm / pass_threads(TILE, OTHER) / PARTS
+                                      : 1)
     sk_pass_kernel(SkArgs a, int it, int finishers) {
     extern __shared__ __align__(128) char pass_smem[];
     constexpr int kThreads = pass_threads(TILE, OTHER);
@@ -1257,13 +1259,13 @@ cudaError_t sinkhorn_setup() {
 
 cudaError_t sinkhorn_row_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s) {
     return with_tiles(l, [&](auto row, auto col) {
-        return run_pass<decltype(row)::value, decltype(col)::value, true>(a, it, l.row_split, s);
+        return run_pass<decltype(row)::value, decltype(col)::value, true>(a, it, l.split, s);
     });
 }
 
 cudaError_t sinkhorn_col_pass(const SkArgs& a, const SkLaunch& l, int it, cudaStream_t s) {
     return with_tiles(l, [&](auto row, auto col) {
-        return run_pass<decltype(col)::value, decltype(row)::value, false>(a, it, l.col_split, s);
+        return run_pass<decltype(col)::value, decltype(row)::value, false>(a, it, l.split, s);
     });
 }
 
