@@ -32,7 +32,7 @@ UNIT = "pairs/s"
 # DRAM bytes of one row-pass launch on the 1000-grain workload, counted by ncu
 # (dram__bytes_read.sum + dram__bytes_write.sum) for the current kernels; None
 # after a kernel change until it is captured again
-SK_PASS_DRAM_BYTES = 351607296
+SK_PASS_DRAM_BYTES = 346988800
 # bytes of a listed pair as the passes stream it: squared ray distance (float)
 # and slot of the other side's spot (16 bits)
 SK_ENTRY_BYTES = 6

@@ -38,7 +38,7 @@ constexpr float kListAlways = 1.0e30f;  // list_share of slices that need not lo
 // 1000-grain configuration at 1 mm^2, where the passes used to evaluate
 // 28.9 %.  A pass then streams 6 bytes per entry (HBM) instead of spending 13
 // packed instructions and two MUFU per evaluated pair.  Measured at that size:
-// listing 1.72 + 1.50 ms once, a pass 1.57 / 1.50 ms before and 0.069 ms now.
+// listing 1.70 + 1.48 ms once, a pass 1.57 / 1.50 ms before and 0.063 ms now.
 // A single iteration is not worth listing for: one sweep of both sides takes
 // about as long (sinkhorn_run).
 //
@@ -694,11 +694,11 @@ __device__ __forceinline__ void pass_release() { asm volatile("griddepcontrol.la
 
 // --------------------------------------------------- row and column passes
 // Iteration `it` of the row (ROWS) or column update.  What bounds it: at the
-// 1000-grain density the lists (324 MB a pass, 48 us at the copy rate, 69 us
-// measured: 4.7 TB/s), below that the chain of a pass: launch, gathers of the
-// potentials, partial sums (100 grains: 53 / 43 us a pass when it evaluated
-// pairs, 4.1 us now; 5 grains: 11 and 3.0 us).  The other side's tile width,
-// for the partials that the first blocks merge, is OTHER.
+// 1000-grain density the lists (324 MB a pass, 48 us at the copy rate, 63 us
+// measured), below that the chain of a pass: launch, gathers of the potentials,
+// partial sums (100 grains: 53 / 43 us a pass when it evaluated pairs, 4.1 us
+// now; 5 grains: 11 and 3.0 us).  The other side's tile width, for the partials
+// that the first blocks merge, is OTHER.
 //
 // Without dustbins (unbalanced OT) a shifted sum underflows for most spots:
 // the potentials of spots far from any partner are the largest, and shift all
